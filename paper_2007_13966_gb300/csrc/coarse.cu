@@ -18,8 +18,8 @@
 // block receives one update from each side. Solve: g_target -= C_e g_pivot
 // along both chains, x_m = S_m^{-1} g_m, then x_pivot = Inv g_pivot - F_e x_target
 // back along both chains. Each inverse is computed in place by a blocked
-// Gauss-Jordan inversion without pivoting (64 x 64 tiles); the off-diagonal
-// blocks are sparse and stored in ELL form.
+// Gauss-Jordan inversion without pivoting; the off-diagonal blocks are sparse and
+// stored in ELL form.
 //
 // The factorisation and the solve each run as ONE cooperative persistent
 // kernel whose phases are separated by a grid barrier; the barrier gives up
@@ -73,10 +73,12 @@ struct Coarse {
     void *lo_v = nullptr, *up_v = nullptr;           // ELL values
     void *g = nullptr, *x = nullptr;                 // [nb*T]
     void *xn = nullptr;                              // [Nc] the coarse solution in natural order
-    void *Zs = nullptr;                              // scratch tile strips [2][TILE][T]
+    void *Zs = nullptr;                              // scratch of the block inverses (gj_scratch per chain)
     void *rx = nullptr, *ry = nullptr;               // restriction passes [cx][ny][nz], [cx][cy][nz]
     int *d_err = nullptr;
     GridBar *d_bar = nullptr;
+    unsigned *d_flags = nullptr;    // ready flags of the FP32 block inverses
+    size_t nflag = 0;
     size_t esz = 8;
     size_t rap_smem = 0, rap125_smem = 0, fac_smem = 0, sol_smem = 0;
     int rap_zs = 0;                 // 0: k_rap (whole support boxes); > 0: k_rap_slab, slabs of rap_zs planes
@@ -84,7 +86,6 @@ struct Coarse {
     int rap125_ng = 25;             // offsets staged per round in k_rap125
     int fac_grid = 0, sol_grid = 0;
     int sol_npf = 0;                // rows per warp prefetched by the solve
-    int use_tc = 0;                 // FP32 inverses: trailing updates on the tcgen05 tensor cores
     int cr = 0;                     // cyclic reduction instead of the two-ended elimination
     int *d_crf = nullptr, *d_crs = nullptr;   // its factorisation and solve schedules
     void *W = nullptr;              // its dense couplings and products [nslot][T][T]
@@ -594,388 +595,15 @@ __device__ bool grid_barrier(GridBar *bar, int *err, unsigned &epoch, unsigned G
 }
 
 // ---------------------------------------------------------------------------
-// 64 x 64 tile helpers (256 threads; thread t owns rows tr..tr+3, cols tc..tc+3)
-// ---------------------------------------------------------------------------
-
-template <typename AT>
-struct TileSmem {
-    AT X[TILE][TILE + 1];
-    AT Y[TILE][TILE + 1];
-    AT rowb[2][4][TILE];   // four pivot rows (double buffered)
-    AT colb[2][TILE][4];   // four pivot columns (double buffered)
-    AT piv[2][4][4];       // inverse of the current / next 4 x 4 pivot block
-};
-
-// correctly rounded reciprocal (IEEE round to nearest)
-__device__ __forceinline__ float recip_rn(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip_rn(double x) { return __drcp_rn(x); }
-
-// In-place inverse of a 4 x 4 block held in registers by the Laplace expansion in the
-// 2 x 2 minors of rows (0, 1) and (2, 3): A^{-1} = adj(A) / det(A), one reciprocal
-// (FP32: the hardware reciprocal, a few ulp; FP64 the correctly rounded one) and a
-// short dependency chain (sequential Gauss-Jordan pivots took ~1 us more per 64 x 64
-// tile inverse). False if the block is singular or not finite.
-__device__ __forceinline__ float recip_fast(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double recip_fast(double x) { return recip_rn(x); }
-template <typename AT>
-__device__ __forceinline__ bool invert4(AT a[4][4]) {
-    const AT s0 = a[0][0] * a[1][1] - a[1][0] * a[0][1], s1 = a[0][0] * a[1][2] - a[1][0] * a[0][2];
-    const AT s2 = a[0][0] * a[1][3] - a[1][0] * a[0][3], s3 = a[0][1] * a[1][2] - a[1][1] * a[0][2];
-    const AT s4 = a[0][1] * a[1][3] - a[1][1] * a[0][3], s5 = a[0][2] * a[1][3] - a[1][2] * a[0][3];
-    const AT c5 = a[2][2] * a[3][3] - a[3][2] * a[2][3], c4 = a[2][1] * a[3][3] - a[3][1] * a[2][3];
-    const AT c3 = a[2][1] * a[3][2] - a[3][1] * a[2][2], c2 = a[2][0] * a[3][3] - a[3][0] * a[2][3];
-    const AT c1 = a[2][0] * a[3][2] - a[3][0] * a[2][2], c0 = a[2][0] * a[3][1] - a[3][0] * a[2][1];
-    const AT det = s0 * c5 - s1 * c4 + s2 * c3 + s3 * c2 - s4 * c1 + s5 * c0;
-    const bool ok = det != (AT)0 && isfinite(det);
-    const AT i = recip_fast(det);
-    AT b[4][4];
-    b[0][0] = ( a[1][1] * c5 - a[1][2] * c4 + a[1][3] * c3) * i;
-    b[0][1] = (-a[0][1] * c5 + a[0][2] * c4 - a[0][3] * c3) * i;
-    b[0][2] = ( a[3][1] * s5 - a[3][2] * s4 + a[3][3] * s3) * i;
-    b[0][3] = (-a[2][1] * s5 + a[2][2] * s4 - a[2][3] * s3) * i;
-    b[1][0] = (-a[1][0] * c5 + a[1][2] * c2 - a[1][3] * c1) * i;
-    b[1][1] = ( a[0][0] * c5 - a[0][2] * c2 + a[0][3] * c1) * i;
-    b[1][2] = (-a[3][0] * s5 + a[3][2] * s2 - a[3][3] * s1) * i;
-    b[1][3] = ( a[2][0] * s5 - a[2][2] * s2 + a[2][3] * s1) * i;
-    b[2][0] = ( a[1][0] * c4 - a[1][1] * c2 + a[1][3] * c0) * i;
-    b[2][1] = (-a[0][0] * c4 + a[0][1] * c2 - a[0][3] * c0) * i;
-    b[2][2] = ( a[3][0] * s4 - a[3][1] * s2 + a[3][3] * s0) * i;
-    b[2][3] = (-a[2][0] * s4 + a[2][1] * s2 - a[2][3] * s0) * i;
-    b[3][0] = (-a[1][0] * c3 + a[1][1] * c1 - a[1][2] * c0) * i;
-    b[3][1] = ( a[0][0] * c3 - a[0][1] * c1 + a[0][2] * c0) * i;
-    b[3][2] = (-a[3][0] * s3 + a[3][1] * s1 - a[3][2] * s0) * i;
-    b[3][3] = ( a[2][0] * s3 - a[2][1] * s1 + a[2][2] * s0) * i;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) a[u][v] = b[u][v];
-    return ok;
-}
-
-// a[u][v] (rows tr + u, columns tc + v of a tile) -= X Y for 64 x 64 tiles X, Y of
-// row stride ld, staged in shared memory: the arithmetic of subtile_product (the same
-// k order, out = prev + (-1) acc), so that a tile update followed by its inverse needs
-// no store and reload of the tile.
-template <typename AT>
-__device__ __forceinline__ void tile_pre_update(TileSmem<AT> &sm, AT (&a)[4][4], const AT *X, const AT *Y,
-                                                int ld, int tr, int tc) {
-    constexpr int VEC = 16 / sizeof(AT);
-    using V16 = typename std::conditional<sizeof(AT) == 4, float4, double2>::type;
-    constexpr int NV = TILE * TILE / VEC / 256;
-    V16 bx[NV], by[NV];
-#pragma unroll
-    for (int m = 0; m < NV; ++m) {
-        const int e = threadIdx.x + 256 * m, r = e / (TILE / VEC), k = (e % (TILE / VEC)) * VEC;
-        bx[m] = __ldcg(reinterpret_cast<const V16 *>(X + (long long)r * ld + k));
-        by[m] = __ldcg(reinterpret_cast<const V16 *>(Y + (long long)r * ld + k));
-    }
-#pragma unroll
-    for (int m = 0; m < NV; ++m) {
-        const int e = threadIdx.x + 256 * m, r = e / (TILE / VEC), k = (e % (TILE / VEC)) * VEC;
-        const AT *vx = reinterpret_cast<const AT *>(&bx[m]), *vy = reinterpret_cast<const AT *>(&by[m]);
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) {
-            sm.X[r][k + q] = vx[q];
-            sm.Y[r][k + q] = vy[q];
-        }
-    }
-    __syncthreads();
-    AT acc[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0;
-#pragma unroll 4
-    for (int k = 0; k < TILE; ++k) {
-        AT xa[4], yb[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) xa[u] = sm.X[tr + u][k];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) yb[v] = sm.Y[k][tc + v];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] += xa[u] * yb[v];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) a[u][v] = a[u][v] + (AT)(-1) * acc[u][v];
-}
-
-// In-place Gauss-Jordan inverse of tile (ti, ti) of M without pivoting, four
-// pivots per step (block column K = kb..kb+3, Pi = A_KK^{-1}):
-//     A_Kj <- Pi A_Kj,  A_ij <- A_ij - A_iK (Pi A_Kj),  A_iK <- -A_iK Pi,  A_KK <- Pi.
-// Thread t owns rows tr..tr+3 and columns tc..tc+3 (no runtime register
-// indexing). Per step: the pivot-row owners form Pi A_Kj and publish it, the
-// pivot-column owners publish A_iK (barrier), every other thread applies the
-// rank-4 update; the owner of the next pivot block inverts it as soon as its
-// own update is done and publishes Pi for the next step (barrier). The 4 x 4
-// inverse takes approximate reciprocals (FP32 preconditioner factors).
-template <typename AT>
-__device__ void tile_invert_b4(TileSmem<AT> &sm, AT *M, int ld, int ti, int *err, const AT *X = nullptr,
-                               const AT *Y = nullptr) {
-    const int tr = (threadIdx.x / 16) * 4, tc = (threadIdx.x % 16) * 4;
-    AT a[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            a[u][v] = __ldcg(M + (long long)(ti * TILE + tr + u) * ld + ti * TILE + tc + v);
-    if (X) tile_pre_update(sm, a, X, Y, ld, tr, tc);   // the tile's last update first
-    auto invert_publish = [&](int par) {
-        AT P[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) P[u][v] = a[u][v];
-        if (!invert4(P)) atomicExch(err, ERR_PIVOT);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) sm.piv[par][u][v] = P[u][v];
-    };
-    if (tr == 0 && tc == 0) invert_publish(0);
-    __syncthreads();
-    for (int kb = 0; kb < TILE; kb += 4) {
-        const int par = (kb >> 2) & 1;
-        AT Pi[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) Pi[u][v] = sm.piv[par][u][v];
-        if (tr == kb && tc == kb) {                  // pivot block -> its inverse
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) a[u][v] = Pi[u][v];
-        } else if (tr == kb) {                       // pivot rows: Pi A_Kj, published
-            AT W[4][4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    AT t = 0;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) t += Pi[u][q] * a[q][v];
-                    W[u][v] = t;
-                }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    a[u][v] = W[u][v];
-                    sm.rowb[par][u][tc + v] = W[u][v];
-                }
-        } else if (tc == kb) {                       // pivot columns: publish A_iK, then -A_iK Pi
-            AT c[4][4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    c[u][v] = a[u][v];
-                    sm.colb[par][tr + u][v] = a[u][v];
-                }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    AT t = 0;
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) t += c[u][m] * Pi[m][v];
-                    a[u][v] = -t;
-                }
-        }
-        __syncthreads();
-        if (tr != kb && tc != kb) {                  // rank-4 update a -= A_iK (Pi A_Kj)
-            AT W[4][4];
-#pragma unroll
-            for (int m = 0; m < 4; ++m)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) W[m][v] = sm.rowb[par][m][tc + v];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                AT c[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) c[m] = sm.colb[par][tr + u][m];
-#pragma unroll
-                for (int v = 0; v < 4; ++v)
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) a[u][v] -= c[m] * W[m][v];
-            }
-            if (tr == kb + 4 && tc == kb + 4) invert_publish(par ^ 1);   // next pivot block
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            M[(long long)(ti * TILE + tr + u) * ld + ti * TILE + tc + v] = a[u][v];
-}
-
-// Scalar Gauss-Jordan (one pivot per barrier): fewest operations, used for
-// FP64 where the arithmetic pipe, not the barrier, bounds the tile inverse.
-template <typename AT>
-__device__ void tile_invert_s(TileSmem<AT> &sm, AT *M, int ld, int ti, int *err, const AT *X = nullptr,
-                              const AT *Y = nullptr) {
-    const int tr = (threadIdx.x / 16) * 4, tc = (threadIdx.x % 16) * 4;
-    AT a[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            a[u][v] = __ldcg(M + (long long)(ti * TILE + tr + u) * ld + ti * TILE + tc + v);
-    if (X) tile_pre_update(sm, a, X, Y, ld, tr, tc);   // the tile's last update first
-    for (int kk = 0; kk < TILE; ++kk) {
-        const int par = kk & 1;
-        if (tr <= kk && kk < tr + 4) {
-            const int u = kk - tr;
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-                sm.rowb[par][0][tc + v] = u == 0 ? a[0][v] : (u == 1 ? a[1][v] : (u == 2 ? a[2][v] : a[3][v]));
-        }
-        if (tc <= kk && kk < tc + 4) {
-            const int v = kk - tc;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                sm.colb[par][tr + u][0] = v == 0 ? a[u][0] : (v == 1 ? a[u][1] : (v == 2 ? a[u][2] : a[u][3]));
-        }
-        __syncthreads();
-        const AT piv = sm.rowb[par][0][kk];
-        if (threadIdx.x == 0 && (!(piv != (AT)0) || !isfinite(piv))) atomicExch(err, ERR_PIVOT);
-        const AT ip = recip_rn(piv);
-        AT rb[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) rb[v] = sm.rowb[par][0][tc + v] * ip;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool ri = (tr + u == kk);
-            const AT ci = sm.colb[par][tr + u][0];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const bool cj = (tc + v == kk);
-                AT nv = a[u][v] - ci * rb[v];
-                if (ri) nv = cj ? ip : rb[v];
-                else if (cj) nv = -ci * ip;
-                a[u][v] = nv;
-            }
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            M[(long long)(ti * TILE + tr + u) * ld + ti * TILE + tc + v] = a[u][v];
-}
-
-// (X, Y: tiles whose product the tile receives first, tile -= X Y; null: none)
-template <typename AT>
-__device__ __forceinline__ void tile_invert(TileSmem<AT> &sm, AT *M, int ld, int ti, int *err,
-                                            const AT *X = nullptr, const AT *Y = nullptr) {
-    if constexpr (sizeof(AT) == 8) tile_invert_s(sm, M, ld, ti, err, X, Y);
-    else tile_invert_b4(sm, M, ld, ti, err, X, Y);
-}
-
-// Sub-tile product: rows [r0, r0 + RR) and columns [c0, c0 + CC) of
-//     out(oi, oj) = sign * tile(xi, xj) * tile(yi, yj)  (+ out if accumulate),
-// 256 threads x BR x BC outputs. In-place use is safe when the output part
-// depends only on the staged part of the aliased input: a row panel
-// (out = P * out) is split by columns, a column panel (out = out * P) by rows.
-template <typename AT, int RR, int CC, int BR, int BC>
-__device__ void subtile_product(TileSmem<AT> &sm, const AT *Xb, const AT *Yb, AT *Ob, int ld, int xi,
-                                int xj, int yi, int yj, int oi, int oj, int r0, int c0, AT sign,
-                                bool accumulate) {
-    static_assert((RR / BR) * (CC / BC) == 256, "256 threads");
-    AT (*X)[TILE + 1] = sm.X;   // X[r][k], r < RR
-    AT (*Y)[TILE + 1] = sm.Y;   // Y[k][c], c < CC
-    // stage both parts with 16-byte loads, all issued before any is consumed
-    constexpr int VEC = 16 / sizeof(AT);
-    using V16 = typename std::conditional<sizeof(AT) == 4, float4, double2>::type;
-    constexpr int NX = RR * TILE / VEC / 256, NY = TILE * CC / VEC / 256;
-    static_assert(NX >= 1 && NY >= 1, "staging split");
-    V16 bx[NX], by[NY];
-#pragma unroll
-    for (int m = 0; m < NX; ++m) {
-        const int e = threadIdx.x + 256 * m;            // vector index
-        const int r = e / (TILE / VEC), k = (e % (TILE / VEC)) * VEC;
-        bx[m] = __ldcg(reinterpret_cast<const V16 *>(Xb + (long long)(xi * TILE + r0 + r) * ld +
-                                                     xj * TILE + k));
-    }
-#pragma unroll
-    for (int m = 0; m < NY; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        const int k = e / (CC / VEC), c = (e % (CC / VEC)) * VEC;
-        by[m] = __ldcg(reinterpret_cast<const V16 *>(Yb + (long long)(yi * TILE + k) * ld + yj * TILE +
-                                                     c0 + c));
-    }
-#pragma unroll
-    for (int m = 0; m < NX; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        const int r = e / (TILE / VEC), k = (e % (TILE / VEC)) * VEC;
-        const AT *v = reinterpret_cast<const AT *>(&bx[m]);
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) X[r][k + q] = v[q];
-    }
-#pragma unroll
-    for (int m = 0; m < NY; ++m) {
-        const int e = threadIdx.x + 256 * m;
-        const int k = e / (CC / VEC), c = (e % (CC / VEC)) * VEC;
-        const AT *v = reinterpret_cast<const AT *>(&by[m]);
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) Y[k][c + q] = v[q];
-    }
-    __syncthreads();
-    constexpr int TPR = CC / BC;
-    const int rr = (threadIdx.x / TPR) * BR, cc = (threadIdx.x % TPR) * BC;
-    AT acc[BR][BC];
-#pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-        for (int v = 0; v < BC; ++v) acc[u][v] = 0;
-#pragma unroll 4
-    for (int k = 0; k < TILE; ++k) {
-        AT xa[BR], yb[BC];
-#pragma unroll
-        for (int u = 0; u < BR; ++u) xa[u] = X[rr + u][k];
-#pragma unroll
-        for (int v = 0; v < BC; ++v) yb[v] = Y[k][cc + v];
-#pragma unroll
-        for (int u = 0; u < BR; ++u)
-#pragma unroll
-            for (int v = 0; v < BC; ++v) acc[u][v] += xa[u] * yb[v];
-    }
-    __syncthreads();   // the output may alias a staged input
-    // all reads of the old output before any store (one round of loads)
-    AT prev[BR][BC];
-#pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-        for (int v = 0; v < BC; ++v)
-            prev[u][v] = accumulate
-                ? __ldcg(Ob + (long long)(oi * TILE + r0 + rr + u) * ld + oj * TILE + c0 + cc + v)
-                : (AT)0;
-#pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-        for (int v = 0; v < BC; ++v)
-            Ob[(long long)(oi * TILE + r0 + rr + u) * ld + oj * TILE + c0 + cc + v] =
-                prev[u][v] + sign * acc[u][v];
-}
-
-// ---------------------------------------------------------------------------
-// trailing updates of the FP32 Gauss-Jordan inverses on the tcgen05 tensor cores
+// FP32 products on the tcgen05 tensor cores: the steps of the block inverses (below) and
+// the dense products of the cyclic reduction
 //
-// Two vertically adjacent 64 x 64 tiles of a block, rows 128 x columns of tile j,
-// are updated together: Out -= X Y with X the 128 x 64 column strip of the pivot
-// panel and Y the 64 x 64 pivot-row tile, one group of MMAs (M = 128, N = 64,
-// K = 8 per instruction) with FP32 accuracy from the TF32 path by the three-term
-// split X Y ~ Xh Yh + Xh Yl + Xl Yh (h: rounded to TF32, l: the FP32 remainder),
-// accumulated in FP32 in tensor memory (64 columns per CTA, allocated for the
-// launch). Operands are split and written by the CTA's threads into shared memory
-// in the canonical K-major layout without swizzle (8-row x 16-byte core matrices,
-// 128 B apart along k, 2048 B apart along rows); one thread issues the MMAs and
-// commits them to an mbarrier that the CTA waits on (bounded).
+// FP32 accuracy comes from the TF32 path (kind::tf32) by splitting each operand into TF32
+// values: X Y ~ Xh Yh + Xh Yl + Xl Yh (h: rounded to TF32, l: the FP32 remainder),
+// accumulated in FP32 in tensor memory. Operands are split and written by the CTA's
+// threads into shared memory in the canonical K-major layout without swizzle (8-row x
+// 16-byte core matrices); one thread issues the MMAs and commits them to an mbarrier that
+// the CTA waits on (bounded).
 // ---------------------------------------------------------------------------
 
 struct TcSmem {
@@ -1015,113 +643,6 @@ __device__ __forceinline__ void tc_put(unsigned char *h, unsigned char *l, int o
     *reinterpret_cast<float *>(l + off) = v - vh;
 }
 
-// Out(tiles i0, i0 + 1; tile column j) -= D(same rows, tile column p) D(p, j), T x T
-// row-major block M. All 256 threads; the CTA's smem overlay is free on entry.
-__device__ void tc_pair_update(TcSmem &ts, TcState &st, float *M, int T, int i0, int p, int j, int *err) {
-    const int tid = threadIdx.x;
-    // the updated tiles (rows 64 i0 .. + 127, column tile j) are read together with the
-    // operands: no other item of the phase writes them, and they overlap neither X
-    // (column tile p) nor Y (row tile p); warp w: rows 32 (w % 4) + lane, columns
-    // 32 (w / 4) .. + 31
-    const int w = tid >> 5, lane = tid & 31, wq = w & 3, wh = w >> 2;
-    float *out = M + (long long)(i0 * TILE + 32 * wq + lane) * T + j * TILE + 32 * wh;
-    float4 prev[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) prev[u] = __ldcg(reinterpret_cast<const float4 *>(out) + u);
-    {   // X: rows 64 i0 .. + 127, columns 64 p .. + 63; thread t: row t / 2, k half (t & 1)
-        const int r = tid >> 1, k0 = (tid & 1) * 32;
-        const float4 *src = reinterpret_cast<const float4 *>(M + (long long)(i0 * TILE + r) * T + p * TILE + k0);
-        float4 v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = __ldcg(src + q);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float *e = reinterpret_cast<const float *>(&v[q]);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) tc_put(ts.xh, ts.xl, tc_off(r, k0 + 4 * q + u), e[u]);
-        }
-    }
-    {   // Y^T: Y = D(p, j), element (k, n) to row n, column k; thread t: k = t / 4, n block (t & 3)
-        const int k = tid >> 2, n0 = (tid & 3) * 16;
-        const float4 *src = reinterpret_cast<const float4 *>(M + (long long)(p * TILE + k) * T + j * TILE + n0);
-        float4 v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = __ldcg(src + q);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float *e = reinterpret_cast<const float *>(&v[q]);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) tc_put(ts.yh, ts.yl, tc_off(n0 + 4 * q + u, k), e[u]);
-        }
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const unsigned xh = (unsigned)__cvta_generic_to_shared(ts.xh), xl = (unsigned)__cvta_generic_to_shared(ts.xl);
-        const unsigned yh = (unsigned)__cvta_generic_to_shared(ts.yh), yl = (unsigned)__cvta_generic_to_shared(ts.yl);
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            const unsigned o = s * 2 * TC_LBO;   // k-step of 8: two core matrices along k
-            const unsigned long long d[3][2] = {{tc_desc(xl + o), tc_desc(yh + o)},
-                                                {tc_desc(xh + o), tc_desc(yl + o)},
-                                                {tc_desc(xh + o), tc_desc(yh + o)}};
-#pragma unroll
-            for (int t3 = 0; t3 < 3; ++t3) {
-                const unsigned acc = (s > 0 || t3 > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n.reg .pred pp;\n"
-                    "setp.ne.b32 pp, %4, 0;\n"
-                    "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, pp;\n}\n"
-                    ::"r"(st.tmem), "l"(d[t3][0]), "l"(d[t3][1]), "r"(TC_IDESC), "r"(acc) : "memory");
-            }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                     ::"r"((unsigned)__cvta_generic_to_shared(st.mbar)) : "memory");
-    }
-    {   // bounded wait for the MMAs
-        const unsigned a = (unsigned)__cvta_generic_to_shared(st.mbar), par = st.phase & 1;
-        bool done = false;
-        for (long long it = 0; it < TC_POLLS && !done; ++it) {
-            unsigned ok;
-            asm volatile(
-                "{\n.reg .pred pp;\n"
-                "mbarrier.try_wait.parity.shared::cta.b64 pp, [%1], %2;\n"
-                "selp.u32 %0, 1, 0, pp;\n}\n"
-                : "=r"(ok) : "r"(a), "r"(par) : "memory");
-            done = ok != 0;
-        }
-        if (!done) atomicExch(err, ERR_TIMEOUT);
-        ++st.phase;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    {
-        unsigned r[32];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-            "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-              "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-              "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-              "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-              "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-            : "r"(st.tmem + ((unsigned)(32 * wq) << 16) + 32u * wh));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            float4 o = prev[u];
-            o.x -= __uint_as_float(r[4 * u]);
-            o.y -= __uint_as_float(r[4 * u + 1]);
-            o.z -= __uint_as_float(r[4 * u + 2]);
-            o.w -= __uint_as_float(r[4 * u + 3]);
-            reinterpret_cast<float4 *>(out)[u] = o;
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();   // the smem overlay and the accumulator are free again
-}
-
 // One product of tc_gemm_core: A (its first row and chunk; leading dimension
 // lda) times B (its first chunk row and column; leading dimension ldb) over nk
 // chunks of 64 along k. With bidx, row k of B is row bidx[k] of B (negative: a
@@ -1134,7 +655,7 @@ struct TcOp {
 
 // Out[0 .. nrows) x [0 .. 64) (leading dimension ldo) (=, +=) sign (o1 [+ o2]) for
 // FP32 row-major operands, on tcgen05 (M = 128, N = 64, K = 8, the three-term TF32
-// split of tc_pair_update), accumulated in tensor memory; the next chunk's global
+// split), accumulated in tensor memory; the next chunk's global
 // loads are issued before the wait for the current chunk's MMAs. nrows is 64 or
 // 128 (rows past it enter as zeros and are not written). All 256 threads; the
 // CTA's shared-memory overlay is free on entry and on return.
@@ -1280,16 +801,16 @@ __device__ __forceinline__ void tc_gemm_pair(TcSmem &ts, TcState &st, float *Out
 template <typename AT>
 struct FacArgs {
     AT *D, *C, *F;
-    AT *Z;   // scratch: per chain 64 rows x T (tile (0, 0) used) for -D_{p+1,p} P_p
+    AT *Z;   // scratch of the block inverses, gj_scratch values per chain
     const int *lo_q, *up_q, *lo_n, *up_n;
     const AT *lo_v, *up_v;
-    int T, nt, nb, mid;
+    int T, nb, mid;
     GridBar *bar;
     int *err;
     int cr;            // cyclic reduction (FP32, tensor cores) instead of the two-ended elimination
     const int *crs;    // its schedule
     AT *W;             // its dense couplings and products, [slot - nb][T][T]
-    int tc;            // FP32 products on the tensor cores (the handle's set-up choice)
+    unsigned *flags;   // ready flags of the FP32 block inverses, gj_flags per chain, zero at launch
 };
 
 // Out[r0+i][c] (=, -=) sum_e M[r0+i][uq[c][e]] uv[c][e] for a chunk of FROWS rows.
@@ -1483,122 +1004,733 @@ __device__ void sparse_rows_times(const AT *Inv, const int *lq, const AT *lv, co
     __syncthreads();                      // the next item may overwrite the staged couplings
 }
 
-// In-place inverses of the blocks blk[0..nblk) (one chain each), panel by
-// panel; the pivot tile of the next panel of each block is updated and
-// inverted by a CTA of its own (when the grid has more CTAs than chains).
+// ---------------------------------------------------------------------------
+// block inverses: distributed Gauss-Jordan
+// ---------------------------------------------------------------------------
+//
+// A T x T block is inverted in place in panels of NB pivots (no pivoting). With P the
+// inverse of panel p's NB x NB pivot block, R the panel's rows and A its columns, all
+// as the earlier panels left them:
+//     rows outside the panel:  q = a_p P,  a_j <- a_j - q R_j (j not in p),  a_p <- -q,
+//     rows of the panel:       a_j <- P R_j (j not in p),  a_p <- P,
+// the second line being the first with a = 0 and q = -P. Every CTA updates its own part
+// of the block straight from A, R and P, so only these cross CTAs: the step of panel p
+// copies the rows and columns of panel p + 1 and the diagonal block of panel p + 2 to
+// strips, and while it runs one CTA per chain forms the next pivot block from the strips
+// of the last step and inverts it. Steps are separated by one grid barrier per panel, or,
+// where every tile of an FP32 block has a CTA of its own, by ready flags: a tile waits
+// only for the two strip parts and the P that it reads.
+//
+// Bound: the chain barrier -> next pivot block -> its inverse, not arithmetic, so NB is
+// small: 32 in FP32 and 16 in FP64, where 2 FMA per cycle and SM make anything that one
+// CTA does expensive. FP32 (GjTile): a CTA owns a 128 x 128 tile and
+// keeps it in registers for the whole inversion; it reads 2 x 16 KB of strips per step,
+// where whole rows per CTA would read the full strip, 128 KB, in every CTA (measured:
+// 17 us per step on a 1024 block, bound by L2, against 7 us). FP64 (gj_rows): a CTA owns rows, so that
+// q costs next to nothing beside the FP64-bound update (a tile of a 256 block would
+// spend a third of its FMA on q). Measured against 64 x 64 pivot tiles with two barriers
+// per tile: 16 blocks of 1024 in FP32 3.8 -> 3.2 ms, 8 blocks of 256 in FP64 5.2 -> 1.2 ms,
+// 16 of 512 in FP64 18.6 -> 7.0 ms (4.3 GFLOP: 3.9 ms of the FP64 pipe).
+template <typename AT> struct Gj;
+template <> struct Gj<float> { static constexpr int NB = 32; };
+template <> struct Gj<double> { static constexpr int NB = 16; };
+
+// scratch per chain: per slot R and A (NB T values each), the diagonal block two panels
+// ahead, P and P transposed (NB^2 each). FP64: two slots, R and A stored [NB][T] (A
+// transposed). FP32: a slot per panel, so that a tile may run ahead of others (see
+// invert_blocks), R stored by column and A by row, [T][NB]: the K-major operands of the
+// tensor-core products.
 template <typename AT>
-__device__ __forceinline__ bool invert_blocks(const FacArgs<AT> &a, TileSmem<AT> &ts, const int *blk, int nblk,
-                              unsigned &epoch, int b, int G, TcState &tcs) {
-    const int T = a.T, nt = a.nt;
-    const long long bsz = (long long)T * T;
-    // prologue: pivot tile 0 and the row panel of step 0
-    for (int c = b; c < nblk; c += G) tile_invert(ts, a.D + blk[c] * bsz, T, 0, a.err);
-    if (!grid_barrier(a.bar, a.err, epoch, G)) return false;
-    {
-        const int n0 = 4 * (nt - 1);
-        for (int it = b; it < nblk * n0; it += G) {
-            AT *Dk = a.D + blk[it / n0] * bsz;
-            const int j = ((it % n0) >> 2) + 1, q = it & 3;
-            subtile_product<AT, 64, 16, 2, 2>(ts, Dk, Dk, Dk, T, 0, 0, 0, j, 0, j, 0, 16 * q, (AT)1, false);
-        }
+__host__ __device__ constexpr int gj_slots(int T) { return sizeof(AT) == 4 ? T / Gj<AT>::NB : 2; }
+template <typename AT>
+__host__ __device__ constexpr size_t gj_scratch(int T) {
+    return (size_t)gj_slots<AT>(T) * (2 * Gj<AT>::NB * (size_t)T + 3 * Gj<AT>::NB * Gj<AT>::NB);
+}
+template <typename AT>
+struct GjStrips {
+    static constexpr int NB = Gj<AT>::NB;
+    AT *R, *A, *D, *P, *Q;      // of panel 0 (Q: P transposed)
+    int strip;                  // NB T
+    __device__ GjStrips(AT *Z, int T) : R(Z), strip(NB * T) {
+        const int n = gj_slots<AT>(T);
+        A = R + (size_t)n * strip;
+        D = A + (size_t)n * strip;
+        P = D + n * NB * NB;
+        Q = P + n * NB * NB;
     }
-    if (!grid_barrier(a.bar, a.err, epoch, G)) return false;
-    const bool own = G > nblk;              // CTAs 0..nblk-1 do only the pivot tiles
-    for (int p = 0; p < nt; ++p) {
-        const bool nxt = p + 1 < nt;
-        // phase A: trailing update D_ij -= D_ip D_pj (i, j != p); the next
-        // pivot tile is updated and inverted by one CTA per chain
-        const int nu = (nt - 1) * (nt - 1);
-        const int nz = nxt ? 4 : 0;           // Z = -D_{p+1,p} P_p into the chain's scratch strip
-        const int dpiv = p * (nt - 1) + p;    // update item of tile (p+1, p+1)
-        const int nreg = nu - (nxt ? 1 : 0) + nz;
-        auto update = [&](int c, int t) {     // update item t (in 0..nu) of chain c
-            AT *Dk = a.D + blk[c] * bsz;
-            const int bi = t / (nt - 1), bj = t % (nt - 1);
-            const int i = bi < p ? bi : bi + 1, j = bj < p ? bj : bj + 1;
-            subtile_product<AT, 64, 64, 4, 4>(ts, Dk, Dk, Dk, T, i, p, p, j, i, j, 0, 0, (AT)-1, true);
-        };
-        // FP32 with the tensor path: the items are pairs of vertically adjacent tiles
-        // (rows 2 pb, 2 pb + 1) of a tile column j != p, one MMA group per pair; a pair
-        // with the pivot row or the next pivot tile (updated by its own CTA) in it
-        // keeps its other tile on the CUDA-core product
-        const bool tcp = sizeof(AT) == 4 && tcs.on;
-        const int npair = (nt + 1) / 2, npi = (nt - 1) * npair;
-        const int nitem = tcp ? npi + nz : nreg;
-        auto z_item = [&](int c, int z) {
-            AT *Dk = a.D + blk[c] * bsz;
-            subtile_product<AT, 16, 64, 2, 2>(ts, Dk, Dk, a.Z + (long long)c * TILE * T, T, p + 1, p,
-                                              p, p, 0, 0, 16 * z, 0, (AT)-1, false);
-        };
-        auto regular = [&](int q) {            // q in 0..nblk*nitem
-            const int c = q / nitem, r = q % nitem;
-            if (r >= nitem - nz) {
-                z_item(c, r - (nitem - nz));
-                return;
+    __device__ int slot(int p) const { return sizeof(AT) == 4 ? p : p & 1; }
+    __device__ AT *r(int p) const { return R + (size_t)slot(p) * strip; }
+    __device__ AT *a(int p) const { return A + (size_t)slot(p) * strip; }
+    __device__ AT *d(int p) const { return D + slot(p) * NB * NB; }
+    __device__ AT *pi(int p) const { return P + slot(p) * NB * NB; }
+    __device__ AT *pt(int p) const { return Q + slot(p) * NB * NB; }
+};
+constexpr int GJ_MAXT = 12;     // most tiles per axis of a block whose tiles all have a CTA (12^2 <= 152 SMs)
+// ready flags of the FP32 inversion: per panel, P, the look-ahead block and, per tile, the
+// strips' parts
+__host__ __device__ constexpr size_t gj_flags(int T) { return (size_t)(T / 32) * (2 + 2 * GJ_MAXT); }
+constexpr int GJ64_MAXR = 7;    // most rows per strip of the FP64 step
+__host__ __device__ constexpr int gj64_strip(int T) { return T / 2 < 256 ? T / 2 : 256; }   // threads per row
+// FP32 step: the tensor-core operands, each value as a sum of TF32 values (A and P: three,
+// exact to FP32; -q, which takes A's place, and R: two)
+struct GjTcSmem {
+    alignas(128) unsigned char a[3][128 * 32 * 4];   // A, then -q: 128 rows x 32 k
+    alignas(128) unsigned char r[2][128 * 32 * 4];   // R by column: 128 columns x 32 k
+    alignas(128) unsigned char p[3][32 * 32 * 4];    // P by column: 32 columns x 32 k
+};
+template <typename AT>
+__host__ __device__ constexpr size_t gj_smem(int T) {
+    constexpr int NB = Gj<AT>::NB;
+    const size_t rows = sizeof(AT) == 4 ? sizeof(GjTcSmem)
+                                        : sizeof(AT) * (size_t)(NB * NB + (256 / gj64_strip(T)) * GJ64_MAXR * 2 * NB);
+    const size_t piv = sizeof(AT) * ((size_t)5 * NB * NB + 256);   // the pivot CTA: P, R, A, D, U, exchanged rows
+    return rows > piv ? rows : piv;
+}
+
+// 1 / x: FP32, the hardware's approximate reciprocal (preconditioner factors); FP64, one
+// third-order step y (1 + e + e^2), e = 1 - x y, from the FP32 reciprocal (24 bits -> 72),
+// where x lies in FP32's normal range (IEEE reciprocal otherwise): three dependent
+// operations on a pipe where each takes ~64 cycles, against ~440 cycles for the IEEE one.
+__device__ __forceinline__ float gj_recip(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ double gj_recip(double x) {
+    const double ax = fabs(x);
+    if (!(ax > 1e-36 && ax < 1e36)) return __drcp_rn(x);
+    const double y = (double)__fdividef(1.0f, (float)x);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// Inverse of an NB x NB block held one column per lane by 8 warps, block row by block
+// row; `ok` is cleared on a zero or non-finite pivot. The warp that owns the next pivot
+// rows solves with their diagonal block for its columns right after its own update
+// (shuffles only) and publishes the scaled rows, the step's only exchange: one CTA
+// barrier per step. FP32: warp I holds rows 4 I .. 4 I + 3, lane c column c, 4 pivots per
+// step, by elimination of the 4 x 4 block on every lane's own right-hand side (its column,
+// or a unit vector in the pivot columns): ~45 instructions, where forming the 4 x 4 inverse
+// first takes ~140 (650 cycles of a 1,000-cycle step: one warp alone issues slowly). FP64:
+// warp I holds rows 2 I, 2 I + 1, lane (u, c) row 2 I + u and column c, 2 pivots per step.
+__device__ __forceinline__ void gj_tile_inverse(float (&a)[4], float *W, bool &ok) {
+    // (the shuffle makes the warp number warp-uniform to the compiler)
+    const int I = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    float4 *Ws = reinterpret_cast<float4 *>(W);   // [2][32]: the pivot rows' column of each lane
+    float c[4][4];                                // this warp's rows in the pivot columns
+    auto columns = [&](int s) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) c[u][m] = __shfl_sync(0xffffffffu, a[u], 4 * s + m);
+    };
+    auto scale = [&](int s) {
+        const bool pc = (lane >> 2) == s;
+        float w[4], inv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = pc ? ((lane & 3) == u ? 1.0f : 0.0f) : a[u];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (!(c[k][k] != 0.0f) || !isfinite(c[k][k])) ok = false;
+            inv[k] = gj_recip(c[k][k]);
+#pragma unroll
+            for (int u = k + 1; u < 4; ++u) {
+                const float l = c[u][k] * inv[k];
+#pragma unroll
+                for (int m = k + 1; m < 4; ++m) c[u][m] = fmaf(-l, c[k][m], c[u][m]);
+                w[u] = fmaf(-l, w[k], w[u]);
             }
-            if (!tcp) {
-                update(c, nxt && r >= dpiv ? r + 1 : r);
-                return;
+        }
+#pragma unroll
+        for (int k = 3; k >= 0; --k) {
+            w[k] *= inv[k];
+#pragma unroll
+            for (int u = 0; u < k; ++u) w[u] = fmaf(-c[u][k], w[k], w[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = w[u];
+        Ws[(s & 1) * 32 + lane] = make_float4(w[0], w[1], w[2], w[3]);
+    };
+    columns(0);
+    if (I == 0) scale(0);
+#pragma unroll 1
+    for (int s = 0; s < 8; ++s) {
+        __syncthreads();
+        const float4 w = Ws[(s & 1) * 32 + lane];
+        const bool pc = (lane >> 2) == s;
+        if (I != s) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float t = pc ? 0.0f : a[u];
+                t = fmaf(-c[u][0], w.x, t);
+                t = fmaf(-c[u][1], w.y, t);
+                t = fmaf(-c[u][2], w.z, t);
+                a[u] = fmaf(-c[u][3], w.w, t);
             }
+        }
+        if (s == 7) break;
+        columns(s + 1);
+        if (I == s + 1) scale(s + 1);
+    }
+}
+__device__ __forceinline__ void gj_tile_inverse(double (&a)[1], double *W, bool &ok) {
+    const int I = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int lane = threadIdx.x & 31, u = lane >> 4, c = lane & 15;
+    auto scale = [&](int s) {                     // W: [2][2][16]
+        const double b00 = __shfl_sync(0xffffffffu, a[0], 2 * s), b01 = __shfl_sync(0xffffffffu, a[0], 2 * s + 1);
+        const double b10 = __shfl_sync(0xffffffffu, a[0], 16 + 2 * s);
+        const double b11 = __shfl_sync(0xffffffffu, a[0], 16 + 2 * s + 1);
+        const double a0 = __shfl_sync(0xffffffffu, a[0], c), a1 = __shfl_sync(0xffffffffu, a[0], 16 + c);
+        const double n0 = u ? -b10 : b11, n1 = u ? b00 : -b01;               // row u of the adjugate
+        const double t = (c >> 1) == s ? ((c & 1) ? n1 : n0) : fma(n1, a1, n0 * a0);
+        const double det = fma(b00, b11, -b01 * b10);
+        if (!(det != 0.0) || !isfinite(det)) ok = false;
+        const double w = t * gj_recip(det);
+        a[0] = w;
+        W[(s & 1) * 32 + lane] = w;
+    };
+    if (I == 0) scale(0);
+#pragma unroll 1
+    for (int s = 0; s < 8; ++s) {
+        const double m0 = __shfl_sync(0xffffffffu, a[0], 16 * u + 2 * s);
+        const double m1 = __shfl_sync(0xffffffffu, a[0], 16 * u + 2 * s + 1);
+        __syncthreads();
+        const double w0 = W[(s & 1) * 32 + c], w1 = W[(s & 1) * 32 + 16 + c];
+        if (I != s) a[0] = fma(-m1, w1, fma(-m0, w0, (c >> 1) == s ? 0.0 : a[0]));
+        if (I == s + 1) scale(s + 1);
+    }
+}
+
+// The inverse P of panel p's pivot block: the block itself for p = 0 (read from M), else
+// the look-ahead block less A P R of the previous panel, from the strips of step p - 2.
+template <typename AT>
+__device__ __noinline__ void gj_pivot(const AT *M, AT *Z, int T, int p, unsigned char *smem, int *err) {
+    constexpr int NB = Gj<AT>::NB, NE = NB * NB / 256;           // values per thread
+    using V = typename std::conditional<sizeof(AT) == 4, float4, double2>::type;
+    constexpr int VE = 16 / sizeof(AT);
+    const GjStrips<AT> S(Z, T);
+    AT *Ps = reinterpret_cast<AT *>(smem), *Xs = Ps + NB * NB, *As = Xs + NB * NB, *Ds = As + NB * NB;
+    AT *Us = Ds + NB * NB, *W = Us + NB * NB;
+    const int I = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // this thread's values: rows rr + u, column c (FP32: 4 rows of a column; FP64: one value)
+    const int c = lane % NB, rr = NB / 8 * I + (sizeof(AT) == 4 ? 0 : lane / NB);
+    AT a[NE];
+    if (p == 0) {
+#pragma unroll
+        for (int u = 0; u < NE; ++u) a[u] = __ldcg(M + (long long)(rr + u) * T + c);
+    } else {
+        const int e = threadIdx.x, k0 = e * VE / NB, j0 = e * VE % NB;
+        if (e * VE < NB * NB) {   // a 16-byte piece of each of P, R, A, D
+            const V vp = __ldcg(reinterpret_cast<const V *>(S.pi(p - 1)) + e);
+            const V vd = __ldcg(reinterpret_cast<const V *>(S.d(p - 1)) + e);
+            V vr, va;
+            if constexpr (sizeof(AT) == 4) {   // R by column (lanes along the columns), A by row
+                vr = __ldcg(reinterpret_cast<const V *>(S.r(p - 1) + (size_t)(p * NB + lane) * NB + I * 4));
+                va = __ldcg(reinterpret_cast<const V *>(S.a(p - 1) + (size_t)p * NB * NB) + e);
+            } else {
+                vr = __ldcg(reinterpret_cast<const V *>(S.r(p - 1) + (size_t)k0 * T + p * NB + j0));
+                va = __ldcg(reinterpret_cast<const V *>(S.a(p - 1) + (size_t)k0 * T + p * NB + j0));
+            }
+            reinterpret_cast<V *>(Ps)[e] = vp;
+            reinterpret_cast<V *>(As)[e] = va;
+            reinterpret_cast<V *>(Ds)[e] = vd;
             if constexpr (sizeof(AT) == 4) {
-                AT *Dk = a.D + blk[c] * bsz;
-                const int bj = r / npair, pb = r % npair;
-                const int j = bj < p ? bj : bj + 1;
-                auto ok = [&](int i) { return i < nt && i != p && !(nxt && i == p + 1 && j == p + 1); };
-                const int i0 = 2 * pb, i1 = 2 * pb + 1;
-                const bool o0 = ok(i0), o1 = ok(i1);
-                if (o0 && o1) {
-                    tc_pair_update(*reinterpret_cast<TcSmem *>(&ts), tcs, Dk, T, i0, p, j, a.err);
-                } else if (o0 || o1) {
-                    const int i = o0 ? i0 : i1;
-                    subtile_product<AT, 64, 64, 4, 4>(ts, Dk, Dk, Dk, T, i, p, p, j, i, j, 0, 0, (AT)-1, true);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) Xs[(I * 4 + m) * NB + lane] = reinterpret_cast<const float *>(&vr)[m];
+            } else {
+                reinterpret_cast<V *>(Xs)[e] = vr;
+            }
+        }
+        __syncthreads();
+        // t[u] (+)= sum_k row(u)[k] col[k]: rows of a row-major block, 16 bytes at a time
+        auto product = [&](const AT *rows, const AT *cols, AT (&t)[NE], AT sign) {
+#pragma unroll
+            for (int k = 0; k < NB; k += VE) {
+                AT x[VE];
+#pragma unroll
+                for (int m = 0; m < VE; ++m) x[m] = sign * cols[(k + m) * NB + c];
+#pragma unroll
+                for (int u = 0; u < NE; ++u) {
+                    const V q = *reinterpret_cast<const V *>(rows + u * NB + k);
+                    const AT *qe = reinterpret_cast<const AT *>(&q);
+#pragma unroll
+                    for (int m = 0; m < VE; ++m) t[u] = fma(qe[m], x[m], t[u]);
                 }
             }
         };
-        auto special = [&](int c) {         // tile (p+1, p+1) -= D_{p+1,p} D_{p,p+1}, then inverted
-            AT *Dk = a.D + blk[c] * bsz;
-            tile_invert(ts, Dk, T, p + 1, a.err, Dk + (long long)(p + 1) * TILE * T + p * TILE,
-                        Dk + (long long)p * TILE * T + (p + 1) * TILE);
-        };
-        if (nxt && own) {
-            if (b < nblk) special(b);
-            else
-                for (int q = b - nblk; q < nblk * nitem; q += G - nblk) regular(q);
+        AT t[NE];
+#pragma unroll
+        for (int u = 0; u < NE; ++u) t[u] = 0;
+        product(Ps + rr * NB, Xs, t, (AT)1);                     // U = P R
+#pragma unroll
+        for (int u = 0; u < NE; ++u) {
+            Us[(rr + u) * NB + c] = t[u];
+            a[u] = Ds[(rr + u) * NB + c];
+        }
+        __syncthreads();
+        if constexpr (sizeof(AT) == 4) {                         // D - A U
+            product(As + rr * NB, Us, a, (AT)-1);
+        } else {                                                 // (A transposed)
+#pragma unroll
+            for (int k = 0; k < NB; ++k) a[0] = fma(-As[k * NB + rr], Us[k * NB + c], a[0]);
+        }
+    }
+    bool ok = true;
+    gj_tile_inverse(a, W, ok);
+    if (!ok) atomicExch(err, ERR_PIVOT);
+    AT *out = S.pi(p);
+#pragma unroll
+    for (int u = 0; u < NE; ++u) out[(rr + u) * NB + c] = a[u];
+    if constexpr (sizeof(AT) == 4)
+        *reinterpret_cast<float4 *>(S.pt(p) + c * NB + rr) = make_float4(a[0], a[1], a[2], a[3]);
+    __syncthreads();   // the shared memory is free again
+}
+
+// Sets a ready flag after the CTA's earlier writes (gj_signal1: the caller has met at a
+// CTA barrier since them).
+__device__ __forceinline__ void gj_signal1(unsigned *f, unsigned v) {
+    if (threadIdx.x == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(f), "r"(v) : "memory");
+}
+__device__ __forceinline__ void gj_signal(unsigned *f, unsigned v) {
+    __syncthreads();
+    gj_signal1(f, v);
+}
+// Waits until three ready flags hold v: three threads poll, at most the launch's poll
+// limit. False (all threads) if the wait ran out, with ERR_TIMEOUT set, or an error is flagged.
+__device__ __forceinline__ bool gj_wait(const unsigned *f0, const unsigned *f1, const unsigned *f2, unsigned v,
+                                        GridBar *bar, int *err) {
+    int ok = 1;
+    if (threadIdx.x < 3) {
+        const unsigned *f = threadIdx.x == 0 ? f0 : (threadIdx.x == 1 ? f1 : f2);
+        const long long lim = bar->polls > 0 ? bar->polls : BAR_POLLS;
+        long long it = 0;
+        while (ld_acquire(f) != v) {
+            if (++it > lim) { atomicExch(err, ERR_TIMEOUT); ok = 0; break; }
+            if ((it & 1023) == 0 && ld_acquire((const unsigned *)err) != 0) { ok = 0; break; }
+        }
+    }
+    return __syncthreads_and(ok) != 0;
+}
+
+// ---- FP32 tiles: 128 x 128 values, products on the tensor cores ----
+//
+// Thread (w, lane) holds row 32 (w % 4) + lane of a tile, columns 64 (w / 4) .. + 63, in
+// registers: the part of tensor memory that its warp may read (32 rows = one panel: the
+// rows of a panel belong to two warps, its columns to one half of the warps).
+// One step is two groups of MMAs (kind::tf32): q = A P (M = 128, N = 32, K = 32), then
+// (-q) R (N = 128), which the threads add to their values with FP32 rounding. Letting the
+// MMAs accumulate on the tile in tensor memory instead cuts every partial sum towards
+// zero, 12 times per panel: the coarse correction's error against FP64 was ten times
+// larger (1.5e-5 for 1.6e-6 on a 64 x 96 x 48 grid). The same step on the CUDA cores took
+// 13,300 cycles, twice the pivot CTA's time.
+constexpr unsigned GJ_TMEM = 256;               // columns held: (-q) R 0 .. 127, q 128 .. 159
+constexpr unsigned GJ_SBO = 1024;               // 8 rows x 32 k of TF32: eight 128-byte core matrices
+constexpr unsigned GJ_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 4) << 24);   // + N / 8 << 17
+
+__device__ __forceinline__ unsigned long long gj_desc(const void *p) {
+    unsigned long long d = (unsigned long long)(((unsigned)__cvta_generic_to_shared(p) & 0x3FFFFu) >> 4);
+    d |= (unsigned long long)(TC_LBO >> 4) << 16;
+    d |= (unsigned long long)(GJ_SBO >> 4) << 32;
+    d |= 1ull << 46;
+    return d;
+}
+// 4 consecutive k (chunk kc) of row `row` of an operand as NS TF32 values each: heads,
+// then remainders (the last is cut to TF32 by the MMA: exact for NS = 3)
+template <int NS, int BYTES>
+__device__ __forceinline__ void gj_put(unsigned char (*op)[BYTES], int row, int kc, float4 v) {
+    const int o = (row >> 3) * (int)GJ_SBO + kc * (int)TC_LBO + (row & 7) * 16;
+#pragma unroll
+    for (int n = 0; n < NS; ++n) {
+        const float4 h = n + 1 < NS ? make_float4(tc_head(v.x), tc_head(v.y), tc_head(v.z), tc_head(v.w)) : v;
+        *reinterpret_cast<float4 *>(op[n] + o) = h;
+        v = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+    }
+}
+__device__ __forceinline__ void gj_ld32(unsigned addr, float (&v)[32]) {
+    unsigned r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
+          "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+          "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+// All threads: the operands in shared memory, then D[tmem] = A B over K = 32 by one
+// thread's MMAs, and the bounded wait for them. NS = 2: the three products of heads and
+// remainders down to 2^-22 of a product; NS = 3: the six down to 2^-33, FP32's accuracy.
+template <int NS, int BA, int BB>
+__device__ __forceinline__ void gj_mma(TcState &st, unsigned dcol, int n, const unsigned char (*A)[BA],
+                                       const unsigned char (*B)[BB], int *err) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const unsigned idesc = GJ_IDESC | ((unsigned)(n >> 3) << 17);
+        unsigned on = 0u;
+#pragma unroll
+        for (int sum = NS - 1; sum >= 0; --sum)          // smallest products first
+#pragma unroll
+            for (int ia = 0; ia <= sum; ++ia) {
+                const unsigned long long da = gj_desc(A[ia]), db = gj_desc(B[sum - ia]);
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    const unsigned long long o = (unsigned long long)(s * 2 * TC_LBO >> 4);   // k-step of 8: two core matrices
+                    asm volatile(
+                        "{\n.reg .pred pp;\n"
+                        "setp.ne.b32 pp, %4, 0;\n"
+                        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, pp;\n}\n"
+                        ::"r"(st.tmem + dcol), "l"(da + o), "l"(db + o), "r"(idesc), "r"(on) : "memory");
+                    on = 1u;
+                }
+            }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                     ::"r"((unsigned)__cvta_generic_to_shared(st.mbar)) : "memory");
+    }
+    const unsigned a = (unsigned)__cvta_generic_to_shared(st.mbar), par = st.phase & 1;
+    bool done = false;
+    for (long long it = 0; it < TC_POLLS && !done; ++it) {
+        unsigned ok;
+        asm volatile(
+            "{\n.reg .pred pp;\n"
+            "mbarrier.try_wait.parity.shared::cta.b64 pp, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, pp;\n}\n"
+            : "=r"(ok) : "r"(a), "r"(par) : "memory");
+        done = ok != 0;
+    }
+    if (!done) atomicExch(err, ERR_TIMEOUT);
+    ++st.phase;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
+struct GjTile {
+    int r0, c0, quad, half, lane;   // tile origin; this warp's rows and columns
+    unsigned tm;                    // tensor memory of this warp's rows and columns
+    unsigned tq;                    // and of its rows of q
+    float v[64];                    // this thread's values
+    __device__ __forceinline__ GjTile(const TcState &st, int ti, int tj) : r0(ti * 128), c0(tj * 128) {
+        const int w = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+        quad = w & 3; half = w >> 2; lane = threadIdx.x & 31;
+        tm = st.tmem + ((unsigned)(32 * quad) << 16) + 64u * half;
+        tq = st.tmem + ((unsigned)(32 * quad) << 16) + 128u;
+    }
+    __device__ __forceinline__ int row() const { return r0 + 32 * quad + lane; }
+    __device__ __forceinline__ bool in(int T) const { return row() < T && c0 + 64 * half < T; }   // (T: of 64s)
+    __device__ __forceinline__ void load(const float *M, int T) {
+        const bool on = in(T);
+        const float4 *src = reinterpret_cast<const float4 *>(M + (long long)row() * T + c0 + 64 * half);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const float4 x = on ? __ldcg(src + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+        }
+    }
+    __device__ __forceinline__ void store(float *M, int T) const {
+        if (!in(T)) return;
+        float4 *dst = reinterpret_cast<float4 *>(M + (long long)row() * T + c0 + 64 * half);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+};
+
+// Step p of one tile (see the section's comment). The caller meets at a CTA barrier
+// before the shared memory is written again.
+__device__ __forceinline__ void gj_tile_step(GjTile &t, TcState &st, float *Z, int T, int p, unsigned char *smem,
+                                          int *err) {
+    constexpr int NB = 32;
+    GjTcSmem &sm = *reinterpret_cast<GjTcSmem *>(smem);
+    const GjStrips<float> S(Z, T);
+    const int w = t.quad + 4 * t.half, lane = t.lane;
+    {   // operands: lanes over 8 rows x 4 chunks of 16 bytes (conflict-free stores)
+        const int rl = lane & 7, kl = lane >> 3;
+        float4 va[4], vr[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int g = w + 8 * m, x = (g >> 1) * 8 + rl, kc = (g & 1) * 4 + kl;
+            if (t.r0 + x < T) va[m] = __ldcg(reinterpret_cast<const float4 *>(S.a(p) + (size_t)(t.r0 + x) * NB) + kc);
+            if (t.c0 + x < T) vr[m] = __ldcg(reinterpret_cast<const float4 *>(S.r(p) + (size_t)(t.c0 + x) * NB) + kc);
+        }
+        const int px = (w >> 1) * 8 + rl, pk = (w & 1) * 4 + kl;
+        const float4 vp = __ldcg(reinterpret_cast<const float4 *>(S.pt(p) + px * NB) + pk);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int g = w + 8 * m, x = (g >> 1) * 8 + rl, kc = (g & 1) * 4 + kl;
+            if (t.r0 + x < T) gj_put<3>(sm.a, x, kc, va[m]);
+            if (t.c0 + x < T) gj_put<2>(sm.r, x, kc, vr[m]);
+        }
+        gj_put<3>(sm.p, px, pk, vp);
+    }
+    gj_mma<3>(st, 128, 32, sm.a, sm.p, err);          // q = A P
+    const int row = t.row();
+    const bool piv = row / NB == p;                                   // (uniform in the warp)
+    float q[32];
+    if (piv) {                                                        // rows of the panel: q = -P
+        const float4 *pr = reinterpret_cast<const float4 *>(S.pi(p) + (row % NB) * NB);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float4 x = __ldcg(pr + k);
+            q[4 * k] = -x.x; q[4 * k + 1] = -x.y; q[4 * k + 2] = -x.z; q[4 * k + 3] = -x.w;
+        }
+#pragma unroll
+        for (int k = 0; k < 64; ++k) t.v[k] = 0.f;
+    } else {
+        gj_ld32(t.tq, q);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {                                     // -q over A (whose MMAs are done), half a row each
+        const int kc = 4 * t.half + k;
+        const float4 v = t.half ? make_float4(-q[16 + 4 * k], -q[17 + 4 * k], -q[18 + 4 * k], -q[19 + 4 * k])
+                                : make_float4(-q[4 * k], -q[4 * k + 1], -q[4 * k + 2], -q[4 * k + 3]);
+        gj_put<2>(sm.a, row - t.r0, kc, v);
+    }
+    gj_mma<2>(st, 0, 128, sm.a, sm.r, err);           // tile -= q R
+    const int h0 = t.c0 + 64 * t.half;                                // this warp's first column
+    const int rp = (t.r0 >> 5) + t.quad, n = p + 1;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {                                     // 32 columns, one panel, at a time
+        float x[32];
+        gj_ld32(t.tm + 32 * h, x);
+        const int col = h0 + 32 * h, cp = col / NB;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) t.v[32 * h + k] = cp == p ? -q[k] : t.v[32 * h + k] + x[k];
+        // the next panel's rows (by column) and columns (by row), and the diagonal block after it
+        if (rp == n && col < T) {
+            float *o = S.r(n) + (size_t)col * NB + lane;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) o[k * NB] = t.v[32 * h + k];
+        }
+        const bool next_a = cp == n && col < T && row < T, next_d = rp == n + 1 && cp == n + 1 && col < T;
+        if (next_a || next_d) {
+            float4 *o = reinterpret_cast<float4 *>(next_a ? S.a(n) + (size_t)row * NB : S.d(n) + lane * NB);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                o[k] = make_float4(t.v[32 * h + 4 * k], t.v[32 * h + 4 * k + 1], t.v[32 * h + 4 * k + 2],
+                                   t.v[32 * h + 4 * k + 3]);
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+
+// FP64: step p of the rows of pass u, strips of RG rows (T / 2 threads each, 256 at most)
+template <int RG>
+__device__ __noinline__ void gj_rows(double *M, double *Z, int T, int p, int u, unsigned char *smem) {
+    constexpr int NB = 16, KB = 8;
+    const GjStrips<double> S(Z, T);
+    const int tw = gj64_strip(T), ns = 256 / tw;
+    const int sub = threadIdx.x / tw, c = threadIdx.x - sub * tw;
+    const int r0 = u * ns * RG, nrow = ns * RG;
+    const double *R = S.r(p);
+    double *Ps = reinterpret_cast<double *>(smem), *as = Ps + NB * NB, *qs = as + nrow * NB;
+    const bool live = sub < ns;
+    const int row0 = r0 + sub * RG;                  // this strip's first row
+    double2 a[RG], pan[KB];
+    auto load_rows = [&](int col) {
+#pragma unroll
+        for (int r = 0; r < RG; ++r) {
+            const int row = row0 + r;
+            a[r] = row < T && row / NB != p ? __ldcg(reinterpret_cast<const double2 *>(M + (long long)row * T + col))
+                                            : make_double2(0.0, 0.0);
+        }
+    };
+    auto load_pan = [&](int col, int k0) {
+#pragma unroll
+        for (int k = 0; k < KB; ++k) pan[k] = __ldcg(reinterpret_cast<const double2 *>(R + (size_t)(k0 + k) * T + col));
+    };
+    if (live && c * 2 < T) {                         // the first loads, in flight during the q step
+        load_pan(c * 2, 0);
+        load_rows(c * 2);
+    }
+    if (threadIdx.x < NB * NB / 2)
+        reinterpret_cast<double2 *>(Ps)[threadIdx.x] = __ldcg(reinterpret_cast<const double2 *>(S.pi(p)) + threadIdx.x);
+    for (int e = threadIdx.x; e < nrow * NB / 2; e += 256) {
+        const int row = r0 + e / (NB / 2);
+        if (row < T)
+            reinterpret_cast<double2 *>(as)[e] =
+                __ldcg(reinterpret_cast<const double2 *>(M + (long long)row * T + p * NB) + e % (NB / 2));
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nrow * NB; e += 256) {
+        const int r = e / NB, j = e % NB, row = r0 + r;
+        double t = 0.0;
+        if (row < T) {
+            if (row / NB == p) {
+                t = -Ps[(row % NB) * NB + j];
+            } else {
+#pragma unroll
+                for (int k = 0; k < NB; ++k) t = fma(as[r * NB + k], Ps[k * NB + j], t);
+            }
+        }
+        qs[e] = t;
+    }
+    __syncthreads();
+    const double *q = qs + (size_t)sub * RG * NB;
+    for (int col = c * 2; live && col < T; col += 512) {
+        if (col != c * 2) {
+            load_pan(col, 0);
+            load_rows(col);
+        }
+#pragma unroll
+        for (int k0 = 0; k0 < NB; k0 += KB) {
+            double2 cur[KB];
+#pragma unroll
+            for (int k = 0; k < KB; ++k) cur[k] = pan[k];
+            if (k0 + KB < NB) load_pan(col, k0 + KB);
+#pragma unroll
+            for (int k = 0; k < KB; ++k)
+#pragma unroll
+                for (int r = 0; r < RG; ++r) {
+                    const double w = q[r * NB + k0 + k];
+                    a[r].x = fma(-w, cur[k].x, a[r].x);
+                    a[r].y = fma(-w, cur[k].y, a[r].y);
+                }
+        }
+        const int cp = col / NB;                     // the column pair's panel
+#pragma unroll
+        for (int r = 0; r < RG; ++r) {
+            const int row = row0 + r;
+            if (row >= T) continue;
+            const double2 o = cp == p ? make_double2(-q[r * NB + col % NB], -q[r * NB + col % NB + 1]) : a[r];
+            *reinterpret_cast<double2 *>(M + (long long)row * T + col) = o;
+            const int rp = row / NB;
+            if (rp == p + 1) *reinterpret_cast<double2 *>(S.r(p + 1) + (size_t)(row % NB) * T + col) = o;
+            if (rp == p + 2 && cp == p + 1) {        // the pivot CTA reads A only for its own panel's rows
+                S.a(p + 1)[(size_t)(col % NB) * T + row] = o.x;
+                S.a(p + 1)[(size_t)(col % NB + 1) * T + row] = o.y;
+            }
+            if (rp == p + 2 && cp == p + 2)
+                *reinterpret_cast<double2 *>(S.d(p + 1) + (row % NB) * NB + col % NB) = o;
+        }
+    }
+    __syncthreads();   // the shared memory is free again
+}
+
+// Rows per strip of the FP64 step: the size whose passes over `ctas` CTAs do the fewest
+// row steps (a pass also costs about one row's time). Every size gives the same bits.
+__device__ __forceinline__ int gj64_rows_per_strip(int T, int ctas) {
+    const int cand[3] = {2, 4, GJ64_MAXR}, ns = 256 / gj64_strip(T);
+    int best = 2, cost = 0x7fffffff;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int pass = (T + ns * cand[i] - 1) / (ns * cand[i]);
+        const int w = ((pass + ctas - 1) / ctas) * (cand[i] + 1);
+        if (w < cost) { cost = w; best = cand[i]; }
+    }
+    return best;
+}
+
+// In-place inverses of the blocks blk[0 .. nblk), one chain each. The pivot blocks have
+// a CTA of their own when every chain can have one and another CTA; the other CTAs are
+// dealt to the chains in turn. Returns false when a barrier gave up.
+template <typename AT>
+__device__ __forceinline__ bool invert_blocks(const FacArgs<AT> &a, unsigned char *smem, const int *blk, int nblk,
+                                              unsigned &epoch, int b, int G, TcState &st) {
+    constexpr int NB = Gj<AT>::NB;
+    const int T = a.T, np = T / NB;
+    const long long bsz = (long long)T * T;
+    const size_t zs = gj_scratch<AT>(T);
+    const bool own = G >= 2 * nblk;
+    // prologue: the strips of panel 0, the diagonal block of panel 1, P of panel 0
+    for (int ch = b; ch < nblk; ch += G) gj_pivot(a.D + blk[ch] * bsz, a.Z + ch * zs, T, 0, smem, a.err);
+    for (int ch = 0; ch < nblk; ++ch) {
+        const AT *M = a.D + blk[ch] * bsz;
+        const GjStrips<AT> S(a.Z + ch * zs, T);
+        for (int e = b * 256 + threadIdx.x; e < 2 * NB * T + NB * NB; e += 256 * G) {
+            if (e < 2 * NB * T) {            // [NB][T] and [T][NB] forms of the first rows and columns
+                const int f = e % (NB * T);
+                const AT row = __ldcg(M + (sizeof(AT) == 4 ? (long long)(f % NB) * T + f / NB : f));
+                const AT col = __ldcg(M + (sizeof(AT) == 4 ? (long long)(f / NB) * T + f % NB
+                                                           : (long long)(f % T) * T + f / T));
+                if (e < NB * T) S.R[f] = row;
+                else S.A[f] = col;
+            } else {
+                const int f = e - 2 * NB * T;
+                S.D[f] = __ldcg(M + (long long)(NB + f / NB) * T + NB + f % NB);
+            }
+        }
+    }
+    if (!grid_barrier(a.bar, a.err, epoch, G)) return false;
+    // chain ch's CTAs are ch, ch + nblk, ... of the nw that take no pivots (all CTAs,
+    // strided over every chain's parts, when !own)
+    const int w = own ? b - nblk : b, nw = own ? G - nblk : G;
+    const int ch = w >= 0 ? w % nblk : 0, nct = own ? (nw - ch + nblk - 1) / nblk : nw;
+    auto pivots = [&](int p) {
+        if (p + 1 >= np) return;
+        if (own) {
+            if (b < nblk) gj_pivot<AT>(nullptr, a.Z + b * zs, T, p + 1, smem, a.err);
         } else {
-            const int ns = nxt ? nblk : 0;
-            for (int it = b; it < ns + nblk * nitem; it += G) {
-                if (it < ns) special(it);
-                else regular(it - ns);
-            }
+            for (int c = b; c < nblk; c += G) gj_pivot<AT>(nullptr, a.Z + c * zs, T, p + 1, smem, a.err);
         }
-        if (!grid_barrier(a.bar, a.err, epoch, G)) return false;
-        // phase B: column panel of step p (D_ip = -D_ip P_p, i != p, p+1),
-        // row panel of step p+1 (D_{p+1,j} = P_{p+1} D_{p+1,j}, j != p, p+1),
-        // and tile (p+1, p) = P_{p+1} (-D_{p+1,p} P_p)
-        const int ncol = nt - 1 - (nxt ? 1 : 0);
-        const int nrow = nxt ? nt - 2 : 0;
-        const int nB = 4 * ncol + 4 * nrow + (nxt ? 4 : 0);
-        for (int it2 = b; it2 < nblk * nB; it2 += G) {
-            const int c = it2 / nB, it = it2 % nB;
-            AT *Dk = a.D + blk[c] * bsz;
-            if (it < 4 * ncol) {
-                const int t = it >> 2, q = it & 3;
-                const int i = t < p ? t : t + 2;      // skip p and p + 1
-                subtile_product<AT, 16, 64, 2, 2>(ts, Dk, Dk, Dk, T, i, p, p, p, i, p, 16 * q, 0,
-                                                  (AT)-1, false);
-            } else if (it < 4 * ncol + 4 * nrow) {
-                const int e = it - 4 * ncol;
-                const int t = e >> 2, q = e & 3;
-                const int j = t < p ? t : t + 2;      // skip p and p + 1
-                subtile_product<AT, 64, 16, 2, 2>(ts, Dk, Dk, Dk, T, p + 1, p + 1, p + 1, j, p + 1, j,
-                                                  0, 16 * q, (AT)1, false);
-            } else {                                  // D_{p+1,p} = P_{p+1} Z (column strips)
-                const int q = it - 4 * ncol - 4 * nrow;
-                subtile_product<AT, 64, 16, 2, 2>(ts, Dk, a.Z + (long long)c * TILE * T, Dk, T, p + 1,
-                                                  p + 1, 0, 0, p + 1, p, 0, 16 * q, (AT)1, false);
+    };
+    if constexpr (sizeof(AT) == 4) {
+        const int nt = (T + 127) / 128;
+        // One tile per CTA, in registers throughout, with ready flags instead of barriers
+        // between the steps: a flag holds the inversion's number (epoch) once its data is
+        // written. A barrier per panel costs ~2.3 us with its skew and makes every step as
+        // long as the slower of pivot and tiles; with flags the pivot chain runs on as soon
+        // as the two tiles it reads are done. Nothing is reused: a slot per panel.
+        if (own && nt <= GJ_MAXT && nt * nt <= nw / nblk) {
+            const int me = w >= 0 ? w / nblk : 0, ti = me / nt, tj = me % nt;
+            GjTile t(st, ti, tj);
+            const bool mine = w >= 0 && w / nblk < nt * nt, pivot = b < nblk;
+            const int c = pivot ? b : ch;
+            float *M = a.D + blk[c] * bsz, *Z = a.Z + c * zs;
+            unsigned *fP = a.flags + c * gj_flags(T), *fD = fP + np, *fR = fD + np, *fA = fR + (size_t)np * nt;
+            const unsigned ep = epoch;
+            bool ok = true;
+            if (pivot) {
+                for (int p = 1; p < np && ok; ++p) {
+                    const int k = p - 1, tp = p / 4;
+                    if (k > 0) ok = gj_wait(fR + k * nt + tp, fA + k * nt + tp, fD + k, ep, a.bar, a.err);
+                    if (!ok) break;
+                    gj_pivot<float>(nullptr, Z, T, p, smem, a.err);
+                    gj_signal(fP + p, ep);
+                }
+            } else if (mine) {
+                t.load(M, T);
+                for (int p = 0; p < np && ok; ++p) {
+                    if (p > 0) ok = gj_wait(fR + p * nt + tj, fA + p * nt + ti, fP + p, ep, a.bar, a.err);
+                    if (!ok) break;
+                    gj_tile_step(t, st, Z, T, p, smem, a.err);
+                    __syncthreads();               // the strips are written, the shared memory is free
+                    if (p + 1 < np) {
+                        if ((p + 1) / 4 == ti) gj_signal1(fR + (p + 1) * nt + tj, ep);
+                        if ((p + 1) / 4 == tj) gj_signal1(fA + (p + 1) * nt + ti, ep);
+                        if ((p + 2) / 4 == ti && ti == tj) gj_signal1(fD + p + 1, ep);
+                    }
+                }
+                if (ok) t.store(M, T);
             }
+            return grid_barrier(a.bar, a.err, epoch, G) && ok;
         }
-        if (!grid_barrier(a.bar, a.err, epoch, G)) return false;
+        for (int p = 0; p < np; ++p) {
+            pivots(p);
+            for (int it = own ? w / nblk : b; w >= 0 && it < (own ? nt * nt : nblk * nt * nt); it += nct) {
+                const int c = own ? ch : it / (nt * nt), q = own ? it : it % (nt * nt);
+                GjTile t(st, q / nt, q % nt);
+                t.load(a.D + blk[c] * bsz, T);
+                gj_tile_step(t, st, a.Z + c * zs, T, p, smem, a.err);
+                t.store(a.D + blk[c] * bsz, T);
+                __syncthreads();   // the next tile overwrites the staged operands and tensor memory
+            }
+            if (!grid_barrier(a.bar, a.err, epoch, G)) return false;
+        }
+    } else {
+        const int rg = gj64_rows_per_strip(T, nw / (own ? nblk : 1));
+        const int per = (256 / gj64_strip(T)) * rg, npass = (T + per - 1) / per;
+        for (int p = 0; p < np; ++p) {
+            pivots(p);
+            for (int it = own ? w / nblk : b; w >= 0 && it < (own ? npass : nblk * npass); it += nct) {
+                const int c = own ? ch : it / npass, u = own ? it : it % npass;
+                double *M = a.D + blk[c] * bsz, *Z = a.Z + c * zs;
+                if (rg == 2) gj_rows<2>(M, Z, T, p, u, smem);
+                else if (rg == 4) gj_rows<4>(M, Z, T, p, u, smem);
+                else gj_rows<GJ64_MAXR>(M, Z, T, p, u, smem);
+            }
+            if (!grid_barrier(a.bar, a.err, epoch, G)) return false;
+        }
     }
     return true;
 }
@@ -1646,12 +1778,11 @@ __device__ __forceinline__ AT *cr_slot(const FacArgs<AT> &a, int s) {
 }
 
 template <typename AT>
-__device__ void cr_factor_body(const FacArgs<AT> &a, int b, int G, TcState &tcs) {
+__device__ __noinline__ void cr_factor_body(const FacArgs<AT> &a, int b, int G, TcState &tcs) {
     if constexpr (sizeof(AT) == 4) {
         extern __shared__ __align__(16) unsigned char smem_raw[];
-        TileSmem<AT> &ts = *reinterpret_cast<TileSmem<AT> *>(smem_raw);
         TcSmem &tsm = *reinterpret_cast<TcSmem *>(smem_raw);
-        const int nt = a.nt, per = ((nt + 1) / 2) * nt;   // items of one product
+        const int nt = a.T / TILE, per = ((nt + 1) / 2) * nt;   // items of one product
         if (!tcs.on) {                     // the reduction needs the tensor path
             if (threadIdx.x == 0) atomicExch(a.err, ERR_ELL);
             return;
@@ -1663,7 +1794,7 @@ __device__ void cr_factor_body(const FacArgs<AT> &a, int b, int G, TcState &tcs)
         unsigned epoch = 0;
         for (int r = 0; r < nround; ++r) {
             const int nE = s[0];
-            if (!invert_blocks(a, ts, s + 1, nE, epoch, b, G, tcs)) return;
+            if (!invert_blocks(a, smem_raw, s + 1, nE, epoch, b, G, tcs)) return;
             s += 1 + nE;
             for (int ph = 0; ph < 2; ++ph) {
                 const int n = s[0];
@@ -1679,7 +1810,7 @@ __device__ void cr_factor_body(const FacArgs<AT> &a, int b, int G, TcState &tcs)
                 if (!grid_barrier(a.bar, a.err, epoch, G)) return;
             }
         }
-        invert_blocks(a, ts, last, 1, epoch, b, G, tcs);
+        invert_blocks(a, smem_raw, last, 1, epoch, b, G, tcs);
     }
 }
 
@@ -1690,7 +1821,6 @@ __device__ __forceinline__ void coarse_factor_body(const FacArgs<AT> &a, int b, 
         return;
     }
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TileSmem<AT> &ts = *reinterpret_cast<TileSmem<AT> *>(smem_raw);
     AT *rows = reinterpret_cast<AT *>(smem_raw);
     const int T = a.T, nb = a.nb, mid = a.mid;
     const long long bsz = (long long)T * T;
@@ -1705,7 +1835,7 @@ __device__ __forceinline__ void coarse_factor_body(const FacArgs<AT> &a, int b, 
         } else {
             blk[nblk++] = mid;
         }
-        if (!invert_blocks(a, ts, blk, nblk, epoch, b, G, tcs)) return;
+        if (!invert_blocks(a, smem_raw, blk, nblk, epoch, b, G, tcs)) return;
         if (s == nsteps) break;
         const long long ell = (long long)T * ELLW;
         const int nchunk = T / FROWS;
@@ -1737,15 +1867,15 @@ __device__ __forceinline__ void coarse_factor_body(const FacArgs<AT> &a, int b, 
 // Tensor memory and the MMA mbarrier of a factorisation CTA (FP32 with the tensor
 // path): allocated before the body, freed after it on every return path.
 template <typename AT>
-__device__ __forceinline__ void tc_begin(TcState &tcs, unsigned *slot, unsigned long long *mbar, bool want) {
+__device__ __forceinline__ void tc_begin(TcState &tcs, unsigned *slot, unsigned long long *mbar) {
     tcs.on = false;
     tcs.tmem = 0;
     tcs.mbar = mbar;
     tcs.phase = 0;
-    if (sizeof(AT) != 4 || !want) return;
+    if (sizeof(AT) != 4) return;
     if (threadIdx.x < 32) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;"
-                     ::"r"((unsigned)__cvta_generic_to_shared(slot)) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"((unsigned)__cvta_generic_to_shared(slot)), "n"(GJ_TMEM) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
@@ -1765,15 +1895,15 @@ __device__ __forceinline__ void tc_end(const TcState &tcs) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (threadIdx.x < 32)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tcs.tmem) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tcs.tmem), "n"(GJ_TMEM) : "memory");
 }
 
 template <typename AT>
-__global__ void __launch_bounds__(256) k_coarse_factor(FacArgs<AT> a, int use_tc) {
+__global__ void __launch_bounds__(256) k_coarse_factor(FacArgs<AT> a) {
     __shared__ unsigned tmem_slot;
     __shared__ unsigned long long mbar;
     TcState tcs;
-    tc_begin<AT>(tcs, &tmem_slot, &mbar, use_tc != 0);
+    tc_begin<AT>(tcs, &tmem_slot, &mbar);
     coarse_factor_body(a, blockIdx.x, gridDim.x, tcs);
     tc_end<AT>(tcs);
 }
@@ -1792,7 +1922,7 @@ __global__ void __launch_bounds__(256) k_coarse_factor_batch(const FacArgs<AT> *
     __shared__ unsigned tmem_slot;
     __shared__ unsigned long long mbar;
     TcState tcs;
-    tc_begin<AT>(tcs, &tmem_slot, &mbar, args[h].tc != 0 || args[h].cr != 0);
+    tc_begin<AT>(tcs, &tmem_slot, &mbar);
     coarse_factor_body(args[h], blockIdx.x - first[h], size[h], tcs);
     tc_end<AT>(tcs);
 }
@@ -2395,20 +2525,17 @@ static int configure_t(Coarse *c) {
                                                25 * WX + 128) + 32 * sizeof(int) + tables;
         if (c->rap125_smem <= (size_t)big || c->rap125_ng == 1) break;
     }
-    c->fac_smem = std::max(sizeof(TileSmem<AT>), sizeof(AT) * (size_t)FROWS * c->T);
+    c->fac_smem = std::max(gj_smem<AT>(c->T), sizeof(AT) * (size_t)FROWS * c->T);
     c->fac_smem = std::max(c->fac_smem, edge_rows_smem(c->T, sizeof(AT)));
-    // FP32: trailing updates of the inverses on the tensor cores (RAS_COARSE_TC=0: CUDA cores)
-    c->use_tc = sizeof(AT) == 4 ? 1 : 0;
-    if (const char *e = getenv("RAS_COARSE_TC")) c->use_tc = c->use_tc && atoi(e) != 0;
-    if (c->use_tc) c->fac_smem = std::max(c->fac_smem, sizeof(TcSmem));
     // RAS_COARSE_CR=1 at set-up (FP32 with the tensor path, at least three
     // blocks): cyclic reduction instead of the two-ended elimination. Not the
     // default: on the 1M-cell workload it takes 9.8 ms per factorisation against
     // 5.3 ms and its solve reads half as many bytes again (the dense products of
     // its rounds outweigh the shorter chain of inversions).
     c->cr = 0;
-    if (const char *e = getenv("RAS_COARSE_CR"))
-        c->cr = sizeof(AT) == 4 && c->use_tc && c->nb >= 3 && atoi(e) != 0 ? 1 : 0;
+    if (const char *e = getenv("RAS_COARSE_CR")) c->cr = sizeof(AT) == 4 && c->nb >= 3 && atoi(e) != 0 ? 1 : 0;
+    if (const char *e = getenv("RAS_COARSE_TC")) c->cr = c->cr && atoi(e) != 0;   // 0: no tensor-core products
+    if (c->cr) c->fac_smem = std::max(c->fac_smem, sizeof(TcSmem));
     // the solve prefetches up to two (FP32) or one (FP64) matrix rows per warp
     // (the reduction's sweeps read theirs directly)
     c->sol_npf = c->cr ? 0 : (sizeof(AT) == 4 ? 2 : 1);
@@ -2557,8 +2684,11 @@ int coarse_setup_grid(Coarse **out, int fnx, int fny, int fnz, const ras_opts &o
         return fail(rc);
     {
         unsigned char *p_z = nullptr, *p_rx = nullptr, *p_ry = nullptr;
-        const size_t nz = (size_t)std::max(2, c->cr_maxE);   // one scratch strip per concurrent inversion
-        if ((rc = dalloc(&p_z, nz * TILE * c->T * c->esz))) return fail(rc);
+        const size_t nz = (size_t)std::max(2, c->cr_maxE);   // scratch of each concurrent inversion
+        const size_t zs = c->prec == 64 ? gj_scratch<double>(c->T) : gj_scratch<float>(c->T);
+        if ((rc = dalloc(&p_z, nz * zs * c->esz))) return fail(rc);
+        c->nflag = c->prec == 64 ? 0 : nz * gj_flags(c->T);
+        if ((rc = dalloc(&c->d_flags, c->nflag))) return fail(rc);
         c->Zs = p_z;
         if ((rc = dalloc(&p_rx, (size_t)c->c[0] * c->n[1] * c->n[2] * c->esz))) return fail(rc);
         c->rx = p_rx;
@@ -2591,7 +2721,7 @@ void coarse_free(Coarse *c) {
         dfree(c->d_ia[a]); dfree(c->d_ib[a]); dfree(c->d_wa[a]); dfree(c->d_wb[a]);
         dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]);
     }
-    dfree(c->d_pos); dfree(c->d_cell); dfree(c->d_err); dfree(c->d_bar);
+    dfree(c->d_pos); dfree(c->d_cell); dfree(c->d_err); dfree(c->d_bar); dfree(c->d_flags);
     dfree(c->lo_q); dfree(c->up_q); dfree(c->lo_n); dfree(c->up_n); dfree(c->d_crf); dfree(c->d_crs);
     for (void *p : {c->Ac, c->D, c->C, c->F, c->lo_v, c->up_v, c->g, c->x, c->Zs, c->rx, c->ry, c->W, c->xn})
         if (p) cudaFree(p);
@@ -2624,10 +2754,10 @@ static int assemble_blocks_t(Coarse *c, cudaStream_t st) {
 }
 
 template <typename AT>
-static FacArgs<AT> fac_args(Coarse *c, GridBar *bar) {
+static FacArgs<AT> fac_args(Coarse *c, GridBar *bar, unsigned *flags) {
     return FacArgs<AT>{(AT *)c->D, (AT *)c->C, (AT *)c->F, (AT *)c->Zs, c->lo_q, c->up_q, c->lo_n, c->up_n,
-                       (const AT *)c->lo_v, (const AT *)c->up_v, c->T, c->T / TILE, c->nb, c->mid, bar, c->d_err,
-                       c->cr, c->d_crf, (AT *)c->W, c->use_tc};
+                       (const AT *)c->lo_v, (const AT *)c->up_v, c->T, c->nb, c->mid, bar, c->d_err,
+                       c->cr, c->d_crf, (AT *)c->W, flags};
 }
 
 template <typename AT>
@@ -2651,9 +2781,9 @@ static int factor_blocks_t(Coarse *c, cudaStream_t st) {
 template <typename AT>
 static int eliminate_t(Coarse *c, cudaStream_t st) {
     RAS_TRY(reset_bar(c, st));
-    FacArgs<AT> fa = fac_args<AT>(c, c->d_bar);
-    int use_tc = c->use_tc;
-    void *args[] = {&fa, &use_tc};
+    if (c->nflag) RAS_CK(cudaMemsetAsync(c->d_flags, 0, c->nflag * sizeof(unsigned), st));
+    FacArgs<AT> fa = fac_args<AT>(c, c->d_bar, c->d_flags);
+    void *args[] = {&fa};
     RAS_CK(cudaLaunchCooperativeKernel((const void *)k_coarse_factor<AT>, dim3(c->fac_grid),
                                        dim3(256), args, c->fac_smem, st));
     RAS_LAUNCHED();
@@ -2745,13 +2875,15 @@ struct CoarseBatch {
     int *d_fcta_inst = nullptr, *d_ffirst = nullptr, *d_fsize = nullptr;
     std::vector<int> fwave0, fwaven;        // factorisation waves: CTA range in d_fcta_inst
     GridBar *d_bars = nullptr;              // [n], one barrier word per handle
+    unsigned *d_flags = nullptr;            // the handles' ready flags, nflag in all
+    size_t nflag = 0;
 };
 
 void coarse_batch_free(CoarseBatch *cb) {
     if (!cb) return;
     if (cb->d_args) cudaFree(cb->d_args);
     if (cb->d_fargs) cudaFree(cb->d_fargs);
-    dfree(cb->d_cta_inst); dfree(cb->d_first); dfree(cb->d_size); dfree(cb->d_bars);
+    dfree(cb->d_cta_inst); dfree(cb->d_first); dfree(cb->d_size); dfree(cb->d_bars); dfree(cb->d_flags);
     dfree(cb->d_fcta_inst); dfree(cb->d_ffirst); dfree(cb->d_fsize);
     delete cb;
 }
@@ -2840,10 +2972,14 @@ static int batch_setup_t(Coarse *const *cs, int n, CoarseBatch *cb) {
     std::vector<SolArgs<AT>> args(n);
     std::vector<FacArgs<AT>> fargs(n);
     RAS_TRY(dalloc(&cb->d_bars, n));
+    for (int i = 0; i < n; ++i) cb->nflag += cs[i]->nflag;
+    RAS_TRY(dalloc(&cb->d_flags, cb->nflag));
+    size_t flag0 = 0;
     for (int i = 0; i < n; ++i) {
         Coarse *c = cs[i];
         args[i] = sol_args<AT>(c, cb->d_bars + i, nullptr, nullptr, 1);
-        fargs[i] = fac_args<AT>(c, cb->d_bars + i);
+        fargs[i] = fac_args<AT>(c, cb->d_bars + i, cb->d_flags + flag0);
+        flag0 += c->nflag;
     }
     RAS_CK(cudaMalloc(&cb->d_args, n * sizeof(SolArgs<AT>)));
     RAS_CK(cudaMalloc(&cb->d_fargs, n * sizeof(FacArgs<AT>)));
@@ -2886,6 +3022,7 @@ int coarse_batch_setup(Coarse *const *cs, int n, CoarseBatch **out) {
 int coarse_factor_batch(CoarseBatch *cb, const unsigned char *d_active, cudaStream_t st) {
     k_reset_bars<<<(cb->n + 127) / 128, 128, 0, st>>>(cb->d_bars, cb->n, barrier_polls());
     RAS_LAUNCHED();
+    if (cb->nflag) RAS_CK(cudaMemsetAsync(cb->d_flags, 0, cb->nflag * sizeof(unsigned), st));
     for (size_t w = 0; w < cb->fwave0.size(); ++w) {
         const int *cta = cb->d_fcta_inst + cb->fwave0[w];
         const dim3 grid(cb->fwaven[w]);
