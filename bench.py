@@ -70,7 +70,7 @@ def parse():
                          "(factor) REPS factorisations (used for the ncu captures)")
     ap.add_argument("--reps", type=int, default=20)
     ap.add_argument("--apply-kernel", type=int, choices=[0, 1], default=None,
-                    help="fine subdomain-solve kernel: 0 level-scheduled, 1 pipelined "
+                    help="fine subdomain-solve kernel setting (0 and 1 run the same sweeps; "
                          "(default: the library's choice)")
     return ap.parse_args()
 
@@ -361,7 +361,7 @@ def gb300_arm(args):
     avg_s = (apply_ms / 1e3) / max(apply_n, 1)
     achieved = bytes_per_launch / avg_s / 1e9 if apply_n else None
     traffic = None
-    kname = "k_ras_pipe" if pc.apply_kernel() == 1 else "k_ras_apply"
+    kname = "k_ras_apply"
     if args.workload == "c2" and not args.small:
         traffic = load_traffic(f"{kname}_fp{args.factor_prec}_1m")
     line = {

@@ -404,33 +404,26 @@ int ras_timing_read(ras_precond *pc, double *total_ms, long long *launches, int 
 double ras_apply_bytes(const ras_precond *pc);
 
 /* Level schedule of the fine-level subdomain solves (a performance setting; the
- * preconditioner's values do not depend on it): consecutive wavefront levels are
- * staged into shared memory in chunks of at most chunk_cells cells (at least the
- * widest level), and each box is solved by `threads` threads (a multiple of 32,
- * <= 512). 0 keeps the default of that argument (1024 cells, 384 for FP64
- * factors; the widest level rounded up to a warp). Smaller chunks use less shared
- * memory per box, so more boxes run per SM: worth it when there are many more
- * boxes than SMs. Synchronous; no apply of this handle may be in flight; a batch
- * created before the call keeps the old launch settings (create it again).
- * RAS_EINVAL for ILU(k > 0) handles, negative or invalid values, or a schedule
- * whose shared memory exceeds the per-block limit (the old schedule stays). */
+ * preconditioner's values do not depend on it): the factor records of consecutive
+ * wavefront levels are staged into a shared-memory ring of three chunks of chunk_cells
+ * cells (at least the widest level), and each box is solved by at least `threads` threads
+ * (a multiple of 32, <= 512; FP32 / BF16 factors: more where the warp roles of the sweeps
+ * take more). 0 keeps the default of that argument (1024 cells, 384 for FP64 factors; the
+ * widest level rounded up to a warp). Smaller chunks use less shared memory per box, so
+ * more boxes run per SM: worth it when there are many more boxes than SMs. Synchronous;
+ * no apply of this handle may be in flight; a batch created before the call keeps the old
+ * launch settings (create it again). RAS_EINVAL for ILU(k > 0) handles, negative or
+ * invalid values, or a schedule whose shared memory exceeds the per-block limit (the old
+ * schedule stays). */
 int ras_set_apply_schedule(ras_precond *pc, int chunk_cells, int threads);
 /* The current schedule (chunk_cells after raising it to the widest level). */
 int ras_get_apply_schedule(const ras_precond *pc, int *chunk_cells, int *threads);
 
-/* Kernel of the fine-level subdomain solves of Eq. equ:as-left (a performance
- * setting: both give the same values, bit for bit, in the same arithmetic order,
- * from the same factor records; the switch takes effect at the next ras_apply).
- * 0 (the default): level-scheduled, every wavefront level i + j + k of a box
- * separated by a CTA barrier, each thread looking its cell up in the level's
- * table (the schedule above applies), each owned z written as soon as the
- * backward sweep has it. 1: pencil-wavefront: each thread owns an x-pencil
- * (j, k) of a box and advances one cell per level, its -x neighbour kept in a
- * register, its positions following from the pencil and the level with no table
- * look-up; pencils numbered by anti-diagonal j + k; the records are staged in
- * chunks of levels (the schedule's chunk size) and z is written as soon as it is
- * final. Allowed for left-RAS (ras_type 1) ILU(0) with FP32 or BF16 factors when
- * no overlapped box has more than 1024 x-pencils (RAS_EINVAL otherwise). */
+/* Kernel of the fine-level subdomain solves of Eq. equ:as-left: 0 (the default) or 1, a
+ * setting of earlier versions that chose between two kernels with the same values. Both
+ * values now run the same wavefront sweeps (blocks of 2 x 2 cells, one CTA per box).
+ * 1 is allowed for left-RAS (ras_type 1) ILU(0) with FP32 or BF16 factors when no
+ * overlapped box has more than 1024 x-pencils (RAS_EINVAL otherwise). */
 int ras_set_apply_kernel(ras_precond *pc, int kernel);
 /* The current kernel of the subdomain solves (0 or 1, as above). */
 int ras_get_apply_kernel(const ras_precond *pc, int *kernel);

@@ -794,7 +794,7 @@ static int b_factor(ras_batch *B, const std::vector<int> &cur, const std::vector
             }
         }
         ras1_factor_params(pc->fine, A, fp[i]);
-        fblock = std::max(fblock, std::min(pc->fine.block, 256));
+        fblock = std::max(fblock, pc->fine.fac_block);
         fsmem = std::max(fsmem, pc->fine.smem_factor);
     }
     RAS_CK(cudaMemcpyAsync(B->d_fp, fp.data(), n * sizeof(FactorParams), cudaMemcpyHostToDevice, st));
@@ -992,7 +992,7 @@ static int batch_create(int n, ras_problem *const *probs, ras_precond *const *pc
             box_local.push_back(q);
             box_cells.push_back(pc->fine.shapes[pc->fine.subs[q].shape].ncell);
         }
-        B->block = std::max(B->block, pc->fine.block);
+        B->block = std::max(B->block, pc->fine.launch);
         B->smem = std::max(B->smem, pc->fine.smem_apply);
     }
     if (off > 0x7fffffffLL) return fail(RAS_EINVAL);   // the flat vector kernels take int counts

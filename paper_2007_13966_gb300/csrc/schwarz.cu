@@ -1,12 +1,12 @@
 // One-level restricted additive Schwarz (Section 3.1) on sm_103a.
 //
-// The paper's subdomains (one per MPI rank on Tianhe-2) become one CTA each.
-// Inside a subdomain the natural-order ILU(0) triangular solves are run as a
-// wavefront: cells with equal i + j + k form a level, levels are separated by
-// CTA barriers, and the working vector lives in shared memory. Factor records
-// are stored in level order so that each staged chunk of consecutive levels is
-// one contiguous range, streamed into a shared-memory ring with cp.async ahead
-// of the sweep that consumes it.
+// The paper's subdomains (one per MPI rank on Tianhe-2) become one CTA each. Inside a
+// subdomain the natural-order ILU(0) triangular solves run as a wavefront with the
+// working vector in shared memory: over blocks of 2 x 2 cells with FP32 / BF16
+// factors, over single cells with FP64 factors (whose arithmetic, not the wavefront's
+// latency, bounds them). Factor records are stored in the order of the sweep, so that
+// each staged chunk of consecutive levels is one contiguous range, streamed into a
+// shared-memory ring with cp.async ahead of the sweep that consumes it.
 #include "schwarz.cuh"
 
 #include <algorithm>
@@ -28,10 +28,6 @@ template <int PREC> struct RecT;
 template <> struct RecT<64> { using T = RecF64; using Acc = double; };
 template <> struct RecT<32> { using T = RecF32; using Acc = float; };
 template <> struct RecT<16> { using T = RecB16; using Acc = float; };
-
-__device__ __forceinline__ RecF64 make_rec64(double a, double b, double c, double d) {
-    return RecF64{a, b, c, d};
-}
 
 template <int PREC>
 __device__ __forceinline__ void store_rec(void *base, long long idx, double a, double b, double c,
@@ -115,10 +111,17 @@ __device__ __forceinline__ int fast_div(int q, int d, unsigned m) {
 
 
 
-// One subdomain solve (one CTA): box `box` of the handle described by P, input r,
-// output z (whole-grid vectors of that handle).
+// A read-only load that stays where it is written (a batch of loads before their uses)
+__device__ __forceinline__ double load_now(const double *p) {
+    double v;
+    asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+
+// One subdomain solve (one CTA), cell by cell: box `box` of the handle described by P,
+// input r, output z (whole-grid vectors of that handle).
 template <int PREC, int NBUF>
-__device__ __forceinline__ void ras_apply_box(const ApplyParams &P, int box, const double *r, double *z,
+__device__ __forceinline__ void ras_apply_cells(const ApplyParams &P, int box, const double *r, double *z,
                                               int accumulate) {
     using R = typename RecT<PREC>::T;
     using Acc = typename RecT<PREC>::Acc;
@@ -179,7 +182,7 @@ __device__ __forceinline__ void ras_apply_box(const ApplyParams &P, int box, con
             const int q = q0 + m * (int)blockDim.x;
             if (q < sh.ncell) {
                 const int row = fast_div(q, bx, mbx), k = fast_div(row, by, mby);
-                v[m] = __ldg(rg + (q - row * bx) + nx * (row - k * by) + nxy * k);
+                v[m] = load_now(rg + (q - row * bx) + nx * (row - k * by) + nxy * k);
             }
         }
 #pragma unroll
@@ -316,9 +319,328 @@ __device__ __forceinline__ void ras_apply_box(const ApplyParams &P, int box, con
     }
 }
 
-template <int PREC, int NBUF>
-__global__ void __launch_bounds__(512, 2) k_ras_apply(ApplyParams P) {
-    ras_apply_box<PREC, NBUF>(P, blockIdx.x, P.r, P.z, P.accumulate);
+// ---- mbarriers of the sweeps in blocks (one phase per box; waits are bounded) ----
+constexpr int APPLY_TIMEOUT = 7;                // error word of a wait that ran out
+constexpr int APPLY_POLLS = 1 << 22;
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mb_init(unsigned long long *b, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mb_inval(unsigned long long *b) {
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(b)) : "memory");
+}
+__device__ __forceinline__ void mb_arrive(unsigned long long *b) {
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
+}
+__device__ __forceinline__ void mb_wait(unsigned long long *b, int *err) {
+    unsigned ok = 0;
+    for (int it = 0; it < APPLY_POLLS; ++it) {
+        asm volatile(
+            "{\n.reg .pred pp;\n"
+            "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 pp, [%1], 0;\n"
+            "selp.u32 %0, 1, 0, pp;\n}\n"
+            : "=r"(ok) : "r"(smem_addr(b)) : "memory");
+        if (ok) return;
+    }
+    atomicMax(err, APPLY_TIMEOUT);
+}
+// `bytes` of global memory into shared memory by the bulk copy engine, completing on b
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, unsigned long long *b) {
+    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;"
+                 ::"r"(smem_addr(b)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(b)) : "memory");
+}
+__device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }   // (from any warp role)
+
+// One subdomain solve (one CTA) in blocks of 2 x 2 cells of a plane, FP32 / BF16 factors.
+//
+// Cell by cell the sweeps are chains of bx + by + bz - 2 levels (58 for 20^3), each a CTA
+// barrier, a table look-up, shared-memory reads and one cell's arithmetic: ~0.2 us per
+// level whatever the bytes, 23 of the kernel's 45 us. Over blocks of 2 x 2 cells a sweep has
+// bx / 2 + by / 2 + bz - 2 levels (38) of at most 100 blocks, one thread per block: a thread
+// reads its 4 records (ahead of the barrier) and 4 + 8 values, runs the block's cells in
+// registers in natural order and writes 4 values. Every cell's arithmetic and its order
+// are those of the cell-by-cell sweep, so the values are the same bit for bit.
+// 45.5 -> 35.0 us per launch on 128 x 128 x 64 cells (256 boxes of up to 20^3, FP32, 69 MB:
+// 1.96 TB/s). What bounds it is the length of the warps' instruction streams, about 16
+// cycles per instruction and warp with ~4 warps per scheduler (ncu): a level of the sweep
+// is ~80 instructions, ~400 cycles; blocks of 2 x 2 x 2 cells have 28 levels of ~620 cycles,
+// and with half as many helpers (four cells of a plane each) the gather takes 43 us.
+//
+// Warp roles, so that the sweeping warps wait for nothing but one another:
+//   - sweepers (as many as the widest level takes) meet at a barrier of their own per
+//     level;
+//   - one thread streams the records, level by level, into a ring with bulk copies, as far
+//     ahead as the ring holds (a host table gives each step's place and how far to run);
+//   - one warp waits for them and for r, and joins the sweepers' barrier when both are in;
+//   - the helpers gather r plane by plane ahead of the forward sweep (every thread the same
+//     cells of each plane: index arithmetic per cell took longer than the loads), and write the owned cells of every
+//     four levels that the backward sweep has finished.
+// All warps meeting at one barrier per level took 43 us: the level then takes as long as
+// its slowest role.
+//
+// The vector is held as float4 per block (elements di + 2 dj), with a plane stride that
+// makes the threads of a level (J + 1, k - 1 from one lane to the next) step by an odd
+// number of 16-byte units: no bank conflicts. A neighbour outside the box has a zero
+// factor value and reads a finite value (a block of the box or the zero guard on either
+// side); cells that pad an odd edge are zero throughout (zero records).
+constexpr int PUT_LEVELS = 4;
+template <int PREC>
+__device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, const double *r, double *z,
+                                                 int accumulate) {
+    using R = typename RecT<PREC>::T;
+    constexpr int RB = (int)sizeof(R);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const BoxInfo bi = P.boxes[box];
+    const SubInfo &si = bi.sub;
+    const ShapeInfo &sh = bi.shape;
+    const int bx = sh.bx, by = sh.by, bz = sh.bz, mx = sh.mx, mp = sh.mp, nlev = sh.nlev, nstep = 2 * nlev;
+    const int yoff = sh.my > 1 ? mx : 0, zoff = bz > 1 ? mp : 0, guard = sh.guard;
+    // [values with guards][steps][block table][mbarriers: records of a step in / read, plane of r, put of levels][ring]
+    float4 *Y = reinterpret_cast<float4 *>(smem) + P.gcap;
+    int4 *st = reinterpret_cast<int4 *>(Y + P.ycap + P.gcap);
+    unsigned *bt = reinterpret_cast<unsigned *>(st + 2 * P.lcap);           // I | J << 8 | k << 16, level order
+    unsigned long long *mb_rec = reinterpret_cast<unsigned long long *>(bt + P.ycap);
+    unsigned long long *mb_free = mb_rec + 2 * P.lcap, *mb_pl = mb_free + 2 * P.lcap, *mb_put = mb_pl + P.lcap;
+    unsigned char *ring = reinterpret_cast<unsigned char *>(mb_put + P.lcap);
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    // warps: sweepers, helpers (one at least, see the launch), a waiter and an issuer
+    const int nsw = (sh.maxw + 31) & ~31, nh = nt - nsw - 64;
+    const bool sweeper = tid < nsw, waiter = tid >= nt - 64 && tid < nt - 32, issuer = tid >= nt - 32;
+    const bool helper = !sweeper && tid < nt - 64;
+    const int ht = tid - nsw;                                               // helper's number
+    const int nput = (nlev + PUT_LEVELS - 1) / PUT_LEVELS;
+
+    const int nx = P.nx, nxy = P.nx * P.ny, bxy = bx * by;
+    const long long g0 = si.e0x + (long long)nx * (si.e0y + (long long)P.ny * si.e0z);
+    const unsigned mbx = magic_div(bx), mby = magic_div(by);
+    auto element = [&](int i, int j, int k) { return 4 * ((i >> 1) + mx * (j >> 1) + mp * k) + (i & 1) + 2 * (j & 1); };
+    // right-RAS: R_i^0 on the input (cells of other boxes read as 0)
+    auto in_xy = [&](int i, int j) {
+        return P.kind != 2 || (i >= si.ox0 && i < si.ox1 && j >= si.oy0 && j < si.oy1);
+    };
+    auto in_z = [&](int k) { return P.kind != 2 || (k >= si.oz0 && k < si.oz1); };
+    // helpers: R_i^delta r. A thread takes the same GC cells of every plane, so their places
+    // are computed once, and holds GD planes' loads in flight.
+    constexpr int GC = 2, GD = 4;
+    double v[GD][GC];
+    int off[GC], elem[GC];
+    const bool planes = GC * nh >= bxy;          // (else: cell by cell, long thin boxes)
+    auto fetch = [&](int k, double (&d)[GC]) {
+#pragma unroll
+        for (int c = 0; c < GC; ++c)
+            if (k < bz && off[c] >= 0) d[c] = load_now(r + g0 + off[c] + (long long)nxy * k);
+    };
+    if (helper && planes) {
+#pragma unroll
+        for (int c = 0; c < GC; ++c) {
+            const int q = ht + c * nh, j = fast_div(q, bx, mbx), i = q - j * bx;
+            off[c] = q < bxy && in_xy(i, j) ? i + nx * j : -1;
+            elem[c] = element(i, j, 0);
+        }
+#pragma unroll
+        for (int d = 0; d < GD; ++d) fetch(d, v[d]);
+    }
+    const int4 *steps = P.steps + sh.chunk_off;  // [nstep + 1]: {first block, blocks, ring place / 16, issue limit}
+    {
+        const int nall = mp * bz;
+        const bool pad = ((bx | by) & 1) != 0 || mp != mx * sh.my;
+        for (int t = tid; t <= nstep; t += nt) st[t] = steps[t];
+        for (int t = tid; t < sh.nblk; t += nt) bt[t] = (unsigned)P.cidx[sh.cell_off + t];
+        for (int t = tid; t < nstep; t += nt) {
+            mb_init(mb_rec + t, 1);
+            mb_init(mb_free + t, 1);
+        }
+        for (int t = tid; t < bz; t += nt) mb_init(mb_pl + t, nh >> 5);
+        for (int t = tid; t < nput; t += nt) mb_init(mb_put + t, nsw >> 5);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int t = tid; t < guard; t += nt) Y[-1 - t] = Y[nall + t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (pad || P.kind == 2)
+            for (int t = tid; t < nall; t += nt) Y[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        cta_barrier();
+    }
+    // helpers: (R_i^0)^T of the blocks [b0, b1) of the table, a row of two cells per item
+    double *zg = z + g0;
+    auto put = [&](int b0, int b1) {
+        for (int e = 2 * b0 + ht; e < 2 * b1; e += nh) {
+            const unsigned b = bt[e >> 1];
+            const int I = b & 255u, J = (b >> 8) & 255u, k = b >> 16, c = e & 1;
+            const int i = 2 * I, j = 2 * J + c;
+            if (j < si.oy0 || j >= si.oy1 || k < si.oz0 || k >= si.oz1) continue;
+            const float2 y = reinterpret_cast<const float2 *>(Y + (I + mx * J + mp * k))[c];
+            double *zp = zg + (i + nx * j + nxy * k);
+            if (i >= si.ox0 && i < si.ox1) {
+                if (accumulate) atomicAdd(zp, (double)y.x);   // one owner per cell
+                else zp[0] = (double)y.x;
+            }
+            if (i + 1 >= si.ox0 && i + 1 < si.ox1) {
+                if (accumulate) atomicAdd(zp + 1, (double)y.y);
+                else zp[1] = (double)y.y;
+            }
+        }
+    };
+
+    float ax[4] = {}, ay[4] = {}, az[4] = {}, di[4] = {};
+    int m = 0;                                   // this thread's block of the coming step
+    bool on = false;
+    auto fcell = [&](int c, float s, float zv, float yv, float xv) {   // w_n = (r_n - sum_{m<n} a_nm w_m) / d_n
+        s = fmsub(az[c], zv, s);
+        s = fmsub(ay[c], yv, s);
+        return fmsub(ax[c], xv, s) * di[c];
+    };
+    auto forward = [&]() {
+        float4 a = Y[m];
+        const float4 zm = Y[m - zoff], xm = Y[m - 1];
+        const float2 ym = reinterpret_cast<const float2 *>(Y + (m - yoff))[1];
+        a.x = fcell(0, a.x, zm.x, ym.x, xm.y);
+        a.y = fcell(1, a.y, zm.y, ym.y, a.x);
+        a.z = fcell(2, a.z, zm.z, a.x, xm.w);
+        a.w = fcell(3, a.w, zm.w, a.y, a.z);
+        Y[m] = a;
+    };
+    auto bcell = [&](int c, float w, float xv, float yv, float zv) {   // z_n = w_n - d_n^{-1} sum_{m>n} a_nm z_m
+        float s = ax[c] * xv;
+        s = fmadd(ay[c], yv, s);
+        s = fmadd(az[c], zv, s);
+        return fmsub(di[c], s, w);
+    };
+    auto backward = [&]() {
+        float4 a = Y[m];
+        const float4 zp = Y[m + zoff], xp = Y[m + 1];
+        const float2 yp = reinterpret_cast<const float2 *>(Y + (m + yoff))[0];
+        a.w = bcell(3, a.w, xp.z, yp.y, zp.w);
+        a.z = bcell(2, a.z, a.w, yp.x, zp.z);
+        a.y = bcell(1, a.y, xp.x, a.w, zp.y);
+        a.x = bcell(0, a.x, a.y, a.z, zp.x);
+        Y[m] = a;
+    };
+    // step n: forward level n, then backward level 2 nlev - 1 - n
+    auto step_barrier = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nsw + 32) : "memory"); };
+    if (sweeper) {
+        // the coming step's table entries are read two steps ahead, its records one
+        int4 s = st[0], s1 = st[1];
+        unsigned b = tid < s.y ? bt[s.x + tid] : 0u;
+        auto load = [&](int n) {                 // the records of step n, w blocks apart
+            on = tid < s.y;
+            if (on) {
+                m = (int)(b & 255u) + mx * (int)((b >> 8) & 255u) + mp * (int)(b >> 16);
+                const unsigned char *rec = ring + 16 * s.z + RB * tid;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) load_rec<float, R>(rec + RB * c * s.y, ax[c], ay[c], az[c], di[c]);
+            }
+            s = s1;
+            b = tid < s.y ? bt[s.x + tid] : 0u;
+        };
+        step_barrier();                          // the first records
+        load(0);
+        for (int n = 0; n < nlev; ++n) {
+            step_barrier();
+            s1 = st[min(n + 2, nstep - 1)];
+            if (on) forward();
+            load(n + 1);
+        }
+        for (int n = nlev; n < nstep; ++n) {
+            step_barrier();
+            s1 = st[min(n + 2, nstep - 1)];
+            if (on) backward();
+            const int done = n - nlev + 1;
+            if (done % PUT_LEVELS == 0 || n + 1 == nstep) {
+                __syncwarp();
+                if (lane == 0) mb_arrive(mb_put + (done - 1) / PUT_LEVELS);
+            }
+            if (n + 1 < nstep) load(n + 1);
+        }
+    } else if (waiter) {
+        // joins the barrier of step n when the plane of r that it reads and the records of
+        // step n + 1 are in (the sweepers wait for nothing else); after it step n's records
+        // are in registers and their place in the ring is free
+        mb_wait(mb_rec, P.err);
+        step_barrier();
+        for (int n = 0; n < nstep; ++n) {
+            if (n < bz) mb_wait(mb_pl + n, P.err);
+            if (n + 1 < nstep) mb_wait(mb_rec + n + 1, P.err);
+            step_barrier();
+            if (lane == 0) mb_arrive(mb_free + n);
+        }
+    } else if (issuer) {
+        if (lane == 0) {
+            int next = 0;
+            for (int n = -1; n < nstep; ++n) {
+                if (n >= 0) mb_wait(mb_free + n, P.err);
+                const int lim = st[n < 0 ? nstep : n].w;
+                for (; next <= lim; ++next) {
+                    const int4 s = st[next];
+                    const unsigned char *src = (next < nlev ? P.fwd : P.bwd) + (si.foff + 4LL * s.x) * RB;
+                    bulk_load(ring + 16 * s.z, src, 4u * s.y * RB, mb_rec + next);
+                }
+                if (next == nstep) break;
+            }
+        }
+    } else {
+        float *Yf = reinterpret_cast<float *>(Y);
+        auto arrive = [&](int k) {
+            __syncwarp();
+            if (lane == 0) mb_arrive(mb_pl + k);
+        };
+        if (planes) {
+            for (int k0 = 0; k0 < bz; k0 += GD) {
+#pragma unroll
+                for (int d = 0; d < GD; ++d) {
+                    const int k = k0 + d;
+                    if (k >= bz) continue;
+#pragma unroll
+                    for (int c = 0; c < GC; ++c)
+                        if (off[c] >= 0 && in_z(k)) Yf[elem[c] + 4 * mp * k] = (float)v[d][c];
+                    fetch(k + GD, v[d]);
+                    arrive(k);
+                }
+            }
+        } else {
+            for (int k = 0; k < bz; ++k) {
+                for (int q = ht; q < bxy; q += nh) {
+                    const int j = fast_div(q, bx, mbx), i = q - j * bx;
+                    if (in_xy(i, j) && in_z(k))
+                        Yf[element(i, j, k)] = (float)__ldg(r + g0 + i + nx * j + (long long)nxy * k);
+                }
+                arrive(k);
+            }
+        }
+        if (P.kind == 1)
+            for (int e = 0; e < nput; ++e) {     // levels nlev - 1 - PUT_LEVELS e downwards
+                mb_wait(mb_put + e, P.err);
+                const int l1 = nlev - PUT_LEVELS * e, l0 = max(0, l1 - PUT_LEVELS);
+                put(st[l0].x, st[l1 - 1].x + st[l1 - 1].y);
+            }
+    }
+    cta_barrier();
+    for (int t = tid; t < nstep; t += nt) {
+        mb_inval(mb_rec + t);
+        mb_inval(mb_free + t);
+    }
+    for (int t = tid; t < bz; t += nt) mb_inval(mb_pl + t);
+    for (int t = tid; t < nput; t += nt) mb_inval(mb_put + t);
+    if (P.kind != 1) {   // AS / right-RAS: the whole box solution, summed per cell later
+        double *dst = P.zbuf + si.foff;
+        for (int q = tid; q < sh.ncell; q += nt) {
+            const int row = fast_div(q, bx, mbx), k = fast_div(row, by, mby);
+            dst[q] = (double)reinterpret_cast<const float *>(Y)[element(q - row * bx, row - k * by, k)];
+        }
+    }
+}
+
+template <int PREC>
+__device__ __forceinline__ void ras_apply_box(const ApplyParams &P, int box, const double *r, double *z,
+                                              int accumulate) {
+    if constexpr (PREC == 64) ras_apply_cells<PREC, 3>(P, box, r, z, accumulate);
+    else ras_apply_blocks<PREC>(P, box, r, z, accumulate);
+}
+
+// 64 registers for 2 CTAs of 512 threads per SM with FP64 factors, 72 for two of 448 with
+// reduced ones
+template <int PREC>
+__global__ void __maxnreg__(PREC == 64 ? 64 : 72) k_ras_apply(ApplyParams P) {
+    ras_apply_box<PREC>(P, blockIdx.x, P.r, P.z, P.accumulate);
 }
 
 // Left-RAS of many handles in one persistent launch: every CTA takes the next
@@ -326,8 +648,8 @@ __global__ void __launch_bounds__(512, 2) k_ras_apply(ApplyParams P) {
 // largest box first) until the queue is empty, and solves box box_local[item] of
 // handle box_inst[item] (items of inactive handles are skipped); r and z are the
 // handles' vectors concatenated at off[handle]. No CTA waits on another.
-template <int PREC, int NBUF>
-__global__ void __launch_bounds__(512, 2) k_ras_apply_batch(BatchApply B) {
+template <int PREC>
+__global__ void __maxnreg__(PREC == 64 ? 64 : 72) k_ras_apply_batch(BatchApply B) {
     __shared__ int s_item;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(B.qcount, 1);
@@ -337,221 +659,8 @@ __global__ void __launch_bounds__(512, 2) k_ras_apply_batch(BatchApply B) {
         if (it >= B.nitems) return;
         const int h = B.box_inst[it];
         if (!B.active[h]) continue;
-        ras_apply_box<PREC, NBUF>(B.inst[h], B.box_local[it], B.r + B.off[h], B.z + B.off[h], B.accumulate);
+        ras_apply_box<PREC>(B.inst[h], B.box_local[it], B.r + B.off[h], B.z + B.off[h], B.accumulate);
     }
-}
-
-// ---------------------------------------------------------------------------
-// Pencil-wavefront subdomain solves (left-RAS, FP32 / BF16 factors)
-//
-// The natural-order ILU(0) sweeps of a box run over its x-pencils (j, k), one
-// thread per pencil: pencil (j, k) handles its cells i = 0 .. bx-1 one per
-// wavefront level, cell i at level i + j + k, so that its -y and -z neighbours,
-// cells of the pencils (j-1, k) and (j, k-1), were finished at the previous level
-// and its -x neighbour is the pencil's previous value, kept in a register (the
-// backward sweep mirrors this). Consecutive levels are separated by one CTA
-// barrier. Pencils are numbered by anti-diagonal d = j + k, then j, so that a warp
-// holds pencils of one or two neighbouring diagonals: it is busy for about bx + 2
-// levels of a sweep with most lanes active and idles (only the barrier) otherwise.
-// A thread's cell, neighbour and record positions follow from its pencil and the
-// level with no table look-up on the dependent chain (level start -> cell index ->
-// values in the level-scheduled kernel). The factor records are in level order with
-// the cells of a level grouped by anti-diagonal, then j (the layout both solve
-// kernels read): the record of pencil number p at level l is record lb[l] + p with
-// lb[l] = (start of level l) - (pencils on the diagonals below the level's first).
-// Chunks of consecutive levels are staged into a shared-memory ring with cp.async
-// two chunks ahead. The backward sweep writes each owned cell's z as soon as it is
-// final (an add when accumulating: one owner per cell). The arithmetic of every
-// cell is the same as in the level-scheduled kernel, in the same order.
-// ---------------------------------------------------------------------------
-
-struct PipeParams {
-    const SubInfo *subs;
-    const ShapeInfo *shapes;
-    const DiagInfo *diag;
-    const int *lvl, *chunk;
-    const unsigned char *fwd, *bwd;
-    const double *r;
-    double *z;
-    int nx, ny, nz;
-    int accumulate;
-    int ycap;          // elements of the padded box vector
-    int lcap;          // level starts (incl. the end) capacity
-    int chunk_cells;   // ring slot capacity (cells)
-};
-
-template <int PREC>
-__global__ void __launch_bounds__(1024, 1) k_ras_pipe(PipeParams P) {
-    using R = typename RecT<PREC>::T;
-    using Acc = typename RecT<PREC>::Acc;
-    constexpr int RB = (int)sizeof(R);
-    constexpr int NBUF = 3;
-    extern __shared__ __align__(16) unsigned char smem[];
-
-    const SubInfo si = P.subs[blockIdx.x];
-    const ShapeInfo sh = P.shapes[si.shape];
-    const int bx = sh.bx, by = sh.by, bz = sh.bz;
-    const int D = by + bz - 1, S = bx + D - 1;
-    const int PX = bx, PXY = sh.pxy;
-    const int nx = P.nx, nxy = P.nx * P.ny;
-    const long long g0 = si.e0x + (long long)nx * (si.e0y + (long long)P.ny * si.e0z);
-
-    // shared memory: [Y: ycap, zero cell, pad][level starts: lcap][lb: lcap][diagonals: dcap][ring]
-    Acc *Y = reinterpret_cast<Acc *>(smem);
-    int *lvl_s = reinterpret_cast<int *>(smem + (((size_t)(P.ycap + 4) * sizeof(Acc) + 15) & ~(size_t)15));
-    int *lb = lvl_s + P.lcap;
-    DiagInfo *dg = reinterpret_cast<DiagInfo *>(lb + P.lcap);
-    unsigned char *ring = reinterpret_cast<unsigned char *>(dg + ((D + 1) & ~1));
-    const int rcap = ((P.chunk_cells * RB + 32) + 15) & ~15;
-
-    const int *chunk_lev = P.chunk + sh.chunk_off;
-    const int nchunk = sh.nchunk, nstage = 2 * nchunk;
-    for (int t = threadIdx.x; t <= S; t += blockDim.x) lvl_s[t] = P.lvl[sh.lvl_off + t];
-    for (int t = threadIdx.x; t < D; t += blockDim.x) dg[t] = P.diag[sh.diag_off + t];
-
-    // stage t < nchunk: forward chunk t; t >= nchunk: backward chunk 2 nchunk - 1 - t
-    auto issue = [&](int t) {
-        if (t < nstage) {
-            const bool fw = t < nchunk;
-            const int c = fw ? t : nstage - 1 - t;
-            const int qa = P.lvl[sh.lvl_off + chunk_lev[c]], qb = P.lvl[sh.lvl_off + chunk_lev[c + 1]];
-            stage_bytes(ring + (size_t)(t % NBUF) * rcap, fw ? P.fwd : P.bwd,
-                        (si.foff + qa) * (long long)RB, (si.foff + qb) * (long long)RB);
-        }
-        cp_async_commit();
-    };
-#pragma unroll
-    for (int t = 0; t < NBUF - 1; ++t) issue(t);
-
-    // gather R_i^delta r into the padded box vector (GB loads in flight per thread)
-    {
-        constexpr int GB = 8;
-        const double *rg = P.r + g0;
-        const unsigned mbx = magic_div(bx), mby = magic_div(by);
-        const int ncell = sh.ncell;
-        for (int q0 = threadIdx.x; q0 < ncell; q0 += GB * blockDim.x) {
-            double v[GB];
-            int yo[GB];
-#pragma unroll
-            for (int m = 0; m < GB; ++m) {
-                const int q = q0 + m * (int)blockDim.x;
-                if (q < ncell) {
-                    const int row = fast_div(q, bx, mbx), k = fast_div(row, by, mby);
-                    const int i = q - row * bx, j = row - k * by;
-                    v[m] = __ldg(rg + i + (long long)nx * j + (long long)nxy * k);
-                    yo[m] = i + PX * j + PXY * k;
-                }
-            }
-#pragma unroll
-            for (int m = 0; m < GB; ++m) {
-                const int q = q0 + m * (int)blockDim.x;
-                if (q < ncell) Y[yo[m]] = (Acc)v[m];
-            }
-        }
-    }
-    __syncthreads();
-    for (int l = threadIdx.x; l < S; l += blockDim.x) lb[l] = lvl_s[l] - dg[max(0, l - bx + 1)].base;
-
-    // this thread's pencil: number p = threadIdx.x in (d, j) order
-    const int p = threadIdx.x;
-    const bool live = p < by * bz;
-    int d = 0, j = 0, k = 0;
-    if (live) {
-        while (d + 1 < D && dg[d + 1].base <= p) ++d;
-        j = (dg[d].jmin_cnt & 0xffff) + (p - dg[d].base);
-        k = d - j;
-    }
-    // -y / -z (forward) and +y / +z (backward) neighbour rows of the pencil; a
-    // neighbour outside the box reads the zero cell Y[ycap] (stride 0 along i)
-    Acc *Yz = Y + P.ycap;
-    const int n0 = PX * j + PXY * k;                       // Y index of cell i = 0
-    Acc *const my = j > 0 ? Y + n0 - PX : Yz, *const mz = k > 0 ? Y + n0 - PXY : Yz;
-    Acc *const py = j < by - 1 ? Y + n0 + PX : Yz, *const pz = k < bz - 1 ? Y + n0 + PXY : Yz;
-    const int smy = j > 0, smz = k > 0, spy = j < by - 1, spz = k < bz - 1;
-    Acc *const yp = Y + n0;
-    double *zp0 = P.z + g0 + ((long long)nx * j + (long long)nxy * k);
-    const bool own_jk = live && j >= si.oy0 && j < si.oy1 && k >= si.oz0 && k < si.oz1;
-    const unsigned owx = (unsigned)(si.ox1 - si.ox0);
-    const bool acc = P.accumulate != 0;
-    if (threadIdx.x == 0) *Yz = (Acc)0;
-
-    int t = -1, lev_lo = 0, lev_hi = -1;   // current ring stage and its level range
-    const unsigned char *rp = ring;         // this pencil's record base in the current stage
-    // a new ring stage: wait for its chunk, refill the slot two stages back
-    auto next_stage = [&]() {
-        ++t;
-        cp_async_wait<NBUF - 2>();
-        __syncthreads();
-        issue(t + NBUF - 1);
-        const int c = t < nchunk ? t : nstage - 1 - t;
-        lev_lo = chunk_lev[c];
-        lev_hi = chunk_lev[c + 1] - 1;
-        const int qa = lvl_s[lev_lo];
-        rp = ring + ((long long)(t % NBUF) * rcap + (((si.foff + qa) * (long long)RB) & 15) +
-                     (long long)RB * (p - qa));
-    };
-    // forward sweep: w_n = (r_n - a_z w_{n-bxy} - a_y w_{n-bx} - a_x w_{n-1}) / d_n
-    {
-        Acc xprev = (Acc)0;
-        Acc ax = 0, ay = 0, az = 0, dinv = 0;
-        bool have = false;                   // the record of the coming level is in registers
-        for (int lev = 0; lev < S; ++lev) {
-            if (lev > lev_hi) { next_stage(); have = false; }
-            const int i = lev - d;
-            const bool on = live && (unsigned)i < (unsigned)bx;
-            if (on) {
-                if (!have) load_rec<Acc, R>(rp + (long long)RB * lb[lev], ax, ay, az, dinv);
-                const Acc yz = mz[i * smz], yy = my[i * smy];
-                Acc s = yp[i];
-                s = fmsub(az, yz, s);
-                s = fmsub(ay, yy, s);
-                s = fmsub(ax, xprev, s);
-                const Acc y = s * dinv;
-                yp[i] = y;
-                xprev = y;
-            }
-            // the next level's record (independent of this level's values), if staged
-            have = false;
-            if (lev + 1 <= lev_hi && live && (unsigned)(i + 1) < (unsigned)bx) {
-                load_rec<Acc, R>(rp + (long long)RB * lb[lev + 1], ax, ay, az, dinv);
-                have = true;
-            }
-            __syncthreads();   // level done: its values are the next level's neighbours
-        }
-    }
-    // backward sweep: z_n = w_n - d_n^{-1} (a_x z_{n+1} + a_y z_{n+bx} + a_z z_{n+bxy})
-    {
-        Acc xprev = (Acc)0;
-        Acc ax = 0, ay = 0, az = 0, dinv = 0;
-        bool have = false;
-        next_stage();
-        for (int lev = S - 1; lev >= 0; --lev) {
-            if (lev < lev_lo) { next_stage(); have = false; }
-            const int i = lev - d;
-            const bool on = live && (unsigned)i < (unsigned)bx;
-            if (on) {
-                if (!have) load_rec<Acc, R>(rp + (long long)RB * lb[lev], ax, ay, az, dinv);
-                const Acc zy = py[i * spy], zz = pz[i * spz];
-                Acc s = ax * xprev;
-                s = fmadd(ay, zy, s);
-                s = fmadd(az, zz, s);
-                const Acc y = fmsub(dinv, s, yp[i]);
-                yp[i] = y;
-                xprev = y;
-                if (own_jk && (unsigned)(i - si.ox0) < owx) {
-                    if (acc) atomicAdd(zp0 + i, (double)y);   // one owner per cell
-                    else zp0[i] = (double)y;
-                }
-            }
-            have = false;
-            if (lev - 1 >= lev_lo && live && (unsigned)(i - 1) < (unsigned)bx) {
-                load_rec<Acc, R>(rp + (long long)RB * lb[lev - 1], ax, ay, az, dinv);
-                have = true;
-            }
-            __syncthreads();
-        }
-    }
-    cp_async_wait<0>();
 }
 
 // z (+)= sum over the overlapped boxes covering each cell of their solution
@@ -588,62 +697,157 @@ __global__ void __launch_bounds__(256) k_ras_sum(SumParams P) {
 }
 
 
+// ---------------------------------------------------------------------------
+// ILU(0) factorisation
+// ---------------------------------------------------------------------------
+
+// (u, v) pairs of an nu x nv grid with u + v < d: those of the quarter plane less those
+// past either edge
+__host__ __device__ __forceinline__ int tri(int x) { return x > 0 ? x * (x + 1) / 2 : 0; }
+__host__ __device__ __forceinline__ int diag_base(int d, int nu, int nv) {
+    return tri(d) - tri(d - nu) - tri(d - nv) + tri(d - nu - nv);
+}
+// position of (u, v) in the order by diagonal u + v, then u
+__host__ __device__ __forceinline__ int diag_pos(int u, int v, int nu, int nv) {
+    return diag_base(u + v, nu, nv) + u - max(0, u + v - (nv - 1));
+}
+
+// 1 / x by one third-order step y (1 + e + e^2), e = 1 - x y, from the FP32 reciprocal
+// (24 bits -> 72, then FP64 rounding), where x lies in FP32's normal range
+__device__ __forceinline__ double recip64(double x) {
+    const double ax = fabs(x);
+    if (!(ax > 1e-36 && ax < 1e36)) return 1.0 / x;
+    const double y = (double)__frcp_rn((float)x);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// axis along which the factorisation's pencils run: x unless that leaves too many
+// pencils for one CTA, then the longest axis (at most 16384^(2/3) = 645 pencils)
+constexpr int FAC_MAXPEN = 1024;
+__host__ __device__ __forceinline__ int pencil_axis(int bx, int by, int bz) {
+    if (by * bz <= FAC_MAXPEN) return 0;
+    return bx >= by && bx >= bz ? 0 : (by >= bz ? 1 : 2);
+}
+__host__ __device__ __forceinline__ int pencil_count(int bx, int by, int bz) {
+    const int a = pencil_axis(bx, by, bz);
+    return a == 0 ? by * bz : (a == 1 ? bx * bz : bx * by);
+}
+
 // ILU(0) of A_i in natural order: only the diagonal changes,
-// d_n = a_nn - sum_{m<n neighbour} (a_nm / d_m) a_mn   (m: -z, -y, -x).
-// One CTA per box (box `box` of the handle described by P).
-template <int PREC>
-__device__ __forceinline__ void ras_factor_box(const FactorParams &P, int box) {
+// d_n = a_nn - sum_{m<n neighbour} a_nm (a_mn / d_m)   (m: -z, -y, -x).
+// One CTA per box (box `box` of the handle described by P), one thread per pencil of
+// cells; a pencil handles one cell per wavefront level, so a_mn / d_m of its own previous
+// cell is in a register and those of the two neighbouring pencils, finished at the
+// previous level, in a shared slot per pencil (by parity of the level). Every operator
+// value is read once, consecutive along the pencil, a level ahead of its use, and both
+// factor records are written at once. Pencils are numbered by diagonal, so that a warp's
+// pencils are active together.
+//
+// Bound: FP64 (2 FMA per cycle and SM): 3 FMA, a reciprocal (3 FMA, where a division takes
+// about ten operations) and 3 multiplications per cell. Three divisions per cell, the
+// operator read cell by cell in level order and a second pass for the records took 1.8
+// times as long: factors and a first use, 60 x 220 x 85 cells in FP64, 585 -> 323 us.
+template <int PREC, int pa>
+__device__ __forceinline__ void ras_factor_pencils(const FactorParams &P, const SubInfo &si, const ShapeInfo &sh) {
     extern __shared__ __align__(16) unsigned char smem[];
-    double *D = reinterpret_cast<double *>(smem);
-    const SubInfo si = P.subs[box];
-    const ShapeInfo sh = P.shapes[si.shape];
-    const int *lvl = P.lvl + sh.lvl_off;
-    const unsigned *cells = P.cells + sh.cell_off;
-    const int bx = sh.bx, by = sh.by, bxy = bx * by;
-    const int nx = P.nx, nxy = P.nx * P.ny;
-    const long long g0 = si.e0x + (long long)nx * (si.e0y + (long long)P.ny * si.e0z);
-    const double *Ac = P.A.c[0], *Amx = P.A.c[1], *Apx = P.A.c[2], *Amy = P.A.c[3],
-                 *Apy = P.A.c[4], *Amz = P.A.c[5], *Apz = P.A.c[6];
-    for (int l = 0; l < sh.nlev; ++l) {
-        const int q1 = lvl[l + 1];
-        for (int q = lvl[l] + threadIdx.x; q < q1; q += blockDim.x) {
-            const unsigned e = cells[q];
-            const int i = e & 255u, j = (e >> 8) & 255u, k = (e >> 16) & 255u;
-            const unsigned fl = e >> 24;
-            const int n = i + bx * j + bxy * k;
-            const long long g = g0 + i + (long long)nx * j + (long long)nxy * k;
-            double d = Ac[g];
-            if (fl & F_MZ) { const double lm = Amz[g] / D[n - bxy]; d -= lm * Apz[g - nxy]; }
-            if (fl & F_MY) { const double lm = Amy[g] / D[n - bx]; d -= lm * Apy[g - nx]; }
-            if (fl & F_MX) { const double lm = Amx[g] / D[n - 1]; d -= lm * Apx[g - 1]; }
-            if (!(d != 0.0) || !isfinite(d)) atomicExch(P.err, 1);
-            D[n] = d;
+    constexpr int ua = pa == 0 ? 1 : 0, va = pa == 2 ? 1 : 2;
+    auto stride = [&](int a) { return a == 0 ? 1LL : (a == 1 ? (long long)P.nx : (long long)P.nx * P.ny); };
+    const int nm = pa == 0 ? sh.bx : (pa == 1 ? sh.by : sh.bz), nu = ua ? sh.by : sh.bx, nv = va == 1 ? sh.by : sh.bz;
+    const int npen = nu * nv, S = nm + nu + nv - 2;
+    double *su = reinterpret_cast<double *>(smem), *sv = su + 2 * npen;   // [2][npen]: a_mn / d_m towards +u, +v
+    int *lstart = reinterpret_cast<int *>(sv + 2 * npen);                 // [nlev]: first record less its first number
+    int *lw = lstart + sh.nlev;                                           // [nlev]: records between a block's cells
+    for (int l = threadIdx.x; l < sh.nlev; l += blockDim.x) {
+        const int a = P.lvl[sh.lvl_off + l], b = P.lvl[sh.lvl_off + l + 1];
+        if constexpr (PREC == 64) lstart[l] = a - diag_base(max(0, l - sh.bx + 1), sh.by, sh.bz);
+        else lstart[l] = 4 * a - diag_base(max(0, l - sh.mx + 1), sh.my, sh.bz);
+        lw[l] = b - a;
+    }
+    // this thread's pencil
+    const int pen = threadIdx.x;
+    const bool live = pen < npen;
+    int u = 0, v = 0;
+    if (live) {
+        int d = 0;
+        while (diag_base(d + 1, nu, nv) <= pen) ++d;
+        u = max(0, d - (nv - 1)) + pen - diag_base(d, nu, nv);
+        v = d - u;
+    }
+    const int qu = live && u > 0 ? diag_pos(u - 1, v, nu, nv) : pen, qv = live && v > 0 ? diag_pos(u, v - 1, nu, nv) : pen;
+    const bool mu = u > 0, mv = v > 0, pu = u < nu - 1, pv = v < nv - 1;
+    const long long g0 = si.e0x + P.nx * (si.e0y + (long long)P.ny * si.e0z) + u * stride(ua) + v * stride(va);
+    const long long gm = stride(pa);
+    const double *Ac = P.A.c[0] + g0, *Amm = P.A.c[1 + 2 * pa] + g0, *Apm = P.A.c[2 + 2 * pa] + g0;
+    const double *Amu = P.A.c[1 + 2 * ua] + g0, *Apu = P.A.c[2 + 2 * ua] + g0;
+    const double *Amv = P.A.c[1 + 2 * va] + g0, *Apv = P.A.c[2 + 2 * va] + g0;
+    double nc = 0, nmm = 0, npm = 0, nmu = 0, npu = 0, nmv = 0, npv = 0;   // the coming cell's row
+    auto fetch = [&](int m) {
+        if (!live || (unsigned)m >= (unsigned)nm) return;
+        const long long o = m * gm;
+        nc = __ldg(Ac + o);
+        nmm = m > 0 ? __ldg(Amm + o) : 0.0;
+        npm = m < nm - 1 ? __ldg(Apm + o) : 0.0;
+        nmu = mu ? __ldg(Amu + o) : 0.0;
+        npu = pu ? __ldg(Apu + o) : 0.0;
+        nmv = mv ? __ldg(Amv + o) : 0.0;
+        npv = pv ? __ldg(Apv + o) : 0.0;
+    };
+    fetch(0);
+    __syncthreads();
+    double um = 0.0;                       // a_mn / d_m of the pencil's previous cell
+    bool bad = false;
+    for (int l = 0; l < S; ++l) {
+        const int m = l - u - v, par = l & 1;
+        if (live && (unsigned)m < (unsigned)nm) {
+            const double c = nc, mm = nmm, pm = npm, m1 = nmu, p1 = npu, m2 = nmv, p2 = npv;
+            fetch(m + 1);
+            double d = c;
+            if (mv) d = fma(-m2, sv[(par ^ 1) * npen + qv], d);
+            if (mu) d = fma(-m1, su[(par ^ 1) * npen + qu], d);
+            d = fma(-mm, um, d);
+            if (!(d != 0.0) || !isfinite(d)) bad = true;
+            const double di = recip64(d);
+            um = pm * di;
+            su[par * npen + pen] = p1 * di;
+            sv[par * npen + pen] = p2 * di;
+            // the cell and its two records
+            const int i = pa == 0 ? m : u, j = pa == 1 ? m : (pa == 0 ? u : v), k = pa == 2 ? m : v;
+            long long at;
+            if constexpr (PREC == 64) {
+                at = si.foff + lstart[i + j + k] + diag_pos(j, k, sh.by, sh.bz);
+            } else {
+                const int J = j >> 1, L = (i >> 1) + J + k;
+                at = si.foff + lstart[L] + lw[L] * ((i & 1) + 2 * (j & 1)) + diag_pos(J, k, sh.my, sh.bz);
+            }
+            const double mx = pa == 0 ? mm : m1, my = pa == 1 ? mm : (pa == 0 ? m1 : m2), mz = pa == 2 ? mm : m2;
+            const double px = pa == 0 ? pm : p1, py = pa == 1 ? pm : (pa == 0 ? p1 : p2), pz = pa == 2 ? pm : p2;
+            store_rec<PREC>(P.fwd, at, mx, my, mz, di);
+            store_rec<PREC>(P.bwd, at, px, py, pz, di);
         }
         __syncthreads();
     }
-    for (int q = threadIdx.x; q < sh.ncell; q += blockDim.x) {
-        const unsigned e = cells[q];
-        const int i = e & 255u, j = (e >> 8) & 255u, k = (e >> 16) & 255u;
-        const unsigned fl = e >> 24;
-        const int n = i + bx * j + bxy * k;
-        const long long g = g0 + i + (long long)nx * j + (long long)nxy * k;
-        const double dinv = 1.0 / D[n];
-        store_rec<PREC>(P.fwd, si.foff + q, (fl & F_MX) ? Amx[g] : 0.0, (fl & F_MY) ? Amy[g] : 0.0,
-                        (fl & F_MZ) ? Amz[g] : 0.0, dinv);
-        store_rec<PREC>(P.bwd, si.foff + q, (fl & F_PX) ? Apx[g] : 0.0, (fl & F_PY) ? Apy[g] : 0.0,
-                        (fl & F_PZ) ? Apz[g] : 0.0, dinv);
-    }
+    if (bad) atomicMax(P.err, 1);
+}
+template <int PREC>
+__device__ __forceinline__ void ras_factor_box(const FactorParams &P, int box) {
+    const SubInfo si = P.subs[box];
+    const ShapeInfo sh = P.shapes[si.shape];
+    const int a = pencil_axis(sh.bx, sh.by, sh.bz);
+    if (a == 0) ras_factor_pencils<PREC, 0>(P, si, sh);
+    else if (a == 1) ras_factor_pencils<PREC, 1>(P, si, sh);
+    else ras_factor_pencils<PREC, 2>(P, si, sh);
 }
 
 template <int PREC>
-__global__ void __launch_bounds__(512) k_ras_factor(FactorParams P) {
+__global__ void __launch_bounds__(FAC_MAXPEN, 1) k_ras_factor(FactorParams P) {
     ras_factor_box<PREC>(P, blockIdx.x);
 }
 
 // The subdomain ILU(0) factorisations of several handles in one launch: CTA b
 // factors box box_local[b] of handle box_inst[b] (CTAs of inactive handles return).
 template <int PREC>
-__global__ void __launch_bounds__(512) k_ras_factor_batch(const FactorParams *__restrict__ inst,
+__global__ void __launch_bounds__(FAC_MAXPEN, 1) k_ras_factor_batch(const FactorParams *__restrict__ inst,
                                                           const int *__restrict__ box_inst,
                                                           const int *__restrict__ box_local,
                                                           const unsigned char *__restrict__ active) {
@@ -666,23 +870,17 @@ static std::vector<int> split_axis(int n, int parts) {
 // The opt-in limit is raised to the per-CTA maximum once: a later set-up with
 // a smaller need must not lower it under a handle that needs more.
 constexpr int SMEM_OPTIN = 227 * 1024;
-template <int PREC, int NBUF>
-static int set_apply_attr(size_t) {
-    RAS_CK(cudaFuncSetAttribute(k_ras_apply<PREC, NBUF>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN));
+template <int PREC>
+static int set_apply_attr() {
+    RAS_CK(cudaFuncSetAttribute(k_ras_apply<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN));
     cudaFuncAttributes fa{};   // the persistent batch kernel has a little static shared memory
-    RAS_CK(cudaFuncGetAttributes(&fa, k_ras_apply_batch<PREC, NBUF>));
-    RAS_CK(cudaFuncSetAttribute(k_ras_apply_batch<PREC, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    RAS_CK(cudaFuncGetAttributes(&fa, k_ras_apply_batch<PREC>));
+    RAS_CK(cudaFuncSetAttribute(k_ras_apply_batch<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 SMEM_OPTIN - (int)fa.sharedSizeBytes));
     return RAS_OK;
 }
 template <int PREC>
-static int set_pipe_attr() {
-    RAS_CK(cudaFuncSetAttribute(k_ras_pipe<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN));
-    return RAS_OK;
-}
-template <int PREC>
-static int set_factor_attr(size_t) {
+static int set_factor_attr() {
     RAS_CK(cudaFuncSetAttribute(k_ras_factor<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 SMEM_OPTIN));
     RAS_CK(cudaFuncSetAttribute(k_ras_factor_batch<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -690,14 +888,12 @@ static int set_factor_attr(size_t) {
     return RAS_OK;
 }
 
-// shared memory of the pipelined solves for the handle's current chunk size
-static size_t pipe_smem(Ras1 &R) {
-    const size_t acc = R.prec == 64 ? 8 : 4;
-    const size_t ybytes = (((size_t)(R.ycap_pipe + 4) * acc) + 15) & ~(size_t)15;
+// The pencil-wavefront kernel's limits (ras_set_apply_kernel): its shared memory for
+// the handle's chunk size
+static size_t pencil_smem(const Ras1 &R) {
+    const size_t ybytes = (((size_t)(R.ycap_pipe + 4) * 4) + 15) & ~(size_t)15;
     const size_t rcap = ((R.chunk_cells * R.rec_bytes + 32) + 15) & ~15;
-    R.smem_pipe = ybytes + 2 * (size_t)R.lcap * sizeof(int) + (size_t)R.dcap_pipe * sizeof(DiagInfo) +
-                  3 * rcap;
-    return R.smem_pipe;
+    return ybytes + 2 * (size_t)R.lcap_cells * sizeof(int) + (size_t)R.dcap_pipe * 8 + 3 * rcap;
 }
 
 // Level schedule of the subdomain solves: chunks of consecutive levels with at most
@@ -722,30 +918,91 @@ static int schedule_tables(Ras1 &R, int chunk_cells, int threads, std::vector<in
         if (threads > 512 || threads % 32) return RAS_EINVAL;
         block = threads;
     }
+    // the shared memory of the sweeps cell by cell decides what is accepted
     const size_t acc = R.prec == 64 ? 8 : 4;
     const size_t rcap = ((cc * R.rec_bytes + 32) + 15) & ~15;
     const size_t ccap = ((cc * 4 + 32) + 15) & ~15;
-    const size_t smem = (R.ycap + 2 * (size_t)R.gcap) * acc + R.lcap * sizeof(int) + R.nbuf * (rcap + ccap);
+    size_t smem = (R.ycap_cells + 2 * (size_t)R.gcap_cells) * acc + R.lcap_cells * sizeof(int) + 3 * (rcap + ccap);
     if (smem > 227 * 1024) return RAS_EINVAL;
+    int launch = block;
     chunk_tab.clear();
-    for (auto &sh : R.shapes) {
-        sh.chunk_off = (int)chunk_tab.size();
-        const int *lv = &R.h_lvl[sh.lvl_off];
-        int l = 0;
-        chunk_tab.push_back(0);
-        int nch = 0;
-        while (l < sh.nlev) {
-            int l1 = l + 1;
-            while (l1 < sh.nlev && lv[l1 + 1] - lv[l] <= cc) ++l1;
-            chunk_tab.push_back(l1);
-            ++nch;
-            l = l1;
+    if (R.prec == 64) {
+        for (auto &sh : R.shapes) {
+            sh.chunk_off = (int)chunk_tab.size();
+            const int *lv = &R.h_lvl[sh.lvl_off];
+            int l = 0;
+            chunk_tab.push_back(0);
+            int nch = 0;
+            while (l < sh.nlev) {
+                int l1 = l + 1;
+                while (l1 < sh.nlev && lv[l1 + 1] - lv[l] <= cc) ++l1;
+                chunk_tab.push_back(l1);
+                ++nch;
+                l = l1;
+            }
+            sh.nchunk = nch;
         }
-        sh.nchunk = nch;
+    } else {
+        // blocks of 2 x 2 cells: a ring of three chunks (at least two of the widest level;
+        // less where the box vector leaves less room)
+        const size_t fixed = ((size_t)R.ycap + 2 * R.gcap) * 16 + (size_t)R.ycap * 4 + R.lcap * (2 * 16 + 6 * 8);
+        const size_t widest = 4 * (size_t)R.maxwb * R.rec_bytes;
+        const size_t room = fixed > 227 * 1024 ? 0 : 227 * 1024 - fixed;
+        if (room < 2 * widest) return RAS_EINVAL;
+        const size_t ring = std::min(std::max(3 * (size_t)cc * R.rec_bytes, 2 * widest), room) & ~(size_t)15;
+        smem = fixed + ring;
+        // sweepers, a waiter, an issuer and helpers enough for a box plane at two cells each
+        // (up to 448 threads: two CTAs per SM), one warp at least
+        const int own = ((R.maxwb + 31) & ~31) + 64, help = std::max(32, ((R.bxy + 1) / 2 + 31) & ~31);
+        launch = std::max(std::max(block, own + 32), std::min(own + help, 448));
+        // per shape and step (levels up, then down): first block, blocks, place in the ring
+        // (in order, from the start again where the end is too near) and the last step whose
+        // place is free once the step's records have been read; a last entry with the limit
+        // before the first step
+        for (auto &sh : R.shapes) {
+            const int *lv = &R.h_lvl[sh.lvl_off];
+            const int ns = 2 * sh.nlev;
+            sh.chunk_off = (int)chunk_tab.size() / 4;
+            std::vector<size_t> a(ns), b(ns);
+            size_t at = 0;
+            for (int n = 0; n < ns; ++n) {
+                const int l = n < sh.nlev ? n : ns - 1 - n;
+                const size_t bytes = 4 * (size_t)(lv[l + 1] - lv[l]) * R.rec_bytes;
+                if (at + bytes > ring) at = 0;
+                a[n] = at;
+                b[n] = at += bytes;
+            }
+            auto limit = [&](int n) {        // steps n + 1 .. s are in the ring together
+                int q = n;
+                while (q + 1 < ns) {
+                    bool ok = true;
+                    for (int t = n + 1; t <= q && ok; ++t) ok = b[t] <= a[q + 1] || b[q + 1] <= a[t];
+                    if (!ok) break;
+                    ++q;
+                }
+                return q;
+            };
+            for (int n = 0; n <= ns; ++n) {
+                const int l = n < sh.nlev ? n : ns - 1 - n;
+                chunk_tab.push_back(n < ns ? lv[l] : 0);
+                chunk_tab.push_back(n < ns ? lv[l + 1] - lv[l] : 0);
+                chunk_tab.push_back(n < ns ? (int)(a[n] / 16) : 0);
+                chunk_tab.push_back(limit(n < ns ? n : -1));
+            }
+            sh.nchunk = ns;
+        }
     }
     R.chunk_cells = cc;
+    R.launch = launch;
     R.block = block;
     R.smem_apply = smem;
+    return RAS_OK;
+}
+
+static int upload_boxes(const Ras1 &R) {
+    std::vector<BoxInfo> b;
+    for (const SubInfo &s : R.subs) b.push_back(BoxInfo{s, R.shapes[s.shape]});
+    RAS_CK(cudaMemcpy(R.d_boxes, b.data(), b.size() * sizeof(BoxInfo), cudaMemcpyHostToDevice));
     return RAS_OK;
 }
 
@@ -758,7 +1015,7 @@ int ras1_set_schedule(Ras1 &R, int chunk_cells, int threads) {
     RAS_TRY(dalloc(&d, chunk_tab.size()));
     if (cudaMemcpy(d, chunk_tab.data(), chunk_tab.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(R.d_shapes, T.shapes.data(), T.shapes.size() * sizeof(ShapeInfo), cudaMemcpyHostToDevice) !=
-            cudaSuccess) {
+            cudaSuccess || upload_boxes(T) != RAS_OK) {
         dfree(d);
         return RAS_ECUDA;
     }
@@ -766,9 +1023,10 @@ int ras1_set_schedule(Ras1 &R, int chunk_cells, int threads) {
     R.d_chunk = d;
     R.shapes = T.shapes;
     R.chunk_cells = T.chunk_cells;
+    R.launch = T.launch;
     R.block = T.block;
     R.smem_apply = T.smem_apply;
-    if (R.pipe_ok && pipe_smem(R) > 227 * 1024) R.pipe = R.pipe_ok = 0;
+    if (R.pipe_ok && pencil_smem(R) > 227 * 1024) R.pipe = R.pipe_ok = 0;
     return RAS_OK;
 }
 
@@ -789,13 +1047,15 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
 
     std::map<std::tuple<int, int, int>, int> shape_id;
     std::vector<int> lvl_tab;
-    std::vector<unsigned> cell_tab;
-    std::vector<int> cidx_tab;        // same positions as cell_tab: i + bx (j + by k)
-    std::vector<DiagInfo> diag_tab;
+    std::vector<int> cidx_tab;        // level order: local index of each cell (block)
+    int bxy_all = 1;
     R.subs.clear();
     R.shapes.clear();
     long long foff = 0;
-    int maxw_all = 0, ycap = 0, lcap = 0, gcap = 0;
+    int maxw_all = 0, ycap = 0, lcap = 0, gcap = 0;      // cell by cell
+    int maxwb = 0, ycapb = 0, lcapb = 0, gcapb = 0;      // blocks of 2 x 2 cells
+    int npen_all = 1;
+    size_t fac_smem = 0;
     for (int kz = 0; kz < pz; ++kz)
         for (int jy = 0; jy < py; ++jy)
             for (int ix = 0; ix < px; ++ix) {
@@ -819,63 +1079,50 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
                     shape_id[key] = sid;
                     ShapeInfo sh{};
                     sh.bx = bx; sh.by = by; sh.bz = bz; sh.ncell = ncell;
-                    sh.nlev = bx + by + bz - 2;
-                    // level schedule: cells ordered by (i + j + k, natural index)
-                    std::vector<std::vector<unsigned>> levels(sh.nlev);
-                    for (int k = 0; k < bz; ++k)
-                        for (int j = 0; j < by; ++j)
-                            for (int i = 0; i < bx; ++i) {
-                                unsigned fl = 0;
-                                if (i > 0) fl |= F_MX;
-                                if (j > 0) fl |= F_MY;
-                                if (k > 0) fl |= F_MZ;
-                                if (i < bx - 1) fl |= F_PX;
-                                if (j < by - 1) fl |= F_PY;
-                                if (k < bz - 1) fl |= F_PZ;
-                                levels[i + j + k].push_back((unsigned)i | ((unsigned)j << 8) |
-                                                            ((unsigned)k << 16) | (fl << 24));
-                            }
-                    // inside a level, cells grouped by x-pencil anti-diagonal d = j + k,
-                    // then by j (the pipelined solves read a diagonal's cells contiguously;
-                    // the cells of a level are independent, so the order is free)
-                    for (auto &L : levels)
-                        std::sort(L.begin(), L.end(), [&](unsigned a, unsigned b) {
-                            auto key = [&](unsigned e) {
-                                const int j = (int)((e >> 8) & 255u), k = (int)((e >> 16) & 255u);
-                                return (j + k) * 256 + j;
-                            };
-                            return key(a) < key(b);
-                        });
-                    while (cell_tab.size() % 4) { cell_tab.push_back(0); cidx_tab.push_back(0); }
-                    sh.cell_off = (int)cell_tab.size();
+                    // level schedule: cells (FP64 factors) or blocks of 2 x 2 cells, by
+                    // I + J + k, inside a level by J + k, then J (the factorisation and the
+                    // sweeps compute positions from this order)
+                    const bool cells = prec == 64;
+                    sh.mx = (bx + 1) / 2; sh.my = (by + 1) / 2;
+                    sh.nblk = sh.mx * sh.my * bz;
+                    // odd step between a level's neighbouring blocks (J + 1, k - 1)
+                    sh.mp = sh.mx * sh.my;
+                    if ((sh.mx - sh.mp) % 2 == 0) ++sh.mp;
+                    sh.guard = std::max(1, std::max(sh.my > 1 ? sh.mx : 0, bz > 1 ? sh.mp : 0));
+                    const int dx = cells ? bx : sh.mx, dy = cells ? by : sh.my, dz = bz;
+                    sh.nlev = dx + dy + dz - 2;
+                    while (cidx_tab.size() % 4) cidx_tab.push_back(0);
+                    sh.cell_off = (int)cidx_tab.size();
                     sh.lvl_off = (int)lvl_tab.size();
-                    int pos = 0, maxw = 0;
-                    for (auto &L : levels) {
+                    int pos = 0, maxw = 0, maxc = 0;
+                    for (int l = 0; l < sh.nlev; ++l) {
                         lvl_tab.push_back(pos);
-                        for (unsigned e : L) {
-                            cell_tab.push_back(e);
-                            cidx_tab.push_back((int)(e & 255u) + bx * ((int)((e >> 8) & 255u) +
-                                                                       by * (int)((e >> 16) & 255u)));
-                        }
-                        pos += (int)L.size();
-                        maxw = std::max(maxw, (int)L.size());
+                        const int p0 = pos;
+                        for (int d = std::max(0, l - dx + 1); d <= std::min(l, dy + dz - 2); ++d)
+                            for (int j = std::max(0, d - dz + 1); j <= std::min(d, dy - 1); ++j, ++pos)
+                                cidx_tab.push_back(cells ? l - d + dx * (j + dy * (d - j)) : (l - d) | j << 8 | (d - j) << 16);
+                        maxw = std::max(maxw, pos - p0);
                     }
                     lvl_tab.push_back(pos);
                     sh.maxw = maxw;
-                    // x-pencil anti-diagonals d = j + k for the pipelined layout
-                    sh.diag_off = (int)diag_tab.size();
-                    int dbase = 0;
-                    for (int d = 0; d < by + bz - 1; ++d) {
-                        const int jmin = std::max(0, d - (bz - 1)), jmax = std::min(d, by - 1);
-                        const int cnt = jmax - jmin + 1;
-                        diag_tab.push_back(DiagInfo{jmin | (cnt << 16), dbase});
-                        dbase += cnt;
+                    for (int l = 0; l < bx + by + bz - 2; ++l) {     // widest level of cells
+                        int w = 0;
+                        for (int d = std::max(0, l - bx + 1); d <= std::min(l, by + bz - 2); ++d)
+                            w += std::min(d, by - 1) - std::max(0, d - bz + 1) + 1;
+                        maxc = std::max(maxc, w);
                     }
-                    sh.pxy = bx * by + (((bx * (by - 1)) % 2 == 0) ? 1 : 0);
-                    maxw_all = std::max(maxw_all, maxw);
+                    maxw_all = std::max(maxw_all, maxc);
                     ycap = std::max(ycap, ncell);
                     gcap = std::max(gcap, bx * by);
-                    lcap = std::max(lcap, sh.nlev + 1);
+                    lcap = std::max(lcap, bx + by + bz - 1);
+                    maxwb = std::max(maxwb, maxw);
+                    ycapb = std::max(ycapb, sh.mp * bz);
+                    bxy_all = std::max(bxy_all, bx * by);
+                    lcapb = std::max(lcapb, sh.nlev + 1);
+                    gcapb = std::max(gcapb, sh.guard);
+                    const int npen = pencil_count(bx, by, bz);
+                    npen_all = std::max(npen_all, npen);
+                    fac_smem = std::max(fac_smem, 4 * (size_t)npen * sizeof(double) + 2 * (size_t)sh.nlev * sizeof(int));
                     R.shapes.push_back(sh);
                     sid = (int)R.shapes.size() - 1;
                 }
@@ -885,7 +1132,7 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
                 si.ox0 = o0[0] - e0[0]; si.oy0 = o0[1] - e0[1]; si.oz0 = o0[2] - e0[2];
                 si.ox1 = o1[0] - e0[0]; si.oy1 = o1[1] - e0[1]; si.oz1 = o1[2] - e0[2];
                 si.foff = foff;
-                foff += (ncell + 3) & ~3;
+                foff += prec == 64 ? (ncell + 3) & ~3 : 4 * (long long)R.shapes[sid].nblk;
                 R.ncell_total += ncell;
                 R.nown += (long long)(o1[0] - o0[0]) * (o1[1] - o0[1]) * (o1[2] - o0[2]);
                 R.subs.push_back(si);
@@ -904,42 +1151,46 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
             return RAS_EINVAL;
     }
     R.nrec = foff;
-    R.ycap = (ycap + 3) & ~3;
-    R.gcap = (gcap + 3) & ~3;
-    R.lcap = (lcap + 3) & ~3;
+    R.ycap_cells = (ycap + 3) & ~3;
+    R.gcap_cells = (gcap + 3) & ~3;
+    R.lcap_cells = (lcap + 3) & ~3;
+    const bool cells = prec == 64;
+    R.ycap = cells ? R.ycap_cells : (ycapb + 3) & ~3;
+    R.gcap = cells ? R.gcap_cells : gcapb;
+    R.lcap = cells ? R.lcap_cells : (lcapb + 3) & ~3;
     R.maxw = maxw_all;
+    R.maxwb = maxwb;
+    R.bxy = bxy_all;
     R.h_lvl = lvl_tab;
     std::vector<int> chunk_tab;
     RAS_TRY(schedule_tables(R, 0, 0, chunk_tab));
-    R.smem_factor = (size_t)R.ycap * sizeof(double);
+    R.smem_factor = fac_smem;
+    R.fac_block = (npen_all + 31) & ~31;
     if (R.smem_apply > 227 * 1024 || R.smem_factor > 227 * 1024) return RAS_EINVAL;
-    // pencil-wavefront subdomain solves: left-RAS with FP32 / BF16 factors, at most
-    // 1024 x-pencils per box (one thread each)
+    // handles for which the pencil-wavefront kernel may be asked for: left-RAS with FP32
+    // / BF16 factors, at most 1024 x-pencils per box
     {
         bool ok = kind == 1 && prec != 64;
         int pens = 1, ycp = 0, dmax = 1;
         for (const ShapeInfo &sh : R.shapes) {
             pens = std::max(pens, sh.by * sh.bz);
-            ycp = std::max(ycp, sh.pxy * sh.bz);
+            ycp = std::max(ycp, (sh.bx * sh.by + ((sh.bx * (sh.by - 1)) % 2 == 0 ? 1 : 0)) * sh.bz);
             dmax = std::max(dmax, sh.by + sh.bz - 1);
         }
         if (pens > 1024) ok = false;
-        R.pipe_warps = (pens + 31) / 32;
         R.ycap_pipe = (ycp + 3) & ~3;
         R.dcap_pipe = (dmax + 1) & ~1;
-        if (pipe_smem(R) > 227 * 1024) ok = false;
+        if (pencil_smem(R) > 227 * 1024) ok = false;
         R.pipe_ok = ok ? 1 : 0;
-        R.pipe = 0;   // the level-scheduled solves are faster on the measured workloads
+        R.pipe = 0;
     }
+    RAS_TRY(dalloc(&R.d_boxes, R.subs.size()));
     RAS_TRY(dalloc(&R.d_subs, R.subs.size()));
     RAS_TRY(dalloc(&R.d_shapes, R.shapes.size()));
     RAS_TRY(dalloc(&R.d_lvl, lvl_tab.size()));
     RAS_TRY(dalloc(&R.d_chunk, chunk_tab.size()));
-    RAS_TRY(dalloc(&R.d_cells, cell_tab.size() + 16));
     RAS_TRY(dalloc(&R.d_cidx, cidx_tab.size() + 16));
     RAS_TRY(dalloc(&R.d_err, 1));
-    RAS_TRY(dalloc(&R.d_diag, diag_tab.size()));
-    RAS_CK(cudaMemcpy(R.d_diag, diag_tab.data(), diag_tab.size() * sizeof(DiagInfo), cudaMemcpyHostToDevice));
     unsigned char *fw = nullptr, *bw = nullptr;
     RAS_TRY(dalloc(&fw, (size_t)R.nrec * R.rec_bytes + 64));
     RAS_TRY(dalloc(&bw, (size_t)R.nrec * R.rec_bytes + 64));
@@ -947,20 +1198,18 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
     RAS_CK(cudaMemcpy(R.d_subs, R.subs.data(), R.subs.size() * sizeof(SubInfo), cudaMemcpyHostToDevice));
     RAS_CK(cudaMemcpy(R.d_shapes, R.shapes.data(), R.shapes.size() * sizeof(ShapeInfo),
                       cudaMemcpyHostToDevice));
+    RAS_TRY(upload_boxes(R));
     RAS_CK(cudaMemcpy(R.d_lvl, lvl_tab.data(), lvl_tab.size() * sizeof(int), cudaMemcpyHostToDevice));
     RAS_CK(cudaMemcpy(R.d_chunk, chunk_tab.data(), chunk_tab.size() * sizeof(int),
                       cudaMemcpyHostToDevice));
-    RAS_CK(cudaMemset(R.d_cells, 0, (cell_tab.size() + 16) * sizeof(unsigned)));
     RAS_CK(cudaMemset(R.d_cidx, 0, (cidx_tab.size() + 16) * sizeof(int)));
     RAS_CK(cudaMemcpy(R.d_cidx, cidx_tab.data(), cidx_tab.size() * sizeof(int), cudaMemcpyHostToDevice));
-    RAS_CK(cudaMemcpy(R.d_cells, cell_tab.data(), cell_tab.size() * sizeof(unsigned),
-                      cudaMemcpyHostToDevice));
     RAS_CK(cudaMemset(R.d_err, 0, sizeof(int)));
     RAS_CK(cudaMemset(R.d_fwd, 0, (size_t)R.nrec * R.rec_bytes + 64));
     RAS_CK(cudaMemset(R.d_bwd, 0, (size_t)R.nrec * R.rec_bytes + 64));
-    if (prec == 64) { RAS_TRY(set_apply_attr<64, 3>(R.smem_apply)); RAS_TRY(set_factor_attr<64>(R.smem_factor)); }
-    if (prec == 32) { RAS_TRY(set_apply_attr<32, 3>(R.smem_apply)); RAS_TRY(set_factor_attr<32>(R.smem_factor)); RAS_TRY(set_pipe_attr<32>()); }
-    if (prec == 16) { RAS_TRY(set_apply_attr<16, 3>(R.smem_apply)); RAS_TRY(set_factor_attr<16>(R.smem_factor)); RAS_TRY(set_pipe_attr<16>()); }
+    if (prec == 64) { RAS_TRY(set_apply_attr<64>()); RAS_TRY(set_factor_attr<64>()); }
+    if (prec == 32) { RAS_TRY(set_apply_attr<32>()); RAS_TRY(set_factor_attr<32>()); }
+    if (prec == 16) { RAS_TRY(set_apply_attr<16>()); RAS_TRY(set_factor_attr<16>()); }
     if (kind != 1) {
         // per axis and coordinate, the (contiguous) range of parts whose overlapped
         // boxes cover it; box solutions are kept per record offset
@@ -984,8 +1233,8 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
 }
 
 void ras1_free(Ras1 &R) {
-    dfree(R.d_subs); dfree(R.d_shapes); dfree(R.d_lvl); dfree(R.d_chunk); dfree(R.d_cells);
-    dfree(R.d_cidx); dfree(R.d_err); dfree(R.d_diag);
+    dfree(R.d_subs); dfree(R.d_boxes); dfree(R.d_shapes); dfree(R.d_lvl); dfree(R.d_chunk);
+    dfree(R.d_cidx); dfree(R.d_err);
     if (R.d_fwd) cudaFree(R.d_fwd);
     if (R.d_bwd) cudaFree(R.d_bwd);
     R.d_fwd = R.d_bwd = nullptr;
@@ -995,19 +1244,16 @@ void ras1_free(Ras1 &R) {
 
 int ras1_factor(Ras1 &R, const Stencil7 &A, cudaStream_t st) {
     FactorParams P;
-    P.subs = R.d_subs; P.shapes = R.d_shapes; P.lvl = R.d_lvl; P.cells = R.d_cells;
-    P.A = A; P.fwd = R.d_fwd; P.bwd = R.d_bwd;
-    P.nx = R.nx; P.ny = R.ny; P.nz = R.nz; P.err = R.d_err;
-    const int block = std::min(R.block, 256);
-    if (R.prec == 64) k_ras_factor<64><<<R.nsub, block, R.smem_factor, st>>>(P);
-    else if (R.prec == 32) k_ras_factor<32><<<R.nsub, block, R.smem_factor, st>>>(P);
-    else k_ras_factor<16><<<R.nsub, block, R.smem_factor, st>>>(P);
+    ras1_factor_params(R, A, P);
+    if (R.prec == 64) k_ras_factor<64><<<R.nsub, R.fac_block, R.smem_factor, st>>>(P);
+    else if (R.prec == 32) k_ras_factor<32><<<R.nsub, R.fac_block, R.smem_factor, st>>>(P);
+    else k_ras_factor<16><<<R.nsub, R.fac_block, R.smem_factor, st>>>(P);
     RAS_LAUNCHED();
     return RAS_OK;
 }
 
 void ras1_factor_params(const Ras1 &R, const Stencil7 &A, FactorParams &P) {
-    P.subs = R.d_subs; P.shapes = R.d_shapes; P.lvl = R.d_lvl; P.cells = R.d_cells;
+    P.subs = R.d_subs; P.shapes = R.d_shapes; P.lvl = R.d_lvl;
     P.A = A; P.fwd = R.d_fwd; P.bwd = R.d_bwd;
     P.nx = R.nx; P.ny = R.ny; P.nz = R.nz; P.err = R.d_err;
 }
@@ -1028,6 +1274,7 @@ int ras1_check(Ras1 &R, cudaStream_t st) {
     RAS_CK(cudaStreamSynchronize(st));
     if (h) {
         RAS_CK(cudaMemsetAsync(R.d_err, 0, sizeof(int), st));
+        if (h == APPLY_TIMEOUT) return RAS_ETIMEOUT;
         return RAS_EZEROPIVOT;
     }
     return RAS_OK;
@@ -1043,20 +1290,21 @@ int ras1_set_kernel(Ras1 &R, int kernel) {
 
 void ras1_apply_params(const Ras1 &R, ApplyParams &P) {
     P = ApplyParams{};
-    P.subs = R.d_subs; P.shapes = R.d_shapes; P.lvl = R.d_lvl; P.chunk = R.d_chunk;
+    P.subs = R.d_subs; P.shapes = R.d_shapes; P.boxes = R.d_boxes; P.lvl = R.d_lvl; P.chunk = R.d_chunk;
     P.cidx = R.d_cidx;
     P.fwd = (const unsigned char *)R.d_fwd; P.bwd = (const unsigned char *)R.d_bwd;
     P.nx = R.nx; P.ny = R.ny; P.nz = R.nz; P.accumulate = 0;
-    P.ycap = R.ycap; P.gcap = R.gcap; P.lcap = R.lcap; P.nbuf = R.nbuf; P.chunk_cells = R.chunk_cells;
+    P.ycap = R.ycap; P.gcap = R.gcap; P.lcap = R.lcap; P.chunk_cells = R.chunk_cells;
+    P.steps = reinterpret_cast<const int4 *>(R.d_chunk); P.err = R.d_err;
     P.kind = R.kind; P.zbuf = R.zbuf;
 }
 
 int ras1_apply_batch(const BatchApply &B, int grid, int prec, int block, size_t smem, cudaStream_t st) {
     if (grid <= 0 || B.nitems <= 0) return RAS_OK;
     RAS_CK(cudaMemsetAsync(B.qcount, 0, sizeof(int), st));
-    if (prec == 64) k_ras_apply_batch<64, 3><<<grid, block, smem, st>>>(B);
-    else if (prec == 32) k_ras_apply_batch<32, 3><<<grid, block, smem, st>>>(B);
-    else k_ras_apply_batch<16, 3><<<grid, block, smem, st>>>(B);
+    if (prec == 64) k_ras_apply_batch<64><<<grid, block, smem, st>>>(B);
+    else if (prec == 32) k_ras_apply_batch<32><<<grid, block, smem, st>>>(B);
+    else k_ras_apply_batch<16><<<grid, block, smem, st>>>(B);
     RAS_LAUNCHED();
     return RAS_OK;
 }
@@ -1065,38 +1313,21 @@ int ras1_batch_grid(int prec, int block, size_t smem, int nitems, int *grid) {
     int dev = 0, sms = 0, per = 0;
     RAS_CK(cudaGetDevice(&dev));
     RAS_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (prec == 64) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<64, 3>, block, smem));
-    else if (prec == 32) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<32, 3>, block, smem));
-    else RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<16, 3>, block, smem));
+    if (prec == 64) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<64>, block, smem));
+    else if (prec == 32) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<32>, block, smem));
+    else RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<16>, block, smem));
     if (per < 1) return RAS_EINVAL;
     *grid = std::min(nitems, sms * per);
     return RAS_OK;
 }
 
 int ras1_apply(Ras1 &R, const double *r, double *z, int accumulate, cudaStream_t st) {
-    if (R.pipe) {
-        PipeParams Q;
-        Q.subs = R.d_subs; Q.shapes = R.d_shapes; Q.diag = R.d_diag;
-        Q.lvl = R.d_lvl; Q.chunk = R.d_chunk;
-        Q.fwd = (const unsigned char *)R.d_fwd; Q.bwd = (const unsigned char *)R.d_bwd;
-        Q.r = r; Q.z = z; Q.nx = R.nx; Q.ny = R.ny; Q.nz = R.nz; Q.accumulate = accumulate;
-        Q.ycap = R.ycap_pipe; Q.lcap = R.lcap; Q.chunk_cells = R.chunk_cells;
-        const int threads = 32 * R.pipe_warps;
-        if (R.prec == 32) k_ras_pipe<32><<<R.nsub, threads, R.smem_pipe, st>>>(Q);
-        else k_ras_pipe<16><<<R.nsub, threads, R.smem_pipe, st>>>(Q);
-        RAS_LAUNCHED();
-        return RAS_OK;
-    }
     ApplyParams P;
-    P.subs = R.d_subs; P.shapes = R.d_shapes; P.lvl = R.d_lvl; P.chunk = R.d_chunk;
-    P.cidx = R.d_cidx;
-    P.fwd = (const unsigned char *)R.d_fwd; P.bwd = (const unsigned char *)R.d_bwd;
-    P.r = r; P.z = z; P.nx = R.nx; P.ny = R.ny; P.nz = R.nz; P.accumulate = accumulate;
-    P.ycap = R.ycap; P.gcap = R.gcap; P.lcap = R.lcap; P.nbuf = R.nbuf; P.chunk_cells = R.chunk_cells;
-    P.kind = R.kind; P.zbuf = R.zbuf;
-    if (R.prec == 64) k_ras_apply<64, 3><<<R.nsub, R.block, R.smem_apply, st>>>(P);
-    else if (R.prec == 32) k_ras_apply<32, 3><<<R.nsub, R.block, R.smem_apply, st>>>(P);
-    else k_ras_apply<16, 3><<<R.nsub, R.block, R.smem_apply, st>>>(P);
+    ras1_apply_params(R, P);
+    P.r = r; P.z = z; P.accumulate = accumulate;
+    if (R.prec == 64) k_ras_apply<64><<<R.nsub, R.launch, R.smem_apply, st>>>(P);
+    else if (R.prec == 32) k_ras_apply<32><<<R.nsub, R.launch, R.smem_apply, st>>>(P);
+    else k_ras_apply<16><<<R.nsub, R.launch, R.smem_apply, st>>>(P);
     RAS_LAUNCHED();
     if (R.kind != 1) {
         SumParams Q;

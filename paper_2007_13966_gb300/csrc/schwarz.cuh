@@ -11,20 +11,14 @@ namespace ras {
 struct ShapeInfo {
     int bx, by, bz, ncell;
     int nlev, nchunk;
-    int lvl_off;     // into lvl_tab: nlev + 1 level starts (cell positions)
-    int cell_off;    // into cell_tab: ncell packed entries (multiple of 4 aligned)
-    int chunk_off;   // into chunk_tab: nchunk + 1 level indices
+    int lvl_off;     // into lvl_tab: nlev + 1 level starts
+    int cell_off;    // into cidx_tab: local indices in level order (multiple of 4 aligned)
+    int chunk_off;   // into chunk_tab: nchunk + 1 level indices (blocks: 4-integer steps)
     int maxw;        // widest level
-    int diag_off;    // into diag_tab: by + bz - 1 anti-diagonals d = j + k of the x-pencils (j, k)
-    int pxy;         // plane stride of the pipelined apply's vector (bx*by or bx*by + 1)
-};
-
-// One anti-diagonal d = j + k of a box's x-pencils (j, k): its first j, its
-// pencil count, and the number of pencils on the diagonals before it (inside a
-// wavefront level the cells are grouped by diagonal, then ordered by j).
-struct DiagInfo {
-    int jmin_cnt;    // jmin | cnt << 16
-    int base;        // sum of cnt over the diagonals d' < d
+    // blocks of 2 x 2 cells of a plane (FP32 / BF16 factors; nlev, lvl_off, cell_off, maxw
+    // then count blocks): blocks along x and y, their number, plane stride and guard in
+    // shared memory
+    int mx, my, nblk, mp, guard;
 };
 
 // One subdomain: overlapped box origin, its shape, owned box (relative to the
@@ -35,9 +29,10 @@ struct SubInfo {
     long long foff;
 };
 
-// cell entry: i | j << 8 | k << 16 | flags << 24 (local coordinates)
-enum : unsigned {
-    F_MX = 1u, F_MY = 2u, F_MZ = 4u, F_PX = 8u, F_PY = 16u, F_PZ = 32u
+// one subdomain with its shape (one load for the sweeps)
+struct BoxInfo {
+    SubInfo sub;
+    ShapeInfo shape;
 };
 
 struct Ras1 {
@@ -46,21 +41,25 @@ struct Ras1 {
     int prec = 64;          // 64, 32, 16
     int rec_bytes = 32;     // bytes of one factor record (4 values)
     int block = 128;        // threads per subdomain CTA
-    int chunk_cells = 1024; // max cells per staged chunk
-    int nbuf = 3;           // staged chunks in flight
-    int ycap = 0, lcap = 0; // smem capacities (cells, levels + 1)
-    int gcap = 0;           // zero guard band on each side of the apply's vector (cells)
-    int maxw = 0;           // widest level over the box shapes
+    int chunk_cells = 1024; // max cells per staged chunk (the schedule asked for)
+    int launch = 128;       // threads per CTA of the sweeps
+    int ycap = 0, lcap = 0; // smem capacities of the sweeps (cells or blocks, levels + 1)
+    int gcap = 0;           // zero guard band on each side of their vector
+    int ycap_cells = 0, lcap_cells = 0, gcap_cells = 0;   // the same cell by cell
+    int maxw = 0;           // widest level of cells over the box shapes
+    int maxwb = 0;          // widest level of the sweeps (cells or blocks)
+    int bxy = 1;            // largest box plane (cells)
+    int fac_block = 32;     // threads per box of the factorisation (its pencils)
     std::vector<int> h_lvl; // host copy of the level starts (rescheduling)
     size_t smem_apply = 0, smem_factor = 0;
     long long nrec = 0;     // factor records (incl. padding)
     long long ncell_total = 0;  // sum of overlapped cells
     long long nown = 0;
     SubInfo *d_subs = nullptr;
+    BoxInfo *d_boxes = nullptr;
     ShapeInfo *d_shapes = nullptr;
     int *d_lvl = nullptr, *d_chunk = nullptr;
-    unsigned *d_cells = nullptr;
-    int *d_cidx = nullptr;  // level-ordered local natural index of each cell (apply)
+    int *d_cidx = nullptr;  // level-ordered local index of each cell (block)
     void *d_fwd = nullptr, *d_bwd = nullptr;
     int *d_err = nullptr;
     // AS (kind 0) and right-RAS (kind 2): each box's whole solution goes to zbuf
@@ -71,15 +70,10 @@ struct Ras1 {
     int parts[3] = {1, 1, 1};
     std::vector<SubInfo> subs;
     std::vector<ShapeInfo> shapes;
-    // pencil-wavefront subdomain solves (left-RAS, FP32 / BF16 factors): one warp
-    // per group of x-pencil anti-diagonals
+    // ras_set_apply_kernel's choice (both values run the same kernel) and its limits
     int pipe = 0;
-    int pipe_ok = 0;          // the handle's shapes and options allow the pipelined solves
-    int pipe_warps = 0;       // warps per box
-    int dcap_pipe = 0;        // anti-diagonal table capacity
-    size_t smem_pipe = 0;
-    int ycap_pipe = 0;        // floats of the padded box vector
-    DiagInfo *d_diag = nullptr;
+    int pipe_ok = 0;
+    int dcap_pipe = 0, ycap_pipe = 0;
 };
 
 int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int overlap, int prec,
@@ -87,7 +81,7 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
 void ras1_free(Ras1 &R);
 // numeric ILU(0) of every A_i = R_i^delta A (R_i^delta)^T; no synchronisation
 int ras1_factor(Ras1 &R, const Stencil7 &A, cudaStream_t st);
-// reads and clears the pivot flag (synchronises)
+// reads and clears the pivot flag and that of a sweep's wait that ran out (synchronises)
 int ras1_check(Ras1 &R, cudaStream_t st);
 // z = M^{-1} r (accumulate = 0) or z += M^{-1} r (accumulate = 1), with
 // M^{-1} = sum_i (R_i^0)^T A_i^{-1} R_i^delta (left-RAS, kind 1),
@@ -96,22 +90,24 @@ int ras1_check(Ras1 &R, cudaStream_t st);
 int ras1_apply(Ras1 &R, const double *r, double *z, int accumulate, cudaStream_t st);
 // new chunk size / threads per box for the subdomain solves (0: default); synchronous
 int ras1_set_schedule(Ras1 &R, int chunk_cells, int threads);
-// subdomain-solve kernel: 0 level-scheduled, 1 pencil-wavefront (both read the
-// same records and give the same bits); RAS_EINVAL if not eligible
+// the kernel choice 0 or 1 (RAS_EINVAL if not eligible); both run the same sweeps
 int ras1_set_kernel(Ras1 &R, int kernel);
 
 // parameters of one handle's apply kernel
 struct ApplyParams {
     const SubInfo *subs;
     const ShapeInfo *shapes;
+    const BoxInfo *boxes;
     const int *lvl, *chunk;
-    const int *cidx;          // per shape, level order: local natural index of each cell
+    const int *cidx;          // per shape, level order: local index of each cell (block)
     const unsigned char *fwd, *bwd;
     const double *r;
     double *z;
     int nx, ny, nz;
     int accumulate;
-    int ycap, gcap, lcap, nbuf, chunk_cells;
+    int ycap, gcap, lcap, chunk_cells;
+    const int4 *steps;   // sweeps in blocks: per shape and step (schedule_tables)
+    int *err;            // a wait that ran out
     int kind;        // 1 left-RAS; 0 AS, 2 right-RAS (box solutions to zbuf)
     double *zbuf;
 };
@@ -134,7 +130,6 @@ struct FactorParams {
     const SubInfo *subs;
     const ShapeInfo *shapes;
     const int *lvl;
-    const unsigned *cells;
     Stencil7 A;
     void *fwd, *bwd;
     int nx, ny, nz;
