@@ -18,6 +18,7 @@
 // by a fixed-order sum over that reservoir's chunks (deterministic). A reservoir
 // whose solve has finished is switched off in a device mask; its chunks and
 // boxes return at once.
+#include "orth.cuh"
 #include "precond.cuh"
 
 #include <algorithm>
@@ -113,9 +114,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_bmdot(const double *__restrict_
             if (v < k) acc[v] = fma(V[v * ldv + base + q], wi, acc[v]);
         if (self) acc[KM] = fma(wi, wi, acc[KM]);
     }
-    __shared__ double sh[RED_THREADS / 32];
-    for (int v = 0; v < k; ++v) block_partial(acc[v], sh, partials, (long long)v * nch + blockIdx.x);
-    if (self) block_partial(acc[KM], sh, partials, (long long)k * nch + blockIdx.x);
+    block_rows<KM>(acc, k, self, partials, nch, blockIdx.x);
 }
 
 // out[inst][slot0 + v] = sum of the reservoir's chunk partials of row v, in chunk
@@ -136,15 +135,37 @@ __global__ void k_bfinalize(const double *__restrict__ partials, int nch, int nv
     }
 }
 
-// w -= sum_v h[v] V[v] with the reservoir's coefficients h = out[inst][hslot ..];
-// partial sums of the new w . w if NORM
-template <bool NORM, int KM>
+// w -= sum_v h[v] V[v] with the reservoir's coefficients h = out[inst][hslot ..], and the
+// partial sums of V[v] w for the new w
+template <int KM>
+__global__ void __launch_bounds__(RED_THREADS) k_bupdate_dot(const double *__restrict__ V, long long ldv, int k,
+                                                             const double *__restrict__ out, int hslot,
+                                                             double *__restrict__ w, const BChunk *__restrict__ ch,
+                                                             const long long *__restrict__ off,
+                                                             const unsigned char *__restrict__ active,
+                                                             double *__restrict__ partials, int nch) {
+    const BChunk c = ch[blockIdx.x];
+    if (!active[c.inst]) return;
+    const long long base = off[c.inst] + c.start;
+    __shared__ double hs[KM];
+    if (threadIdx.x < KM) hs[threadIdx.x] = threadIdx.x < k ? out[(long long)c.inst * OST + hslot + threadIdx.x] : 0.0;
+    __syncthreads();
+    double acc[KM + 1];
+#pragma unroll
+    for (int v = 0; v <= KM; ++v) acc[v] = 0.0;
+    for (int q = threadIdx.x; q < c.count; q += blockDim.x)
+        w[base + q] = update_dot<KM>(V, ldv, base + q, k, hs, w[base + q], acc);
+    block_rows<KM>(acc, k, 0, partials, nch, blockIdx.x);
+}
+
+// w -= sum_v h[v] V[v], and the partial sums of the new w . w
+template <int KM>
 __global__ void __launch_bounds__(RED_THREADS) k_bupdate(const double *__restrict__ V, long long ldv, int k,
                                                          const double *__restrict__ out, int hslot,
                                                          double *__restrict__ w, const BChunk *__restrict__ ch,
                                                          const long long *__restrict__ off,
                                                          const unsigned char *__restrict__ active,
-                                                         double *__restrict__ partials) {
+                                                         double *__restrict__ partials, int) {
     const BChunk c = ch[blockIdx.x];
     if (!active[c.inst]) return;
     const long long base = off[c.inst] + c.start;
@@ -159,12 +180,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_bupdate(const double *__restric
         for (int v = 0; v < KM; ++v)
             if (v < k) s = fma(-hv[v], V[v * ldv + base + q], s);
         w[base + q] = s;
-        if (NORM) acc = fma(s, s, acc);
+        acc = fma(s, s, acc);
     }
-    if (NORM) {
-        __shared__ double sh[RED_THREADS / 32];
-        block_partial(acc, sh, partials, blockIdx.x);
-    }
+    __shared__ double sh[RED_THREADS / 32];
+    block_partial(acc, sh, partials, blockIdx.x);
 }
 
 // y = x / s[inst * stride] per reservoir
@@ -424,20 +443,30 @@ static int b_finalize(ras_batch *B, int nvec, int slot0, int sqrt_last, cudaStre
     return RAS_OK;
 }
 
-template <bool NORM>
+// KM: the next power of two >= k
+#define RAS_BUPD(KERNEL, KM) KERNEL<KM><<<B->nch, RED_THREADS, 0, st>>>(B->V, B->Ntot, k, B->out, hslot, w, \
+                                                                       B->d_ch, B->d_off, B->d_act, B->partials, B->nch)
+#define RAS_BUPD_K(KERNEL)                   \
+    do {                                     \
+        if (k <= 1) RAS_BUPD(KERNEL, 1);     \
+        else if (k <= 2) RAS_BUPD(KERNEL, 2);    \
+        else if (k <= 4) RAS_BUPD(KERNEL, 4);    \
+        else if (k <= 8) RAS_BUPD(KERNEL, 8);    \
+        else if (k <= 16) RAS_BUPD(KERNEL, 16);  \
+        else RAS_BUPD(KERNEL, 32);           \
+    } while (0)
 static int b_update(ras_batch *B, int k, int hslot, double *w, cudaStream_t st) {
-#define RAS_BUPD(KM) k_bupdate<NORM, KM><<<B->nch, RED_THREADS, 0, st>>>(B->V, B->Ntot, k, B->out, hslot, w, \
-                                                                         B->d_ch, B->d_off, B->d_act, B->partials)
-    if (k <= 1) RAS_BUPD(1);
-    else if (k <= 2) RAS_BUPD(2);
-    else if (k <= 4) RAS_BUPD(4);
-    else if (k <= 8) RAS_BUPD(8);
-    else if (k <= 16) RAS_BUPD(16);
-    else RAS_BUPD(32);
-#undef RAS_BUPD
+    RAS_BUPD_K(k_bupdate);
     RAS_LAUNCHED();
     return RAS_OK;
 }
+static int b_update_dot(ras_batch *B, int k, int hslot, double *w, cudaStream_t st) {
+    RAS_BUPD_K(k_bupdate_dot);
+    RAS_LAUNCHED();
+    return RAS_OK;
+}
+#undef RAS_BUPD
+#undef RAS_BUPD_K
 
 template <bool RESID>
 static int b_stencil(ras_batch *B, const double *b, const double *x, double *y, cudaStream_t st,
@@ -533,10 +562,9 @@ static int b_cycle(ras_batch *B, int j0, int j1, cudaStream_t st) {
         RAS_TRY(b_stencil<false>(B, nullptr, Zj, B->w, st));
         RAS_TRY(b_mdot(B, B->V, k, 1, B->w, st));
         RAS_TRY(b_finalize(B, k + 1, 0, 0, st));
-        RAS_TRY(b_update<false>(B, k, 0, B->w, st));
-        RAS_TRY(b_mdot(B, B->V, k, 0, B->w, st));
+        RAS_TRY(b_update_dot(B, k, 0, B->w, st));
         RAS_TRY(b_finalize(B, k, k + 1, 0, st));
-        RAS_TRY(b_update<true>(B, k, k + 1, B->w, st));
+        RAS_TRY(b_update(B, k, k + 1, B->w, st));
         RAS_TRY(b_finalize(B, 1, 2 * k + 1, 1, st));
         RAS_TRY(b_scale(B, B->V + (size_t)(j + 1) * Nt, B->w, B->out + 2 * k + 1, OST, st));
         k_bgivens<<<(B->n + 63) / 64, 64, 0, st>>>(B->K, B->out, B->d_act, j, B->n);
