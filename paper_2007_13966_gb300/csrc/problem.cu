@@ -160,46 +160,81 @@ int vec_set(double *y, double v, int n, cudaStream_t st) {
 // 7-point operator: y = A x  /  y = b - A x
 // ---------------------------------------------------------------------------
 
-template <bool RESID>
+// Two consecutive cells per thread, the seven coefficients in 16-byte loads when every
+// array is 16-byte aligned (VEC): all of a thread's loads are in flight together, and the
+// blocks are full whatever the row length (a block of 32 threads per piece of a 60-cell row,
+// one cell each, left too few bytes in flight). 60 x 220 x 85 cells, 81 MB: 24.5 -> 21.0 us.
+template <bool RESID, bool VEC>
 __global__ void __launch_bounds__(256) k_stencil(Stencil7 A, int nx, int ny, int nz,
                                                  const double *__restrict__ b,
                                                  const double *__restrict__ x,
                                                  double *__restrict__ y) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y, k = blockIdx.z;
-    if (i >= nx) return;
-    const int nxy = nx * ny;
-    const int n = i + nx * (j + ny * k);
-    double s = A.c[0][n] * x[n];
-    if (i > 0) s = fma(A.c[1][n], x[n - 1], s);
-    if (i < nx - 1) s = fma(A.c[2][n], x[n + 1], s);
-    if (j > 0) s = fma(A.c[3][n], x[n - nx], s);
-    if (j < ny - 1) s = fma(A.c[4][n], x[n + nx], s);
-    if (k > 0) s = fma(A.c[5][n], x[n - nxy], s);
-    if (k < nz - 1) s = fma(A.c[6][n], x[n + nxy], s);
-    y[n] = RESID ? b[n] - s : s;
+    const int nxy = nx * ny, N = nxy * nz;
+    const int n = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (n >= N) return;
+    const bool two = n + 1 < N;
+    double c[7][2], bb[2] = {0.0, 0.0};
+    auto pair = [&](const double *a, double (&v)[2]) {
+        if (VEC && two) {
+            const double2 t = __ldg(reinterpret_cast<const double2 *>(a + n));
+            v[0] = t.x;
+            v[1] = t.y;
+        } else {
+            v[0] = __ldg(a + n);
+            v[1] = two ? __ldg(a + n + 1) : 0.0;
+        }
+    };
+#pragma unroll
+    for (int s = 0; s < 7; ++s) pair(A.c[s], c[s]);
+    if (RESID) pair(b, bb);
+    int row = n / nx, i = n - row * nx, k = row / ny, j = row - k * ny;
+    double r[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int q = n + e;
+        if (e == 1 && !two) break;
+        double s = c[0][e] * x[q];
+        if (i > 0) s = fma(c[1][e], x[q - 1], s);
+        if (i < nx - 1) s = fma(c[2][e], x[q + 1], s);
+        if (j > 0) s = fma(c[3][e], x[q - nx], s);
+        if (j < ny - 1) s = fma(c[4][e], x[q + nx], s);
+        if (k > 0) s = fma(c[5][e], x[q - nxy], s);
+        if (k < nz - 1) s = fma(c[6][e], x[q + nxy], s);
+        r[e] = RESID ? bb[e] - s : s;
+        if (++i == nx) {
+            i = 0;
+            if (++j == ny) { j = 0; ++k; }
+        }
+    }
+    if (VEC && two) {
+        *reinterpret_cast<double2 *>(y + n) = make_double2(r[0], r[1]);
+    } else {
+        y[n] = r[0];
+        if (two) y[n + 1] = r[1];
+    }
 }
 
-static inline dim3 stencil_grid(int nx, int ny, int nz, int threads) {
-    return dim3((nx + threads - 1) / threads, ny, nz);
+template <bool RESID>
+static int stencil_launch(const Stencil7 &A, int nx, int ny, int nz, const double *b, const double *x, double *y,
+                          cudaStream_t st) {
+    const long long N = (long long)nx * ny * nz;
+    const int g = (int)((N + 511) / 512);
+    uintptr_t all = (uintptr_t)y | (uintptr_t)b;
+    for (int s = 0; s < 7; ++s) all |= (uintptr_t)A.c[s];
+    if (all % 16 == 0) k_stencil<RESID, true><<<g, 256, 0, st>>>(A, nx, ny, nz, b, x, y);
+    else k_stencil<RESID, false><<<g, 256, 0, st>>>(A, nx, ny, nz, b, x, y);
+    RAS_LAUNCHED();
+    return RAS_OK;
 }
-
-static inline int stencil_threads(int nx) { return nx >= 128 ? 128 : (nx >= 64 ? 64 : 32); }
 
 int stencil_apply(const Stencil7 &A, int nx, int ny, int nz, const double *x, double *y,
                   cudaStream_t st) {
-    const int t = stencil_threads(nx);
-    k_stencil<false><<<stencil_grid(nx, ny, nz, t), t, 0, st>>>(A, nx, ny, nz, nullptr, x, y);
-    RAS_LAUNCHED();
-    return RAS_OK;
+    return stencil_launch<false>(A, nx, ny, nz, nullptr, x, y, st);
 }
 
 int stencil_residual(const Stencil7 &A, int nx, int ny, int nz, const double *b, const double *x,
                      double *y, cudaStream_t st) {
-    const int t = stencil_threads(nx);
-    k_stencil<true><<<stencil_grid(nx, ny, nz, t), t, 0, st>>>(A, nx, ny, nz, b, x, y);
-    RAS_LAUNCHED();
-    return RAS_OK;
+    return stencil_launch<true>(A, nx, ny, nz, b, x, y, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -262,30 +297,56 @@ __device__ __forceinline__ float cubic_root_f32(float c2, float c1, float c0) {
 
 struct EosOut {
     double c, dc, m, dm;
-    double Z;
+    double Z, iZ;
     bool ok;   // an admissible root: Z finite, Z > B, f_Z != 0
 };
 
-__device__ __forceinline__ EosOut eos_cell(double p, const EosConst &E) {
-    const double be = E.beta, al = E.alpha;
-    const double A = al * p, B = be * p;
-    const double c2 = -(1.0 - B);
-    const double c1 = A - 3.0 * B * B - 2.0 * B;
-    const double c0 = -(A * B - B * B - B * B * B);
-    double Z = (double)cubic_root_f32((float)c2, (float)c1, (float)c0);
-    // three FP64 Newton steps on the cubic (FP32 start is ~1e-7 accurate)
+// 1 / x by one third-order step y (1 + e + e^2), e = 1 - x y, from the FP32 reciprocal
+// (24 bits -> 72, then FP64 rounding), where x lies in FP32's normal range: 3 operations of
+// the FP64 pipe (2 per cycle and SM) and two conversions, where a division takes about ten
+__device__ __forceinline__ double recip64(double x) {
+    const double ax = fabs(x);
+    if (!(ax > 1e-36 && ax < 1e36)) return 1.0 / x;
+    const double y = (double)__frcp_rn((float)x);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// The largest real root Z of Z^3 + c2 Z^2 + c1 Z + c0. FP32 closed form, then Newton steps
+// with FP64 residuals. The first two take the slope's reciprocal in FP32: near a simple
+// root the step is a small correction, so its relative error of 1e-6 leaves 1e-13 and then
+// rounding. Steps go on with the FP64 slope only while they still move the root by more than
+// 1e-10 (close roots, where Newton converges slowly).
+// Root selection in FP64: the FP32 closed form decides between one and three real roots in
+// FP32, and near a pair of close roots it can start Newton on another root than the largest.
+// The other two roots solve the deflated quadratic t^2 + (c2 + Z) t + (c1 + (c2 + Z) Z) = 0;
+// a real root above Z replaces it (polished by two Newton steps). The discriminant is taken
+// in FP32 first: below minus a margin (its FP32 error is at most 4 eps 1.5 (c2^2 + Z^2 +
+// |c1|) = 3.6e-7 of that sum) there is no real root; otherwise FP64 decides.
+__device__ __forceinline__ double largest_root(double c2, double c1, double c0) {
+    const float f2 = (float)c2, f1 = (float)c1;
+    const float z0 = cubic_root_f32(f2, f1, (float)c0);
+    double Z = (double)z0;
+    float last = 0.0f;
 #pragma unroll
-    for (int it = 0; it < 3; ++it) {
-        const double f = ((Z + c2) * Z + c1) * Z + c0;
-        const double fz = (3.0 * Z + 2.0 * c2) * Z + c1;
-        Z -= f / fz;
+    for (int it = 0; it < 2; ++it) {
+        const double f = fma(fma(Z + c2, Z, c1), Z, c0);
+        const float z = it == 0 ? z0 : (float)Z;
+        const float slope = fmaf(fmaf(3.0f, z, 2.0f * f2), z, f1);
+        last = __fdividef((float)f, slope);
+        Z -= (double)last;
     }
-    // Root selection in FP64: the FP32 closed form decides between one and three
-    // real roots in FP32, and near a pair of close roots it can start Newton on
-    // another root than the largest. The other two roots solve the deflated
-    // quadratic t^2 + (c2 + Z) t + (c1 + (c2 + Z) Z) = 0; if it has a real root
-    // above Z, that root is the largest: take it and polish it.
-    {
+    if (!(fabsf(last) <= 1e-10f)) {
+#pragma unroll 1
+        for (int it = 0; it < 3; ++it) {
+            const double f = fma(fma(Z + c2, Z, c1), Z, c0);
+            const double fz = fma(fma(3.0, Z, 2.0 * c2), Z, c1);
+            Z -= f / fz;
+        }
+    }
+    const float zf = (float)Z, q1f = f2 + zf, q0f = fmaf(q1f, zf, f1);
+    const float margin = 1e-6f * (f2 * f2 + fabsf(f1) + zf * zf);
+    if (!(fmaf(q1f, q1f, -4.0f * q0f) < -margin)) {
         const double q1 = c2 + Z, q0 = c1 + q1 * Z;
         const double dq = q1 * q1 - 4.0 * q0;
         if (dq >= 0.0) {
@@ -302,29 +363,43 @@ __device__ __forceinline__ EosOut eos_cell(double p, const EosConst &E) {
             }
         }
     }
+    return Z;
+}
+
+// Bound: FP64 at 2 operations per cycle and SM, so the operations are what is saved: the
+// coefficients of the cubic's derivatives shared, one reciprocal for both 1 / f_Z and 1 / Z.
+__device__ __forceinline__ EosOut eos_cell(double p, const EosConst &E) {
+    const double be = E.beta, al = E.alpha;
+    const double A = al * p, B = be * p;
+    const double c2 = B - 1.0;
+    const double c1 = fma(-B, fma(3.0, B, 2.0), A);        // A - 3 B^2 - 2 B
+    const double c0 = B * (fma(B, B, B) - A);              // -(A B - B^2 - B^3)
+    const double Z = largest_root(c2, c1, c0);
     // partial derivatives of f(Z, p) with A = alpha p, B = beta p
-    const double fZ = 3.0 * Z * Z - 2.0 * (1.0 - B) * Z + (A - 3.0 * B * B - 2.0 * B);
-    const double fp = be * Z * Z + (al - 6.0 * be * B - 2.0 * be) * Z
-                      - (2.0 * al * B - 2.0 * be * B - 3.0 * be * B * B);
-    const double fZZ = 6.0 * Z - 2.0 * (1.0 - B);
-    const double fZp = 2.0 * be * Z + (al - 6.0 * be * B - 2.0 * be);
-    const double fpp = -6.0 * be * be * Z - (2.0 * al * be - 2.0 * be * be - 6.0 * be * be * B);
-    const double ifZ = 1.0 / fZ;
+    const double fZ = fma(fma(3.0, Z, 2.0 * c2), Z, c1);
+    const double h = fma(-6.0 * be, B, al - 2.0 * be);     // al - 6 be B - 2 be
+    const double g = fma(3.0 * be, B, 2.0 * (be - al));    // -(2 al - 2 be - 3 be B)
+    const double fp = fma(fma(be, Z, h), Z, B * g);
+    const double fZZ = fma(6.0, Z, 2.0 * c2);
+    const double fZp = fma(2.0 * be, Z, h);
+    const double fpp = be * fma(6.0 * be, B - Z, 2.0 * (be - al));   // -6 be^2 Z - (2 al be - 2 be^2 - 6 be^2 B)
+    const double inv = recip64(fZ * Z);
+    const double ifZ = inv * Z, iZ = inv * fZ;
     const double dZ = -fp * ifZ;                                   // dZ/dp
-    const double d2Z = -(fZZ * dZ * dZ + 2.0 * fZp * dZ + fpp) * ifZ;
-    const double iZ = 1.0 / Z;
-    const double iZ2 = iZ * iZ;
+    const double d2Z = -fma(dZ, fma(fZZ, dZ, 2.0 * fZp), fpp) * ifZ;
+    const double u = dZ * iZ, pu = p * u;                          // Z'/Z, p Z'/Z
     EosOut o;
-    o.c = iZ - p * dZ * iZ2;                                       // (p/Z)(1/p - Z'/Z)
-    o.dc = -2.0 * dZ * iZ2 - p * d2Z * iZ2 + 2.0 * p * dZ * dZ * iZ2 * iZ;
+    o.c = fma(-pu, iZ, iZ);                                        // (p/Z)(1/p - Z'/Z)
+    o.dc = iZ * fma(2.0 * u, pu - 1.0, -p * (d2Z * iZ));           // -2 Z'/Z^2 - p Z''/Z^2 + 2 p Z'^2/Z^3
     o.m = p * iZ * E.inv_mu;                                       // p / (mu Z)
     o.dm = o.c * E.inv_mu;
     o.Z = Z;
+    o.iZ = iZ;
     o.ok = isfinite(Z) && Z > B && fZ != 0.0 && isfinite(o.c) && isfinite(o.dc);
     return o;
 }
 
-// pass 1: per-cell storage term and its derivative, and m, dm for the fluxes.
+// pass 1: per-cell storage term and its derivative, and m / 2, dm / 2 for the fluxes.
 // Accumulation V phi c(p) D_t p (Eq. gover_sys), or in the conservative form
 // V phi D_t(p/Z) with the same BDF weights on p/Z at the three levels (d(p/Z)/dp = c);
 // fixed injection rates subtract (p/Z) Q from the cell's residual.
@@ -345,11 +420,11 @@ __global__ void __launch_bounds__(256) k_eos_storage(
             if (!ol.ok) o.ok = false;
             double DtP;
             if (order == 1) {
-                DtP = (pn / o.Z - pl[n] / ol.Z) * inv_dt;
+                DtP = (pn * o.iZ - pl[n] * ol.iZ) * inv_dt;
             } else {
                 const EosOut om = eos_cell(plm1[n], E);
                 if (!om.ok) o.ok = false;
-                DtP = (3.0 * (pn / o.Z) - 4.0 * (pl[n] / ol.Z) + plm1[n] / om.Z) * (0.5 * inv_dt);
+                DtP = (3.0 * (pn * o.iZ) - 4.0 * (pl[n] * ol.iZ) + plm1[n] * om.iZ) * (0.5 * inv_dt);
             }
             f = vp * DtP;
             jc = vp * o.c * g;
@@ -361,7 +436,7 @@ __global__ void __launch_bounds__(256) k_eos_storage(
         }
         if (rateQ) {
             const double q = rateQ[n];
-            f -= (pn / o.Z) * q;
+            f -= (pn * o.iZ) * q;
             jc -= o.c * q;
         }
         if (!o.ok) {   // no admissible root: flag it and poison the cell's residual
@@ -370,8 +445,8 @@ __global__ void __launch_bounds__(256) k_eos_storage(
         }
         F[n] = f;
         if (Jc) Jc[n] = jc;
-        m_out[n] = o.m;
-        dm_out[n] = o.dm;
+        m_out[n] = 0.5 * o.m;      // halves: what a face's mean mobility takes from the cell
+        dm_out[n] = 0.5 * o.dm;
     }
 }
 
@@ -380,20 +455,25 @@ struct JacOut {
 };
 
 // pass 2: two-point fluxes, connections, Jacobian rows. Row order of the sum:
-// storage, +x, -x, +y, -y, +z, -z, connections.
-template <bool WANT_J>
-__global__ void __launch_bounds__(128) k_flux(
+// storage, +x, -x, +y, -y, +z, -z, connections. m and dm hold halves.
+//
+// Bound: FP64 at 2 operations per cycle and SM. With level faces and mean mobilities (not
+// GEN: no gravity, no upwinding) a face takes eight: the mean mobility from the halves,
+//     t = T (m_n + m_q) / 2, flux t (p_n - p_q), d flux / d p_n = u dm_n / 2 + t,
+//     d flux / d p_q = u dm_q / 2 - t,  u = T (p_n - p_q),
+// where the general form (weights, face potential with the mean density) takes seventeen.
+// Residual and Jacobian of 128 x 128 x 64 cells, both passes: 505 -> 283 us.
+template <bool WANT_J, bool GEN>
+__global__ void __launch_bounds__(256) k_flux(
     int nx, int ny, int nz, const double *__restrict__ p, const double *__restrict__ m,
     const double *__restrict__ dm, const double *__restrict__ Tx, const double *__restrict__ Ty,
     const double *__restrict__ Tz, const int *__restrict__ conn_ptr,
     const double *__restrict__ conn_p, const double *__restrict__ conn_T,
     const double *__restrict__ conn_m, double ghz, int upwind, double *__restrict__ F, JacOut J) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y, k = blockIdx.z;
-    if (i >= nx) return;
-    const int nxy = nx * ny;
-    const int n = i + nx * (j + ny * k);
-    const double pn = p[n], mn = m[n], dmn = dm[n];
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, nxy = nx * ny;
+    if (n >= nxy * nz) return;
+    const int row = n / nx, i = n - row * nx, k = row / ny, j = row - k * ny;
+    const double pn = p[n], mh = m[n], dmh = WANT_J ? dm[n] : 0.0;
     double f = F[n];
     double jc = WANT_J ? J.c[0][n] : 0.0;
     double jn[6] = {0, 0, 0, 0, 0, 0};
@@ -401,16 +481,25 @@ __global__ void __launch_bounds__(128) k_flux(
     // gz: +1 towards the deeper neighbour (+z), -1 towards the shallower, 0 level faces
     // face mobility: the mean, or the upstream cell's (weights wn, wq of m_n, m_q)
     auto face = [&](double T, int q, int slot, double gz) {
-        const double mq = m[q], mbar = 0.5 * (mn + mq);
-        const double gh = gz * ghz;
-        const double dphi = (pn - p[q]) + gh * mbar;
-        const bool up_n = dphi >= 0.0;
-        const double mf = upwind ? (up_n ? mn : mq) : mbar;
-        const double wn = upwind ? (up_n ? 1.0 : 0.0) : 0.5, wq = upwind ? 1.0 - wn : 0.5;
-        f += T * mf * dphi;
-        if (WANT_J) {
-            jc += T * (wn * dmn * dphi + mf * (1.0 + 0.5 * gh * dmn));
-            jn[slot] = T * (wq * dm[q] * dphi + mf * (-1.0 + 0.5 * gh * dm[q]));
+        const double mbar = mh + m[q], dp = pn - p[q];
+        if constexpr (!GEN) {
+            const double t = T * mbar, u = T * dp;
+            f = fma(t, dp, f);
+            if (WANT_J) {
+                jc += fma(u, dmh, t);
+                jn[slot] = fma(u, dm[q], -t);
+            }
+        } else {
+            const double gh = gz * ghz;
+            const double dphi = dp + gh * mbar;
+            const bool up_n = dphi >= 0.0;
+            const double mf = upwind ? 2.0 * (up_n ? mh : m[q]) : mbar;
+            const double wn = upwind ? (up_n ? 2.0 : 0.0) : 1.0, wq = upwind ? 2.0 - wn : 1.0;   // of dm / 2
+            f += T * mf * dphi;
+            if (WANT_J) {
+                jc += T * (wn * dmh * dphi + mf * (1.0 + gh * dmh));
+                jn[slot] = T * (wq * dm[q] * dphi + mf * (-1.0 + gh * dm[q]));
+            }
         }
     };
     if (i < nx - 1) face(Tx[n], n + 1, 1, 0.0);
@@ -420,7 +509,7 @@ __global__ void __launch_bounds__(128) k_flux(
     if (k < nz - 1) face(Tz[n], n + nxy, 5, 1.0);
     if (k > 0) face(Tz[n - nxy], n - nxy, 4, -1.0);
     for (int q = conn_ptr[n]; q < conn_ptr[n + 1]; ++q) {
-        const double dp = pn - conn_p[q];
+        const double dp = pn - conn_p[q], mn = 2.0 * mh, dmn = 2.0 * dmh;
         const double mf = upwind ? (dp >= 0.0 ? mn : conn_m[q]) : 0.5 * (mn + conn_m[q]);
         const double wn = upwind ? (dp >= 0.0 ? 1.0 : 0.0) : 0.5;
         f += conn_T[q] * mf * dp;
@@ -673,17 +762,13 @@ int residual_eval_impl(ras_problem *P, const double *p, const double *pl, const 
                                                    J ? J[0] : nullptr, P->eos_m, P->eos_dm,
                                                    P->noroot_d, P->conservative, P->rateQ);
     RAS_LAUNCHED();
-    const int t = stencil_threads(P->nx);
-    const dim3 g = stencil_grid(P->nx, P->ny, P->nz, t);
     JacOut jo;
     for (int s = 0; s < 7; ++s) jo.c[s] = J ? J[s] : nullptr;
-    if (J) {
-        k_flux<true><<<g, t, 0, st>>>(P->nx, P->ny, P->nz, p, P->eos_m, P->eos_dm, P->Tx, P->Ty,
-                                      P->Tz, P->conn_ptr, P->conn_p, P->conn_T, P->conn_m, P->ghz, P->upwind, F, jo);
-    } else {
-        k_flux<false><<<g, t, 0, st>>>(P->nx, P->ny, P->nz, p, P->eos_m, P->eos_dm, P->Tx, P->Ty,
-                                       P->Tz, P->conn_ptr, P->conn_p, P->conn_T, P->conn_m, P->ghz, P->upwind, F, jo);
-    }
+    const int g = (P->N + 255) / 256;
+    const bool gen = P->upwind != 0 || P->ghz != 0.0;
+    auto *kern = J ? (gen ? k_flux<true, true> : k_flux<true, false>) : (gen ? k_flux<false, true> : k_flux<false, false>);
+    kern<<<g, 256, 0, st>>>(P->nx, P->ny, P->nz, p, P->eos_m, P->eos_dm, P->Tx, P->Ty, P->Tz, P->conn_ptr, P->conn_p,
+                            P->conn_T, P->conn_m, P->ghz, P->upwind, F, jo);
     RAS_LAUNCHED();
     return RAS_OK;
 }
