@@ -142,6 +142,11 @@ template <int PREC>
 __global__ void __launch_bounds__(512) k_ras125_factor(Fac125 P) {
     extern __shared__ int posq[];                 // natural local index -> level-order row
     __shared__ Shape125 sh;
+    // pivot slot s and this lane's offsets lane + 32 r: the slot of the pivot's U row that
+    // the offset's column takes, or -1 (the same for every row; computing it per pivot was
+    // most of the instructions), and the pivot's natural distance
+    __shared__ char4 umap[64][32];
+    __shared__ int sdm[64];
     const Sub125 si = P.subs[blockIdx.x];
     copy_shape(sh, P.shapes[si.shape]);
     __syncthreads();
@@ -167,6 +172,20 @@ __global__ void __launch_bounds__(512) k_ras125_factor(Fac125 P) {
         od[r] = ox[r] + bx * oy[r] + bxy * oz[r];
     }
     const int nL = sh.nL;
+    for (int s = wid; s < nL; s += nw) {
+        const int om = sh.lowo[s], mx = off_dx(om), my = off_dy(om), mz = off_dz(om);
+        const int dm = mx + bx * my + bxy * mz;
+        signed char t[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int cx = ox[r] - mx, cy = oy[r] - my, cz = oz[r] - mz;
+            t[r] = live[r] && od[r] > dm && cx >= -2 && cx <= 2 && cy >= -2 && cy <= 2 && cz >= -2 && cz <= 2
+                       ? sh.uslot[off_enc(cx, cy, cz)] : (signed char)-1;
+        }
+        umap[s][lane] = make_char4(t[0], t[1], t[2], t[3]);
+        if (lane == 0) sdm[s] = dm;
+    }
+    __syncthreads();
     double *work = P.work + si.foff * RREC;
     auto inbox = [&](int i, int j, int k) {
         return (unsigned)i < (unsigned)bx && (unsigned)j < (unsigned)by && (unsigned)k < (unsigned)bz;
@@ -210,23 +229,16 @@ __global__ void __launch_bounds__(512) k_ras125_factor(Fac125 P) {
                 if (m1) { const int s = 31 + __ffs(m1); m1 &= m1 - 1; return s; }
                 return -1;
             };
-            struct Pivot { int om; unsigned need; double pinv; double u[4]; };
+            struct Pivot { int om; double pinv; double u[4]; };
             auto fetch = [&](int s, Pivot &f) {
-                const int om = sh.lowo[s];
-                const int mx = off_dx(om), my = off_dy(om), mz = off_dz(om);
-                const int dm = mx + bx * my + bxy * mz;
-                const double *wr = work + (long long)posq[n + dm] * RREC;
-                f.om = om;
-                f.need = 0;
+                const double *wr = work + (long long)posq[n + sdm[s]] * RREC;
+                const char4 t = umap[s][lane];
+                f.om = sh.lowo[s];
                 f.pinv = wr[RREC - 1];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int cx = ox[r] - mx, cy = oy[r] - my, cz = oz[r] - mz;
-                    const bool need = pat[r] && od[r] > dm && cx >= -2 && cx <= 2 && cy >= -2 &&
-                                      cy <= 2 && cz >= -2 && cz <= 2;
-                    f.u[r] = need ? wr[sh.uslot[off_enc(cx, cy, cz)]] : 0.0;
-                    if (need) f.need |= 1u << r;
-                }
+                f.u[0] = pat[0] && t.x >= 0 ? wr[t.x] : 0.0;
+                f.u[1] = pat[1] && t.y >= 0 ? wr[t.y] : 0.0;
+                f.u[2] = pat[2] && t.z >= 0 ? wr[t.z] : 0.0;
+                f.u[3] = pat[3] && t.w >= 0 ? wr[t.w] : 0.0;
             };
             // pivots in order, their U rows fetched PD pivots ahead (register ring)
             Pivot pb[PD];
@@ -254,8 +266,7 @@ __global__ void __launch_bounds__(512) k_ras125_factor(Fac125 P) {
                         else w[3] = lm;
                     }
 #pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        if (cur.need & (1u << r)) w[r] -= lm * cur.u[r];
+                    for (int r = 0; r < 4; ++r) w[r] -= lm * cur.u[r];   // (0 off the pattern)
                 }
             }
             const double piv = __shfl_sync(0xffffffffu, w[1], CENTRE125 - 32);
@@ -298,7 +309,7 @@ struct App125 {
     double *z;
     int nx, ny, nz;
     int accumulate;
-    int ycap;
+    int ycap, guard;
 };
 
 // z = sum_i (R_i^0)^T U_i^{-1} L_i^{-1} R_i^delta r with, per row (one warp),
@@ -307,12 +318,17 @@ struct App125 {
 // lane t taking the couplings of slots t and t + 32 (slot 63 of the backward
 // record holds 1/u_nn). Accumulation in FP64 (64) or FP32 (32, 16). Each
 // warp's first row of a level is loaded AD levels ahead (register ring).
-template <int PREC>
+// Bound: ~110 dependent levels per sweep of a 10^3 box, each the instruction stream of one
+// row. GUARD: the vector has zeros on either side as far as the couplings reach (guard
+// cells), a coupling leaving the box has factor value 0, and no row tests its 62 couplings
+// against the box: that was most of a row's instructions. Without room for the guard (large
+// flat boxes) every coupling is tested; the values are the same.
+template <int PREC, bool GUARD>
 __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
     using Acc = typename Val125<PREC>::Acc;
     extern __shared__ __align__(16) unsigned char smem[];
-    Acc *Y = reinterpret_cast<Acc *>(smem);
-    int *lvl_s = reinterpret_cast<int *>(smem + (size_t)P.ycap * sizeof(Acc));
+    Acc *Y = reinterpret_cast<Acc *>(smem) + P.guard;
+    int *lvl_s = reinterpret_cast<int *>(smem + ((size_t)P.ycap + 2 * P.guard) * sizeof(Acc));
     __shared__ Shape125 sh;
     const Sub125 si = P.subs[blockIdx.x];
     copy_shape(sh, P.shapes[si.shape]);
@@ -323,6 +339,8 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
     const int nx = P.nx;
     const long long nxy = (long long)P.nx * P.ny;
     const long long g0 = si.e0x + nx * (long long)si.e0y + nxy * si.e0z;
+    if (GUARD)
+        for (int t = threadIdx.x; t < P.guard; t += blockDim.x) Y[-1 - t] = Y[sh.ncell + t] = (Acc)0;
     for (int t = threadIdx.x; t < sh.ncell; t += blockDim.x) {
         const int i = t % bx, j = (t / bx) % by, k = t / bxy;
         Y[t] = (Acc)__ldg(P.r + g0 + i + nx * (long long)j + nxy * k);
@@ -340,6 +358,10 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
         ld[h] = lx[h] + bx * ly[h] + bxy * lz[h];
         ux[h] = off_dx(ou); uy[h] = off_dy(ou); uz[h] = off_dz(ou);
         ud[h] = ux[h] + bx * uy[h] + bxy * uz[h];
+        if (GUARD) {   // couplings longer than the box never hold: read the cell itself
+            if (abs(lx[h]) >= bx || abs(ly[h]) >= by || abs(lz[h]) >= bz) ld[h] = 0;
+            if (abs(ux[h]) >= bx || abs(uy[h]) >= by || abs(uz[h]) >= bz) ud[h] = 0;
+        }
     }
     auto inbox = [&](int i, int j, int k) {
         return (unsigned)i < (unsigned)bx && (unsigned)j < (unsigned)by && (unsigned)k < (unsigned)bz;
@@ -349,8 +371,10 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
     __syncthreads();
 
     // the first row of each level for this warp, fetched AD levels ahead
+    const typename Val125<PREC>::T *fw = reinterpret_cast<const typename Val125<PREC>::T *>(P.fwd) + fbase + lane;
+    const typename Val125<PREC>::T *bw = reinterpret_cast<const typename Val125<PREC>::T *>(P.bwd) + fbase + lane;
     struct Row { int q; unsigned e; Acc v0, v1; };
-    auto fetch = [&](int l, const void *rec) {
+    auto fetch = [&](int l, const typename Val125<PREC>::T *rec) {
         Row rw;
         rw.q = -1;
         rw.e = 0;
@@ -358,11 +382,10 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
         if (l >= 0 && l < sh.nlev) {
             const int q = lvl_s[l] + wid;
             if (q < lvl_s[l + 1]) {
-                const long long rb = fbase + (long long)q * RREC;
                 rw.q = q;
                 rw.e = __ldg(cells + q);
-                rw.v0 = load_val<PREC>(rec, rb + lane);
-                rw.v1 = load_val<PREC>(rec, rb + lane + 32);
+                rw.v0 = load_val<PREC>(rec, q * RREC);
+                rw.v1 = load_val<PREC>(rec, q * RREC + 32);
             }
         }
         return rw;
@@ -372,8 +395,13 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
         const int i = e & 255u, j = (e >> 8) & 255u, k = (e >> 16) & 255u;
         const int n = i + bx * j + bxy * k;
         Acc acc = 0;
-        if (lv[0] && inbox(i + lx[0], j + ly[0], k + lz[0])) acc += a0 * Y[n + ld[0]];
-        if (lv[1] && inbox(i + lx[1], j + ly[1], k + lz[1])) acc += a1 * Y[n + ld[1]];
+        if (GUARD) {
+            acc = a0 * Y[n + ld[0]];
+            if (lv[1]) acc += a1 * Y[n + ld[1]];
+        } else {
+            if (lv[0] && inbox(i + lx[0], j + ly[0], k + lz[0])) acc += a0 * Y[n + ld[0]];
+            if (lv[1] && inbox(i + lx[1], j + ly[1], k + lz[1])) acc += a1 * Y[n + ld[1]];
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) Y[n] -= acc;
@@ -383,8 +411,13 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
         const int i = e & 255u, j = (e >> 8) & 255u, k = (e >> 16) & 255u;
         const int n = i + bx * j + bxy * k;
         Acc acc = 0;
-        if (lv[0] && inbox(i + ux[0], j + uy[0], k + uz[0])) acc += b0 * Y[n + ud[0]];
-        if (lv[1] && inbox(i + ux[1], j + uy[1], k + uz[1])) acc += b1 * Y[n + ud[1]];
+        if (GUARD) {
+            acc = b0 * Y[n + ud[0]];
+            if (lv[1]) acc += b1 * Y[n + ud[1]];
+        } else {
+            if (lv[0] && inbox(i + ux[0], j + uy[0], k + uz[0])) acc += b0 * Y[n + ud[0]];
+            if (lv[1] && inbox(i + ux[1], j + uy[1], k + uz[1])) acc += b1 * Y[n + ud[1]];
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         const Acc dinv = __shfl_sync(0xffffffffu, b1, 31);
@@ -393,38 +426,34 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
 
     Row ring[AD];
 #pragma unroll
-    for (int u = 0; u < AD; ++u) ring[u] = fetch(u, P.fwd);
+    for (int u = 0; u < AD; ++u) ring[u] = fetch(u, fw);
     for (int lb = 0; lb < sh.nlev; lb += AD) {
 #pragma unroll
         for (int u = 0; u < AD; ++u) {
             const int l = lb + u;
             if (l < sh.nlev) {
                 const Row cur = ring[u];
-                ring[u] = fetch(l + AD, P.fwd);
+                ring[u] = fetch(l + AD, fw);
                 if (cur.q >= 0) fwd_row(cur.e, cur.v0, cur.v1);
                 for (int q = lvl_s[l] + wid + nw; q < lvl_s[l + 1]; q += nw) {
-                    const long long rb = fbase + (long long)q * RREC;
-                    fwd_row(__ldg(cells + q), load_val<PREC>(P.fwd, rb + lane),
-                            load_val<PREC>(P.fwd, rb + lane + 32));
+                    fwd_row(__ldg(cells + q), load_val<PREC>(fw, q * RREC), load_val<PREC>(fw, q * RREC + 32));
                 }
                 __syncthreads();
             }
         }
     }
 #pragma unroll
-    for (int u = 0; u < AD; ++u) ring[u] = fetch(sh.nlev - 1 - u, P.bwd);
+    for (int u = 0; u < AD; ++u) ring[u] = fetch(sh.nlev - 1 - u, bw);
     for (int lb = 0; lb < sh.nlev; lb += AD) {
 #pragma unroll
         for (int u = 0; u < AD; ++u) {
             const int l = sh.nlev - 1 - (lb + u);
             if (l >= 0) {
                 const Row cur = ring[u];
-                ring[u] = fetch(l - AD, P.bwd);
+                ring[u] = fetch(l - AD, bw);
                 if (cur.q >= 0) bwd_row(cur.e, cur.v0, cur.v1);
                 for (int q = lvl_s[l] + wid + nw; q < lvl_s[l + 1]; q += nw) {
-                    const long long rb = fbase + (long long)q * RREC;
-                    bwd_row(__ldg(cells + q), load_val<PREC>(P.bwd, rb + lane),
-                            load_val<PREC>(P.bwd, rb + lane + 32));
+                    bwd_row(__ldg(cells + q), load_val<PREC>(bw, q * RREC), load_val<PREC>(bw, q * RREC + 32));
                 }
                 __syncthreads();
             }
@@ -654,6 +683,14 @@ int ras125_setup(Ras125 &R, int nx, int ny, int nz, int px, int py, int pz, int 
     const size_t acc = prec == 64 ? 8 : 4;
     R.ycap = (ycap + 3) & ~3;
     R.smem_apply = (size_t)R.ycap * acc + (size_t)lcap * sizeof(int);
+    // guard of the solves' vector: the longest coupling that some cell of a box has
+    int guard = 0;
+    for (const Shape125 &sh : R.shapes)
+        guard = std::max(guard, std::min(2, sh.bx - 1) + sh.bx * std::min(2, sh.by - 1) +
+                                    sh.bx * sh.by * std::min(2, sh.bz - 1));
+    guard = (guard + 3) & ~3;
+    R.guard = R.smem_apply + 2 * (size_t)guard * acc <= (size_t)SMEM125_MAX ? guard : -1;
+    if (R.guard > 0) R.smem_apply += 2 * (size_t)R.guard * acc;
     R.smem_factor = (size_t)ycap * sizeof(int);
     if (R.smem_apply > (size_t)SMEM125_MAX || R.smem_factor > (size_t)SMEM125_MAX) return RAS_EINVAL;
     const size_t esz = prec == 64 ? 8 : (prec == 32 ? 4 : 2);
@@ -688,13 +725,16 @@ int ras125_setup(Ras125 &R, int nx, int ny, int nz, int px, int py, int pz, int 
     const int big = SMEM125_MAX;
     if (prec == 64) {
         RAS_CK(cudaFuncSetAttribute(k_ras125_factor<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     } else if (prec == 32) {
         RAS_CK(cudaFuncSetAttribute(k_ras125_factor<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     } else {
         RAS_CK(cudaFuncSetAttribute(k_ras125_factor<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     }
     return RAS_OK;
 }
@@ -740,9 +780,12 @@ int ras125_apply(Ras125 &R, const double *r, double *z, int accumulate, cudaStre
     P.nx = R.nx; P.ny = R.ny; P.nz = R.nz; P.accumulate = accumulate;
     P.ycap = R.ycap;
     const int threads = 32 * R.nwarps;
-    if (R.prec == 64) k_ras125_apply<64><<<R.nsub, threads, R.smem_apply, st>>>(P);
-    else if (R.prec == 32) k_ras125_apply<32><<<R.nsub, threads, R.smem_apply, st>>>(P);
-    else k_ras125_apply<16><<<R.nsub, threads, R.smem_apply, st>>>(P);
+    P.guard = std::max(R.guard, 0);
+    auto run = [&](auto kernel) { kernel<<<R.nsub, threads, R.smem_apply, st>>>(P); };
+    const bool g = R.guard >= 0;
+    if (R.prec == 64) g ? run(k_ras125_apply<64, true>) : run(k_ras125_apply<64, false>);
+    else if (R.prec == 32) g ? run(k_ras125_apply<32, true>) : run(k_ras125_apply<32, false>);
+    else g ? run(k_ras125_apply<16, true>) : run(k_ras125_apply<16, false>);
     RAS_LAUNCHED();
     return RAS_OK;
 }

@@ -39,6 +39,7 @@ struct Ras125 {
     int nx = 0, ny = 0, nz = 0, N = 0;
     int prec = 64;
     int nsub = 0, nwarps = 8, ycap = 0, lcap = 0;
+    int guard = -1;                      // zeros on either side of the solves' vector (-1: none, tested couplings)
     long long nrow = 0;                  // factor rows (sum of box cells)
     size_t smem_apply = 0, smem_factor = 0;
     std::vector<Sub125> subs;
