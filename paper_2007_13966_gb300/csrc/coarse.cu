@@ -451,25 +451,26 @@ __host__ __device__ __forceinline__ int nbr_index(const CGeom &G, int I, int o) 
     return x + G.cx * (y + G.cy * z);
 }
 
-// D_k = within-block entries of A_c; identity on padding positions
+// D_k = within-block entries of A_c; identity on padding positions. A thread per block
+// position and offset (a thread per position, looping over its 125 offsets, took 54 us
+// whatever the size).
 template <typename AT>
-__global__ void k_assemble(const AT *__restrict__ Ac, const int *__restrict__ pos,
-                           const int *__restrict__ cell, CGeom G, AT *__restrict__ D) {
-    const long long tot = (long long)G.nb * G.T;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < tot;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(p / G.T), r = (int)(p % G.T);
-        AT *Dk = D + (long long)k * G.T * G.T;
-        const int I = cell[p];
-        if (I < 0) { Dk[(long long)r * G.T + r] = (AT)1; continue; }
-        for (int o = 0; o < 125; ++o) {
-            const int J = nbr_index(G, I, o);
-            if (J < 0) continue;
-            const int pj = pos[J];
-            if (pj / G.T != k) continue;
-            Dk[(long long)r * G.T + (pj % G.T)] = Ac[(long long)o * G.Nc + I];
-        }
+__global__ void __launch_bounds__(256) k_assemble(const AT *__restrict__ Ac, const int *__restrict__ pos,
+                                                  const int *__restrict__ cell, CGeom G, AT *__restrict__ D) {
+    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const int o = blockIdx.y;
+    if (p >= (long long)G.nb * G.T) return;
+    const int k = (int)(p / G.T), r = (int)(p % G.T);
+    AT *Dr = D + ((long long)k * G.T + r) * G.T;
+    const int I = cell[p];
+    if (I < 0) {
+        if (o == 0) Dr[r] = (AT)1;
+        return;
     }
+    const int J = nbr_index(G, I, o);
+    if (J < 0) return;
+    const int c = pos[J] - k * G.T;
+    if (c >= 0 && c < G.T) Dr[c] = Ac[(long long)o * G.Nc + I];
 }
 
 // pivot / target block of edge e (see the header)
@@ -479,46 +480,45 @@ __host__ __device__ __forceinline__ int edge_target(int e, int mid) { return e <
 // ELL forms of the couplings across edge e:
 //   row ELL: rows of the target block -> (column in the pivot block, A_c value)  [A(target, pivot)]
 //   col ELL: columns of the target block -> (row in the pivot block, A_c value)  [A(pivot, target), by column]
+// A warp per row of a target block, its lanes over the offsets (32 at a time, entries placed
+// in ascending offset order by ballot ranks): a thread per row took 86 us whatever the size.
 template <typename AT>
-__global__ void k_ell(const AT *__restrict__ Ac, const int *__restrict__ pos,
-                      const int *__restrict__ cell, CGeom G, int *__restrict__ lo_q,
-                      AT *__restrict__ lo_v, int *__restrict__ up_q, AT *__restrict__ up_v,
-                      int *__restrict__ lo_n, int *__restrict__ up_n, int *__restrict__ err) {
-    const long long tot = (long long)(G.nb - 1) * G.T;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < tot;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int e = (int)(p / G.T);
-        const int pv = edge_pivot(e, G.mid), tg = edge_target(e, G.mid);
-        const int I = cell[(long long)tg * G.T + p % G.T];   // row of the target block
-        int nl = 0, nu = 0;
-        if (I >= 0) {
-            for (int o = 0; o < 125; ++o) {
-                const int J = nbr_index(G, I, o);
-                if (J < 0) continue;
-                const int pj = pos[J];
-                if (pj / G.T != pv) continue;
-                if (nl < ELLW) {   // A(target, pivot)[I][J] (offset o of row I)
-                    lo_q[p * ELLW + nl] = pj % G.T;
-                    lo_v[p * ELLW + nl] = Ac[(long long)o * G.Nc + I];
-                }
-                ++nl;
-                if (nu < ELLW) {   // A(pivot, target)[J][I] (offset -o of row J), [e][T] layout
-                    const long long u = (long long)e * ELLW * G.T + (long long)nu * G.T + (p % G.T);
-                    up_q[u] = pj % G.T;
-                    up_v[u] = Ac[(long long)(124 - o) * G.Nc + J];
-                }
-                ++nu;
+__global__ void __launch_bounds__(256) k_ell(const AT *__restrict__ Ac, const int *__restrict__ pos,
+                                             const int *__restrict__ cell, CGeom G, int *__restrict__ lo_q,
+                                             AT *__restrict__ lo_v, int *__restrict__ up_q, AT *__restrict__ up_v,
+                                             int *__restrict__ lo_n, int *__restrict__ up_n, int *__restrict__ err) {
+    const long long p = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (p >= (long long)(G.nb - 1) * G.T) return;
+    const int e = (int)(p / G.T), c = (int)(p % G.T);
+    const int pv = edge_pivot(e, G.mid), tg = edge_target(e, G.mid);
+    const int I = cell[(long long)tg * G.T + c];         // row of the target block
+    const long long ub = (long long)e * ELLW * G.T + c;  // [e][ELLW][T] layout of the column form
+    int n = 0;
+    if (I >= 0) {
+        for (int o0 = 0; o0 < 125; o0 += 32) {
+            const int o = o0 + lane;
+            const int J = o < 125 ? nbr_index(G, I, o) : -1;
+            const int q = J >= 0 ? pos[J] - pv * G.T : -1;
+            const bool in = q >= 0 && q < G.T;
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            const int at = n + __popc(m & ((1u << lane) - 1u));
+            if (in && at < ELLW) {
+                lo_q[p * ELLW + at] = q;                 // A(target, pivot)[I][J] (offset o of row I)
+                lo_v[p * ELLW + at] = Ac[(long long)o * G.Nc + I];
+                up_q[ub + (long long)at * G.T] = q;      // A(pivot, target)[J][I] (offset -o of row J)
+                up_v[ub + (long long)at * G.T] = Ac[(long long)(124 - o) * G.Nc + J];
             }
+            n += __popc(m);
         }
-        if (nl > ELLW || nu > ELLW) atomicExch(err, ERR_ELL);
-        lo_n[p] = min(nl, ELLW);
-        up_n[p] = min(nu, ELLW);
-        for (int q = min(nl, ELLW); q < ELLW; ++q) { lo_q[p * ELLW + q] = 0; lo_v[p * ELLW + q] = 0; }
-        for (int q = min(nu, ELLW); q < ELLW; ++q) {
-            const long long u = (long long)e * ELLW * G.T + (long long)q * G.T + (p % G.T);
-            up_q[u] = 0;
-            up_v[u] = 0;
-        }
+    }
+    if (lane == 0) {
+        if (n > ELLW) atomicExch(err, ERR_ELL);
+        lo_n[p] = up_n[p] = min(n, ELLW);
+    }
+    for (int at = min(n, ELLW) + lane; at < ELLW; at += 32) {
+        lo_q[p * ELLW + at] = up_q[ub + (long long)at * G.T] = 0;
+        lo_v[p * ELLW + at] = up_v[ub + (long long)at * G.T] = (AT)0;
     }
 }
 
@@ -2735,10 +2735,10 @@ static int assemble_blocks_t(Coarse *c, cudaStream_t st) {
     AT *Ac = (AT *)c->Ac, *D = (AT *)c->D;
     const size_t bsz = (size_t)c->T * c->T;
     RAS_CK(cudaMemsetAsync(D, 0, c->nb * bsz * sizeof(AT), st));
-    k_assemble<AT><<<grid_of((long long)c->nb * c->T), 256, 0, st>>>(Ac, c->d_pos, c->d_cell, G, D);
+    k_assemble<AT><<<dim3((unsigned)(((long long)c->nb * c->T + 255) / 256), 125), 256, 0, st>>>(Ac, c->d_pos, c->d_cell, G, D);
     RAS_LAUNCHED();
     if (c->nb > 1) {
-        k_ell<AT><<<grid_of((long long)(c->nb - 1) * c->T), 256, 0, st>>>(
+        k_ell<AT><<<(unsigned)(((long long)(c->nb - 1) * c->T + 7) / 8), 256, 0, st>>>(
             Ac, c->d_pos, c->d_cell, G, c->lo_q, (AT *)c->lo_v, c->up_q, (AT *)c->up_v, c->lo_n,
             c->up_n, c->d_err);
         RAS_LAUNCHED();
