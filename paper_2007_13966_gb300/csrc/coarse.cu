@@ -61,6 +61,7 @@ struct Coarse {
     double *d_wa[3] = {}, *d_wb[3] = {};
     int *d_lo[3] = {}, *d_hi[3] = {};
     double *d_wt[3] = {};           // per coarse index: the weights of its fine support (w1's values)
+    double *d_ww[3] = {};           // per coarse index: the Galerkin product's pair weights [5][5][wmax]
     int af, am, as;                 // axis order: fastest, middle, slowest
     int T = 0, nb = 0;              // block size (multiple of TILE), number of blocks
     int mid = 0;                    // middle block of the two-ended elimination
@@ -102,6 +103,7 @@ struct Interp {
     const double *wa[3], *wb[3];
     const int *lo[3], *hi[3];
     const double *wt[3];   // [I][m]: P(lo[I] + m, I), m < W (the same values as w1)
+    const double *ww[3];   // [I][d][t][m]: P(lo[I] + m, I) P(lo[I] + m + t - 2, I + d - 2), m < W (0 outside)
     int W[3];
 };
 
@@ -208,33 +210,35 @@ __global__ void __launch_bounds__(256) k_rap(Stencil7 A, Interp P, CGeom G, RapD
 
     const int I = blockIdx.x;
     const int Ic[3] = {I % G.cx, (I / G.cx) % G.cy, I / (G.cx * G.cy)};
-    const int cdim[3] = {G.cx, G.cy, G.cz};
-    const int ndim[3] = {G.nx, G.ny, G.nz};
     const int lo[3] = {P.lo[0][Ic[0]], P.lo[1][Ic[1]], P.lo[2][Ic[2]]};
     const int wx = P.hi[0][Ic[0]] - lo[0], wy = P.hi[1][Ic[1]] - lo[1], wz = P.hi[2][Ic[2]] - lo[2];
     const int box = wx * wy * wz;
     const long long nxy = (long long)G.nx * G.ny;
     rap_tables(uix, vix, wx, wy, WX);
 
-    for (int e = threadIdx.x; e < 7 * box; e += blockDim.x) {
-        const int s = e / box, q = e % box;
-        const int ax = q % wx, ay = (q / wx) % wy, az = q / (wx * wy);
-        const long long g = (lo[0] + ax) + (long long)G.nx * (lo[1] + ay) + nxy * (lo[2] + az);
-        const double *src = s == 0 ? A.c[0] : s == 1 ? A.c[1] : s == 2 ? A.c[2] : s == 3 ? A.c[3]
-                          : s == 4 ? A.c[4] : s == 5 ? A.c[5] : A.c[6];   // no indexed parameter copy
-        Abox[((s * WZ + az) * WY + ay) * WX + ax] = (AT)src[g];
+    // the seven terms' support boxes: a cell's places are computed once for the seven
+    // (divisions per value were most of the kernel's instructions)
+    const long long gl = lo[0] + (long long)G.nx * lo[1] + nxy * lo[2];
+    const int vol = WZ * WY * WX;
+    for (int q = threadIdx.x; q < box; q += blockDim.x) {
+        const int row = q / wx, ax = q - row * wx, az = row / wy, ay = row - az * wy;
+        const long long g = gl + ax + (long long)G.nx * ay + nxy * az;
+        AT *dst = Abox + (az * WY + ay) * WX + ax;
+        double v[7];
+#pragma unroll
+        for (int s = 0; s < 7; ++s) v[s] = __ldg(A.c[s] + g);
+#pragma unroll
+        for (int s = 0; s < 7; ++s) dst[s * vol] = (AT)v[s];
     }
-    // pair weights W[axis][d][s][a] = P(a, I) P(a + s, I + d)
-    for (int e = threadIdx.x; e < 45 * WM; e += blockDim.x) {
-        const int q = e % WM, si = (e / WM) % 3, d = (e / (3 * WM)) % 5, axis = e / (15 * WM);
-        const int wa = axis == 0 ? wx : (axis == 1 ? wy : wz);
-        double w = 0.0;
-        if (q < wa) {
-            const int a = lo[axis] + q, as = a + si - 1, J = Ic[axis] + d - 2;
-            if (J >= 0 && J < cdim[axis] && as >= 0 && as < ndim[axis])
-                w = w1(P, axis, a, Ic[axis]) * w1(P, axis, as, J);
+    // pair weights W[axis][d][s][a] = P(a, I) P(a + s, I + d) from the tables of each axis
+#pragma unroll
+    for (int axis = 0; axis < 3; ++axis) {
+        const int W1 = P.W[axis];
+        const double *src = P.ww[axis] + (long long)Ic[axis] * 25 * W1;
+        for (int e = threadIdx.x; e < 15 * W1; e += blockDim.x) {
+            const int ds = e / W1, d = ds / 3, t = ds - 3 * d + 1;
+            Wt[(axis * 15 + ds) * WM + e - ds * W1] = (AT)__ldg(src + (d * 5 + t) * W1 + e - ds * W1);
         }
-        Wt[e] = (AT)w;
     }
     if (threadIdx.x < 125) out[threadIdx.x] = 0;
     __syncthreads();
@@ -434,6 +438,88 @@ __global__ void __launch_bounds__(256) k_rap125(const double *__restrict__ Af, I
         }
     }
     if (threadIdx.x < 125) Ac[(long long)threadIdx.x * G.Nc + I] = out[threadIdx.x];
+}
+
+// The same when the support boxes of all 125 offsets fit in shared memory (ratio 2): the
+// sum over offsets t = (tx, ty, tz) is factorised too, each pass summing over one component,
+//     U[ty, tx][dz] = sum_tz Wz(tz) A_t,  V[tx][dz, dy] = sum_ty Wy(ty) U[ty, tx],
+//     out[dz, dy, dx] = sum_tx Wx(tx) V[tx],
+// so that a coarse row takes three barrier-separated passes of 2,000, 500 and 125 sums where
+// offset by offset it takes 3 x 81 passes of about 100 sums (half the operations, and the
+// barriers bounded it: 2.0 ms on 15 x 55 x 22 coarse cells, 7 % of a three-level step
+// there). The FP32 error against FP64 halves (rms 3.3e-8 of the largest entry for 6.5e-8):
+// a value is the end of 15 sums instead of 81 terms added up.
+static size_t rap125_all_smem(const int w[3], size_t esz) {
+    const size_t WX = w[0], WY = w[1], WZ = w[2], WM = std::max(WX, std::max(WY, WZ));
+    return esz * (125 * WX * WY * WZ + 75 * WM + 125 * WY * WX + 125 * WX) + sizeof(int) * (5 * WY * WX + 25 * WX);
+}
+template <typename AT>
+__global__ void __launch_bounds__(256) k_rap125_all(const double *__restrict__ Af, Interp P, CGeom G, RapDims W,
+                                                    AT *__restrict__ Ac) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int WX = W.wx, WY = W.wy, WZ = W.wz, WM = max(WX, max(WY, WZ)), plane = WY * WX, vol = plane * WZ;
+    AT *Abox = reinterpret_cast<AT *>(smem_raw);     // [125][WZ][WY][WX]
+    AT *Wt = Abox + 125 * vol;                       // [3][5 d][5 t][WM]
+    AT *U = Wt + 75 * WM;                            // [25][5][WY][WX]
+    AT *V = U + 125 * plane;                         // [5][25][WX]
+    int *uix = reinterpret_cast<int *>(V + 125 * WX);
+    int *vix = uix + 5 * plane;
+    const int I = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    const int Ic[3] = {I % G.cx, (I / G.cx) % G.cy, I / (G.cx * G.cy)};
+    const int lo[3] = {P.lo[0][Ic[0]], P.lo[1][Ic[1]], P.lo[2][Ic[2]]};
+    const int wx = P.hi[0][Ic[0]] - lo[0], wy = P.hi[1][Ic[1]] - lo[1], wz = P.hi[2][Ic[2]] - lo[2];
+    const int box = wx * wy * wz, nU = 5 * wy * wx, nV = 25 * wx;
+    const long long nxy = (long long)G.nx * G.ny, Nf = nxy * G.nz;
+    const long long gl = lo[0] + (long long)G.nx * lo[1] + nxy * lo[2];
+    rap_tables(uix, vix, wx, wy, WX);
+#pragma unroll
+    for (int axis = 0; axis < 3; ++axis) {
+        const int W1 = P.W[axis];
+        const double *src = P.ww[axis] + (long long)Ic[axis] * 25 * W1;
+        for (int e = tid; e < 25 * W1; e += nt) {
+            const int dt = e / W1;
+            Wt[(axis * 25 + dt) * WM + e - dt * W1] = (AT)__ldg(src + e);
+        }
+    }
+    // a thread keeps one cell of the box and walks over the offsets
+    const int per = max(1, nt / box), t0 = tid / box;
+    for (int q = tid - t0 * box; q < box && t0 < per; q += nt) {
+        const int row = q / wx, ax = q - row * wx, az = row / wy, ay = row - az * wy;
+        const double *src = Af + gl + ax + (long long)G.nx * ay + nxy * az;
+        AT *dst = Abox + (az * WY + ay) * WX + ax;
+#pragma unroll 8
+        for (int t = t0; t < 125; t += per) dst[t * vol] = (AT)__ldg(src + t * Nf);
+    }
+    __syncthreads();
+    for (int e = tid; e < 25 * nU; e += nt) {
+        const int tyx = e / nU, code = uix[e - tyx * nU], dz = code >> 16, ab = code & 0xffff;
+        AT acc = 0;
+        for (int tz = 0; tz < 5; ++tz) {
+            const AT *w = Wt + (2 * 25 + dz * 5 + tz) * WM, *a = Abox + (tz * 25 + tyx) * vol + ab;
+            for (int az = 0; az < wz; ++az) acc += w[az] * a[az * plane];
+        }
+        U[(tyx * 5 + dz) * plane + ab] = acc;
+    }
+    __syncthreads();
+    for (int e = tid; e < 5 * nV; e += nt) {
+        const int tx = e / nV, code = vix[e - tx * nV], dz = code >> 16, dy = (code >> 8) & 0xff, ax = code & 0xff;
+        AT acc = 0;
+        for (int ty = 0; ty < 5; ++ty) {
+            const AT *w = Wt + (25 + dy * 5 + ty) * WM, *u = U + ((ty * 5 + tx) * 5 + dz) * plane + ax;
+            for (int ay = 0; ay < wy; ++ay) acc += w[ay] * u[ay * WX];
+        }
+        V[(tx * 25 + dz * 5 + dy) * WX + ax] = acc;
+    }
+    __syncthreads();
+    if (tid < 125) {
+        const int dx = tid % 5, dzy = tid / 5;
+        AT acc = 0;
+        for (int tx = 0; tx < 5; ++tx) {
+            const AT *w = Wt + (dx * 5 + tx) * WM, *v = V + (tx * 25 + dzy) * WX;
+            for (int ax = 0; ax < wx; ++ax) acc += w[ax] * v[ax];
+        }
+        Ac[(long long)tid * G.Nc + I] = acc;
+    }
 }
 
 // FP32 Galerkin values into the FP64 level-operator storage
@@ -2402,7 +2488,7 @@ static Interp interp_of(const Coarse *c) {
         P.ia[a] = c->d_ia[a]; P.ib[a] = c->d_ib[a];
         P.wa[a] = c->d_wa[a]; P.wb[a] = c->d_wb[a];
         P.lo[a] = c->d_lo[a]; P.hi[a] = c->d_hi[a];
-        P.wt[a] = c->d_wt[a]; P.W[a] = c->wmax[a];
+        P.wt[a] = c->d_wt[a]; P.ww[a] = c->d_ww[a]; P.W[a] = c->wmax[a];
     }
     return P;
 }
@@ -2511,6 +2597,7 @@ static int configure_t(Coarse *c) {
     RAS_CK(cudaFuncSetAttribute(k_rap<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     RAS_CK(cudaFuncSetAttribute(k_rap_slab<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     RAS_CK(cudaFuncSetAttribute(k_rap125<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+    RAS_CK(cudaFuncSetAttribute(k_rap125_all<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     RAS_CK(cudaFuncSetAttribute(k_coarse_factor<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     RAS_CK(cudaFuncSetAttribute(k_coarse_factor_batch<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     RAS_CK(cudaFuncSetAttribute(k_coarse_solve<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
@@ -2567,7 +2654,7 @@ static int configure_t(Coarse *c) {
 
 // interpolation tables of one axis on the device
 static int upload_axis(int n, int r, int order, int *&d_ia, int *&d_ib, double *&d_wa, double *&d_wb, int *&d_lo,
-                       int *&d_hi, double *&d_wt, int &nc, int &wmax) {
+                       int *&d_hi, double *&d_wt, double *&d_ww, int &nc, int &wmax) {
     std::vector<int> ia, ib, lo, hi;
     std::vector<double> wa, wb;
     interp_axis(n, r, ia, ib, wa, wb, lo, hi, nc, order);
@@ -2578,6 +2665,18 @@ static int upload_axis(int n, int r, int order, int *&d_ia, int *&d_ib, double *
     for (int I = 0; I < nc; ++I)
         for (int a = lo[I]; a < hi[I]; ++a)
             wt[(size_t)I * wmax + (a - lo[I])] = ia[a] == I ? wa[a] : (ib[a] == I ? wb[a] : 0.0);
+    auto weight = [&](int a, int I) { return ia[a] == I ? wa[a] : (ib[a] == I ? wb[a] : 0.0); };
+    std::vector<double> ww((size_t)nc * 25 * wmax, 0.0);
+    for (int I = 0; I < nc; ++I)
+        for (int d = 0; d < 5; ++d)
+            for (int t = 0; t < 5; ++t)
+                for (int a = lo[I]; a < hi[I]; ++a) {
+                    const int as = a + t - 2, J = I + d - 2;
+                    if (J >= 0 && J < nc && as >= 0 && as < n)
+                        ww[(((size_t)I * 5 + d) * 5 + t) * wmax + (a - lo[I])] = weight(a, I) * weight(as, J);
+                }
+    RAS_TRY(dalloc(&d_ww, ww.size()));
+    RAS_CK(cudaMemcpy(d_ww, ww.data(), ww.size() * 8, cudaMemcpyHostToDevice));
     RAS_TRY(dalloc(&d_wt, wt.size()));
     RAS_CK(cudaMemcpy(d_wt, wt.data(), wt.size() * 8, cudaMemcpyHostToDevice));
     RAS_TRY(dalloc(&d_ia, ia.size()));
@@ -2618,7 +2717,7 @@ int coarse_setup_grid(Coarse **out, int fnx, int fny, int fnz, const ras_opts &o
     for (int a = 0; a < 3; ++a) {
         c->r[a] = o.coarsen[a];
         const int rc = upload_axis(c->n[a], c->r[a], o.interp_order, c->d_ia[a], c->d_ib[a], c->d_wa[a], c->d_wb[a],
-                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->c[a], c->wmax[a]);
+                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->d_ww[a], c->c[a], c->wmax[a]);
         if (rc) return fail(rc);
     }
     c->Nc = c->c[0] * c->c[1] * c->c[2];
@@ -2719,7 +2818,7 @@ void coarse_free(Coarse *c) {
     if (!c) return;
     for (int a = 0; a < 3; ++a) {
         dfree(c->d_ia[a]); dfree(c->d_ib[a]); dfree(c->d_wa[a]); dfree(c->d_wb[a]);
-        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]);
+        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]); dfree(c->d_ww[a]);
     }
     dfree(c->d_pos); dfree(c->d_cell); dfree(c->d_err); dfree(c->d_bar); dfree(c->d_flags);
     dfree(c->lo_q); dfree(c->up_q); dfree(c->lo_n); dfree(c->up_n); dfree(c->d_crf); dfree(c->d_crs);
@@ -2808,8 +2907,13 @@ static int factor_t(Coarse *c, const Stencil7 &A, cudaStream_t st) {
 template <typename AT>
 static int factor125_t(Coarse *c, const double *Af, cudaStream_t st) {
     RapDims W{c->wmax[0], c->wmax[1], c->wmax[2]};
-    k_rap125<AT><<<c->Nc, 256, c->rap125_smem, st>>>(Af, interp_of(c), geom_of(c), W, c->rap125_ng,
-                                                      (AT *)c->Ac);
+    const size_t all = rap125_all_smem(c->wmax, sizeof(AT));
+    if (all <= 100 * 1024) {   // (two CTAs per SM at least)
+        k_rap125_all<AT><<<c->Nc, 256, all, st>>>(Af, interp_of(c), geom_of(c), W, (AT *)c->Ac);
+    } else {
+        k_rap125<AT><<<c->Nc, 256, c->rap125_smem, st>>>(Af, interp_of(c), geom_of(c), W, c->rap125_ng,
+                                                          (AT *)c->Ac);
+    }
     RAS_LAUNCHED();
     return factor_blocks_t<AT>(c, st);
 }
@@ -3143,7 +3247,7 @@ int transfer_setup(Transfer **out, int nx, int ny, int nz, const int ratio[3], i
     for (int a = 0; a < 3; ++a) {
         c->r[a] = ratio[a];
         const int rc = upload_axis(c->n[a], c->r[a], order, c->d_ia[a], c->d_ib[a], c->d_wa[a], c->d_wb[a],
-                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->c[a], c->wmax[a]);
+                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->d_ww[a], c->c[a], c->wmax[a]);
         if (rc) { transfer_free(t); return rc; }
     }
     c->Nc = c->c[0] * c->c[1] * c->c[2];
@@ -3172,7 +3276,7 @@ void transfer_free(Transfer *t) {
     Coarse *c = &t->geo;
     for (int a = 0; a < 3; ++a) {
         dfree(c->d_ia[a]); dfree(c->d_ib[a]); dfree(c->d_wa[a]); dfree(c->d_wb[a]);
-        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]);
+        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]); dfree(c->d_ww[a]);
     }
     delete t;
 }
