@@ -61,6 +61,7 @@ struct Coarse {
     double *d_wa[3] = {}, *d_wb[3] = {};
     int *d_lo[3] = {}, *d_hi[3] = {};
     double *d_wt[3] = {};           // per coarse index: the weights of its fine support (w1's values)
+    float *d_wf[3] = {};            // FP32: wa, wb, then wt
     double *d_ww[3] = {};           // per coarse index: the Galerkin product's pair weights [5][5][wmax]
     int af, am, as;                 // axis order: fastest, middle, slowest
     int T = 0, nb = 0;              // block size (multiple of TILE), number of blocks
@@ -86,7 +87,7 @@ struct Coarse {
     int need125 = 0;                // the handle's operator is 125-point (three levels): k_rap125 must fit
     int rap125_ng = 25;             // offsets staged per round in k_rap125
     int fac_grid = 0, sol_grid = 0;
-    int sol_npf = 0;                // rows per warp prefetched by the solve
+    int sol_npf = 0;                // rows per warp in flight in the solve
     int cr = 0;                     // cyclic reduction instead of the two-ended elimination
     int *d_crf = nullptr, *d_crs = nullptr;   // its factorisation and solve schedules
     void *W = nullptr;              // its dense couplings and products [nslot][T][T]
@@ -103,6 +104,7 @@ struct Interp {
     const double *wa[3], *wb[3];
     const int *lo[3], *hi[3];
     const double *wt[3];   // [I][m]: P(lo[I] + m, I), m < W (the same values as w1)
+    const float *fa[3], *fb[3], *ft[3];   // wa, wb, wt in FP32
     const double *ww[3];   // [I][d][t][m]: P(lo[I] + m, I) P(lo[I] + m + t - 2, I + d - 2), m < W (0 outside)
     int W[3];
 };
@@ -448,7 +450,7 @@ __global__ void __launch_bounds__(256) k_rap125(const double *__restrict__ Af, I
 // offset by offset it takes 3 x 81 passes of about 100 sums (half the operations, and the
 // barriers bounded it: 2.0 ms on 15 x 55 x 22 coarse cells, 7 % of a three-level step
 // there). The FP32 error against FP64 halves (rms 3.3e-8 of the largest entry for 6.5e-8):
-// a value is the end of 15 sums instead of 81 terms added up.
+// a value is three sums of 20 terms where 81 terms were added up.
 static size_t rap125_all_smem(const int w[3], size_t esz) {
     const size_t WX = w[0], WY = w[1], WZ = w[2], WM = std::max(WX, std::max(WY, WZ));
     return esz * (125 * WX * WY * WZ + 75 * WM + 125 * WY * WX + 125 * WX) + sizeof(int) * (5 * WY * WX + 25 * WX);
@@ -658,16 +660,22 @@ __device__ __forceinline__ void red_add_release(unsigned *p, unsigned v) {
 // the grid; a group of co-resident CTAs with a barrier word of its own). Returns
 // false if this or any CTA has flagged an error or the wait ran out (ERR_TIMEOUT
 // is then set).
-__device__ bool grid_barrier(GridBar *bar, int *err, unsigned &epoch, unsigned G = 0) {
+// meanwhile() is what every thread does between the arrival and the wait.
+template <typename F>
+__device__ __forceinline__ bool grid_barrier_with(GridBar *bar, int *err, unsigned &epoch, unsigned G, F meanwhile) {
     __shared__ int s_ok;
     ++epoch;
     __syncthreads();
+    unsigned e0 = 0;
     if (threadIdx.x == 0) {
-        const unsigned e0 = *reinterpret_cast<volatile const unsigned *>(err);
+        e0 = *reinterpret_cast<volatile const unsigned *>(err);
+        red_add_release(&bar->count, 1u);
+    }
+    meanwhile();
+    if (threadIdx.x == 0) {
         int ok = 1;
         const long long lim = bar->polls > 0 ? bar->polls : BAR_POLLS;
         const unsigned target = epoch * (G ? G : gridDim.x);
-        red_add_release(&bar->count, 1u);
         long long it = 0;
         while (ld_acquire(&bar->count) < target) {
             if (++it > lim) { atomicExch(err, ERR_TIMEOUT); ok = 0; break; }
@@ -678,6 +686,9 @@ __device__ bool grid_barrier(GridBar *bar, int *err, unsigned &epoch, unsigned G
     }
     __syncthreads();
     return s_ok != 0;
+}
+__device__ bool grid_barrier(GridBar *bar, int *err, unsigned &epoch, unsigned G = 0) {
+    return grid_barrier_with(bar, err, epoch, G, [] {});
 }
 
 // ---------------------------------------------------------------------------
@@ -2050,7 +2061,7 @@ struct SolArgs {
     AT *rx, *ry;
     GridBar *bar;
     int *err;
-    int npf;   // matrix rows per warp prefetched into shared memory per stage (0..2)
+    int npf;   // matrix rows per warp coming into shared memory (0..3)
     int cr;            // cyclic reduction: the block sweeps follow its solve schedule
     const int *crs;
     const AT *W;
@@ -2064,7 +2075,9 @@ __device__ __forceinline__ void cp_async16_cg(void *smem, const void *gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit_all() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { cp_async_wait<0>(); }
 
 // dot of a shared-memory matrix row with a shared-memory vector; lane l reads the
 // 16-byte pieces l, l + 32, ... (the pieces it copied itself)
@@ -2118,21 +2131,23 @@ __device__ __forceinline__ AT row_dot(const AT *row, const AT *xs, int T, int la
     return acc;
 }
 
-// xs <- xsrc (T values, 16-byte loads, read through L2 only)
+// xs <- x0, x1 (T values each, x1 only when n == 2; 16-byte loads in flight together, read
+// through L2 only)
 template <typename AT>
-__device__ void stage_vector(const AT *xsrc, AT *xs, int T) {
+__device__ void stage_vectors(const AT *x0, const AT *x1, int n, AT *xs, int T) {
     using V16 = typename std::conditional<sizeof(AT) == 4, float4, double2>::type;
     const int nv = T / (16 / (int)sizeof(AT));
-    const V16 *src = reinterpret_cast<const V16 *>(xsrc);
     V16 *dst = reinterpret_cast<V16 *>(xs);
-    for (int base = threadIdx.x; base < nv; base += 4 * blockDim.x) {
+    for (int base = threadIdx.x; base < n * nv; base += 4 * blockDim.x) {
         V16 buf[4];
 #pragma unroll
-        for (int m = 0; m < 4; ++m)
-            if (base + m * (int)blockDim.x < nv) buf[m] = __ldcg(src + base + m * blockDim.x);
+        for (int m = 0; m < 4; ++m) {
+            const int e = base + m * (int)blockDim.x;
+            if (e < n * nv) buf[m] = __ldcg(reinterpret_cast<const V16 *>(e < nv ? x0 : x1) + (e < nv ? e : e - nv));
+        }
 #pragma unroll
         for (int m = 0; m < 4; ++m)
-            if (base + m * (int)blockDim.x < nv) dst[base + m * blockDim.x] = buf[m];
+            if (base + m * (int)blockDim.x < n * nv) dst[base + m * blockDim.x] = buf[m];
     }
     __syncthreads();
 }
@@ -2175,10 +2190,27 @@ __device__ bool cr_sweeps(const SolArgs<AT> &a, int b, int ng, unsigned &epoch) 
     return true;
 }
 
+// An axis's interpolation weights in the solve's type. (Rounding them where they are used
+// costs: a conversion from FP64 takes as long as an FP64 operation, two a cycle and SM, and
+// the x pass of the restriction made 16 per coarse value, the prolongation 7 per cell.)
+template <typename AT>
+__device__ __forceinline__ const AT *wa_of(const Interp &P, int ax) {
+    if constexpr (sizeof(AT) == 4) return P.fa[ax]; else return P.wa[ax];
+}
+template <typename AT>
+__device__ __forceinline__ const AT *wb_of(const Interp &P, int ax) {
+    if constexpr (sizeof(AT) == 4) return P.fb[ax]; else return P.wb[ax];
+}
+template <typename AT>
+__device__ __forceinline__ const AT *wt_of(const Interp &P, int ax) {
+    if constexpr (sizeof(AT) == 4) return P.ft[ax]; else return P.wt[ax];
+}
+
 // z (+)= P x for the fine cells p0, p0 + stride, ..., four at a time with their loads
 // in flight together; the coarse values from the natural-order copy (the cyclic
-// reduction's sweeps leave x in block order only)
-template <typename AT>
+// reduction's sweeps leave x in block order only). OWN: a kernel of its own, which may read
+// them through L1 (neighbouring cells share them).
+template <typename AT, bool OWN>
 __device__ __forceinline__ void coarse_prolong_range(const SolArgs<AT> &a, double *z, long long start,
                                                      long long stride) {
     const CGeom &G = a.G;
@@ -2191,14 +2223,14 @@ __device__ __forceinline__ void coarse_prolong_range(const SolArgs<AT> &a, doubl
             const long long p = p0 + m * stride;
             sv[m] = 0;
             if (p >= N) continue;
-            const int ax = (int)(p % G.nx), ay = (int)((p / G.nx) % G.ny),
-                      az = (int)(p / ((long long)G.nx * G.ny));
+            const unsigned row = (unsigned)p / (unsigned)G.nx;   // (a device holds fewer than 2^32 cells)
+            const int ax = (int)((unsigned)p - row * G.nx), az = (int)(row / (unsigned)G.ny), ay = (int)row - az * G.ny;
             const int Ix[2] = {P.ia[0][ax], P.ib[0][ax]};
             const int Iy[2] = {P.ia[1][ay], P.ib[1][ay]};
             const int Iz[2] = {P.ia[2][az], P.ib[2][az]};
-            const AT Wx[2] = {(AT)P.wa[0][ax], (AT)P.wb[0][ax]};
-            const AT Wy[2] = {(AT)P.wa[1][ay], (AT)P.wb[1][ay]};
-            const AT Wz[2] = {(AT)P.wa[2][az], (AT)P.wb[2][az]};
+            const AT Wx[2] = {__ldg(wa_of<AT>(P, 0) + ax), __ldg(wb_of<AT>(P, 0) + ax)};
+            const AT Wy[2] = {__ldg(wa_of<AT>(P, 1) + ay), __ldg(wb_of<AT>(P, 1) + ay)};
+            const AT Wz[2] = {__ldg(wa_of<AT>(P, 2) + az), __ldg(wb_of<AT>(P, 2) + az)};
             AT s = 0;
 #pragma unroll
             for (int u = 0; u < 2; ++u)
@@ -2208,7 +2240,7 @@ __device__ __forceinline__ void coarse_prolong_range(const SolArgs<AT> &a, doubl
                     for (int w = 0; w < 2; ++w) {
                         const AT wt = Wx[w] * Wy[v] * Wz[u];
                         const int I = Ix[w] + G.cx * (Iy[v] + G.cy * Iz[u]);
-                        if (wt != (AT)0) s += wt * (a.cr ? __ldcg(a.x + a.pos[I]) : __ldcg(a.xn + I));
+                        if (wt != (AT)0) s += wt * (a.cr ? __ldcg(a.x + a.pos[I]) : OWN ? __ldg(a.xn + I) : __ldcg(a.xn + I));
                     }
             sv[m] = s;
         }
@@ -2233,14 +2265,18 @@ __device__ __forceinline__ void coarse_solve_body(const SolArgs<AT> &a, int b, i
     // Block sweeps as 2 nsteps + 1 stages separated by grid barriers: forward along
     // both chains (g_target -= C_e g_pivot, and x_pivot = Inv_pivot g_pivot), the
     // middle block (x_mid = Inv_mid g_mid), back along both chains
-    // (x_pivot -= F_e x_target). The matrix rows of a stage do not depend on the
-    // vectors, so each warp copies its first npf rows of the next stage into shared
-    // memory before the barrier (the copies overlap the barrier and the next
-    // vector staging); further rows are read directly.
+    // (x_pivot -= F_e x_target). The matrix rows do not depend on the vectors, so each warp
+    // keeps the next D rows of its sequence over all stages coming into a ring in shared
+    // memory, across the barriers (D = 3 is up to three stages ahead). A row of a later stage
+    // is asked for between the arrival at the barrier and the wait, so that its address
+    // arithmetic is not part of the chain; asked for before the arrival, the ring gave
+    // nothing. With the weight tables: FP32 step on 128x128x64 21.5 -> 20.8 ms (about 29
+    // coarse solves), batch of 12 33.3 -> 32.5 ms.
     const int nb = G.nb, mid = G.mid, ntop = mid, nbot = nb - 1 - mid;
     const int nsteps = max(ntop, nbot), nstage = 2 * nsteps + 1;
     const int wg = b * wpb + (threadIdx.x >> 5), nwt = ng * wpb;
-    AT *rbuf = xs + 2 * (long long)T + (long long)(threadIdx.x >> 5) * a.npf * T;
+    const int D = a.npf;
+    AT *rbuf = xs + 2 * (long long)T + (long long)(threadIdx.x >> 5) * D * T;
     constexpr int VEC = 16 / sizeof(AT);
     auto edges_of = [&](int st, int *edg) {
         int ne = 0;
@@ -2257,27 +2293,30 @@ __device__ __forceinline__ void coarse_solve_body(const SolArgs<AT> &a, int b, i
     auto nrows_of = [&](int st, int ne) { return st < nsteps ? ne * 2 * T : (st == nsteps ? T : ne * T); };
     auto row_ptr = [&](int st, const int *edg, int r) -> const AT * {
         if (st < nsteps) {
-            const int c = r / (2 * T), rr = r % (2 * T), e = edg[c];
+            const int c = r >= 2 * T, rr = r - c * 2 * T, e = edg[c];
             return rr < T ? a.E + edge_pivot(e, mid) * bsz + (long long)rr * T
                           : a.C + e * bsz + (long long)(rr - T) * T;
         }
         if (st == nsteps) return a.E + mid * bsz + (long long)r * T;
-        return a.F + edg[r / T] * bsz + (long long)(r % T) * T;
+        const int c = r >= T;
+        return a.F + edg[c] * bsz + (long long)(r - c * T) * T;
     };
-    auto prefetch = [&](int st) {
-        if (st < nstage) {
+    // the next row to copy (stage, row, slot), the next slot to read, free slots
+    int ist = 0, ir = wg, islot = 0, slot = 0, due = 0;
+    auto issue = [&] {
+        for (; ist < nstage; ++ist, ir = wg) {
             int edg[2];
-            const int nr = nrows_of(st, edges_of(st, edg));
-            for (int k = 0; k < a.npf; ++k) {
-                const int r = wg + k * nwt;
-                if (r >= nr) break;
-                const AT *src = row_ptr(st, edg, r);
-                for (int v = lane; v < T / VEC; v += 32) cp_async16_cg(rbuf + (long long)k * T + v * VEC, src + v * VEC);
-            }
+            if (ir >= nrows_of(ist, edges_of(ist, edg))) continue;
+            const AT *src = row_ptr(ist, edg, ir);
+            AT *dst = rbuf + (long long)islot * T;
+            for (int v = lane; v < T / VEC; v += 32) cp_async16_cg(dst + v * VEC, src + v * VEC);
+            ir += nwt;
+            break;
         }
+        islot = islot + 1 == D ? 0 : islot + 1;
         cp_async_commit_all();
     };
-    prefetch(0);   // lands during the restriction
+    for (int k = 0; k < D; ++k) issue();   // land during the restriction
     // g = R t with R = P^T = Pz^T Py^T Px^T, one axis per pass
     const long long gtid = b * (long long)blockDim.x + threadIdx.x;
     const long long gstride = (long long)ng * blockDim.x;
@@ -2285,44 +2324,45 @@ __device__ __forceinline__ void coarse_solve_body(const SolArgs<AT> &a, int b, i
     // (each pass: the support's weights from the per-axis table and its values
     // loaded in batches of 8 before any is used; terms summed in index order)
     for (long long e = gtid; e < n1; e += gstride) {          // x pass
-        const int Ix = (int)(e % G.cx);
-        const long long yz = e / G.cx;
+        const unsigned yz = (unsigned)e / (unsigned)G.cx;
+        const int Ix = (int)((unsigned)e - yz * G.cx);
         const int x0 = P.lo[0][Ix], nw = P.hi[0][Ix] - x0;
-        const double *src = t + yz * G.nx + x0, *wt = P.wt[0] + (long long)Ix * P.W[0];
+        const double *src = t + (long long)yz * G.nx + x0;
+        const AT *wt = wt_of<AT>(P, 0) + (long long)Ix * P.W[0];
         AT acc = 0;
         for (int m0 = 0; m0 < nw; m0 += 8) {
-            double tv[8], wv[8];
+            double tv[8];
+            AT wv[8];
 #pragma unroll
             for (int m = 0; m < 8; ++m) {
                 tv[m] = m0 + m < nw ? __ldg(src + m0 + m) : 0.0;
-                wv[m] = m0 + m < nw ? __ldg(wt + m0 + m) : 0.0;
+                wv[m] = m0 + m < nw ? __ldg(wt + m0 + m) : (AT)0;
             }
 #pragma unroll
             for (int m = 0; m < 8; ++m)
-                if (m0 + m < nw) acc += (AT)wv[m] * (AT)tv[m];
+                if (m0 + m < nw) acc += wv[m] * (AT)tv[m];
         }
         a.rx[e] = acc;
     }
     if (!grid_barrier(a.bar, a.err, epoch, ng)) { cp_async_wait_all(); return; }
     const long long n2 = (long long)G.cx * G.cy * G.nz;
     for (long long e = gtid; e < n2; e += gstride) {          // y pass
-        const int Ix = (int)(e % G.cx), Iy = (int)((e / G.cx) % G.cy);
-        const long long az = e / ((long long)G.cx * G.cy);
+        const unsigned q = (unsigned)e / (unsigned)G.cx, az = q / (unsigned)G.cy;
+        const int Ix = (int)((unsigned)e - q * G.cx), Iy = (int)(q - az * G.cy);
         const int y0 = P.lo[1][Iy], nw = P.hi[1][Iy] - y0;
         const AT *src = a.rx + Ix + (long long)G.cx * (y0 + (long long)G.ny * az);
-        const double *wt = P.wt[1] + (long long)Iy * P.W[1];
+        const AT *wt = wt_of<AT>(P, 1) + (long long)Iy * P.W[1];
         AT acc = 0;
         for (int m0 = 0; m0 < nw; m0 += 8) {
-            AT v[8];
-            double wv[8];
+            AT v[8], wv[8];
 #pragma unroll
             for (int m = 0; m < 8; ++m) {
                 v[m] = m0 + m < nw ? __ldcg(src + (long long)G.cx * (m0 + m)) : (AT)0;
-                wv[m] = m0 + m < nw ? __ldg(wt + m0 + m) : 0.0;
+                wv[m] = m0 + m < nw ? __ldg(wt + m0 + m) : (AT)0;
             }
 #pragma unroll
             for (int m = 0; m < 8; ++m)
-                if (m0 + m < nw) acc += (AT)wv[m] * v[m];
+                if (m0 + m < nw) acc += wv[m] * v[m];
         }
         a.ry[e] = acc;
     }
@@ -2332,20 +2372,19 @@ __device__ __forceinline__ void coarse_solve_body(const SolArgs<AT> &a, int b, i
         const int z0 = P.lo[2][Iz], nw = P.hi[2][Iz] - z0;
         const long long cxy = (long long)G.cx * G.cy;
         const AT *src = a.ry + Ix + (long long)G.cx * Iy + cxy * z0;
-        const double *wt = P.wt[2] + (long long)Iz * P.W[2];
+        const AT *wt = wt_of<AT>(P, 2) + (long long)Iz * P.W[2];
         const int dst = a.pos[I];
         AT acc = 0;
         for (int m0 = 0; m0 < nw; m0 += 8) {
-            AT v[8];
-            double wv[8];
+            AT v[8], wv[8];
 #pragma unroll
             for (int m = 0; m < 8; ++m) {
                 v[m] = m0 + m < nw ? __ldcg(src + cxy * (m0 + m)) : (AT)0;
-                wv[m] = m0 + m < nw ? __ldg(wt + m0 + m) : 0.0;
+                wv[m] = m0 + m < nw ? __ldg(wt + m0 + m) : (AT)0;
             }
 #pragma unroll
             for (int m = 0; m < 8; ++m)
-                if (m0 + m < nw) acc += (AT)wv[m] * v[m];
+                if (m0 + m < nw) acc += wv[m] * v[m];
         }
         a.g[dst] = acc;
     }
@@ -2354,53 +2393,64 @@ __device__ __forceinline__ void coarse_solve_body(const SolArgs<AT> &a, int b, i
     for (int st = 0; st < (a.cr ? 0 : nstage); ++st) {
         int edg[2];
         const int ne = edges_of(st, edg);
-        if (st < nsteps)
-            for (int c = 0; c < ne; ++c)
-                stage_vector(a.g + (long long)edge_pivot(edg[c], mid) * T, xs + (long long)c * T, T);
-        else if (st == nsteps)
-            stage_vector(a.g + (long long)mid * T, xs, T);
-        else
-            for (int c = 0; c < ne; ++c)
-                stage_vector(a.x + (long long)edge_target(edg[c], mid) * T, xs + (long long)c * T, T);
-        cp_async_wait_all();
-        __syncwarp();
+        const AT *xv[2];
+        for (int c = 0; c < 2; ++c)
+            xv[c] = st < nsteps ? a.g + (long long)edge_pivot(edg[c < ne ? c : 0], mid) * T
+                  : st == nsteps ? a.g + (long long)mid * T
+                                 : a.x + (long long)edge_target(edg[c < ne ? c : 0], mid) * T;
+        stage_vectors(xv[0], xv[1], st == nsteps ? 1 : ne, xs, T);
         const int nr = nrows_of(st, ne);
-        int k = 0;
-        for (int r = wg; r < nr; r += nwt, ++k) {
+        for (int r = wg; r < nr; r += nwt) {
             // lane 0 first reads what the row updates (the target entry of g, or the
             // pivot entry of x on the way back) and the natural index of a row whose x
             // value becomes final in this stage (the middle block, and the pivot blocks
             // on the way back), so that those loads overlap the dot product
             AT *y = nullptr;
+            const AT *xr = xs;
             long long qf = -1;
+            bool rmw = true;                                       // y -= acc
             if (st < nsteps) {
-                const int c = r / (2 * T), rr = r % (2 * T), e = edg[c];
-                y = rr < T ? a.x + (long long)edge_pivot(e, mid) * T + rr
-                           : a.g + (long long)edge_target(e, mid) * T + (rr - T);
+                const int c = r >= 2 * T, rr = r - c * 2 * T, e = edg[c];
+                rmw = rr >= T;
+                xr += c * T;
+                y = rmw ? a.g + (long long)edge_target(e, mid) * T + (rr - T)
+                        : a.x + (long long)edge_pivot(e, mid) * T + rr;
             } else if (st == nsteps) {
+                rmw = false;
                 qf = (long long)mid * T + r;
                 y = a.x + qf;
             } else {
-                qf = (long long)edge_pivot(edg[r / T], mid) * T + (r % T);
+                const int c = r >= T;
+                xr += c * T;
+                qf = (long long)edge_pivot(edg[c], mid) * T + (r - c * T);
                 y = a.x + qf;
             }
-            const bool rmw = st > nsteps || (st < nsteps && r % (2 * T) >= T);   // y -= acc
             const AT prev = lane == 0 && rmw ? __ldcg(y) : (AT)0;
             const int cf = lane == 0 && qf >= 0 ? a.cell[qf] : -1;
-            const AT *xv = xs + (long long)(st < nsteps ? r / (2 * T) : (st == nsteps ? 0 : r / T)) * T;
-            const AT acc = k < a.npf ? row_dot_s(rbuf + (long long)k * T, xv, T, lane)
-                                     : row_dot(row_ptr(st, edg, r), xv, T, lane);
+            AT acc;
+            if (D > 0) {
+                const int left = D - 1 - due;                      // younger copies in flight
+                if (left >= 2) cp_async_wait<2>(); else if (left == 1) cp_async_wait<1>(); else cp_async_wait<0>();
+                acc = row_dot_s(rbuf + (long long)slot * T, xr, T, lane);   // (a lane reads what it copied)
+                slot = slot + 1 == D ? 0 : slot + 1;
+                ++due;
+            } else {
+                acc = row_dot(row_ptr(st, edg, r), xr, T, lane);
+            }
             if (lane == 0) {
                 const AT v = rmw ? prev - acc : acc;
                 *y = v;
                 if (cf >= 0) a.xn[cf] = v;
             }
+            if (D > 0 && ist == st) { issue(); --due; }            // a row of this stage
         }
-        __syncwarp();                      // this warp's reads of its row buffer are done
-        prefetch(st + 1);
-        if (!grid_barrier(a.bar, a.err, epoch, ng)) { cp_async_wait_all(); return; }
+        // later stages' rows, between the arrival at the barrier and the wait
+        if (!grid_barrier_with(a.bar, a.err, epoch, ng, [&] { for (; due > 0; --due) issue(); })) {
+            cp_async_wait_all();
+            return;
+        }
     }
-    if (a.prolong) coarse_prolong_range(a, z, gtid, gstride);
+    if (a.prolong) coarse_prolong_range<AT, false>(a, z, gtid, gstride);
 }
 
 template <typename AT>
@@ -2412,8 +2462,8 @@ __global__ void __launch_bounds__(256, 2) k_coarse_solve(SolArgs<AT> a) {
 // occupancy: the loop is bound by the latency of its table and coarse loads, which
 // the cooperative kernel's two CTAs per SM do not hide)
 template <typename AT>
-__global__ void __launch_bounds__(256) k_coarse_prolong(SolArgs<AT> a) {
-    coarse_prolong_range(a, a.z, blockIdx.x * (long long)blockDim.x + threadIdx.x,
+__global__ void __launch_bounds__(256, 4) k_coarse_prolong(SolArgs<AT> a) {
+    coarse_prolong_range<AT, true>(a, a.z, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                          (long long)gridDim.x * blockDim.x);
 }
 
@@ -2509,6 +2559,7 @@ static Interp interp_of(const Coarse *c) {
         P.wa[a] = c->d_wa[a]; P.wb[a] = c->d_wb[a];
         P.lo[a] = c->d_lo[a]; P.hi[a] = c->d_hi[a];
         P.wt[a] = c->d_wt[a]; P.ww[a] = c->d_ww[a]; P.W[a] = c->wmax[a];
+        P.fa[a] = c->d_wf[a]; P.fb[a] = c->d_wf[a] + c->n[a]; P.ft[a] = c->d_wf[a] + 2 * c->n[a];
     }
     return P;
 }
@@ -2645,7 +2696,10 @@ static int configure_t(Coarse *c) {
     if (c->cr) c->fac_smem = std::max(c->fac_smem, sizeof(TcSmem));
     // the solve prefetches up to two (FP32) or one (FP64) matrix rows per warp
     // (the reduction's sweeps read theirs directly)
-    c->sol_npf = c->cr ? 0 : (sizeof(AT) == 4 ? 2 : 1);
+    // rows in flight: three if two CTAs fit an SM with them, fewer down to one before the
+    // second CTA goes
+    c->sol_npf = c->cr ? 0 : 3;
+    while (c->sol_npf > 1 && sizeof(AT) * (size_t)(2 + 8 * c->sol_npf) * c->T > 112 * 1024) --c->sol_npf;
     while (c->sol_npf > 0 && sizeof(AT) * (size_t)(2 + 8 * c->sol_npf) * c->T > (size_t)big) --c->sol_npf;
     c->sol_smem = sizeof(AT) * (size_t)(2 + 8 * c->sol_npf) * c->T;
     if (c->rap_smem > (size_t)big || (c->need125 && c->rap125_smem > (size_t)big) || c->fac_smem > (size_t)big ||
@@ -2674,7 +2728,7 @@ static int configure_t(Coarse *c) {
 
 // interpolation tables of one axis on the device
 static int upload_axis(int n, int r, int order, int *&d_ia, int *&d_ib, double *&d_wa, double *&d_wb, int *&d_lo,
-                       int *&d_hi, double *&d_wt, double *&d_ww, int &nc, int &wmax) {
+                       int *&d_hi, double *&d_wt, double *&d_ww, float *&d_wf, int &nc, int &wmax) {
     std::vector<int> ia, ib, lo, hi;
     std::vector<double> wa, wb;
     interp_axis(n, r, ia, ib, wa, wb, lo, hi, nc, order);
@@ -2695,6 +2749,11 @@ static int upload_axis(int n, int r, int order, int *&d_ia, int *&d_ib, double *
                     if (J >= 0 && J < nc && as >= 0 && as < n)
                         ww[(((size_t)I * 5 + d) * 5 + t) * wmax + (a - lo[I])] = weight(a, I) * weight(as, J);
                 }
+    std::vector<float> wf(wa.begin(), wa.end());
+    wf.insert(wf.end(), wb.begin(), wb.end());
+    wf.insert(wf.end(), wt.begin(), wt.end());
+    RAS_TRY(dalloc(&d_wf, wf.size()));
+    RAS_CK(cudaMemcpy(d_wf, wf.data(), wf.size() * 4, cudaMemcpyHostToDevice));
     RAS_TRY(dalloc(&d_ww, ww.size()));
     RAS_CK(cudaMemcpy(d_ww, ww.data(), ww.size() * 8, cudaMemcpyHostToDevice));
     RAS_TRY(dalloc(&d_wt, wt.size()));
@@ -2737,7 +2796,7 @@ int coarse_setup_grid(Coarse **out, int fnx, int fny, int fnz, const ras_opts &o
     for (int a = 0; a < 3; ++a) {
         c->r[a] = o.coarsen[a];
         const int rc = upload_axis(c->n[a], c->r[a], o.interp_order, c->d_ia[a], c->d_ib[a], c->d_wa[a], c->d_wb[a],
-                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->d_ww[a], c->c[a], c->wmax[a]);
+                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->d_ww[a], c->d_wf[a], c->c[a], c->wmax[a]);
         if (rc) return fail(rc);
     }
     c->Nc = c->c[0] * c->c[1] * c->c[2];
@@ -2838,7 +2897,7 @@ void coarse_free(Coarse *c) {
     if (!c) return;
     for (int a = 0; a < 3; ++a) {
         dfree(c->d_ia[a]); dfree(c->d_ib[a]); dfree(c->d_wa[a]); dfree(c->d_wb[a]);
-        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]); dfree(c->d_ww[a]);
+        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]); dfree(c->d_ww[a]); dfree(c->d_wf[a]);
     }
     dfree(c->d_pos); dfree(c->d_cell); dfree(c->d_err); dfree(c->d_bar); dfree(c->d_flags);
     dfree(c->lo_q); dfree(c->up_q); dfree(c->lo_n); dfree(c->up_n); dfree(c->d_crf); dfree(c->d_crs);
@@ -3267,7 +3326,7 @@ int transfer_setup(Transfer **out, int nx, int ny, int nz, const int ratio[3], i
     for (int a = 0; a < 3; ++a) {
         c->r[a] = ratio[a];
         const int rc = upload_axis(c->n[a], c->r[a], order, c->d_ia[a], c->d_ib[a], c->d_wa[a], c->d_wb[a],
-                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->d_ww[a], c->c[a], c->wmax[a]);
+                                   c->d_lo[a], c->d_hi[a], c->d_wt[a], c->d_ww[a], c->d_wf[a], c->c[a], c->wmax[a]);
         if (rc) { transfer_free(t); return rc; }
     }
     c->Nc = c->c[0] * c->c[1] * c->c[2];
@@ -3296,7 +3355,7 @@ void transfer_free(Transfer *t) {
     Coarse *c = &t->geo;
     for (int a = 0; a < 3; ++a) {
         dfree(c->d_ia[a]); dfree(c->d_ib[a]); dfree(c->d_wa[a]); dfree(c->d_wb[a]);
-        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]); dfree(c->d_ww[a]);
+        dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]); dfree(c->d_ww[a]); dfree(c->d_wf[a]);
     }
     delete t;
 }
