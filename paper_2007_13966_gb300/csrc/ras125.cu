@@ -605,6 +605,37 @@ double ras125_bytes(const Ras125 &R) {
     return 2.0 * RREC * esz * (double)R.nrow + 16.0 * (double)R.N;
 }
 
+// Warps per box (a warp per row of a level): the number whose waves of boxes times the
+// rounds over its levels are fewest, the larger one of equals. A warp for every row of the
+// widest level is the fastest box, but its registers let fewer boxes share an SM, and a
+// second wave of boxes costs as much as the first: on 336 boxes of 10^3 cells (152 SMs,
+// levels of up to 14 rows, 7.5 on average) 14 warps took two waves of solves and three of
+// factorisations. With no more boxes than SMs every number takes one wave and the widest
+// level decides.
+template <typename K>
+static int pick_warps(K kernel, size_t smem, int widest, int nsub, int sms, const std::vector<Shape125> &shapes,
+                      const std::vector<int> &lvl_tab, int &warps) {
+    warps = widest;
+    long long best = -1;
+    for (int w = widest; w >= 4; --w) {
+        int occ = 0;
+        RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32 * w, smem));
+        if (occ < 1) continue;
+        long long rounds = 0;
+        for (const Shape125 &sh : shapes) {
+            long long n = 0;
+            for (int l = 0; l < sh.nlev; ++l) {
+                const int *c = lvl_tab.data() + sh.lvl_off + l;
+                n += (c[1] - c[0] + w - 1) / w;
+            }
+            rounds = std::max(rounds, n);
+        }
+        const long long cost = rounds * ((nsub + (long long)occ * sms - 1) / ((long long)occ * sms));
+        if (best < 0 || cost < best) { best = cost; warps = w; }
+    }
+    return RAS_OK;
+}
+
 constexpr int SMEM125_MAX = 200 * 1024;
 
 int ras125_setup(Ras125 &R, int nx, int ny, int nz, int px, int py, int pz, int overlap, int prec,
@@ -679,7 +710,6 @@ int ras125_setup(Ras125 &R, int nx, int ny, int nz, int px, int py, int pz, int 
     R.nrow = foff;
     R.ycap = ycap;
     R.lcap = lcap;
-    R.nwarps = std::min(16, std::max(4, maxw));
     const size_t acc = prec == 64 ? 8 : 4;
     R.ycap = (ycap + 3) & ~3;
     R.smem_apply = (size_t)R.ycap * acc + (size_t)lcap * sizeof(int);
@@ -723,18 +753,26 @@ int ras125_setup(Ras125 &R, int nx, int ny, int nz, int px, int py, int pz, int 
     RAS_CK(cudaMemset(R.d_fwd, 0, nval * esz));
     RAS_CK(cudaMemset(R.d_bwd, 0, nval * esz));
     const int big = SMEM125_MAX;
+    int dev = 0, sms = 1;
+    RAS_CK(cudaGetDevice(&dev));
+    RAS_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    auto prepare = [&](auto kernel, size_t smem, int &warps) -> int {
+        RAS_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        return pick_warps(kernel, smem, std::min(16, std::max(4, maxw)), R.nsub, sms, R.shapes, lvl_tab, warps);
+    };
+    const bool g = R.guard >= 0;
     if (prec == 64) {
-        RAS_CK(cudaFuncSetAttribute(k_ras125_factor<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_TRY(prepare(k_ras125_factor<64>, R.smem_factor, R.warps_factor));
+        RAS_TRY(g ? prepare(k_ras125_apply<64, true>, R.smem_apply, R.warps_apply)
+                  : prepare(k_ras125_apply<64, false>, R.smem_apply, R.warps_apply));
     } else if (prec == 32) {
-        RAS_CK(cudaFuncSetAttribute(k_ras125_factor<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_TRY(prepare(k_ras125_factor<32>, R.smem_factor, R.warps_factor));
+        RAS_TRY(g ? prepare(k_ras125_apply<32, true>, R.smem_apply, R.warps_apply)
+                  : prepare(k_ras125_apply<32, false>, R.smem_apply, R.warps_apply));
     } else {
-        RAS_CK(cudaFuncSetAttribute(k_ras125_factor<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        RAS_CK(cudaFuncSetAttribute(k_ras125_apply<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+        RAS_TRY(prepare(k_ras125_factor<16>, R.smem_factor, R.warps_factor));
+        RAS_TRY(g ? prepare(k_ras125_apply<16, true>, R.smem_apply, R.warps_apply)
+                  : prepare(k_ras125_apply<16, false>, R.smem_apply, R.warps_apply));
     }
     return RAS_OK;
 }
@@ -754,7 +792,7 @@ int ras125_factor(Ras125 &R, const double *A, cudaStream_t st) {
     P.A = A; P.nx = R.nx; P.ny = R.ny; P.nz = R.nz;
     P.work = R.d_work; P.fwd = R.d_fwd; P.bwd = R.d_bwd; P.err = R.d_err;
     P.mask = R.d_mask;
-    const int threads = 32 * R.nwarps;
+    const int threads = 32 * R.warps_factor;
     if (R.prec == 64) k_ras125_factor<64><<<R.nsub, threads, R.smem_factor, st>>>(P);
     else if (R.prec == 32) k_ras125_factor<32><<<R.nsub, threads, R.smem_factor, st>>>(P);
     else k_ras125_factor<16><<<R.nsub, threads, R.smem_factor, st>>>(P);
@@ -779,7 +817,7 @@ int ras125_apply(Ras125 &R, const double *r, double *z, int accumulate, cudaStre
     P.fwd = R.d_fwd; P.bwd = R.d_bwd; P.r = r; P.z = z;
     P.nx = R.nx; P.ny = R.ny; P.nz = R.nz; P.accumulate = accumulate;
     P.ycap = R.ycap;
-    const int threads = 32 * R.nwarps;
+    const int threads = 32 * R.warps_apply;
     P.guard = std::max(R.guard, 0);
     auto run = [&](auto kernel) { kernel<<<R.nsub, threads, R.smem_apply, st>>>(P); };
     const bool g = R.guard >= 0;

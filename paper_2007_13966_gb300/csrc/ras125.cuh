@@ -38,7 +38,7 @@ struct Sub125 {
 struct Ras125 {
     int nx = 0, ny = 0, nz = 0, N = 0;
     int prec = 64;
-    int nsub = 0, nwarps = 8, ycap = 0, lcap = 0;
+    int nsub = 0, warps_factor = 8, warps_apply = 8, ycap = 0, lcap = 0;
     int guard = -1;                      // zeros on either side of the solves' vector (-1: none, tested couplings)
     long long nrow = 0;                  // factor rows (sum of box cells)
     size_t smem_apply = 0, smem_factor = 0;
