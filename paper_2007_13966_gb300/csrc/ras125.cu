@@ -89,11 +89,22 @@ __device__ __forceinline__ void store_val(void *base, long long idx, double v) {
     else reinterpret_cast<__nv_bfloat16 *>(base)[idx] = __float2bfloat16_rn((float)v);
 }
 
+// slots 4 h .. 4 h + 3 of a record row
 template <int PREC>
-__device__ __forceinline__ typename Val125<PREC>::Acc load_val(const void *base, long long idx) {
-    if constexpr (PREC == 64) return __ldg(reinterpret_cast<const double *>(base) + idx);
-    else if constexpr (PREC == 32) return __ldg(reinterpret_cast<const float *>(base) + idx);
-    else return __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(base)[idx]);
+__device__ __forceinline__ void load_slots(const void *base, long long row, int h, typename Val125<PREC>::Acc (&v)[4]) {
+    const long long at = row * (RREC / 4) + h;
+    if constexpr (PREC == 64) {
+        const double2 *p = reinterpret_cast<const double2 *>(base) + 2 * at;
+        const double2 a = __ldg(p), b = __ldg(p + 1);
+        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    } else if constexpr (PREC == 32) {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(base) + at);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    } else {
+        const uint2 a = __ldg(reinterpret_cast<const uint2 *>(base) + at);
+        v[0] = __uint_as_float(a.x << 16); v[1] = __uint_as_float(a.x & 0xffff0000u);
+        v[2] = __uint_as_float(a.y << 16); v[3] = __uint_as_float(a.y & 0xffff0000u);
+    }
 }
 
 // shape tables copied to shared memory by the whole CTA
@@ -312,14 +323,17 @@ struct App125 {
     int ycap, guard;
 };
 
-// z = sum_i (R_i^0)^T U_i^{-1} L_i^{-1} R_i^delta r with, per row (one warp),
+// z = sum_i (R_i^0)^T U_i^{-1} L_i^{-1} R_i^delta r with, per row (half a warp),
 //     forward   y_n = r_n - sum_{m<n} l_nm y_m,
 //     backward  z_n = (y_n - sum_{m>n} u_nm z_m) / u_nn,
-// lane t taking the couplings of slots t and t + 32 (slot 63 of the backward
-// record holds 1/u_nn). Accumulation in FP64 (64) or FP32 (32, 16). Each
-// warp's first row of a level is loaded AD levels ahead (register ring).
+// lane h of 16 taking the couplings of slots 4 h .. 4 h + 3 (slot 63 of the backward record
+// holds 1/u_nn). Accumulation in FP64 (64) or FP32 (32, 16). Each half warp's first row of a
+// level is loaded AD levels ahead (register ring).
 // Bound: ~110 dependent levels per sweep of a 10^3 box, each the instruction stream of one
-// row. GUARD: the vector has zeros on either side as far as the couplings reach (guard
+// row, and the instructions of three boxes on an SM: a row per half warp halves them (one
+// 16-byte load instead of two and four shuffles instead of five, for two rows at a time):
+// 207 -> 173 us on 336 boxes in FP32.
+// GUARD: the vector has zeros on either side as far as the couplings reach (guard
 // cells), a coupling leaving the box has factor value 0, and no row tests its 62 couplings
 // against the box: that was most of a row's instructions. Without room for the guard (large
 // flat boxes) every coupling is tested; the values are the same.
@@ -345,22 +359,21 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
         const int i = t % bx, j = (t / bx) % by, k = t / bxy;
         Y[t] = (Acc)__ldg(P.r + g0 + i + nx * (long long)j + nxy * k);
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int h = threadIdx.x & 15, wid = threadIdx.x >> 4, nw = blockDim.x >> 4;   // half warps
     const int nL = sh.nL;
-    int lx[2], ly[2], lz[2], ld[2], ux[2], uy[2], uz[2], ud[2];
-    bool lv[2];
+    int ld[4], ud[4], lo[4], uo[4];   // natural distances; the offsets themselves (packed)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int s = lane + 32 * h;
-        lv[h] = s < nL;
-        const int ol = lv[h] ? sh.lowo[s] : CENTRE125, ou = lv[h] ? sh.upo[s] : CENTRE125;
-        lx[h] = off_dx(ol); ly[h] = off_dy(ol); lz[h] = off_dz(ol);
-        ld[h] = lx[h] + bx * ly[h] + bxy * lz[h];
-        ux[h] = off_dx(ou); uy[h] = off_dy(ou); uz[h] = off_dz(ou);
-        ud[h] = ux[h] + bx * uy[h] + bxy * uz[h];
+    for (int m = 0; m < 4; ++m) {
+        const int s = 4 * h + m;
+        lo[m] = s < nL ? sh.lowo[s] : CENTRE125;
+        uo[m] = s < nL ? sh.upo[s] : CENTRE125;
+        const int lx = off_dx(lo[m]), ly = off_dy(lo[m]), lz = off_dz(lo[m]);
+        const int ux = off_dx(uo[m]), uy = off_dy(uo[m]), uz = off_dz(uo[m]);
+        ld[m] = lx + bx * ly + bxy * lz;
+        ud[m] = ux + bx * uy + bxy * uz;
         if (GUARD) {   // couplings longer than the box never hold: read the cell itself
-            if (abs(lx[h]) >= bx || abs(ly[h]) >= by || abs(lz[h]) >= bz) ld[h] = 0;
-            if (abs(ux[h]) >= bx || abs(uy[h]) >= by || abs(uz[h]) >= bz) ud[h] = 0;
+            if (abs(lx) >= bx || abs(ly) >= by || abs(lz) >= bz) ld[m] = 0;
+            if (abs(ux) >= bx || abs(uy) >= by || abs(uz) >= bz) ud[m] = 0;
         }
     }
     auto inbox = [&](int i, int j, int k) {
@@ -370,59 +383,60 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
     for (int t = threadIdx.x; t <= sh.nlev; t += blockDim.x) lvl_s[t] = lvl[t];
     __syncthreads();
 
-    // the first row of each level for this warp, fetched AD levels ahead
-    const typename Val125<PREC>::T *fw = reinterpret_cast<const typename Val125<PREC>::T *>(P.fwd) + fbase + lane;
-    const typename Val125<PREC>::T *bw = reinterpret_cast<const typename Val125<PREC>::T *>(P.bwd) + fbase + lane;
-    struct Row { int q; unsigned e; Acc v0, v1; };
-    auto fetch = [&](int l, const typename Val125<PREC>::T *rec) {
+    // the first row of each level for this half warp, fetched AD levels ahead
+    const typename Val125<PREC>::T *fw = reinterpret_cast<const typename Val125<PREC>::T *>(P.fwd) + fbase;
+    const typename Val125<PREC>::T *bw = reinterpret_cast<const typename Val125<PREC>::T *>(P.bwd) + fbase;
+    struct Row { int q; unsigned e; Acc v[4]; };
+    auto load = [&](int q, const typename Val125<PREC>::T *rec) {
         Row rw;
-        rw.q = -1;
-        rw.e = 0;
-        rw.v0 = rw.v1 = 0;
-        if (l >= 0 && l < sh.nlev) {
-            const int q = lvl_s[l] + wid;
-            if (q < lvl_s[l + 1]) {
-                rw.q = q;
-                rw.e = __ldg(cells + q);
-                rw.v0 = load_val<PREC>(rec, q * RREC);
-                rw.v1 = load_val<PREC>(rec, q * RREC + 32);
-            }
-        }
+        rw.q = q;
+        rw.e = __ldg(cells + q);
+        load_slots<PREC>(rec, q, h, rw.v);
         return rw;
     };
-    // forward row: y_n = r_n - sum_{m<n} l_nm y_m
-    auto fwd_row = [&](unsigned e, Acc a0, Acc a1) {
-        const int i = e & 255u, j = (e >> 8) & 255u, k = (e >> 16) & 255u;
-        const int n = i + bx * j + bxy * k;
+    auto fetch = [&](int l, const typename Val125<PREC>::T *rec) {
+        if (l >= 0 && l < sh.nlev) {
+            const int q = lvl_s[l] + wid;
+            if (q < lvl_s[l + 1]) return load(q, rec);
+        }
+        return Row{-1, 0u, {0, 0, 0, 0}};
+    };
+    // sum of a row's couplings over its half warp (a half without a row sums zeros at cell 0)
+    auto row_sum = [&](const Row &rw, const int *d, const int *o, int n) {
         Acc acc = 0;
         if (GUARD) {
-            acc = a0 * Y[n + ld[0]];
-            if (lv[1]) acc += a1 * Y[n + ld[1]];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) acc += rw.v[m] * Y[n + d[m]];
         } else {
-            if (lv[0] && inbox(i + lx[0], j + ly[0], k + lz[0])) acc += a0 * Y[n + ld[0]];
-            if (lv[1] && inbox(i + lx[1], j + ly[1], k + lz[1])) acc += a1 * Y[n + ld[1]];
+            const int i = rw.e & 255u, j = (rw.e >> 8) & 255u, k = (rw.e >> 16) & 255u;
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (4 * h + m < nL && inbox(i + off_dx(o[m]), j + off_dy(o[m]), k + off_dz(o[m])))
+                    acc += rw.v[m] * Y[n + d[m]];
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) Y[n] -= acc;
+        for (int q = 8; q > 0; q >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, q);
+        return acc;
+    };
+    auto cell_of = [&](unsigned e) {
+        return (int)(e & 255u) + bx * (int)((e >> 8) & 255u) + bxy * (int)((e >> 16) & 255u);
+    };
+    // forward row: y_n = r_n - sum_{m<n} l_nm y_m
+    auto fwd_row = [&](const Row &rw) {
+        const int n = cell_of(rw.e);
+        const Acc acc = row_sum(rw, ld, lo, n);
+        if (h == 0 && rw.q >= 0) Y[n] -= acc;
     };
     // backward row: z_n = (y_n - sum_{m>n} u_nm z_m) / u_nn (slot 63 = 1/u_nn)
-    auto bwd_row = [&](unsigned e, Acc b0, Acc b1) {
-        const int i = e & 255u, j = (e >> 8) & 255u, k = (e >> 16) & 255u;
-        const int n = i + bx * j + bxy * k;
-        Acc acc = 0;
-        if (GUARD) {
-            acc = b0 * Y[n + ud[0]];
-            if (lv[1]) acc += b1 * Y[n + ud[1]];
-        } else {
-            if (lv[0] && inbox(i + ux[0], j + uy[0], k + uz[0])) acc += b0 * Y[n + ud[0]];
-            if (lv[1] && inbox(i + ux[1], j + uy[1], k + uz[1])) acc += b1 * Y[n + ud[1]];
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        const Acc dinv = __shfl_sync(0xffffffffu, b1, 31);
-        if (lane == 0) Y[n] = (Y[n] - acc) * dinv;
+    auto bwd_row = [&](Row rw) {
+        const int n = cell_of(rw.e);
+        const Acc dinv = __shfl_sync(0xffffffffu, rw.v[3], 15, 16);
+        if (h == 15) rw.v[3] = 0;
+        const Acc acc = row_sum(rw, ud, uo, n);
+        if (h == 0 && rw.q >= 0) Y[n] = (Y[n] - acc) * dinv;
     };
+    // (both halves of a warp go on together: a half without a row in a round takes none)
+    const int wid0 = wid & ~1;
 
     Row ring[AD];
 #pragma unroll
@@ -434,10 +448,10 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
             if (l < sh.nlev) {
                 const Row cur = ring[u];
                 ring[u] = fetch(l + AD, fw);
-                if (cur.q >= 0) fwd_row(cur.e, cur.v0, cur.v1);
-                for (int q = lvl_s[l] + wid + nw; q < lvl_s[l + 1]; q += nw) {
-                    fwd_row(__ldg(cells + q), load_val<PREC>(fw, q * RREC), load_val<PREC>(fw, q * RREC + 32));
-                }
+                const int end = lvl_s[l + 1];
+                if (lvl_s[l] + wid0 < end) fwd_row(cur);
+                for (int q = lvl_s[l] + wid + nw; q - (wid & 1) < end; q += nw)
+                    fwd_row(q < end ? load(q, fw) : Row{-1, 0u, {0, 0, 0, 0}});
                 __syncthreads();
             }
         }
@@ -451,10 +465,10 @@ __global__ void __launch_bounds__(512) k_ras125_apply(App125 P) {
             if (l >= 0) {
                 const Row cur = ring[u];
                 ring[u] = fetch(l - AD, bw);
-                if (cur.q >= 0) bwd_row(cur.e, cur.v0, cur.v1);
-                for (int q = lvl_s[l] + wid + nw; q < lvl_s[l + 1]; q += nw) {
-                    bwd_row(__ldg(cells + q), load_val<PREC>(bw, q * RREC), load_val<PREC>(bw, q * RREC + 32));
-                }
+                const int end = lvl_s[l + 1];
+                if (lvl_s[l] + wid0 < end) bwd_row(cur);
+                for (int q = lvl_s[l] + wid + nw; q - (wid & 1) < end; q += nw)
+                    bwd_row(q < end ? load(q, bw) : Row{-1, 0u, {0, 0, 0, 0}});
                 __syncthreads();
             }
         }
@@ -605,19 +619,19 @@ double ras125_bytes(const Ras125 &R) {
     return 2.0 * RREC * esz * (double)R.nrow + 16.0 * (double)R.N;
 }
 
-// Warps per box (a warp per row of a level): the number whose waves of boxes times the
+// Warps per box (each takes `rows` rows of a level at a time): the number whose waves of boxes times the
 // rounds over its levels are fewest, the larger one of equals. A warp for every row of the
 // widest level is the fastest box, but its registers let fewer boxes share an SM, and a
 // second wave of boxes costs as much as the first: on 336 boxes of 10^3 cells (152 SMs,
 // levels of up to 14 rows, 7.5 on average) 14 warps took two waves of solves and three of
-// factorisations. With no more boxes than SMs every number takes one wave and the widest
-// level decides.
+// factorisations (328 us and 5.19 ms; 207 us and 3.98 ms by this rule). With no more boxes
+// than SMs every number takes one wave and the widest level decides.
 template <typename K>
 static int pick_warps(K kernel, size_t smem, int widest, int nsub, int sms, const std::vector<Shape125> &shapes,
-                      const std::vector<int> &lvl_tab, int &warps) {
+                      const std::vector<int> &lvl_tab, int rows, int &warps) {
     warps = widest;
     long long best = -1;
-    for (int w = widest; w >= 4; --w) {
+    for (int w = widest; w >= std::min(widest, 4 / rows); --w) {
         int occ = 0;
         RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32 * w, smem));
         if (occ < 1) continue;
@@ -626,7 +640,7 @@ static int pick_warps(K kernel, size_t smem, int widest, int nsub, int sms, cons
             long long n = 0;
             for (int l = 0; l < sh.nlev; ++l) {
                 const int *c = lvl_tab.data() + sh.lvl_off + l;
-                n += (c[1] - c[0] + w - 1) / w;
+                n += (c[1] - c[0] + rows * w - 1) / (rows * w);
             }
             rounds = std::max(rounds, n);
         }
@@ -756,23 +770,24 @@ int ras125_setup(Ras125 &R, int nx, int ny, int nz, int px, int py, int pz, int 
     int dev = 0, sms = 1;
     RAS_CK(cudaGetDevice(&dev));
     RAS_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    auto prepare = [&](auto kernel, size_t smem, int &warps) -> int {
+    auto prepare = [&](auto kernel, size_t smem, int rows, int &warps) -> int {
         RAS_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-        return pick_warps(kernel, smem, std::min(16, std::max(4, maxw)), R.nsub, sms, R.shapes, lvl_tab, warps);
+        return pick_warps(kernel, smem, std::min(16, std::max(4, (maxw + rows - 1) / rows)), R.nsub, sms, R.shapes, lvl_tab,
+                          rows, warps);
     };
     const bool g = R.guard >= 0;
     if (prec == 64) {
-        RAS_TRY(prepare(k_ras125_factor<64>, R.smem_factor, R.warps_factor));
-        RAS_TRY(g ? prepare(k_ras125_apply<64, true>, R.smem_apply, R.warps_apply)
-                  : prepare(k_ras125_apply<64, false>, R.smem_apply, R.warps_apply));
+        RAS_TRY(prepare(k_ras125_factor<64>, R.smem_factor, 1, R.warps_factor));
+        RAS_TRY(g ? prepare(k_ras125_apply<64, true>, R.smem_apply, 2, R.warps_apply)
+                  : prepare(k_ras125_apply<64, false>, R.smem_apply, 2, R.warps_apply));
     } else if (prec == 32) {
-        RAS_TRY(prepare(k_ras125_factor<32>, R.smem_factor, R.warps_factor));
-        RAS_TRY(g ? prepare(k_ras125_apply<32, true>, R.smem_apply, R.warps_apply)
-                  : prepare(k_ras125_apply<32, false>, R.smem_apply, R.warps_apply));
+        RAS_TRY(prepare(k_ras125_factor<32>, R.smem_factor, 1, R.warps_factor));
+        RAS_TRY(g ? prepare(k_ras125_apply<32, true>, R.smem_apply, 2, R.warps_apply)
+                  : prepare(k_ras125_apply<32, false>, R.smem_apply, 2, R.warps_apply));
     } else {
-        RAS_TRY(prepare(k_ras125_factor<16>, R.smem_factor, R.warps_factor));
-        RAS_TRY(g ? prepare(k_ras125_apply<16, true>, R.smem_apply, R.warps_apply)
-                  : prepare(k_ras125_apply<16, false>, R.smem_apply, R.warps_apply));
+        RAS_TRY(prepare(k_ras125_factor<16>, R.smem_factor, 1, R.warps_factor));
+        RAS_TRY(g ? prepare(k_ras125_apply<16, true>, R.smem_apply, 2, R.warps_apply)
+                  : prepare(k_ras125_apply<16, false>, R.smem_apply, 2, R.warps_apply));
     }
     return RAS_OK;
 }
