@@ -3267,51 +3267,73 @@ struct Transfer {
     size_t smem32 = 0;
 };
 
-// tc[I] = sum_a P(a, I) t[a] over the fine support box of I (FP64)
-__global__ void __launch_bounds__(256) k_restrict(Interp P, CGeom G, const double *__restrict__ t,
+// tc[I] = sum_a P(a, I) t[a] over the fine support box of I (FP64), summed axis by axis:
+// FP64 arithmetic bounds it (two operations per cycle and SM), and 64 + 16 + 4 of them for
+// a box of 4^3 cells take the place of 192 and a search for every weight. Four rows of four
+// values are in flight at once.
+__global__ void __launch_bounds__(256, 4) k_restrict(Interp P, CGeom G, const double *__restrict__ t,
                                                   double *__restrict__ tc) {
     const long long nxy = (long long)G.nx * G.ny;
     for (int I = blockIdx.x * blockDim.x + threadIdx.x; I < G.Nc; I += gridDim.x * blockDim.x) {
-        const int Ix = I % G.cx, Iy = (I / G.cx) % G.cy, Iz = I / (G.cx * G.cy);
+        const int row = I / G.cx, Ix = I - row * G.cx, Iz = row / G.cy, Iy = row - Iz * G.cy;
+        const int x0 = P.lo[0][Ix], wx = P.hi[0][Ix] - x0, y0 = P.lo[1][Iy], wy = P.hi[1][Iy] - y0;
+        const int z0 = P.lo[2][Iz], wz = P.hi[2][Iz] - z0;
+        const double *vx = P.wt[0] + (long long)Ix * P.W[0], *vy = P.wt[1] + (long long)Iy * P.W[1];
+        const double *vz = P.wt[2] + (long long)Iz * P.W[2];
+        const double *src = t + x0 + G.nx * (long long)y0 + nxy * z0;
         double acc = 0.0;
-        for (int az = P.lo[2][Iz]; az < P.hi[2][Iz]; ++az) {
-            const double wz = w1(P, 2, az, Iz);
-            for (int ay = P.lo[1][Iy]; ay < P.hi[1][Iy]; ++ay) {
-                const double wyz = wz * w1(P, 1, ay, Iy);
-                const double *row = t + G.nx * (long long)ay + nxy * az;
-                for (int ax = P.lo[0][Ix]; ax < P.hi[0][Ix]; ++ax)
-                    acc += wyz * w1(P, 0, ax, Ix) * __ldg(row + ax);
-            }
+        for (int az = 0; az < wz; ++az) {
+            double sy = 0.0;
+            for (int ay = 0; ay < wy; ay += 4)
+                for (int ax = 0; ax < wx; ax += 4) {
+                    double v[4][4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int m = 0; m < 4; ++m)
+                            if (ay + q < wy && ax + m < wx)
+                                v[q][m] = __ldg(src + nxy * az + G.nx * (long long)(ay + q) + ax + m);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (ay + q >= wy) break;
+                        double sx = 0.0;
+#pragma unroll
+                        for (int m = 0; m < 4; ++m)
+                            if (ax + m < wx) sx += __ldg(vx + ax + m) * v[q][m];
+                        sy += __ldg(vy + ay + q) * sx;
+                    }
+                }
+            acc += __ldg(vz + az) * sy;
         }
         tc[I] = acc;
     }
 }
 
-// x[a] += sum_I P(a, I) xc[I] (eight coarse cells per fine cell, FP64)
+// x[a] += sum_I P(a, I) xc[I] (eight coarse cells per fine cell, FP64; axis by axis, 14
+// operations for the eight terms where their weights' products took 24: FP64 bounds it)
 __global__ void __launch_bounds__(256) k_prolong(Interp P, CGeom G, const double *__restrict__ xc,
                                                  double *__restrict__ x) {
     const long long N = (long long)G.nx * G.ny * G.nz;
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N;
          p += (long long)gridDim.x * blockDim.x) {
-        const int ax = (int)(p % G.nx), ay = (int)((p / G.nx) % G.ny),
-                  az = (int)(p / ((long long)G.nx * G.ny));
+        const unsigned row = (unsigned)p / (unsigned)G.nx;   // (a device holds fewer than 2^32 cells)
+        const int ax = (int)((unsigned)p - row * G.nx), az = (int)(row / (unsigned)G.ny), ay = (int)row - az * G.ny;
         const int Ix[2] = {P.ia[0][ax], P.ib[0][ax]};
         const int Iy[2] = {P.ia[1][ay], P.ib[1][ay]};
         const int Iz[2] = {P.ia[2][az], P.ib[2][az]};
-        const double Wx[2] = {P.wa[0][ax], P.wb[0][ax]};
-        const double Wy[2] = {P.wa[1][ay], P.wb[1][ay]};
-        const double Wz[2] = {P.wa[2][az], P.wb[2][az]};
-        double s = 0.0;
+        double v[2][2][2];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
-            for (int v = 0; v < 2; ++v)
+            for (int q = 0; q < 2; ++q)
 #pragma unroll
-                for (int w = 0; w < 2; ++w) {
-                    const double wt = Wx[w] * Wy[v] * Wz[u];
-                    if (wt != 0.0) s += wt * __ldg(xc + Ix[w] + G.cx * (Iy[v] + G.cy * Iz[u]));
-                }
-        x[p] += s;
+                for (int w = 0; w < 2; ++w) v[u][q][w] = __ldg(xc + Ix[w] + G.cx * (Iy[q] + G.cy * Iz[u]));
+        const double xa = P.wa[0][ax], xb = P.wb[0][ax], ya = P.wa[1][ay], yb = P.wb[1][ay];
+        double s[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            s[u] = ya * (xa * v[u][0][0] + xb * v[u][0][1]) + yb * (xa * v[u][1][0] + xb * v[u][1][1]);
+        x[p] += P.wa[2][az] * s[0] + P.wb[2][az] * s[1];
     }
 }
 
