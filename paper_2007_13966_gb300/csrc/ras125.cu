@@ -7,9 +7,9 @@
 // 81 are used for a 7-point fine operator). The subdomain solver is ILU(0) in
 // the natural order of each overlapped box on the operator's nonzero pattern.
 //
-// GPU mapping: one CTA per subdomain, one warp per matrix row. A row's 62
-// lower (or upper) couplings are spread over the 32 lanes and reduced with
-// shuffles; rows with no mutual dependency form a level (a static wavefront
+// GPU mapping: one CTA per subdomain; a matrix row takes a warp in the factorisation
+// and half a warp in the solves, its 62 lower (or upper) couplings spread over the
+// lanes and reduced with shuffles; rows with no mutual dependency form a level (a static wavefront
 // schedule computed per box shape on the host from the full 5x5x5
 // neighbourhood, a superset of every pattern), and levels are separated by CTA
 // barriers. The working vector of a subdomain lives in shared memory.
