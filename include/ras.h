@@ -419,6 +419,19 @@ int ras_set_apply_schedule(ras_precond *pc, int chunk_cells, int threads);
 /* The current schedule (chunk_cells after raising it to the widest level). */
 int ras_get_apply_schedule(const ras_precond *pc, int *chunk_cells, int *threads);
 
+/* The staging steps of the FP32 / BF16 subdomain solves as the library builds them for a
+ * grid of nx x ny x nz cells, the subdomains and factor precision of *o and a schedule of
+ * chunk_cells (0: the default), for inspection and host-side checks: host only, no CUDA
+ * call. tab: ring bytes, bytes of a factor record, shapes; then per box shape its edges,
+ * its number of steps ns (the levels of 2 x 2-cell blocks upwards, then downwards) and
+ * ns + 1 entries of 4 ints {first block, blocks, place / 16, limit}: step n takes
+ * 4 blocks x record bytes of the ring at its place, and steps up to its limit may be
+ * copied in once its records have been read (entry ns: before any have). The sweeps read
+ * step n only when step n + 1 is in too. The length goes to *len even when cap is too
+ * small (then RAS_EINVAL); RAS_EINVAL also for what ras_setup or ras_set_apply_schedule
+ * refuse of these arguments and for other factors than FP32 / BF16 ILU(0). */
+int ras_apply_steps(int nx, int ny, int nz, const ras_opts *o, int chunk_cells, int *tab, int cap, int *len);
+
 /* Kernel of the fine-level subdomain solves of Eq. equ:as-left: 0 (the default) or 1, a
  * setting of earlier versions that chose between two kernels with the same values. Both
  * values now run the same wavefront sweeps (blocks of 2 x 2 cells, one CTA per box).

@@ -908,7 +908,7 @@ static int schedule_tables(Ras1 &R, int chunk_cells, int threads, std::vector<in
         if (v >= 64 && v <= 8192) base_chunk = v;
     }
     if (chunk_cells > 0) base_chunk = chunk_cells;
-    const int cc = std::max(base_chunk, R.maxw);
+    int cc = std::max(base_chunk, R.maxw);
     int block = std::min(512, std::max(64, ((R.maxw + 31) / 32) * 32));
     if (const char *e = getenv("RAS_APPLY_THREADS")) {   // tuning knob
         const int v = atoi(e);
@@ -943,14 +943,18 @@ static int schedule_tables(Ras1 &R, int chunk_cells, int threads, std::vector<in
             sh.nchunk = nch;
         }
     } else {
-        // blocks of 2 x 2 cells: a ring of three chunks (at least two of the widest level;
-        // less where the box vector leaves less room)
+        // blocks of 2 x 2 cells: a ring of three chunks of at least the widest level (less
+        // where the box vector leaves less room). The sweeps read step n only when step
+        // n + 1 is in, and free its place after that, so the two must lie side by side: with
+        // three widest levels they do whichever of them wraps (step n then starts past the
+        // first of the three, and n + 1 fits into that); a smaller ring is checked below.
+        cc = std::max(cc, 4 * R.maxwb);
         const size_t fixed = ((size_t)R.ycap + 2 * R.gcap) * 16 + (size_t)R.ycap * 4 + R.lcap * (2 * 16 + 6 * 8);
-        const size_t widest = 4 * (size_t)R.maxwb * R.rec_bytes;
         const size_t room = fixed > 227 * 1024 ? 0 : 227 * 1024 - fixed;
-        if (room < 2 * widest) return RAS_EINVAL;
-        const size_t ring = std::min(std::max(3 * (size_t)cc * R.rec_bytes, 2 * widest), room) & ~(size_t)15;
+        const size_t ring = std::min(3 * (size_t)cc * R.rec_bytes, room) & ~(size_t)15;
+        if (ring < 4 * (size_t)R.maxwb * R.rec_bytes) return RAS_EINVAL;
         smem = fixed + ring;
+        R.ring_bytes = ring;
         // sweepers, a waiter, an issuer and helpers enough for a box plane at two cells each
         // (up to 448 threads: two CTAs per SM), one warp at least
         const int own = ((R.maxwb + 31) & ~31) + 64, help = std::max(32, ((R.bxy + 1) / 2 + 31) & ~31);
@@ -982,6 +986,8 @@ static int schedule_tables(Ras1 &R, int chunk_cells, int threads, std::vector<in
                 }
                 return q;
             };
+            for (int n = 0; n + 1 < ns; ++n)
+                if (limit(n - 1) < n + 1) return RAS_EINVAL;
             for (int n = 0; n <= ns; ++n) {
                 const int l = n < sh.nlev ? n : ns - 1 - n;
                 chunk_tab.push_back(n < ns ? lv[l] : 0);
@@ -1030,8 +1036,11 @@ int ras1_set_schedule(Ras1 &R, int chunk_cells, int threads) {
     return RAS_OK;
 }
 
-int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int overlap, int prec,
-               int kind) {
+// The host side of the set-up: boxes, their shapes and the shapes' level tables (no CUDA
+// call). cuts: the owned parts along each axis; cidx_tab: level order, local index of each
+// cell (block).
+static int ras1_geometry(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int overlap, int prec, int kind,
+                         std::vector<int> (&cuts)[3], std::vector<int> &cidx_tab) {
     if (px < 1 || py < 1 || pz < 1 || overlap < 0) return RAS_EINVAL;
     if (kind < 0 || kind > 2) return RAS_EINVAL;
     R.kind = kind;
@@ -1042,12 +1051,10 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
     R.rec_bytes = prec == 64 ? 32 : (prec == 32 ? 16 : 8);
     const int dims[3] = {nx, ny, nz};
     const int parts[3] = {px, py, pz};
-    std::vector<int> cuts[3];
     for (int a = 0; a < 3; ++a) cuts[a] = split_axis(dims[a], parts[a]);
 
     std::map<std::tuple<int, int, int>, int> shape_id;
     std::vector<int> lvl_tab;
-    std::vector<int> cidx_tab;        // level order: local index of each cell (block)
     int bxy_all = 1;
     R.subs.clear();
     R.shapes.clear();
@@ -1162,10 +1169,18 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
     R.maxwb = maxwb;
     R.bxy = bxy_all;
     R.h_lvl = lvl_tab;
-    std::vector<int> chunk_tab;
-    RAS_TRY(schedule_tables(R, 0, 0, chunk_tab));
     R.smem_factor = fac_smem;
     R.fac_block = (npen_all + 31) & ~31;
+    return RAS_OK;
+}
+
+int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int overlap, int prec,
+               int kind) {
+    const int dims[3] = {nx, ny, nz}, parts[3] = {px, py, pz};
+    std::vector<int> cuts[3], cidx_tab, chunk_tab;
+    RAS_TRY(ras1_geometry(R, nx, ny, nz, px, py, pz, overlap, prec, kind, cuts, cidx_tab));
+    RAS_TRY(schedule_tables(R, 0, 0, chunk_tab));
+    const std::vector<int> &lvl_tab = R.h_lvl;
     if (R.smem_apply > 227 * 1024 || R.smem_factor > 227 * 1024) return RAS_EINVAL;
     // handles for which the pencil-wavefront kernel may be asked for: left-RAS with FP32
     // / BF16 factors, at most 1024 x-pencils per box
@@ -1353,3 +1368,23 @@ double ras1_bytes(const Ras1 &R) {
 }
 
 }  // namespace ras
+
+using namespace ras;
+
+extern "C" int ras_apply_steps(int nx, int ny, int nz, const ras_opts *o, int chunk_cells, int *tab, int cap, int *len) {
+    if (!o || !len || nx < 1 || ny < 1 || nz < 1 || chunk_cells < 0 || o->ilu_k != 0) return RAS_EINVAL;
+    if (o->factor_prec != 32 && o->factor_prec != 16) return RAS_EINVAL;
+    Ras1 R;
+    std::vector<int> cuts[3], cidx_tab, steps;
+    RAS_TRY(ras1_geometry(R, nx, ny, nz, o->px, o->py, o->pz, o->overlap, o->factor_prec, o->ras_type, cuts, cidx_tab));
+    RAS_TRY(schedule_tables(R, chunk_cells, 0, steps));
+    std::vector<int> t{(int)R.ring_bytes, R.rec_bytes, R.nshape};
+    for (const ShapeInfo &sh : R.shapes) {
+        t.insert(t.end(), {sh.bx, sh.by, sh.bz, sh.nchunk});
+        t.insert(t.end(), steps.begin() + 4 * sh.chunk_off, steps.begin() + 4 * (sh.chunk_off + sh.nchunk + 1));
+    }
+    *len = (int)t.size();
+    if (!tab || cap < *len) return RAS_EINVAL;
+    std::copy(t.begin(), t.end(), tab);
+    return RAS_OK;
+}

@@ -52,6 +52,7 @@ struct Ras1 {
     int fac_block = 32;     // threads per box of the factorisation (its pencils)
     std::vector<int> h_lvl; // host copy of the level starts (rescheduling)
     size_t smem_apply = 0, smem_factor = 0;
+    size_t ring_bytes = 0;  // record ring of the sweeps in blocks
     long long nrec = 0;     // factor records (incl. padding)
     long long ncell_total = 0;  // sum of overlapped cells
     long long nown = 0;

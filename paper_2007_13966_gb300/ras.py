@@ -27,7 +27,7 @@ EXPORTED = ["ras_problem_create", "ras_problem_destroy", "residual_eval", "ras_s
             "ras_stencil_transpose", "ras_adjoint_rhs", "ras_grad_logk", "ras_batch_create",
             "ras_batch_destroy", "ras_batch_gmres", "ras_batch_newton_step", "ras_set_apply_schedule",
             "ras_get_apply_schedule", "ras_set_apply_kernel", "ras_get_apply_kernel", "ras_gemm_f32",
-            "ras_coarse_cr_schedule"]
+            "ras_coarse_cr_schedule", "ras_apply_steps"]
 
 
 class Grid(C.Structure):
@@ -125,6 +125,7 @@ def lib():
             "ras_gemm_f32": (i, [i, i, i, C.c_float, vp, i, vp, i, C.c_float, vp, i, vp]),
             "ras_coarse_cr_schedule": (i, [i, C.POINTER(i), i, C.POINTER(i), i, C.POINTER(i), C.POINTER(i),
                                            C.POINTER(i)]),
+            "ras_apply_steps": (i, [i, i, i, C.POINTER(Opts), i, C.POINTER(i), i, C.POINTER(i)]),
             "ras_batch_create": (i, [i, vp, vp, C.POINTER(vp)]),
             "ras_batch_destroy": (None, [vp]),
             "ras_batch_gmres": (i, [vp, vp, vp, vp, C.POINTER(KrylovOpts), vp, vp]),
@@ -188,6 +189,27 @@ def gemm_f32(A, B, C, alpha=1.0, beta=0.0, stream=None):
     n = B.shape[1]
     check(lib().ras_gemm_f32(m, n, k, float(alpha), _ptr(A), A.stride(0), _ptr(B), B.stride(0),
                              float(beta), _ptr(C), C.stride(0), _stream(stream)), "ras_gemm_f32")
+
+
+def apply_steps(dims, parts, overlap, factor_prec=32, chunk_cells=0):
+    """The staging steps of the FP32 / BF16 subdomain solves (host only): (ring bytes, record
+    bytes, [((bx, by, bz), [(first block, blocks, place / 16, limit), ...]), ...])."""
+    o = Opts()
+    o.px, o.py, o.pz = parts
+    o.overlap, o.ras_type, o.factor_prec = int(overlap), 1, int(factor_prec)
+    n = C.c_int(0)
+    st = lib().ras_apply_steps(*dims, C.byref(o), int(chunk_cells), None, 0, C.byref(n))
+    tab = (C.c_int * max(n.value, 1))()
+    if n.value:
+        st = lib().ras_apply_steps(*dims, C.byref(o), int(chunk_cells), tab, n.value, C.byref(n))
+    check(st, "ras_apply_steps")
+    shapes, at = [], 3
+    for _ in range(tab[2]):
+        edges, ns = tuple(tab[at:at + 3]), tab[at + 3]
+        at += 4
+        shapes.append((edges, [tuple(tab[at + 4 * q:at + 4 * q + 4]) for q in range(ns + 1)]))
+        at += 4 * (ns + 1)
+    return tab[0], tab[1], shapes
 
 
 def coarse_cr_schedule(nb):
