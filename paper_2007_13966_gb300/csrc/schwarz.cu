@@ -455,6 +455,9 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
         for (int t = tid; t < bz; t += nt) mb_init(mb_pl + t, nh >> 5);
         for (int t = tid; t < nput; t += nt) mb_init(mb_put + t, nsw >> 5);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // a batch's boxes of other handles have their vectors and tables where this one has
+        // its ring: their ordinary writes come before the bulk copies
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         for (int t = tid; t < guard; t += nt) Y[-1 - t] = Y[nall + t] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (pad || P.kind == 2)
             for (int t = tid; t < nall; t += nt) Y[t] = make_float4(0.f, 0.f, 0.f, 0.f);
