@@ -240,7 +240,7 @@ void ras_precond_destroy(ras_precond *pc);
  * A_0 = P_0^T A_1 P_0. The multilevel preconditioners also keep a private copy
  * of J for the fine-level residuals, so J may be freed after the call.
  * Synchronises the stream to check pivots: RAS_EZEROPIVOT on a zero or
- * non-finite pivot. */
+ * non-finite pivot (RAS_ETIMEOUT also for an earlier ras_apply, see there). */
 int ras_factor(ras_precond *pc, const ras_stencil *J, void *stream);
 
 /* z = M^{-1} r. One level: left-RAS, Eq. equ:as-left,
@@ -251,7 +251,10 @@ int ras_factor(ras_precond *pc, const ras_stencil *J, void *stream);
  * default). Three levels: Algorithm 1 with one RAS-Richardson pre- and
  * post-smoothing step on the fine and middle levels and the exact block-LU
  * solve on the coarsest. r, z: device [N], must not alias. Requires a prior
- * ras_factor. */
+ * ras_factor. Asynchronous: a bounded device wait that gave up inside it (z is then
+ * not M^{-1} r) is reported as RAS_ETIMEOUT by the next call on this handle that
+ * synchronises (ras_factor, a linear solve, a Newton step); the solves read the waits
+ * of their own applies and report them themselves. */
 int ras_apply(ras_precond *pc, const double *r, double *z, void *stream);
 
 /* Right-preconditioned flexible GMRES(m) (Section 3, Eq. jacobian, Remark 2)

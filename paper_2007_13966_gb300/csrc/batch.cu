@@ -340,7 +340,8 @@ struct ras_batch {
     std::vector<cudaGraphExec_t> cycle_exec; // the cycle's Arnoldi steps, CYC_CHUNK per graph
     std::vector<long long> cycle_launches;   // kernels in each (counted at every replay)
     int cycle_m = 0;                         // m of the captured cycle
-    long long cycle_polls = 0;               // coarse barrier poll limit captured in it
+    long long cycle_polls = 0;               // poll limit of the waits captured in it
+    int *h_err = nullptr;                    // pinned copies of the handles' error words
     unsigned char *h_act = nullptr;          // pinned host copy of the mask (between chunks)
     bool graph_off = false;                  // capture failed or disabled: direct launches
     cudaStream_t gstream = nullptr;          // the graph's own stream (joined to the caller's by events)
@@ -364,6 +365,7 @@ static void batch_free(ras_batch *B) {
     dfree(B->d_act); dfree(B->d_ap); dfree(B->d_box_inst); dfree(B->d_box_local); dfree(B->d_qcount); dfree(B->d_fp);
     dfree(B->partials); dfree(B->out); dfree(B->d_y); dfree(B->d_beta);
     if (B->h_out) cudaFreeHost(B->h_out);
+    if (B->h_err) cudaFreeHost(B->h_err);
     dfree(B->V); dfree(B->Z); dfree(B->w); dfree(B->r); dfree(B->b); dfree(B->x); dfree(B->tmp);
     dfree(B->K.H); dfree(B->K.cs); dfree(B->K.sn); dfree(B->K.g); dfree(B->K.tol); dfree(B->K.res);
     dfree(B->K.it); dfree(B->K.jend); dfree(B->K.bad); dfree(B->d_cyc); dfree(B->d_lastg);
@@ -486,7 +488,8 @@ static int b_scale(ras_batch *B, double *y, const double *x, const double *s, in
 //   z = M v;  t = v - A z;  z += P A_c^{-1} R t;  t = v - A z;  z += M t
 // (A: the operator of each reservoir's last factorisation)
 static int b_precond(ras_batch *B, const double *v, double *z, cudaStream_t st) {
-    BatchApply A{B->d_ap, B->d_box_inst, B->d_box_local, B->d_off, B->d_act, v, z, 0, B->nbox, B->d_qcount};
+    BatchApply A{B->d_ap, B->d_box_inst, B->d_box_local, B->d_off, B->d_act, v, z, 0, B->nbox, B->d_qcount,
+                 ras1_polls()};
     RAS_TRY(ras1_apply_batch(A, B->qgrid, B->prec, B->block, B->smem, st));
     if (!B->twolevel) return RAS_OK;
     RAS_TRY(b_stencil<true>(B, v, z, B->t, st, B->d_opsM));
@@ -593,7 +596,7 @@ static int b_run_cycle(ras_batch *B, int m, cudaStream_t st) {
         }
     }
     const int nchk = (m + CYC_CHUNK - 1) / CYC_CHUNK;
-    const long long polls = B->twolevel ? coarse_barrier_polls() : 0;
+    const long long polls = barrier_polls();
     if (use_graph && (B->cycle_m != m || B->cycle_polls != polls || (int)B->cycle_exec.size() != nchk)) {
         for (auto &g : B->cycle_exec)
             if (g) cudaGraphExecDestroy(g);
@@ -648,21 +651,20 @@ static int b_run_cycle(ras_batch *B, int m, cudaStream_t st) {
     return RAS_OK;
 }
 
-// Reads and clears the deferred error words of every selected reservoir (the
-// fine factors' and the coarse level's after a factorisation, the
-// preconditioner's after a solve), so that an error of one launch is not left
-// set for a later call; returns the first error found.
+// Reads and clears the deferred error words of every selected reservoir (after a
+// factorisation, or after a solve: FP64 subdomain solves leave none), so that an error of
+// one launch is not left set for a later call; returns the first error found. The words of
+// all reservoirs come with one synchronisation.
 static int drain_checks(ras_batch *B, const std::vector<unsigned char> &sel, bool factor, cudaStream_t st) {
+    if (!factor && !B->twolevel && B->prec == 64) return RAS_OK;
+    for (int i = 0; i < B->n; ++i)
+        if (sel[i])
+            RAS_CK(cudaMemcpyAsync(B->h_err + 2 * i, B->pc[i]->fine.d_err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    RAS_CK(cudaStreamSynchronize(st));
     int first = RAS_OK;
-    auto keep = [&](int rc) { if (rc != RAS_OK && first == RAS_OK) first = rc; };
     for (int i = 0; i < B->n; ++i) {
-        if (!sel[i]) continue;
-        if (factor) {
-            keep(ras1_check(B->pc[i]->fine, st));
-            if (B->twolevel) keep(coarse_check(B->pc[i]->coarse, st));
-        } else {
-            keep(precond_check(B->pc[i], st));
-        }
+        const int rc = sel[i] ? precond_words_status(B->pc[i], B->h_err + 2 * i, st) : RAS_OK;
+        if (rc != RAS_OK && first == RAS_OK) first = rc;
     }
     return first;
 }
@@ -1055,6 +1057,10 @@ static int batch_create(int n, ras_problem *const *probs, ras_precond *const *pc
         return fail(rc);
     if (cudaMallocHost((void **)&B->h_out, (size_t)n * OST * sizeof(double)) != cudaSuccess) {
         B->h_out = nullptr;
+        return fail(RAS_ENOMEM);
+    }
+    if (cudaMallocHost((void **)&B->h_err, 2 * (size_t)n * sizeof(int)) != cudaSuccess) {
+        B->h_err = nullptr;
         return fail(RAS_ENOMEM);
     }
     if (cudaMallocHost((void **)&B->h_act, (size_t)n) != cudaSuccess) {

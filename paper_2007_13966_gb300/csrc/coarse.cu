@@ -78,6 +78,7 @@ struct Coarse {
     void *Zs = nullptr;                              // scratch of the block inverses (gj_scratch per chain)
     void *rx = nullptr, *ry = nullptr;               // restriction passes [cx][ny][nz], [cx][cy][nz]
     int *d_err = nullptr;
+    bool own_err = true;            // d_err is this level's own word
     GridBar *d_bar = nullptr;
     unsigned *d_flags = nullptr;    // ready flags of the FP32 block inverses
     size_t nflag = 0;
@@ -2538,13 +2539,11 @@ __global__ void k_reset_bars(GridBar *bars, int n, long long polls) {
     }
 }
 
-static long long barrier_polls() {
+long long barrier_polls() {
     long long polls = 0;
     if (const char *e = getenv("RAS_BARRIER_POLLS")) polls = atoll(e);
     return polls;
 }
-
-long long coarse_barrier_polls() { return barrier_polls(); }
 
 static int reset_bar(Coarse *c, cudaStream_t st) {
     k_reset_bars<<<1, 32, 0, st>>>(c->d_bar, 1, barrier_polls());
@@ -2897,7 +2896,8 @@ void coarse_free(Coarse *c) {
         dfree(c->d_ia[a]); dfree(c->d_ib[a]); dfree(c->d_wa[a]); dfree(c->d_wb[a]);
         dfree(c->d_lo[a]); dfree(c->d_hi[a]); dfree(c->d_wt[a]); dfree(c->d_ww[a]); dfree(c->d_wf[a]);
     }
-    dfree(c->d_pos); dfree(c->d_cell); dfree(c->d_err); dfree(c->d_bar); dfree(c->d_flags);
+    if (c->own_err) dfree(c->d_err);
+    dfree(c->d_pos); dfree(c->d_cell); dfree(c->d_bar); dfree(c->d_flags);
     dfree(c->lo_q); dfree(c->up_q); dfree(c->lo_n); dfree(c->up_n); dfree(c->d_crf); dfree(c->d_crs);
     for (void *p : {c->Ac, c->D, c->C, c->F, c->lo_v, c->up_v, c->g, c->x, c->Zs, c->rx, c->ry, c->W, c->xn})
         if (p) cudaFree(p);
@@ -3022,10 +3022,19 @@ int coarse_check(Coarse *c, cudaStream_t st) {
     int h = 0;
     RAS_CK(cudaMemcpyAsync(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     RAS_CK(cudaStreamSynchronize(st));
-    if (h) {
-        RAS_CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), st));
-        return h == ERR_TIMEOUT ? RAS_ETIMEOUT : (h == ERR_ELL ? RAS_EINVAL : RAS_EZEROPIVOT);
-    }
+    if (h) RAS_CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), st));
+    return coarse_status(h);
+}
+
+int coarse_status(int word) {
+    return word == 0 ? RAS_OK : (word == ERR_TIMEOUT ? RAS_ETIMEOUT : (word == ERR_ELL ? RAS_EINVAL : RAS_EZEROPIVOT));
+}
+
+int coarse_share_err(Coarse *c, int *word) {
+    RAS_CK(cudaMemset(word, 0, sizeof(int)));
+    if (c->own_err) dfree(c->d_err);
+    c->d_err = word;
+    c->own_err = false;
     return RAS_OK;
 }
 

@@ -18,6 +18,11 @@ extern std::atomic<long long> g_launches;
 
 void record_error(cudaError_t e, const char *what, const char *file, int line);
 
+// The poll limit that the kernels' bounded waits take at their next launch
+// (RAS_BARRIER_POLLS; 0: the default). A captured launch keeps the value it was
+// captured with, so a graph holding one is captured again when this changes.
+long long barrier_polls();
+
 inline void counted() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
 #define RAS_CK(x)                                                                  \

@@ -292,7 +292,7 @@ int fgmres(ras_problem *P, const Stencil7 &A, ras_precond *pc, const double *b, 
     if (o.restart < 1 || o.restart > MAX_MDOT - 1 || o.maxit < 1) return RAS_EINVAL;
     RAS_TRY(ensure_krylov(P, o.restart));
     const int nx = P->nx, ny = P->ny, nz = P->nz;
-    return fgmres_core(
+    const int rc = fgmres_core(
         P->N, P->kV, P->kZ, P->kw, P->kr, P->red,
         [&](const double *v, double *z) { return precond_apply(pc, v, z, st); },
         [&](const double *z, double *y) { return stencil_apply(A, nx, ny, nz, z, y, st); },
@@ -300,6 +300,10 @@ int fgmres(ras_problem *P, const Stencil7 &A, ras_precond *pc, const double *b, 
             return stencil_residual(A, nx, ny, nz, bb, xx, rr, st);
         },
         [&]() { return precond_check(pc, st); }, b, x, o, stats, st);
+    if (rc >= 0) return rc;
+    // a device wait that ran out explains a non-finite value, say: it is reported instead
+    const int d = precond_check(pc, st);
+    return d != RAS_OK ? d : rc;
 }
 
 // ---------------------------------------------------------------------------

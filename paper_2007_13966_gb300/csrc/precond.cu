@@ -25,6 +25,21 @@ static int fine_apply(ras_precond *pc, const double *r, double *z, int accumulat
     return RAS_OK;
 }
 
+int precond_words_status(ras_precond *pc, const int *words, cudaStream_t st) {
+    for (int q = 0; q < 2; ++q)
+        if (words[q]) RAS_CK(cudaMemsetAsync(pc->fine.d_err + q, 0, sizeof(int), st));
+    const int s = ras1_status(words[0]);
+    return s != RAS_OK ? s : coarse_status(words[1]);
+}
+
+// both levels' error words in one copy
+static int words_check(ras_precond *pc, cudaStream_t st) {
+    int h[2] = {0, 0};
+    RAS_CK(cudaMemcpyAsync(h, pc->fine.d_err, sizeof(h), cudaMemcpyDeviceToHost, st));
+    RAS_CK(cudaStreamSynchronize(st));
+    return precond_words_status(pc, h, st);
+}
+
 int precond_factor(ras_precond *pc, const ras_stencil *J, cudaStream_t st) {
     Stencil7 A;
     for (int s = 0; s < 7; ++s) A.c[s] = J->c[s];
@@ -75,9 +90,9 @@ int precond_factor(ras_precond *pc, const ras_stencil *J, cudaStream_t st) {
         RAS_TRY(itcoarse_factor(pc->icoarse, A, st));
     }
     if (pc->use125) RAS_TRY(ras125_check(pc->fine125, st));
-    else RAS_TRY(ras1_check(pc->fine, st));
+    else RAS_TRY(words_check(pc, st));
     if (pc->xfer) RAS_TRY(ras125_check(pc->mid, st));
-    if (pc->coarse) RAS_TRY(coarse_check(pc->coarse, st));
+    if (pc->use125 && pc->coarse) RAS_TRY(coarse_check(pc->coarse, st));
     if (pc->icoarse) RAS_TRY(itcoarse_check(pc->icoarse, st));
     return RAS_OK;
 }
@@ -114,7 +129,9 @@ static int three_level_apply(ras_precond *pc, const double *r, double *z, cudaSt
 }
 
 int precond_check(ras_precond *pc, cudaStream_t st) {
-    return pc->coarse ? coarse_check(pc->coarse, st) : RAS_OK;   // the inexact coarse solve has no deferred error
+    // (the FP64 subdomain sweeps, ILU(k > 0) and the inexact coarse solve have no deferred error)
+    if (pc->use125) return pc->coarse ? coarse_check(pc->coarse, st) : RAS_OK;
+    return pc->coarse || pc->fine.prec != 64 ? words_check(pc, st) : RAS_OK;
 }
 
 // z = M^{-1} r for the configured preconditioner
@@ -210,6 +227,7 @@ extern "C" int ras_setup(const ras_problem *P, const ras_opts *o, ras_precond **
         if (!rc) rc = dalloc(&pc->t2, P->N);
         if (!rc) rc = dalloc(&pc->t3, P->N);
         for (int s = 0; s < 7 && !rc; ++s) rc = dalloc(&pc->Acopy[s], P->N);
+        if (!rc && pc->coarse && !pc->use125) rc = coarse_share_err(pc->coarse, pc->fine.d_err + 1);
         if (rc) { ras_precond_destroy(pc); return rc; }
     }
     *out = pc;

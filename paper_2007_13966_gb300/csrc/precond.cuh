@@ -16,10 +16,9 @@ int coarse_factor(Coarse *c, const Stencil7 &A, cudaStream_t st);
 int coarse_factor125(Coarse *c, const double *Af, cudaStream_t st);
 // reads and clears the coarse pivot / layout flag (synchronises)
 int coarse_check(Coarse *c, cudaStream_t st);
-// The poll limit the coarse kernels' grid barriers take at their next launch
-// (RAS_BARRIER_POLLS; 0: the default). A captured launch keeps the value it was
-// captured with, so a graph holding one is captured again when this changes.
-long long coarse_barrier_polls();
+int coarse_status(int word);
+// the level's error word from now on (device; the caller's, cleared here)
+int coarse_share_err(Coarse *c, int *word);
 // bytes of the dense block factors read by one coarse solve
 double coarse_bytes(const Coarse *c);
 // ec = A_c^{-1} R t, then z (+)= P ec  (accumulate selects += )
@@ -99,8 +98,11 @@ struct ras_precond {
 namespace ras {
 int precond_factor(ras_precond *pc, const ras_stencil *J, cudaStream_t st);
 int precond_apply(ras_precond *pc, const double *r, double *z, cudaStream_t st);
-// reports (and clears) an error recorded by the asynchronous coarse solves
+// reports (and clears) an error recorded by the asynchronous subdomain and coarse solves
 int precond_check(ras_precond *pc, cudaStream_t st);
+// the status in the error words of a handle with ILU(0) subdomains (fine.d_err on the host:
+// the fine level's, then the coarse level's); nonzero words are cleared
+int precond_words_status(ras_precond *pc, const int *words, cudaStream_t st);
 // Newton helpers shared by the single and the batched drivers
 int ensure_newton(ras_problem *P);
 double backtrack(double lam, double lam_prev, double phi0, double slope, double phi_lam,

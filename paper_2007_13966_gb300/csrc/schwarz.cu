@@ -322,6 +322,14 @@ __device__ __forceinline__ void ras_apply_cells(const ApplyParams &P, int box, c
 // ---- mbarriers of the sweeps in blocks (one phase per box; waits are bounded) ----
 constexpr int APPLY_TIMEOUT = 7;                // error word of a wait that ran out
 constexpr int APPLY_POLLS = 1 << 22;
+// what a wait needs: the handle's error word, the CTA's flag of a wait that ran out (the
+// others then give up too: the box is lost, and every role still runs to its end; the steps
+// copied follow it), and the launch's poll limit (0: the default)
+struct Waits {
+    int *err;
+    volatile int *failed;
+    int polls;
+};
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mb_init(unsigned long long *b, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
@@ -332,17 +340,34 @@ __device__ __forceinline__ void mb_inval(unsigned long long *b) {
 __device__ __forceinline__ void mb_arrive(unsigned long long *b) {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
 }
-__device__ __forceinline__ void mb_wait(unsigned long long *b, int *err) {
-    unsigned ok = 0;
-    for (int it = 0; it < APPLY_POLLS; ++it) {
-        asm volatile(
-            "{\n.reg .pred pp;\n"
-            "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 pp, [%1], 0;\n"
-            "selp.u32 %0, 1, 0, pp;\n}\n"
-            : "=r"(ok) : "r"(smem_addr(b)) : "memory");
-        if (ok) return;
+// one poll (the hardware suspends it for a while), or a test without a wait
+__device__ __forceinline__ bool mb_poll(unsigned long long *b) {
+    unsigned ok;
+    asm volatile(
+        "{\n.reg .pred pp;\n"
+        "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 pp, [%1], 0;\n"
+        "selp.u32 %0, 1, 0, pp;\n}\n"
+        : "=r"(ok) : "r"(smem_addr(b)) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mb_test(unsigned long long *b) {
+    unsigned ok;
+    asm volatile(
+        "{\n.reg .pred pp;\n"
+        "mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 pp, [%1], 0;\n"
+        "selp.u32 %0, 1, 0, pp;\n}\n"
+        : "=r"(ok) : "r"(smem_addr(b)) : "memory");
+    return ok != 0;
+}
+template <bool LIMIT>
+__device__ __forceinline__ bool mb_wait(unsigned long long *b, const Waits &w) {
+    for (int it = 0; it < (LIMIT ? w.polls : APPLY_POLLS); ++it) {
+        if (LIMIT ? mb_test(b) : mb_poll(b)) return true;
+        if (*w.failed) return false;
     }
-    atomicMax(err, APPLY_TIMEOUT);
+    *w.failed = 1;
+    atomicMax(w.err, APPLY_TIMEOUT);
+    return false;
 }
 // `bytes` of global memory into shared memory by the bulk copy engine, completing on b
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, unsigned long long *b) {
@@ -386,9 +411,9 @@ __device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 0;" ::: "
 // factor value and reads a finite value (a block of the box or the zero guard on either
 // side); cells that pad an odd edge are zero throughout (zero records).
 constexpr int PUT_LEVELS = 4;
-template <int PREC>
+template <int PREC, bool LIMIT>
 __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, const double *r, double *z,
-                                                 int accumulate) {
+                                                 int accumulate, int polls) {
     using R = typename RecT<PREC>::T;
     constexpr int RB = (int)sizeof(R);
     extern __shared__ __align__(16) unsigned char smem[];
@@ -404,6 +429,8 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
     unsigned long long *mb_rec = reinterpret_cast<unsigned long long *>(bt + P.ycap);
     unsigned long long *mb_free = mb_rec + 2 * P.lcap, *mb_pl = mb_free + 2 * P.lcap, *mb_put = mb_pl + P.lcap;
     unsigned char *ring = reinterpret_cast<unsigned char *>(mb_put + P.lcap);
+    // (the last of mb_free's places is beyond the last step)
+    const Waits wt{P.err, reinterpret_cast<volatile int *>(mb_free + 2 * P.lcap - 1), polls};
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     // warps: sweepers, helpers (one at least, see the launch), a waiter and an issuer
     const int nsw = (sh.maxw + 31) & ~31, nh = nt - nsw - 64;
@@ -459,6 +486,7 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
         // its ring: their ordinary writes come before the bulk copies
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         for (int t = tid; t < guard; t += nt) Y[-1 - t] = Y[nall + t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid == 0) *wt.failed = 0;
         if (pad || P.kind == 2)
             for (int t = tid; t < nall; t += nt) Y[t] = make_float4(0.f, 0.f, 0.f, 0.f);
         cta_barrier();
@@ -558,11 +586,11 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
         // joins the barrier of step n when the plane of r that it reads and the records of
         // step n + 1 are in (the sweepers wait for nothing else); after it step n's records
         // are in registers and their place in the ring is free
-        mb_wait(mb_rec, P.err);
+        mb_wait<LIMIT>(mb_rec, wt);
         step_barrier();
         for (int n = 0; n < nstep; ++n) {
-            if (n < bz) mb_wait(mb_pl + n, P.err);
-            if (n + 1 < nstep) mb_wait(mb_rec + n + 1, P.err);
+            if (n < bz) mb_wait<LIMIT>(mb_pl + n, wt);
+            if (n + 1 < nstep) mb_wait<LIMIT>(mb_rec + n + 1, wt);
             step_barrier();
             if (lane == 0) mb_arrive(mb_free + n);
         }
@@ -570,7 +598,7 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
         if (lane == 0) {
             int next = 0;
             for (int n = -1; n < nstep; ++n) {
-                if (n >= 0) mb_wait(mb_free + n, P.err);
+                if (n >= 0 && !mb_wait<LIMIT>(mb_free + n, wt)) break;
                 const int lim = st[n < 0 ? nstep : n].w;
                 for (; next <= lim; ++next) {
                     const int4 s = st[next];
@@ -579,6 +607,7 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
                 }
                 if (next == nstep) break;
             }
+            wt.failed[1] = next;                 // steps whose copies were started
         }
     } else {
         float *Yf = reinterpret_cast<float *>(Y);
@@ -611,12 +640,17 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
         }
         if (P.kind == 1)
             for (int e = 0; e < nput; ++e) {     // levels nlev - 1 - PUT_LEVELS e downwards
-                mb_wait(mb_put + e, P.err);
+                mb_wait<LIMIT>(mb_put + e, wt);
                 const int l1 = nlev - PUT_LEVELS * e, l0 = max(0, l1 - PUT_LEVELS);
                 put(st[l0].x, st[l1 - 1].x + st[l1 - 1].y);
             }
     }
     cta_barrier();
+    if (*wt.failed) {                            // the box is lost: its last copies land before the CTA goes on
+        for (int t = tid; t < wt.failed[1]; t += nt)
+            for (int it = 0; !mb_poll(mb_rec + t) && it < APPLY_POLLS; ++it) {}
+        cta_barrier();
+    }
     for (int t = tid; t < nstep; t += nt) {
         mb_inval(mb_rec + t);
         mb_inval(mb_free + t);
@@ -632,18 +666,18 @@ __device__ __forceinline__ void ras_apply_blocks(const ApplyParams &P, int box, 
     }
 }
 
-template <int PREC>
+template <int PREC, bool LIMIT>
 __device__ __forceinline__ void ras_apply_box(const ApplyParams &P, int box, const double *r, double *z,
-                                              int accumulate) {
+                                              int accumulate, int polls) {
     if constexpr (PREC == 64) ras_apply_cells<PREC, 3>(P, box, r, z, accumulate);
-    else ras_apply_blocks<PREC>(P, box, r, z, accumulate);
+    else ras_apply_blocks<PREC, LIMIT>(P, box, r, z, accumulate, polls);
 }
 
 // 64 registers for 2 CTAs of 512 threads per SM with FP64 factors, 72 for two of 448 with
-// reduced ones
-template <int PREC>
+// reduced ones. LIMIT: the waits take the launch's poll limit.
+template <int PREC, bool LIMIT>
 __global__ void __maxnreg__(PREC == 64 ? 64 : 72) k_ras_apply(ApplyParams P) {
-    ras_apply_box<PREC>(P, blockIdx.x, P.r, P.z, P.accumulate);
+    ras_apply_box<PREC, LIMIT>(P, blockIdx.x, P.r, P.z, P.accumulate, P.polls);
 }
 
 // Left-RAS of many handles in one persistent launch: every CTA takes the next
@@ -651,7 +685,7 @@ __global__ void __maxnreg__(PREC == 64 ? 64 : 72) k_ras_apply(ApplyParams P) {
 // largest box first) until the queue is empty, and solves box box_local[item] of
 // handle box_inst[item] (items of inactive handles are skipped); r and z are the
 // handles' vectors concatenated at off[handle]. No CTA waits on another.
-template <int PREC>
+template <int PREC, bool LIMIT>
 __global__ void __maxnreg__(PREC == 64 ? 64 : 72) k_ras_apply_batch(BatchApply B) {
     __shared__ int s_item;
     for (;;) {
@@ -662,7 +696,7 @@ __global__ void __maxnreg__(PREC == 64 ? 64 : 72) k_ras_apply_batch(BatchApply B
         if (it >= B.nitems) return;
         const int h = B.box_inst[it];
         if (!B.active[h]) continue;
-        ras_apply_box<PREC>(B.inst[h], B.box_local[it], B.r + B.off[h], B.z + B.off[h], B.accumulate);
+        ras_apply_box<PREC, LIMIT>(B.inst[h], B.box_local[it], B.r + B.off[h], B.z + B.off[h], B.accumulate, B.polls);
     }
 }
 
@@ -873,12 +907,12 @@ static std::vector<int> split_axis(int n, int parts) {
 // The opt-in limit is raised to the per-CTA maximum once: a later set-up with
 // a smaller need must not lower it under a handle that needs more.
 constexpr int SMEM_OPTIN = 227 * 1024;
-template <int PREC>
+template <int PREC, bool LIMIT>
 static int set_apply_attr() {
-    RAS_CK(cudaFuncSetAttribute(k_ras_apply<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN));
+    RAS_CK(cudaFuncSetAttribute(k_ras_apply<PREC, LIMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_OPTIN));
     cudaFuncAttributes fa{};   // the persistent batch kernel has a little static shared memory
-    RAS_CK(cudaFuncGetAttributes(&fa, k_ras_apply_batch<PREC>));
-    RAS_CK(cudaFuncSetAttribute(k_ras_apply_batch<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    RAS_CK(cudaFuncGetAttributes(&fa, k_ras_apply_batch<PREC, LIMIT>));
+    RAS_CK(cudaFuncSetAttribute(k_ras_apply_batch<PREC, LIMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 SMEM_OPTIN - (int)fa.sharedSizeBytes));
     return RAS_OK;
 }
@@ -1208,7 +1242,7 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
     RAS_TRY(dalloc(&R.d_lvl, lvl_tab.size()));
     RAS_TRY(dalloc(&R.d_chunk, chunk_tab.size()));
     RAS_TRY(dalloc(&R.d_cidx, cidx_tab.size() + 16));
-    RAS_TRY(dalloc(&R.d_err, 1));
+    RAS_TRY(dalloc(&R.d_err, 2));
     unsigned char *fw = nullptr, *bw = nullptr;
     RAS_TRY(dalloc(&fw, (size_t)R.nrec * R.rec_bytes + 64));
     RAS_TRY(dalloc(&bw, (size_t)R.nrec * R.rec_bytes + 64));
@@ -1222,12 +1256,15 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
                       cudaMemcpyHostToDevice));
     RAS_CK(cudaMemset(R.d_cidx, 0, (cidx_tab.size() + 16) * sizeof(int)));
     RAS_CK(cudaMemcpy(R.d_cidx, cidx_tab.data(), cidx_tab.size() * sizeof(int), cudaMemcpyHostToDevice));
-    RAS_CK(cudaMemset(R.d_err, 0, sizeof(int)));
+    RAS_CK(cudaMemset(R.d_err, 0, 2 * sizeof(int)));
     RAS_CK(cudaMemset(R.d_fwd, 0, (size_t)R.nrec * R.rec_bytes + 64));
     RAS_CK(cudaMemset(R.d_bwd, 0, (size_t)R.nrec * R.rec_bytes + 64));
-    if (prec == 64) { RAS_TRY(set_apply_attr<64>()); RAS_TRY(set_factor_attr<64>()); }
-    if (prec == 32) { RAS_TRY(set_apply_attr<32>()); RAS_TRY(set_factor_attr<32>()); }
-    if (prec == 16) { RAS_TRY(set_apply_attr<16>()); RAS_TRY(set_factor_attr<16>()); }
+    if (prec == 64) RAS_TRY(set_apply_attr<64, false>());
+    if (prec == 32) { RAS_TRY(set_apply_attr<32, false>()); RAS_TRY(set_apply_attr<32, true>()); }
+    if (prec == 16) { RAS_TRY(set_apply_attr<16, false>()); RAS_TRY(set_apply_attr<16, true>()); }
+    if (prec == 64) RAS_TRY(set_factor_attr<64>());
+    if (prec == 32) RAS_TRY(set_factor_attr<32>());
+    if (prec == 16) RAS_TRY(set_factor_attr<16>());
     if (kind != 1) {
         // per axis and coordinate, the (contiguous) range of parts whose overlapped
         // boxes cover it; box solutions are kept per record offset
@@ -1290,13 +1327,11 @@ int ras1_check(Ras1 &R, cudaStream_t st) {
     int h = 0;
     RAS_CK(cudaMemcpyAsync(&h, R.d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     RAS_CK(cudaStreamSynchronize(st));
-    if (h) {
-        RAS_CK(cudaMemsetAsync(R.d_err, 0, sizeof(int), st));
-        if (h == APPLY_TIMEOUT) return RAS_ETIMEOUT;
-        return RAS_EZEROPIVOT;
-    }
-    return RAS_OK;
+    if (h) RAS_CK(cudaMemsetAsync(R.d_err, 0, sizeof(int), st));
+    return ras1_status(h);
 }
+
+int ras1_status(int word) { return word == 0 ? RAS_OK : (word == APPLY_TIMEOUT ? RAS_ETIMEOUT : RAS_EZEROPIVOT); }
 
 int ras1_set_kernel(Ras1 &R, int kernel) {
     if (kernel != 0 && kernel != 1) return RAS_EINVAL;
@@ -1305,6 +1340,8 @@ int ras1_set_kernel(Ras1 &R, int kernel) {
     return RAS_OK;
 }
 
+
+int ras1_polls() { return (int)std::min<long long>(barrier_polls(), APPLY_POLLS); }
 
 void ras1_apply_params(const Ras1 &R, ApplyParams &P) {
     P = ApplyParams{};
@@ -1320,9 +1357,10 @@ void ras1_apply_params(const Ras1 &R, ApplyParams &P) {
 int ras1_apply_batch(const BatchApply &B, int grid, int prec, int block, size_t smem, cudaStream_t st) {
     if (grid <= 0 || B.nitems <= 0) return RAS_OK;
     RAS_CK(cudaMemsetAsync(B.qcount, 0, sizeof(int), st));
-    if (prec == 64) k_ras_apply_batch<64><<<grid, block, smem, st>>>(B);
-    else if (prec == 32) k_ras_apply_batch<32><<<grid, block, smem, st>>>(B);
-    else k_ras_apply_batch<16><<<grid, block, smem, st>>>(B);
+    auto kern = prec == 64 ? k_ras_apply_batch<64, false>
+              : prec == 32 ? (B.polls > 0 ? k_ras_apply_batch<32, true> : k_ras_apply_batch<32, false>)
+                           : (B.polls > 0 ? k_ras_apply_batch<16, true> : k_ras_apply_batch<16, false>);
+    kern<<<grid, block, smem, st>>>(B);
     RAS_LAUNCHED();
     return RAS_OK;
 }
@@ -1331,9 +1369,9 @@ int ras1_batch_grid(int prec, int block, size_t smem, int nitems, int *grid) {
     int dev = 0, sms = 0, per = 0;
     RAS_CK(cudaGetDevice(&dev));
     RAS_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (prec == 64) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<64>, block, smem));
-    else if (prec == 32) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<32>, block, smem));
-    else RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<16>, block, smem));
+    if (prec == 64) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<64, false>, block, smem));
+    else if (prec == 32) RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<32, false>, block, smem));
+    else RAS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply_batch<16, false>, block, smem));
     if (per < 1) return RAS_EINVAL;
     *grid = std::min(nitems, sms * per);
     return RAS_OK;
@@ -1343,9 +1381,11 @@ int ras1_apply(Ras1 &R, const double *r, double *z, int accumulate, cudaStream_t
     ApplyParams P;
     ras1_apply_params(R, P);
     P.r = r; P.z = z; P.accumulate = accumulate;
-    if (R.prec == 64) k_ras_apply<64><<<R.nsub, R.launch, R.smem_apply, st>>>(P);
-    else if (R.prec == 32) k_ras_apply<32><<<R.nsub, R.launch, R.smem_apply, st>>>(P);
-    else k_ras_apply<16><<<R.nsub, R.launch, R.smem_apply, st>>>(P);
+    P.polls = ras1_polls();
+    auto kern = R.prec == 64 ? k_ras_apply<64, false>
+              : R.prec == 32 ? (P.polls > 0 ? k_ras_apply<32, true> : k_ras_apply<32, false>)
+                             : (P.polls > 0 ? k_ras_apply<16, true> : k_ras_apply<16, false>);
+    kern<<<R.nsub, R.launch, R.smem_apply, st>>>(P);
     RAS_LAUNCHED();
     if (R.kind != 1) {
         SumParams Q;

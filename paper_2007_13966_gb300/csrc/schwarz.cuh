@@ -62,7 +62,7 @@ struct Ras1 {
     int *d_lvl = nullptr, *d_chunk = nullptr;
     int *d_cidx = nullptr;  // level-ordered local index of each cell (block)
     void *d_fwd = nullptr, *d_bwd = nullptr;
-    int *d_err = nullptr;
+    int *d_err = nullptr;   // the factors' and the sweeps' error word, then one for the handle's coarse level
     // AS (kind 0) and right-RAS (kind 2): each box's whole solution goes to zbuf
     // (at the box's record offset), then every cell sums the boxes covering it
     int kind = 1;
@@ -84,6 +84,7 @@ void ras1_free(Ras1 &R);
 int ras1_factor(Ras1 &R, const Stencil7 &A, cudaStream_t st);
 // reads and clears the pivot flag and that of a sweep's wait that ran out (synchronises)
 int ras1_check(Ras1 &R, cudaStream_t st);
+int ras1_status(int word);
 // z = M^{-1} r (accumulate = 0) or z += M^{-1} r (accumulate = 1), with
 // M^{-1} = sum_i (R_i^0)^T A_i^{-1} R_i^delta (left-RAS, kind 1),
 // sum_i (R_i^delta)^T A_i^{-1} R_i^delta (AS, kind 0) or
@@ -109,6 +110,7 @@ struct ApplyParams {
     int ycap, gcap, lcap, chunk_cells;
     const int4 *steps;   // sweeps in blocks: per shape and step (schedule_tables)
     int *err;            // a wait that ran out
+    int polls;           // its poll limit (0: the default)
     int kind;        // 1 left-RAS; 0 AS, 2 right-RAS (box solutions to zbuf)
     double *zbuf;
 };
@@ -124,7 +126,10 @@ struct BatchApply {
     int accumulate;                   // z += (instead of =) the correction
     int nitems;                       // boxes in the work queue (box_inst / box_local order)
     int *qcount;                      // device work counter, cleared before each launch
+    int polls;                        // poll limit of the sweeps' waits (0: the default)
 };
+// the poll limit of the sweeps' waits for the next launch (barrier_polls)
+int ras1_polls();
 void ras1_apply_params(const Ras1 &R, ApplyParams &P);
 // parameters of one handle's ILU(0) factorisation kernel on operator A
 struct FactorParams {
