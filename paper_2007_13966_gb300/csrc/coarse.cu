@@ -1267,11 +1267,11 @@ __device__ __forceinline__ void gj_tile_inverse(float (&a)[4], float *W, bool &o
         if (I != s) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                float t = pc ? 0.0f : a[u];
-                t = fmaf(-c[u][0], w.x, t);
-                t = fmaf(-c[u][1], w.y, t);
-                t = fmaf(-c[u][2], w.z, t);
-                a[u] = fmaf(-c[u][3], w.w, t);
+                float t = c[u][0] * w.x;                         // (summed before it meets a: see gj_pivot)
+                t = fmaf(c[u][1], w.y, t);
+                t = fmaf(c[u][2], w.z, t);
+                t = fmaf(c[u][3], w.w, t);
+                a[u] = (pc ? 0.0f : a[u]) - t;
             }
         }
         if (s == 7) break;
@@ -1309,6 +1309,9 @@ __device__ __forceinline__ void gj_tile_inverse(double (&a)[1], double *W, bool 
 
 // The inverse P of panel p's pivot block: the block itself for p = 0 (read from M), else
 // the look-ahead block less A P R of the previous panel, from the strips of step p - 2.
+// FP32: A P R is summed by itself and subtracted once. Subtracted term by term, its many
+// small terms are rounded at the block's own size, and those below half a unit of it are
+// lost, all to one side: that was most of the error of the inverses.
 template <typename AT>
 __device__ __noinline__ void gj_pivot(const AT *M, AT *Z, int T, int p, unsigned char *smem, int *err) {
     constexpr int NB = Gj<AT>::NB, NE = NB * NB / 256;           // values per thread
@@ -1349,12 +1352,12 @@ __device__ __noinline__ void gj_pivot(const AT *M, AT *Z, int T, int p, unsigned
         }
         __syncthreads();
         // t[u] (+)= sum_k row(u)[k] col[k]: rows of a row-major block, 16 bytes at a time
-        auto product = [&](const AT *rows, const AT *cols, AT (&t)[NE], AT sign) {
+        auto product = [&](const AT *rows, const AT *cols, AT (&t)[NE]) {
 #pragma unroll
             for (int k = 0; k < NB; k += VE) {
                 AT x[VE];
 #pragma unroll
-                for (int m = 0; m < VE; ++m) x[m] = sign * cols[(k + m) * NB + c];
+                for (int m = 0; m < VE; ++m) x[m] = cols[(k + m) * NB + c];
 #pragma unroll
                 for (int u = 0; u < NE; ++u) {
                     const V q = *reinterpret_cast<const V *>(rows + u * NB + k);
@@ -1367,15 +1370,18 @@ __device__ __noinline__ void gj_pivot(const AT *M, AT *Z, int T, int p, unsigned
         AT t[NE];
 #pragma unroll
         for (int u = 0; u < NE; ++u) t[u] = 0;
-        product(Ps + rr * NB, Xs, t, (AT)1);                     // U = P R
+        product(Ps + rr * NB, Xs, t);                            // U = P R
 #pragma unroll
         for (int u = 0; u < NE; ++u) {
             Us[(rr + u) * NB + c] = t[u];
             a[u] = Ds[(rr + u) * NB + c];
+            t[u] = 0;
         }
         __syncthreads();
         if constexpr (sizeof(AT) == 4) {                         // D - A U
-            product(As + rr * NB, Us, a, (AT)-1);
+            product(As + rr * NB, Us, t);
+#pragma unroll
+            for (int u = 0; u < NE; ++u) a[u] -= t[u];
         } else {                                                 // (A transposed)
 #pragma unroll
             for (int k = 0; k < NB; ++k) a[0] = fma(-As[k * NB + rr], Us[k * NB + c], a[0]);
@@ -1429,6 +1435,17 @@ __device__ __forceinline__ bool gj_wait(const unsigned *f0, const unsigned *f1, 
 // zero, 12 times per panel: the coarse correction's error against FP64 was ten times
 // larger (1.5e-5 for 1.6e-6 on a 64 x 96 x 48 grid). The same step on the CUDA cores took
 // 13,300 cycles, twice the pivot CTA's time.
+// Precision: the MMAs cut addends and running sums towards zero. On these products, of 32
+// terms mostly of one sign, that loses 0.8 to 2.1 x 2^-23 of a result (a CPU emulation of
+// the rounding, checked against ras_gemm_f32, on seven coarse operators), so 1 + 2^-23 times
+// it is taken (GJ_CUT: an FMA in the place of the addition). With that and the pivot block's
+// sums taken apart (gj_pivot) the FP32 coarse correction is nearer to the FP64 one than with
+// the 64 x 64 pivot tiles that this form replaced: relative error, geometric means over 5 to
+// 10 reservoirs and 4 vectors, those tiles / neither / both: 50 x 50 coarse cells
+// 1.30e-5 / 2.33e-5 / 0.65e-5, 20 x 12 x 12 3.6e-5 / 5.5e-5 / 1.3e-5, 16 x 24 x 12
+// 5.1e-5 / 6.5e-5 / 3.3e-5, 32 x 32 x 16 1.53e-4 / 2.19e-4 / 1.28e-4. Three values of -q and
+// R where the panel's rows are formed (P R) give the same errors, for 1 to 2 % of an FP32 step.
+constexpr float GJ_CUT = 1.0f + 1.1920929e-7f;  // 1 + 2^-23
 constexpr unsigned GJ_TMEM = 256;               // columns held: (-q) R 0 .. 127, q 128 .. 159
 constexpr unsigned GJ_SBO = 1024;               // 8 rows x 32 k of TF32: eight 128-byte core matrices
 constexpr unsigned GJ_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 4) << 24);   // + N / 8 << 17
@@ -1595,6 +1612,8 @@ __device__ __forceinline__ void gj_tile_step(GjTile &t, TcState &st, float *Z, i
         for (int k = 0; k < 64; ++k) t.v[k] = 0.f;
     } else {
         gj_ld32(t.tq, q);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) q[k] *= GJ_CUT;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {                                     // -q over A (whose MMAs are done), half a row each
@@ -1613,7 +1632,7 @@ __device__ __forceinline__ void gj_tile_step(GjTile &t, TcState &st, float *Z, i
         gj_ld32(t.tm + 32 * h, x);
         const int col = h0 + 32 * h, cp = col / NB;
 #pragma unroll
-        for (int k = 0; k < 32; ++k) t.v[32 * h + k] = cp == p ? -q[k] : t.v[32 * h + k] + x[k];
+        for (int k = 0; k < 32; ++k) t.v[32 * h + k] = cp == p ? -q[k] : fmaf(x[k], GJ_CUT, t.v[32 * h + k]);
         // the next panel's rows (by column) and columns (by row), and the diagonal block after it
         if (rp == n && col < T) {
             float *o = S.r(n) + (size_t)col * NB + lane;
