@@ -3,15 +3,22 @@ against the FP64 one of the same handle options: relative error over several res
 right-hand sides, geometric mean. The bounds are the errors measured with the 64 x 64 pivot
 tiles (panels by FP32 multiply-adds) that the present block inverses replaced and must not
 exceed: 50 x 50, 20 x 12 x 12 and 16 x 24 x 12 coarse cells (blocks of T = 128, 320 and
-384, and so edge tiles of 128 rows and tiles partly beyond the block)."""
+384, and so edge tiles of 128 rows and tiles partly beyond the block). The FP64 correction
+the same against the oracle's operator, solved with residuals in extended precision, on
+16^3 coarse cells (8 blocks of 512)."""
 import math
 
+import numpy as np
 import pytest
+import scipy.sparse as sp
+import scipy.sparse.linalg as sla
 import torch
 
+from oracle import discretization as disc
+from oracle import multilevel as ml
 from paper_2007_13966_gb300 import synthetic as syn
 
-from gpu_util import dev
+from gpu_util import dev, host, j_to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -46,3 +53,37 @@ def test_no_further_from_fp64_than_the_tiles_replaced(dims, ratio, count, bound)
                 pc.apply(v, zz)
         logs += [math.log(float((a - b).norm() / b.norm())) for a, b in zip(z[32], z[64])]
     assert math.exp(sum(logs) / len(logs)) < bound
+
+
+def _refined(A, b):
+    """A x = b in FP64 with residuals in extended precision."""
+    A = sp.csr_matrix(A)
+    A.sort_indices()
+    lu = sla.splu(sp.csc_matrix(A))
+    L = np.longdouble
+    x, data = lu.solve(b).astype(L), A.data.astype(L)
+    for _ in range(4):
+        r = b.astype(L) - np.add.reduceat(data * x[A.indices], A.indptr[:-1])
+        x = x + lu.solve(r.astype(np.float64))
+    return x.astype(np.float64)
+
+
+def test_fp64_sums_are_taken_apart():
+    """Bound: 1.5 times the 2.03e-13 of the tiles replaced (single reservoirs 1.7e-13 to
+    3.0e-13); with every term of an update rounded at the value's own size: 4.1e-13."""
+    from paper_2007_13966_gb300 import ras
+    dims, ratio, logs = (64, 64, 64), (4, 4, 4), []
+    for seed in (5, 15, 25, 35):
+        res = _reservoir(dims, seed)
+        p = syn.random_pressure(res, seed)
+        F, J = disc.residual(disc.Problem(res), p, 0.99 * p, 0.98 * p, res.dt, 2, want_jac=True)
+        A, P = disc.jacobian_csr(res.grid, J), ml.interpolation(dims, ratio, 2)
+        b = -np.asarray(F).ravel()
+        ref = P @ _refined(P.T @ A @ P, P.T @ b)
+        pc = ras.Precond(ras.Problem(res), (4, 4, 4), 1, factor_prec=64, nlevels=2, coarsen=ratio, coarse_prec=64,
+                         mlevel_type=4)
+        pc.factor(j_to_dev(J))
+        z = torch.zeros(res.grid.n, dtype=torch.float64, device="cuda")
+        pc.apply(dev(b), z)
+        logs.append(math.log(np.linalg.norm(host(z) - ref) / np.linalg.norm(ref)))
+    assert math.exp(sum(logs) / len(logs)) < 1.5 * 2.03e-13
