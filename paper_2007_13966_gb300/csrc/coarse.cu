@@ -1634,7 +1634,7 @@ __device__ __forceinline__ void gj_tile_step(GjTile &t, TcState &st, float *Z, i
 #pragma unroll
         for (int k = 0; k < 32; ++k) t.v[32 * h + k] = cp == p ? -q[k] : fmaf(x[k], GJ_CUT, t.v[32 * h + k]);
         // the next panel's rows (by column) and columns (by row), and the diagonal block after it
-        if (rp == n && col < T) {
+        if (rp == n && row < T && col < T) {                          // (no strip of rows beyond the block)
             float *o = S.r(n) + (size_t)col * NB + lane;
 #pragma unroll
             for (int k = 0; k < 32; ++k) o[k * NB] = t.v[32 * h + k];
