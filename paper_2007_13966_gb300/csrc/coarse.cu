@@ -1217,8 +1217,43 @@ __device__ __forceinline__ double gj_recip(double x) {
 // barrier per step. FP32: warp I holds rows 4 I .. 4 I + 3, lane c column c, 4 pivots per
 // step, by elimination of the 4 x 4 block on every lane's own right-hand side (its column,
 // or a unit vector in the pivot columns): ~45 instructions, where forming the 4 x 4 inverse
-// first takes ~140 (650 cycles of a 1,000-cycle step: one warp alone issues slowly). FP64:
+// first takes ~140 (650 cycles of a 1,000-cycle step: one warp alone issues slowly). `ok` is
+// also cleared where a pivot inside a 4 x 4 block is small beside the values below it; such
+// a block may be regular all the same, and with EXCHANGE its rows are exchanged. FP64:
 // warp I holds rows 2 I, 2 I + 1, lane (u, c) row 2 I + u and column c, 2 pivots per step.
+constexpr float GJ_GROW = 64.0f;   // sum of a 4 x 4 block's six multipliers beyond which rows are exchanged
+// c w' = w for a 4 x 4 block c by elimination with row exchanges; false if c is singular
+// or not finite
+__device__ __forceinline__ bool gj_solve4(float (&c)[4][4], float (&w)[4]) {
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int u = k + 1; u < 4; ++u)              // the largest of the column's rest comes to row k
+            if (fabsf(c[u][k]) > fabsf(c[k][k])) {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) { const float t = c[k][m]; c[k][m] = c[u][m]; c[u][m] = t; }
+                const float t = w[k];
+                w[k] = w[u];
+                w[u] = t;
+            }
+        if (!(c[k][k] != 0.0f) || !isfinite(c[k][k])) ok = false;
+        const float inv = gj_recip(c[k][k]);
+#pragma unroll
+        for (int m = k; m < 4; ++m) c[k][m] *= inv;
+        w[k] *= inv;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (u != k) {
+                const float l = c[u][k];
+#pragma unroll
+                for (int m = k; m < 4; ++m) c[u][m] = fmaf(-l, c[k][m], c[u][m]);
+                w[u] = fmaf(-l, w[k], w[u]);
+            }
+    }
+    return ok;
+}
+template <bool EXCHANGE>
 __device__ __forceinline__ void gj_tile_inverse(float (&a)[4], float *W, bool &ok) {
     // (the shuffle makes the warp number warp-uniform to the compiler)
     const int I = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -1232,26 +1267,33 @@ __device__ __forceinline__ void gj_tile_inverse(float (&a)[4], float *W, bool &o
     };
     auto scale = [&](int s) {
         const bool pc = (lane >> 2) == s;
-        float w[4], inv[4];
+        float w[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) w[u] = pc ? ((lane & 3) == u ? 1.0f : 0.0f) : a[u];
+        if constexpr (EXCHANGE) {
+            if (!gj_solve4(c, w)) ok = false;
+        } else {
+            float inv[4], grow = 0.0f;               // the multipliers, and 1 per pivot (not a number: 0 or infinite)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (!(c[k][k] != 0.0f) || !isfinite(c[k][k])) ok = false;
-            inv[k] = gj_recip(c[k][k]);
+            for (int k = 0; k < 4; ++k) {
+                inv[k] = gj_recip(c[k][k]);
+                grow = fmaf(c[k][k], inv[k], grow);
 #pragma unroll
-            for (int u = k + 1; u < 4; ++u) {
-                const float l = c[u][k] * inv[k];
+                for (int u = k + 1; u < 4; ++u) {
+                    const float l = c[u][k] * inv[k];
+                    grow += fabsf(l);
 #pragma unroll
-                for (int m = k + 1; m < 4; ++m) c[u][m] = fmaf(-l, c[k][m], c[u][m]);
-                w[u] = fmaf(-l, w[k], w[u]);
+                    for (int m = k + 1; m < 4; ++m) c[u][m] = fmaf(-l, c[k][m], c[u][m]);
+                    w[u] = fmaf(-l, w[k], w[u]);
+                }
             }
-        }
 #pragma unroll
-        for (int k = 3; k >= 0; --k) {
-            w[k] *= inv[k];
+            for (int k = 3; k >= 0; --k) {
+                w[k] *= inv[k];
 #pragma unroll
-            for (int u = 0; u < k; ++u) w[u] = fmaf(-c[u][k], w[k], w[u]);
+                for (int u = 0; u < k; ++u) w[u] = fmaf(-c[u][k], w[k], w[u]);
+            }
+            if (!(grow <= GJ_GROW)) ok = false;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) a[u] = w[u];
@@ -1279,6 +1321,7 @@ __device__ __forceinline__ void gj_tile_inverse(float (&a)[4], float *W, bool &o
         if (I == s + 1) scale(s + 1);
     }
 }
+template <bool>
 __device__ __forceinline__ void gj_tile_inverse(double (&a)[1], double *W, bool &ok) {
     const int I = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31, u = lane >> 4, c = lane & 15;
@@ -1290,7 +1333,7 @@ __device__ __forceinline__ void gj_tile_inverse(double (&a)[1], double *W, bool 
         const double n0 = u ? -b10 : b11, n1 = u ? b00 : -b01;               // row u of the adjugate
         const double t = (c >> 1) == s ? ((c & 1) ? n1 : n0) : fma(n1, a1, n0 * a0);
         const double det = fma(b00, b11, -b01 * b10);
-        if (!(det != 0.0) || !isfinite(det)) ok = false;
+        if (!(b00 != 0.0) || !(det != 0.0) || !isfinite(det)) ok = false;   // (the pivots b00, det / b00)
         const double w = t * gj_recip(det);
         a[0] = w;
         W[(s & 1) * 32 + lane] = w;
@@ -1305,6 +1348,16 @@ __device__ __forceinline__ void gj_tile_inverse(double (&a)[1], double *W, bool 
         if (I != s) a[0] = fma(-m1, w1, fma(-m0, w0, (c >> 1) == s ? 0.0 : a[0]));
         if (I == s + 1) scale(s + 1);
     }
+}
+
+// The inverse of the block that the CTA's threads left in `block` (4 values each), with row
+// exchanges inside the 4 x 4 pivot blocks
+__device__ __noinline__ void gj_exchange(float *block, float *W, bool &ok) {
+    float4 &v = reinterpret_cast<float4 *>(block)[threadIdx.x];
+    float a[4] = {v.x, v.y, v.z, v.w};
+    ok = true;
+    gj_tile_inverse<true>(a, W, ok);
+    v = make_float4(a[0], a[1], a[2], a[3]);
 }
 
 // The inverse P of panel p's pivot block: the block itself for p = 0 (read from M), else
@@ -1387,15 +1440,30 @@ __device__ __noinline__ void gj_pivot(const AT *M, AT *Z, int T, int p, unsigned
             for (int k = 0; k < NB; ++k) a[0] = fma(-As[k * NB + rr], Us[k * NB + c], a[0]);
         }
     }
-    bool ok = true;
-    gj_tile_inverse(a, W, ok);
-    if (!ok) atomicExch(err, ERR_PIVOT);
     AT *out = S.pi(p);
+    auto store = [&] {
 #pragma unroll
-    for (int u = 0; u < NE; ++u) out[(rr + u) * NB + c] = a[u];
-    if constexpr (sizeof(AT) == 4)
-        *reinterpret_cast<float4 *>(S.pt(p) + c * NB + rr) = make_float4(a[0], a[1], a[2], a[3]);
-    __syncthreads();   // the shared memory is free again
+        for (int u = 0; u < NE; ++u) out[(rr + u) * NB + c] = a[u];
+        if constexpr (sizeof(AT) == 4)
+            *reinterpret_cast<float4 *>(S.pt(p) + c * NB + rr) = make_float4(a[0], a[1], a[2], a[3]);
+    };
+    bool ok = true;
+    if constexpr (sizeof(AT) == 4)      // (P's place is free)
+        *reinterpret_cast<float4 *>(Ps + threadIdx.x * NE) = make_float4(a[0], a[1], a[2], a[3]);
+    gj_tile_inverse<false>(a, W, ok);
+    store();
+    const bool bad = __syncthreads_or(!ok) != 0;   // (the shared memory is free again)
+    if (bad && sizeof(AT) == 8 && threadIdx.x == 0) atomicExch(err, ERR_PIVOT);
+    if constexpr (sizeof(AT) == 4) {
+        if (bad) {
+            gj_exchange(Ps, W, ok);
+#pragma unroll
+            for (int u = 0; u < NE; ++u) a[u] = Ps[threadIdx.x * NE + u];
+            if (!ok) atomicExch(err, ERR_PIVOT);
+            store();
+            __syncthreads();
+        }
+    }
 }
 
 // Sets a ready flag after the CTA's earlier writes (gj_signal1: the caller has met at a
