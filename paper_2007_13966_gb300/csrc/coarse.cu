@@ -29,6 +29,7 @@
 // natural order; FP32 handles may take the cyclic reduction of the block
 // tridiagonal system instead of the two-ended elimination (RAS_COARSE_CR=1).
 #include "precond.cuh"
+#include "recip.cuh"
 
 #include <algorithm>
 #include <cstddef>
@@ -1197,18 +1198,9 @@ __host__ __device__ constexpr size_t gj_smem(int T) {
     return rows > piv ? rows : piv;
 }
 
-// 1 / x: FP32, the hardware's approximate reciprocal (preconditioner factors); FP64, one
-// third-order step y (1 + e + e^2), e = 1 - x y, from the FP32 reciprocal (24 bits -> 72),
-// where x lies in FP32's normal range (IEEE reciprocal otherwise): three dependent
-// operations on a pipe where each takes ~64 cycles, against ~440 cycles for the IEEE one.
+// 1 / x (FP32: the hardware's approximate reciprocal, preconditioner factors)
 __device__ __forceinline__ float gj_recip(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double gj_recip(double x) {
-    const double ax = fabs(x);
-    if (!(ax > 1e-36 && ax < 1e36)) return __drcp_rn(x);
-    const double y = (double)__fdividef(1.0f, (float)x);
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
+__device__ __forceinline__ double gj_recip(double x) { return recip64(x); }
 
 // Inverse of an NB x NB block held one column per lane by 8 warps, block row by block
 // row; `ok` is cleared on a zero or non-finite pivot. The warp that owns the next pivot

@@ -1,6 +1,7 @@
 // Discrete problem: Peng-Robinson EOS per cell, two-point-flux residual and
 // exact Jacobian with BDF1/BDF2 (Section 2), 7-point operator products and
 // deterministic reductions.
+#include "recip.cuh"
 #include "common.cuh"
 
 #include <cstring>
@@ -300,17 +301,6 @@ struct EosOut {
     double Z, iZ;
     bool ok;   // an admissible root: Z finite, Z > B, f_Z != 0
 };
-
-// 1 / x by one third-order step y (1 + e + e^2), e = 1 - x y, from the FP32 reciprocal
-// (24 bits -> 72, then FP64 rounding), where x lies in FP32's normal range: 3 operations of
-// the FP64 pipe (2 per cycle and SM) and two conversions, where a division takes about ten
-__device__ __forceinline__ double recip64(double x) {
-    const double ax = fabs(x);
-    if (!(ax > 1e-36 && ax < 1e36)) return 1.0 / x;
-    const double y = (double)__frcp_rn((float)x);
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
 
 // The largest real root Z of Z^3 + c2 Z^2 + c1 Z + c0. FP32 closed form, then Newton steps
 // with FP64 residuals. The first two take the slope's reciprocal in FP32: near a simple

@@ -9,6 +9,8 @@
 // shared-memory ring with cp.async ahead of the sweep that consumes it.
 #include "schwarz.cuh"
 
+#include "recip.cuh"
+
 #include <algorithm>
 #include <cstdlib>
 #include <map>
@@ -747,16 +749,6 @@ __host__ __device__ __forceinline__ int diag_base(int d, int nu, int nv) {
 // position of (u, v) in the order by diagonal u + v, then u
 __host__ __device__ __forceinline__ int diag_pos(int u, int v, int nu, int nv) {
     return diag_base(u + v, nu, nv) + u - max(0, u + v - (nv - 1));
-}
-
-// 1 / x by one third-order step y (1 + e + e^2), e = 1 - x y, from the FP32 reciprocal
-// (24 bits -> 72, then FP64 rounding), where x lies in FP32's normal range
-__device__ __forceinline__ double recip64(double x) {
-    const double ax = fabs(x);
-    if (!(ax > 1e-36 && ax < 1e36)) return 1.0 / x;
-    const double y = (double)__frcp_rn((float)x);
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
 }
 
 // axis along which the factorisation's pencils run: x unless that leaves too many
