@@ -71,7 +71,7 @@ def parse():
     ap.add_argument("--reps", type=int, default=20)
     ap.add_argument("--apply-kernel", type=int, choices=[0, 1], default=None,
                     help="fine subdomain-solve kernel setting (0 and 1 run the same sweeps; "
-                         "(default: the library's choice)")
+                         "default: the library's choice)")
     return ap.parse_args()
 
 

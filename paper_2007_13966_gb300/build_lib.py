@@ -36,8 +36,8 @@ def source_hash(files=None) -> str:
     return h.hexdigest()[:16]
 
 
-# files that define the fine-level subdomain-solve kernels (k_ras_apply, k_ras_pipe):
-# their own source; the shared header holds host-side declarations only
+# files that define the fine-level subdomain-solve kernel (k_ras_apply): its own source; the
+# shared headers hold declarations and the factorisation's reciprocal only
 RAS_APPLY_FILES = ("schwarz.cuh", "schwarz.cu")
 
 

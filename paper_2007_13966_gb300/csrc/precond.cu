@@ -303,7 +303,7 @@ extern "C" int ras_set_apply_kernel(ras_precond *pc, int kernel) {
 
 extern "C" int ras_get_apply_kernel(const ras_precond *pc, int *kernel) {
     if (!pc || !kernel) return RAS_EINVAL;
-    *kernel = pc->use125 ? 0 : pc->fine.pipe;
+    *kernel = pc->use125 ? 0 : pc->fine.kernel;
     return RAS_OK;
 }
 

@@ -917,14 +917,6 @@ static int set_factor_attr() {
     return RAS_OK;
 }
 
-// The pencil-wavefront kernel's limits (ras_set_apply_kernel): its shared memory for
-// the handle's chunk size
-static size_t pencil_smem(const Ras1 &R) {
-    const size_t ybytes = (((size_t)(R.ycap_pipe + 4) * 4) + 15) & ~(size_t)15;
-    const size_t rcap = ((R.chunk_cells * R.rec_bytes + 32) + 15) & ~15;
-    return ybytes + 2 * (size_t)R.lcap_cells * sizeof(int) + (size_t)R.dcap_pipe * 8 + 3 * rcap;
-}
-
 // Level schedule of the subdomain solves: chunks of consecutive levels with at most
 // chunk_cells cells (staged into the shared-memory ring together) and threads per
 // box. 0 takes the default (chunk 1024 cells, 384 in FP64; threads: the widest
@@ -947,7 +939,8 @@ static int schedule_tables(Ras1 &R, int chunk_cells, int threads, std::vector<in
         if (threads > 512 || threads % 32) return RAS_EINVAL;
         block = threads;
     }
-    // the shared memory of the sweeps cell by cell decides what is accepted
+    // what a schedule may ask for: the shared memory of the sweeps cell by cell (the sweeps in
+    // blocks cut their ring to the room there is, and would take any chunk)
     const size_t acc = R.prec == 64 ? 8 : 4;
     const size_t rcap = ((cc * R.rec_bytes + 32) + 15) & ~15;
     const size_t ccap = ((cc * 4 + 32) + 15) & ~15;
@@ -1061,7 +1054,6 @@ int ras1_set_schedule(Ras1 &R, int chunk_cells, int threads) {
     R.launch = T.launch;
     R.block = T.block;
     R.smem_apply = T.smem_apply;
-    if (R.pipe_ok && pencil_smem(R) > 227 * 1024) R.pipe = R.pipe_ok = 0;
     return RAS_OK;
 }
 
@@ -1211,23 +1203,6 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
     RAS_TRY(schedule_tables(R, 0, 0, chunk_tab));
     const std::vector<int> &lvl_tab = R.h_lvl;
     if (R.smem_apply > 227 * 1024 || R.smem_factor > 227 * 1024) return RAS_EINVAL;
-    // handles for which the pencil-wavefront kernel may be asked for: left-RAS with FP32
-    // / BF16 factors, at most 1024 x-pencils per box
-    {
-        bool ok = kind == 1 && prec != 64;
-        int pens = 1, ycp = 0, dmax = 1;
-        for (const ShapeInfo &sh : R.shapes) {
-            pens = std::max(pens, sh.by * sh.bz);
-            ycp = std::max(ycp, (sh.bx * sh.by + ((sh.bx * (sh.by - 1)) % 2 == 0 ? 1 : 0)) * sh.bz);
-            dmax = std::max(dmax, sh.by + sh.bz - 1);
-        }
-        if (pens > 1024) ok = false;
-        R.ycap_pipe = (ycp + 3) & ~3;
-        R.dcap_pipe = (dmax + 1) & ~1;
-        if (pencil_smem(R) > 227 * 1024) ok = false;
-        R.pipe_ok = ok ? 1 : 0;
-        R.pipe = 0;
-    }
     RAS_TRY(dalloc(&R.d_boxes, R.subs.size()));
     RAS_TRY(dalloc(&R.d_subs, R.subs.size()));
     RAS_TRY(dalloc(&R.d_shapes, R.shapes.size()));
@@ -1327,8 +1302,12 @@ int ras1_status(int word) { return word == 0 ? RAS_OK : (word == APPLY_TIMEOUT ?
 
 int ras1_set_kernel(Ras1 &R, int kernel) {
     if (kernel != 0 && kernel != 1) return RAS_EINVAL;
-    if (kernel == 1 && !R.pipe_ok) return RAS_EINVAL;
-    R.pipe = kernel;
+    if (kernel == 1) {
+        if (R.kind != 1 || R.prec == 64) return RAS_EINVAL;
+        for (const ShapeInfo &sh : R.shapes)
+            if (sh.by * sh.bz > 1024) return RAS_EINVAL;
+    }
+    R.kernel = kernel;
     return RAS_OK;
 }
 

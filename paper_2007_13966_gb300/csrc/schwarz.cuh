@@ -71,10 +71,7 @@ struct Ras1 {
     int parts[3] = {1, 1, 1};
     std::vector<SubInfo> subs;
     std::vector<ShapeInfo> shapes;
-    // ras_set_apply_kernel's choice (both values run the same kernel) and its limits
-    int pipe = 0;
-    int pipe_ok = 0;
-    int dcap_pipe = 0, ycap_pipe = 0;
+    int kernel = 0;   // ras_set_apply_kernel's value (0 and 1 run the same sweeps)
 };
 
 int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int overlap, int prec,
