@@ -414,8 +414,8 @@ double ras_apply_bytes(const ras_precond *pc);
  * take more). 0 keeps the default of that argument (1024 cells, 384 for FP64 factors; the
  * widest level rounded up to a warp). Smaller chunks use less shared memory per box, so
  * more boxes run per SM: worth it when there are many more boxes than SMs. Synchronous;
- * no apply of this handle may be in flight; a batch created before the call keeps the old
- * launch settings (create it again). RAS_EINVAL for ILU(k > 0) handles, negative or
+ * no apply of this handle may be in flight; a batch created before the call takes the new
+ * schedule at its next call. RAS_EINVAL for ILU(k > 0) handles, negative or
  * invalid values, or a schedule whose shared memory exceeds the per-block limit (the old
  * schedule stays). */
 int ras_set_apply_schedule(ras_precond *pc, int chunk_cells, int threads);

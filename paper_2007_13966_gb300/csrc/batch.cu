@@ -311,6 +311,7 @@ struct ras_batch {
     int n = 0;
     std::vector<ras_problem *> P;
     std::vector<ras_precond *> pc;
+    std::vector<int> sched;                  // the handles' schedules that the launch settings were made for
     std::vector<long long> off;              // cell offset of each reservoir
     long long Ntot = 0;
     int nch = 0, nbox = 0, qgrid = 0;       // chunks; boxes in the work queue; persistent CTAs
@@ -768,11 +769,44 @@ static int bfgmres_run(ras_batch *B, const std::vector<unsigned char> &want, con
     return status;
 }
 
+// The launch settings of the batched subdomain solves and the handles' parameters, from the
+// handles' present schedules
+static int launch_settings(ras_batch *B) {
+    std::vector<ApplyParams> ap(B->n);
+    B->block = 0;
+    B->smem = 0;
+    B->sched.assign(B->n, 0);
+    for (int i = 0; i < B->n; ++i) {
+        const Ras1 &R = B->pc[i]->fine;
+        ras1_apply_params(R, ap[i]);
+        B->block = std::max(B->block, R.launch);
+        B->smem = std::max(B->smem, R.smem_apply);
+        B->sched[i] = R.sched;
+    }
+    RAS_TRY(ras1_batch_grid(B->prec, B->block, B->smem, B->nbox, &B->qgrid));
+    RAS_CK(cudaMemcpy(B->d_ap, ap.data(), B->n * sizeof(ApplyParams), cudaMemcpyHostToDevice));
+    return RAS_OK;
+}
+
+// ... made again when a handle's schedule has changed since (its tables moved): also the
+// captured cycles, which hold them
+static int refresh_schedules(ras_batch *B, cudaStream_t st) {
+    bool same = true;
+    for (int i = 0; i < B->n; ++i) same = same && B->sched[i] == B->pc[i]->fine.sched;
+    if (same) return RAS_OK;
+    RAS_CK(cudaStreamSynchronize(st));
+    for (auto &g : B->cycle_exec)
+        if (g) cudaGraphExecDestroy(g);
+    B->cycle_exec.clear();
+    return launch_settings(B);
+}
+
 // The batched FGMRES; on an early error return (a non-finite value after a coarse
 // solve whose barrier wait ran out, say) the deferred error words are still read
 // and cleared, and the device error, which explains the other, is reported.
 static int bfgmres(ras_batch *B, const std::vector<unsigned char> &want, const ras_krylov_opts &o,
                    ras_krylov_stats *stats, cudaStream_t st) {
+    RAS_TRY(refresh_schedules(B, st));
     const int rc = bfgmres_run(B, want, o, stats, st);
     if (rc >= 0) return rc;
     const int d = drain_checks(B, want, false, st);
@@ -991,7 +1025,6 @@ static int batch_create(int n, ras_problem *const *probs, ras_precond *const *pc
     B->P.assign(probs, probs + n);
     B->pc.assign(pcs, pcs + n);
     std::vector<BChunk> ch;
-    std::vector<ApplyParams> ap(n);
     std::vector<int> box_inst, box_local, box_cells;
     long long off = 0;
     for (int i = 0; i < n; ++i) {
@@ -1016,20 +1049,13 @@ static int batch_create(int n, ras_problem *const *probs, ras_precond *const *pc
         op.nx = P->nx; op.ny = P->ny; op.nz = P->nz;
         op.mx = bmagic(P->nx); op.my = bmagic(P->ny);
         B->ops.push_back(op);
-        ras1_apply_params(pc->fine, ap[i]);
         for (int q = 0; q < pc->fine.nsub; ++q) {
             box_inst.push_back(i);
             box_local.push_back(q);
             box_cells.push_back(pc->fine.shapes[pc->fine.subs[q].shape].ncell);
         }
-        B->block = std::max(B->block, pc->fine.launch);
-        B->smem = std::max(B->smem, pc->fine.smem_apply);
     }
     if (off > 0x7fffffffLL) return fail(RAS_EINVAL);   // the flat vector kernels take int counts
-    {
-        const int rq = ras1_batch_grid(B->prec, B->block, B->smem, (int)box_inst.size(), &B->qgrid);
-        if (rq < 0) return fail(rq);
-    }
     B->Ntot = off;
     B->nch = (int)ch.size();
     B->nbox = (int)box_inst.size();
@@ -1073,10 +1099,10 @@ static int batch_create(int n, ras_problem *const *probs, ras_precond *const *pc
     if (!up(B->d_ops, B->ops.data(), n * sizeof(BOp)) || !up(B->d_ch, ch.data(), ch.size() * sizeof(BChunk)) ||
         !up(B->d_off, B->off.data(), n * sizeof(long long)) || !up(B->d_ch0, B->ch0.data(), n * sizeof(int)) ||
         !up(B->d_chn, B->chn.data(), n * sizeof(int)) || !up(B->d_act, B->act.data(), n) ||
-        !up(B->d_ap, ap.data(), n * sizeof(ApplyParams)) ||
         !up(B->d_box_inst, box_inst.data(), box_inst.size() * sizeof(int)) ||
         !up(B->d_box_local, box_local.data(), box_local.size() * sizeof(int)))
         return fail(RAS_ECUDA);
+    if ((rc = launch_settings(B)) < 0) return fail(rc);
     // the padding between reservoirs stays zero in every vector
     if (cudaMemset(B->w, 0, Nt * sizeof(double)) != cudaSuccess || cudaMemset(B->r, 0, Nt * sizeof(double)) ||
         cudaMemset(B->b, 0, Nt * sizeof(double)) || cudaMemset(B->x, 0, Nt * sizeof(double)) ||

@@ -1050,6 +1050,7 @@ int ras1_set_schedule(Ras1 &R, int chunk_cells, int threads) {
     dfree(R.d_chunk);
     R.d_chunk = d;
     R.shapes = T.shapes;
+    ++R.sched;
     R.chunk_cells = T.chunk_cells;
     R.launch = T.launch;
     R.block = T.block;

@@ -43,6 +43,7 @@ struct Ras1 {
     int block = 128;        // threads per subdomain CTA
     int chunk_cells = 1024; // max cells per staged chunk (the schedule asked for)
     int launch = 128;       // threads per CTA of the sweeps
+    int sched = 0;          // counts the changes of the schedule
     int ycap = 0, lcap = 0; // smem capacities of the sweeps (cells or blocks, levels + 1)
     int gcap = 0;           // zero guard band on each side of their vector
     int ycap_cells = 0, lcap_cells = 0, gcap_cells = 0;   // the same cell by cell
