@@ -306,7 +306,10 @@ struct EosOut {
 // with FP64 residuals. The first two take the slope's reciprocal in FP32: near a simple
 // root the step is a small correction, so its relative error of 1e-6 leaves 1e-13 and then
 // rounding. Steps go on with the FP64 slope only while they still move the root by more than
-// 1e-10 (close roots, where Newton converges slowly).
+// 1e-10 (close roots, where Newton converges slowly); where three of them do not settle
+// either (a start beside a minimum that just fails to be a pair of roots), they start again
+// from Cauchy's bound of the roots: above it if the cubic reaches 0 right of its turning
+// point or in its minimum, else below it, Newton comes to the largest root without passing it.
 // Root selection in FP64: the FP32 closed form decides between one and three real roots in
 // FP32, and near a pair of close roots it can start Newton on another root than the largest.
 // The other two roots solve the deflated quadratic t^2 + (c2 + Z) t + (c1 + (c2 + Z) Z) = 0;
@@ -327,11 +330,23 @@ __device__ __forceinline__ double largest_root(double c2, double c1, double c0) 
         Z -= (double)last;
     }
     if (!(fabsf(last) <= 1e-10f)) {
+        auto cubic = [&](double x) { return fma(fma(x + c2, x, c1), x, c0); };
+        double d = 0.0;
+        auto newton = [&] {
+            d = cubic(Z) / fma(fma(3.0, Z, 2.0 * c2), Z, c1);
+            Z -= d;
+        };
 #pragma unroll 1
-        for (int it = 0; it < 3; ++it) {
-            const double f = fma(fma(Z + c2, Z, c1), Z, c0);
-            const double fz = fma(fma(3.0, Z, 2.0 * c2), Z, c1);
-            Z -= f / fz;
+        for (int it = 0; it < 3; ++it) newton();
+        if (!(fabs(d) <= 1e-10)) {
+            const double turn = -c2 / 3.0, low = turn + sqrt(fmax(turn * turn - c1 / 3.0, 0.0));
+            Z = 1.0 + fmax(fabs(c2), fmax(fabs(c1), fabs(c0)));
+            if (cubic(low) > 0.0) Z = -Z;
+#pragma unroll 1
+            for (int it = 0; it < 100; ++it) {
+                newton();
+                if (!(fabs(d) > 1e-16 * fabs(Z))) break;
+            }
         }
     }
     const float zf = (float)Z, q1f = f2 + zf, q0f = fmaf(q1f, zf, f1);
@@ -348,6 +363,7 @@ __device__ __forceinline__ double largest_root(double c2, double c1, double c0) 
                     const double fz = (3.0 * Zq + 2.0 * c2) * Zq + c1;
                     const double step = f / fz;
                     if (isfinite(step)) Zq -= step;
+                    if (fabs(step) > 1e-3) Zq = Z;   // (no root there: dq >= 0 by rounding)
                 }
                 Z = Zq;
             }
