@@ -598,6 +598,7 @@ static int b_run_cycle(ras_batch *B, int m, cudaStream_t st) {
     }
     const int nchk = (m + CYC_CHUNK - 1) / CYC_CHUNK;
     const long long polls = barrier_polls();
+    if (polls > 0) RAS_TRY(ras1_limit_ready(B->prec));
     if (use_graph && (B->cycle_m != m || B->cycle_polls != polls || (int)B->cycle_exec.size() != nchk)) {
         for (auto &g : B->cycle_exec)
             if (g) cudaGraphExecDestroy(g);

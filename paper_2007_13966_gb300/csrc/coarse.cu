@@ -1140,8 +1140,8 @@ __device__ void sparse_rows_times(const AT *Inv, const int *lq, const AT *lv, co
 // 17 us per step on a 1024 block, bound by L2, against 7 us). FP64 (gj_rows): a CTA owns rows, so that
 // q costs next to nothing beside the FP64-bound update (a tile of a 256 block would
 // spend a third of its FMA on q). Measured against 64 x 64 pivot tiles with two barriers
-// per tile: 16 blocks of 1024 in FP32 3.8 -> 3.2 ms, 8 blocks of 256 in FP64 5.2 -> 1.2 ms,
-// 16 of 512 in FP64 18.6 -> 7.0 ms (4.3 GFLOP: 3.9 ms of the FP64 pipe).
+// per tile: 16 blocks of 1024 in FP32 3.8 -> 2.8 ms, 8 blocks of 256 in FP64 5.2 -> 1.2 ms,
+// 16 of 512 in FP64 18.6 -> 7.1 ms (4.3 GFLOP: 3.9 ms of the FP64 pipe).
 template <typename AT> struct Gj;
 template <> struct Gj<float> { static constexpr int NB = 32; };
 template <> struct Gj<double> { static constexpr int NB = 16; };

@@ -389,11 +389,12 @@ __device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 0;" ::: "
 // reads its 4 records (ahead of the barrier) and 4 + 8 values, runs the block's cells in
 // registers in natural order and writes 4 values. Every cell's arithmetic and its order
 // are those of the cell-by-cell sweep, so the values are the same bit for bit.
-// 45.5 -> 35.0 us per launch on 128 x 128 x 64 cells (256 boxes of up to 20^3, FP32, 69 MB:
-// 1.96 TB/s). What bounds it is the length of the warps' instruction streams, about 16
-// cycles per instruction and warp with ~4 warps per scheduler (ncu): a level of the sweep
-// is ~80 instructions, ~400 cycles; blocks of 2 x 2 x 2 cells have 28 levels of ~620 cycles,
-// and with half as many helpers (four cells of a plane each) the gather takes 43 us.
+// 45.5 -> 34.8 us per launch on 128 x 128 x 64 cells (256 boxes of up to 20^3, FP32, 69 MB:
+// 1.97 TB/s). What bounds it is the length of the warps' instruction streams, about 18
+// cycles per instruction and warp with ~5 warps per scheduler (ncu): a level of the sweep
+// is ~80 instructions, ~400 cycles. Blocks of 2 x 2 x 2 cells have 28 levels of ~620 cycles:
+// the same time, and more padding on flat boxes. With half as many helpers (four cells of a
+// plane each) the gather takes 43 us.
 //
 // Warp roles, so that the sweeping warps wait for nothing but one another:
 //   - sweepers (as many as the widest level takes) meet at a barrier of their own per
@@ -1008,15 +1009,14 @@ static int schedule_tables(Ras1 &R, int chunk_cells, int threads, std::vector<in
                 }
                 return q;
             };
-            for (int n = 0; n + 1 < ns; ++n)
-                if (limit(n - 1) < n + 1) return RAS_EINVAL;
-            for (int n = 0; n <= ns; ++n) {
-                const int l = n < sh.nlev ? n : ns - 1 - n;
-                chunk_tab.push_back(n < ns ? lv[l] : 0);
-                chunk_tab.push_back(n < ns ? lv[l + 1] - lv[l] : 0);
-                chunk_tab.push_back(n < ns ? (int)(a[n] / 16) : 0);
-                chunk_tab.push_back(limit(n < ns ? n : -1));
+            const int first = limit(-1);     // before any step has been read
+            for (int n = 0; n < ns; ++n) {
+                const int l = n < sh.nlev ? n : ns - 1 - n, lim = limit(n);
+                if (lim < std::min(n + 2, ns - 1)) return RAS_EINVAL;
+                chunk_tab.insert(chunk_tab.end(), {lv[l], lv[l + 1] - lv[l], (int)(a[n] / 16), lim});
             }
+            if (first < std::min(1, ns - 1)) return RAS_EINVAL;
+            chunk_tab.insert(chunk_tab.end(), {0, 0, 0, first});
             sh.nchunk = ns;
         }
     }
@@ -1227,12 +1227,9 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
     RAS_CK(cudaMemset(R.d_err, 0, 2 * sizeof(int)));
     RAS_CK(cudaMemset(R.d_fwd, 0, (size_t)R.nrec * R.rec_bytes + 64));
     RAS_CK(cudaMemset(R.d_bwd, 0, (size_t)R.nrec * R.rec_bytes + 64));
-    if (prec == 64) RAS_TRY(set_apply_attr<64, false>());
-    if (prec == 32) { RAS_TRY(set_apply_attr<32, false>()); RAS_TRY(set_apply_attr<32, true>()); }
-    if (prec == 16) { RAS_TRY(set_apply_attr<16, false>()); RAS_TRY(set_apply_attr<16, true>()); }
-    if (prec == 64) RAS_TRY(set_factor_attr<64>());
-    if (prec == 32) RAS_TRY(set_factor_attr<32>());
-    if (prec == 16) RAS_TRY(set_factor_attr<16>());
+    if (prec == 64) { RAS_TRY((set_apply_attr<64, false>())); RAS_TRY(set_factor_attr<64>()); }
+    if (prec == 32) { RAS_TRY((set_apply_attr<32, false>())); RAS_TRY(set_factor_attr<32>()); }
+    if (prec == 16) { RAS_TRY((set_apply_attr<16, false>())); RAS_TRY(set_factor_attr<16>()); }
     if (kind != 1) {
         // per axis and coordinate, the (contiguous) range of parts whose overlapped
         // boxes cover it; box solutions are kept per record offset
@@ -1313,6 +1310,10 @@ int ras1_set_kernel(Ras1 &R, int kernel) {
 }
 
 
+int ras1_limit_ready(int prec) {
+    return prec == 64 ? RAS_OK : (prec == 32 ? set_apply_attr<32, true>() : set_apply_attr<16, true>());
+}
+
 int ras1_polls() { return (int)std::min<long long>(barrier_polls(), APPLY_POLLS); }
 
 void ras1_apply_params(const Ras1 &R, ApplyParams &P) {
@@ -1354,6 +1355,7 @@ int ras1_apply(Ras1 &R, const double *r, double *z, int accumulate, cudaStream_t
     ras1_apply_params(R, P);
     P.r = r; P.z = z; P.accumulate = accumulate;
     P.polls = ras1_polls();
+    if (P.polls > 0) RAS_TRY(ras1_limit_ready(R.prec));
     auto kern = R.prec == 64 ? k_ras_apply<64, false>
               : R.prec == 32 ? (P.polls > 0 ? k_ras_apply<32, true> : k_ras_apply<32, false>)
                              : (P.polls > 0 ? k_ras_apply<16, true> : k_ras_apply<16, false>);

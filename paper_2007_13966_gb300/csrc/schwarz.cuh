@@ -128,6 +128,8 @@ struct BatchApply {
 };
 // the poll limit of the sweeps' waits for the next launch (barrier_polls)
 int ras1_polls();
+// makes the sweeps that take it ready to launch (before a capture)
+int ras1_limit_ready(int prec);
 void ras1_apply_params(const Ras1 &R, ApplyParams &P);
 // parameters of one handle's ILU(0) factorisation kernel on operator A
 struct FactorParams {
