@@ -1288,14 +1288,6 @@ int ras1_factor_batch(const FactorParams *d_inst, const int *d_box_inst, const i
     return RAS_OK;
 }
 
-int ras1_check(Ras1 &R, cudaStream_t st) {
-    int h = 0;
-    RAS_CK(cudaMemcpyAsync(&h, R.d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RAS_CK(cudaStreamSynchronize(st));
-    if (h) RAS_CK(cudaMemsetAsync(R.d_err, 0, sizeof(int), st));
-    return ras1_status(h);
-}
-
 int ras1_status(int word) { return word == 0 ? RAS_OK : (word == APPLY_TIMEOUT ? RAS_ETIMEOUT : RAS_EZEROPIVOT); }
 
 int ras1_set_kernel(Ras1 &R, int kernel) {

@@ -80,8 +80,7 @@ int ras1_setup(Ras1 &R, int nx, int ny, int nz, int px, int py, int pz, int over
 void ras1_free(Ras1 &R);
 // numeric ILU(0) of every A_i = R_i^delta A (R_i^delta)^T; no synchronisation
 int ras1_factor(Ras1 &R, const Stencil7 &A, cudaStream_t st);
-// reads and clears the pivot flag and that of a sweep's wait that ran out (synchronises)
-int ras1_check(Ras1 &R, cudaStream_t st);
+// the status in the error word d_err[0]: a zero or non-finite pivot, a sweep's wait that ran out
 int ras1_status(int word);
 // z = M^{-1} r (accumulate = 0) or z += M^{-1} r (accumulate = 1), with
 // M^{-1} = sum_i (R_i^0)^T A_i^{-1} R_i^delta (left-RAS, kind 1),
@@ -144,7 +143,7 @@ struct FactorParams {
 void ras1_factor_params(const Ras1 &R, const Stencil7 &A, FactorParams &P);
 // the ILU(0) factorisations of several handles in one launch: CTA b factors box
 // d_box_local[b] of handle d_box_inst[b] (d_inst: device copies of the handles'
-// parameters); no synchronisation (each handle's ras1_check reads its pivot flag)
+// parameters); no synchronisation (a zero pivot is left in the handle's error word)
 int ras1_factor_batch(const FactorParams *d_inst, const int *d_box_inst, const int *d_box_local,
                       const unsigned char *d_active, int nbox, int prec, int block, size_t smem, cudaStream_t st);
 // persistent launch of `grid` CTAs over the B.nitems boxes of the work queue
