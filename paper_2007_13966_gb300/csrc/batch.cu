@@ -774,26 +774,27 @@ static int bfgmres_run(ras_batch *B, const std::vector<unsigned char> &want, con
 // handles' present schedules
 static int launch_settings(ras_batch *B) {
     std::vector<ApplyParams> ap(B->n);
+    std::vector<int> sched(B->n);
     B->block = 0;
     B->smem = 0;
-    B->sched.assign(B->n, 0);
     for (int i = 0; i < B->n; ++i) {
         const Ras1 &R = B->pc[i]->fine;
         ras1_apply_params(R, ap[i]);
         B->block = std::max(B->block, R.launch);
         B->smem = std::max(B->smem, R.smem_apply);
-        B->sched[i] = R.sched;
+        sched[i] = R.sched;
     }
     RAS_TRY(ras1_batch_grid(B->prec, B->block, B->smem, B->nbox, &B->qgrid));
     RAS_CK(cudaMemcpy(B->d_ap, ap.data(), B->n * sizeof(ApplyParams), cudaMemcpyHostToDevice));
+    B->sched = sched;                        // (only settings that can be launched count as made)
     return RAS_OK;
 }
 
 // ... made again when a handle's schedule has changed since (its tables moved): also the
 // captured cycles, which hold them
 static int refresh_schedules(ras_batch *B, cudaStream_t st) {
-    bool same = true;
-    for (int i = 0; i < B->n; ++i) same = same && B->sched[i] == B->pc[i]->fine.sched;
+    bool same = (int)B->sched.size() == B->n;
+    for (int i = 0; same && i < B->n; ++i) same = same && B->sched[i] == B->pc[i]->fine.sched;
     if (same) return RAS_OK;
     RAS_CK(cudaStreamSynchronize(st));
     for (auto &g : B->cycle_exec)
